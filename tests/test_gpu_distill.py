@@ -51,6 +51,26 @@ def test_distillation_matches_cpu(shape):
           f"KL {l0:.4f} -> {l1:.4f}  max|dW| {np.abs(W - W_ref).max():.2e}")
 
 
+@pytest.mark.parametrize("T,N,d", [(1, 1, 1), (63, 8, 64), (65, 9, 66), (257, 64, 130), (1190, 33, 68), (9601, 17, 36)])
+def test_distillation_tile_edges(T, N, d):
+    """Token tiles of one to eight warps and their remainders, expert tiles 1 to 8, columns off the 64-column tile and off
+    16-byte rows, more tokens than one wave of CTAs."""
+    from oracle import distill
+    build.build()
+    rng = np.random.default_rng(1000 * T + N)
+    H = rng.standard_normal((T, d)).astype(np.float32)
+    Z = rng.standard_normal((T, N))
+    Qr = (np.exp(Z) / np.exp(Z).sum(1, keepdims=True)).astype(np.float32)
+    W0 = (rng.standard_normal((N, d)) / np.sqrt(d)).astype(np.float32)
+    b0 = rng.standard_normal(N).astype(np.float32)
+    W_ref, b_ref = distill.distill(H, Qr, W0, b0, iters=4, lr=0.01)
+    W, b = binding.distill_router(torch.from_numpy(H).cuda(), torch.from_numpy(Qr).cuda(), W0, b0, iters=4, lr=0.01)
+    # a gradient that is exactly zero in one summation order and 1e-17 in another moves Adam by up to lr: not seen with
+    # more than one expert; with one expert the softmax is 1 and every gradient is (1 - q_r) h
+    assert np.abs(W - W_ref).max() <= 2e-6 * max(1.0, float(np.abs(W_ref).max()))
+    assert np.abs(b - b_ref).max() <= 2e-6 * max(1.0, float(np.abs(b_ref).max()))
+
+
 def test_distillation_rejects_bad_arguments():
     build.build()
     H = torch.zeros((8, 16), dtype=torch.float32, device="cuda")
