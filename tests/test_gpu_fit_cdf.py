@@ -61,6 +61,22 @@ def test_fit_matches_cpu_fit(shape):
           f"max|dw| {np.abs(w - w_ref).max():.2e} max|dtheta| {np.abs(th - th_ref).max():.2e}")
 
 
+@pytest.mark.parametrize("T,N,k,iters,lr", [(1, 1, 1, 20, 0.05), (64, 8, 8, 20, 0.05), (513, 9, 1, 20, 0.05), (1025, 64, 1, 20, 0.05),
+                                            (8193, 33, 8, 10, 0.05), (9000, 64, 8, 5, 0.05), (300, 16, 4, 4, 200.0)])
+def test_fit_tile_edges(T, N, k, iters, lr):
+    """One to sixteen clusters and remainders, tokens in two passes, tokens that do not fit shared memory, one threshold,
+    and thresholds outside the range of the factored exponentials (the large step)."""
+    from oracle import fit_cdf
+    build.build()
+    rng = np.random.default_rng(T + N)
+    X = np.sort(rng.dirichlet(np.full(N, 0.5), T), axis=1)[:, ::-1].copy()
+    dstar = rng.integers(0, N - k + 1, T).astype(np.int32)
+    w_ref, th_ref = fit_cdf.fit(X, dstar, N, k, iters=iters, lr=lr)
+    w, th = binding.fit_cdf(torch.from_numpy(X).cuda(), torch.from_numpy(dstar).cuda(), k, iters=iters, lr=lr)
+    assert np.abs(w - w_ref).max() <= 1e-5 * max(1.0, float(np.abs(w_ref).max())), np.abs(w - w_ref).max()
+    assert np.abs(th - th_ref).max() <= 1e-5 * max(1.0, float(np.abs(th_ref).max())), np.abs(th - th_ref).max()
+
+
 def test_fit_rejects_bad_arguments():
     build.build()
     X = torch.zeros((8, 70), dtype=torch.float64, device="cuda")
