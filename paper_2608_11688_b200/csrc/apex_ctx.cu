@@ -111,35 +111,31 @@ int apex_create(const apex_config* cfg, apex_ctx** out) {
   CR(cudaMemset(ctx->d_spec, 0xff, L * APEX_MAX_TOPK * sizeof(int32_t)));
   CR(dev_alloc(&ctx->d_counters, 2));
   CR(cudaMemset(ctx->d_counters, 0, 2 * sizeof(unsigned long long)));
-  const size_t max_pairs = MB * (k + 1);
-  CR(dev_alloc(&ctx->d_plan_exec_idx, MB * k));
-  CR(dev_alloc(&ctx->d_plan_exec_gate, MB * k));
-  CR(dev_alloc(&ctx->d_pair_tok, max_pairs));
-  CR(dev_alloc(&ctx->d_pair_gate, max_pairs));
-  CR(dev_alloc(&ctx->d_pair_expert, max_pairs));
-  CR(dev_alloc(&ctx->d_n_pairs, 4));
-  CR(dev_alloc(&ctx->d_grp, 4 + 3 * (N + 1)));
   CR(dev_alloc(&ctx->d_cand, MB * C));
   CR(dev_alloc(&ctx->d_idx, L * MB * k));
   CR(dev_alloc(&ctx->d_exec_idx, MB * k));
   CR(dev_alloc(&ctx->d_alpha, L * MB * N));
   CR(dev_alloc(&ctx->d_exec_gate, MB * k));
   CR(dev_alloc(&ctx->d_cand_ncand, MB));
-  // batched tensor-core path: scratch and tensor maps (only for contexts that will see large batches)
-  if (MB >= kTcMinBatch && tc_shape_supported(c.d, c.I, c.I_shared, ctx->fmt)) {
-    const size_t rows = max_pairs + 256;
-    const size_t i_max = (size_t)(c.I > c.I_shared ? c.I : c.I_shared);
+  // batched path (only for contexts that will see batches): pair list, scratch and tensor maps of the grouped GEMM
+  if (MB > 1) {
+    const size_t max_pairs = MB * (k + 1);
+    const size_t rows = max_pairs + 64;  // (boxes of the last group reach past its rows)
+    const size_t i_max = ((size_t)(c.I > c.I_shared ? c.I : c.I_shared) + 63) / 64 * 64;
+    CR(dev_alloc(&ctx->d_pair_tok, max_pairs));
+    CR(dev_alloc(&ctx->d_pair_gate, max_pairs));
+    CR(dev_alloc(&ctx->d_grp, 4 + 3 * (N + 1)));
+    CR(dev_alloc(&ctx->d_tc_sync, (size_t)kTcSyncWords));
+    CR(dev_alloc(&ctx->d_plan_masks, 2));
     ctx->act_stride = (int)i_max;
-    CR(dev_alloc(&ctx->d_xg, rows * d));
-    ctx->act_plane = rows * i_max;
+    ctx->act_rows = (int)rows;
+    CR(dev_alloc(&ctx->d_xb, MB * d));
     CR(dev_alloc(&ctx->d_act, 2 * rows * i_max));
-    CR(cudaMemset(ctx->d_xg, 0, rows * d * 2));
+    CR(cudaMemset(ctx->d_xb, 0, MB * d * 2));
     CR(cudaMemset(ctx->d_act, 0, 2 * rows * i_max * 2));
-    ctx->tc_ok = tc_make_store_maps(ctx->fmt, ctx->tc_maps.w_gateup, ctx->tc_maps.w_down, ctx->tc_maps.sc_gateup, ctx->tc_maps.sc_down,
-                                    ctx->d_cache, c.d, c.I, L * C, ctx->expert_bytes) &&
-                 tc_make_rows_map(ctx->tc_maps.xg, ctx->d_xg, c.d, rows, d) &&
-                 tc_make_rows_map(ctx->tc_maps.act, ctx->d_act, (int)i_max, rows, i_max) &&
-                 tc_make_rows_map(ctx->tc_maps.act_lo, ctx->d_act + ctx->act_plane, (int)i_max, rows, i_max);
+    if (!tc_make_store_maps(ctx->fmt, ctx->tc_maps.w, ctx->tc_maps.sc, ctx->d_cache, c.d, c.I, L * C, ctx->expert_bytes) ||
+        !tc_make_activation_maps(&ctx->tc_maps, ctx->d_xb, c.d, (int)MB, ctx->d_act, rows, (int)i_max))
+      return bail(APEX_ECUDA, "apex_create: a tensor map of the batched path could not be encoded", cudaSuccess);
     ctx->tc_shared_maps.assign(L, ctx->tc_maps);
   }
   ctx->attn_bytes = (4 * d * d + 2 * (size_t)ctx->cfg.ctx_len * d) * 2;
@@ -151,15 +147,11 @@ int apex_create(const apex_config* cfg, apex_ctx** out) {
   // mapped mailbox
   MailboxLayout& ml = ctx->ml;
   size_t off = sizeof(MailboxHeader);
-  ml.off_exec_seq = off;  off += L * sizeof(uint32_t);
   off = (off + 15) & ~(size_t)15;
   ml.off_sel_rec = off;   off += 16;
-  ml.off_exec_rec = off;  off += L * 32;   // per layer: routed-set record, execution-set record (B = 1)
+  ml.off_exec_rec = off;  off += L * 32;   // per layer: routed-set record, execution-set record
   ml.off_ncand = off; off += MB * sizeof(int32_t);
   ml.off_cand = off;  off += MB * C * sizeof(int32_t);
-  ml.kr_stride = MB * k * sizeof(int32_t);
-  ml.off_kr = off;    off += L * ml.kr_stride;
-  ml.off_exec = off;  off += L * ml.kr_stride;
   ml.bytes = off;
   ctx->exec_seq.assign(L, 0u);
   CR(cudaHostAlloc(reinterpret_cast<void**>(&ctx->mbox), ml.bytes, cudaHostAllocMapped | cudaHostAllocPortable));
@@ -219,8 +211,8 @@ int apex_destroy(apex_ctx* ctx) {
   cudaDeviceSynchronize();
   cudaGetLastError();
   void* dev[] = {ctx->d_Wr, ctx->d_br, ctx->d_Wp, ctx->d_bp, ctx->d_w, ctx->d_theta, ctx->d_cache, ctx->d_slot_ready, ctx->d_zp,
-                 ctx->d_qp, ctx->d_zr, ctx->d_demand, ctx->d_pi, ctx->d_ncand, ctx->d_stats, ctx->d_counters, ctx->d_tickets, ctx->d_spec, ctx->d_plan_exec_idx,
-                 ctx->d_plan_exec_gate, ctx->d_pair_tok, ctx->d_pair_gate, ctx->d_pair_expert, ctx->d_n_pairs, ctx->d_grp, ctx->d_xg, ctx->d_act, ctx->d_cand,
+                 ctx->d_qp, ctx->d_zr, ctx->d_demand, ctx->d_pi, ctx->d_ncand, ctx->d_stats, ctx->d_counters, ctx->d_tickets, ctx->d_spec, ctx->d_pair_tok,
+                 ctx->d_pair_gate, ctx->d_grp, ctx->d_tc_sync, ctx->d_plan_masks, ctx->d_xb, ctx->d_act, ctx->d_cand,
                  ctx->d_idx, ctx->d_exec_idx, ctx->d_alpha, ctx->d_exec_gate, ctx->d_cand_ncand, ctx->d_attn, ctx->d_attn_sink,
                  ctx->d_h_stage, ctx->d_hp_stage, ctx->d_y_stage};
   for (void* p : dev)
@@ -303,10 +295,9 @@ int apex_set_shared_expert(apex_ctx* ctx, int layer, const void* dev_weights) {
   ctx->shared_dev[layer] = static_cast<const uint8_t*>(dev_weights);
   if (ctx->d_shared_ptrs)
     CU_TRY(ctx, cudaMemcpy(ctx->d_shared_ptrs + layer, &dev_weights, sizeof(void*), cudaMemcpyHostToDevice));
-  if (ctx->tc_ok) {
+  if (!ctx->tc_shared_maps.empty()) {
     TcMaps& m = ctx->tc_shared_maps[layer];
-    if (!tc_make_store_maps(ctx->fmt, m.ws_gateup, m.ws_down, m.ssc_gateup, m.ssc_down, dev_weights, ctx->cfg.d, ctx->cfg.I_shared, 1,
-                            ctx->shared_bytes))
+    if (!tc_make_store_maps(ctx->fmt, m.ws, m.ssc, dev_weights, ctx->cfg.d, ctx->cfg.I_shared, 1, ctx->shared_bytes))
       return fail(ctx, APEX_ECUDA, "tensor map for the shared expert could not be encoded");
   }
   return APEX_OK;

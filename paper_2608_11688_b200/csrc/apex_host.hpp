@@ -50,15 +50,9 @@ inline cudaError_t dev_alloc(T** p, size_t n) {
 inline MailboxHeader* mhdr(apex_ctx* ctx) { return reinterpret_cast<MailboxHeader*>(ctx->mbox); }
 inline int32_t* mbox_i32(apex_ctx* ctx, size_t off) { return reinterpret_cast<int32_t*>(ctx->mbox + off); }
 inline volatile uint32_t* mbox_sel_rec(apex_ctx* ctx) { return reinterpret_cast<volatile uint32_t*>(ctx->mbox + ctx->ml.off_sel_rec); }
-inline volatile uint32_t* mbox_exec_seq(apex_ctx* ctx, int l) {
-  return reinterpret_cast<volatile uint32_t*>(ctx->mbox + ctx->ml.off_exec_seq) + l;
-}
 inline volatile uint32_t* mbox_exec_rec(apex_ctx* ctx, int l) {
   return reinterpret_cast<volatile uint32_t*>(ctx->mbox + ctx->ml.off_exec_rec) + 8 * l;
 }
-inline int32_t* mbox_kr(apex_ctx* ctx, int l) { return mbox_i32(ctx, ctx->ml.off_kr + (size_t)l * ctx->ml.kr_stride); }
-inline int32_t* mbox_exec(apex_ctx* ctx, int l) { return mbox_i32(ctx, ctx->ml.off_exec + (size_t)l * ctx->ml.kr_stride); }
-
 // A 32-bit word written in stream order (after everything queued before it on that stream).
 inline int stream_write32(apex_ctx* ctx, cudaStream_t cs, uint32_t* dev, uint32_t value) {
   if (ctx->fn_write_value32) {

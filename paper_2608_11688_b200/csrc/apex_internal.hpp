@@ -47,10 +47,10 @@ struct MailboxHeader {
   uint32_t pad[2];
 };
 
-// Byte offsets inside the mailbox.  Per layer: route_seq[l] is written by the gate kernel after
-// K_r of that layer, exec_seq[l] by the FFN's plan step after the execution sets.
+// Byte offsets inside the mailbox.  Per layer: two records of the FFN step, routed and execution set (B > 1: their
+// unions over the tokens), each with its sequence number.
 struct MailboxLayout {
-  size_t off_exec_seq, off_sel_rec, off_exec_rec, off_ncand, off_cand, off_kr, off_exec, kr_stride, bytes;
+  size_t off_sel_rec, off_exec_rec, off_ncand, off_cand, bytes;
 };
 
 // Device-side counters of one layer (S9), accumulated with 64-bit atomics.
@@ -121,17 +121,13 @@ struct FfnParams {
   const float* shared_gate; // [d] gate vector of the shared expert, or null: weight 1
   const uint32_t* slot_ready;  // [C]
   // batched plan (B > 1), context-owned
-  int32_t* plan_exec_idx;   // [B][k]
-  float* plan_exec_gate;    // [B][k]
-  int32_t* pair_tok;        // [B*k + B]
+  int32_t* pair_tok;        // [B*k + B] token of each (expert, token) pair, sorted by expert; the shared expert's pairs last
   float* pair_gate;         // [B*k + B]
-  int32_t* pair_expert;     // [B*k + B]   (N = shared expert)
-  int32_t* n_pairs;         // [1]
   int32_t* grp;             // [4 + 3*(N+1)]: routed groups, all groups, 0, 0, then (expert, pair offset, tokens) per group
-  int32_t* mbox_exec;       // mapped host [B][k]
-  int32_t* mbox_kr;         // mapped host [B][k]: the routed sets, posted with the execution sets
-  uint32_t* mbox_rec;       // mapped host, B = 1: two 16-byte records {mask lo, mask hi, sequence number, 0}: routed set, execution set
-  volatile uint32_t* mbox_seq;
+  unsigned* tc_sync;        // [kTcSyncWords] zeroed by the plan
+  unsigned long long* plan_masks;  // [2] union of the routed sets, of the execution sets
+  __nv_bfloat16* xb;        // [B][d] h' in bf16
+  uint32_t* mbox_rec;       // mapped host: two 16-byte records {mask lo, mask hi, sequence number, 0}: routed set, execution set (B > 1: their unions)
   volatile uint32_t* mbox_status;
   uint32_t seq_value;
   DevStats* stats;
@@ -155,23 +151,29 @@ struct FfnParams {
 
 constexpr int kMaxDevices = 64;  // per-device launch attributes are remembered for this many devices
 
-// Batched tensor-core path (kernels_ffn_tc.cu)
-constexpr int kTcMinBatch = 2;  // from this many tokens per step the tensor-core grouped GEMM runs (it beats the per-pair kernel at every B > 1)
+// Batched tensor-core path (kernels_ffn_tc.cu): B > 1
+// Words of the synchronisation block, zeroed by the plan kernel of every step
+constexpr int kTcTicket = 0;                 // units handed out
+constexpr int kTcAbort = 1;                  // somebody gave up
+constexpr int kTcDone = 2;                   // [N + 1] gate/up units counted in, per group
+constexpr int kTcSyncWords = kTcDone + APEX_MAX_EXPERTS + 1;
+struct TcShifts { uint32_t up2, up4, up6, up8, up12; };  // powers of two (see the code converters)
 struct TcParams {
   FfnParams f;
-  const int32_t* grp;
-  __nv_bfloat16* xg;    // [pairs][d] gathered activations, bf16
-  __nv_bfloat16* act;   // two planes [2][rows][act_stride]: bf16(a) and bf16(a - bf16(a))
-  size_t act_plane;     // elements per plane
-  int act_stride;
-  int layer_slot0;      // index of this layer's slot 0 in the all-layers weight tensor map
-  int nmax1, nmax2;     // tokens per unit of the gate/up and of the down kernel (set by the launcher)
-  int nstage1, nstage2; // pipeline depths
+  unsigned* sync;                        // [kTcSyncWords]
+  const unsigned long long* plan_masks;  // union of the routed sets, of the execution sets
+  __nv_bfloat16* act;                    // the intermediate, two planes [2][act_rows][act_stride]: bf16(a) and bf16(a - bf16(a))
+  size_t act_plane;                      // elements per plane
+  int act_rows, act_stride;
+  int layer_slot0;                       // index of this layer's slot 0 in the all-layers weight tensor map
+  int nmax1, nmax2;                      // tokens per unit of the gate/up and of the down projection (set by the launcher)
+  int nstage, nraw, stage_bytes;         // ring depths and stage size
+  TcShifts shifts;
 };
 struct TcMaps {          // opaque 128-byte CUtensorMap objects
-  alignas(64) unsigned char w_gateup[128], w_down[128], ws_gateup[128], ws_down[128], xg[128], act[128], act_lo[128];
-  // e2m1 stores only: the same bytes as w_* / ws_* with 16-byte boxes, for the block-scale bytes
-  alignas(64) unsigned char sc_gateup[128], sc_down[128], ssc_gateup[128], ssc_down[128];
+  alignas(64) unsigned char w[128], ws[128];    // weights of the slots / of the layer's shared expert
+  alignas(64) unsigned char sc[128], ssc[128];  // quantised stores: the same bytes in 16-byte boxes, for the e2m1 block scales
+  alignas(64) unsigned char x[128], xc[128], act[128];
 };
 
 // Persistent decode kernel (kernels_decode.cu): all layers of one token in one cooperative launch.
@@ -245,15 +247,12 @@ struct AttnParams {
 cudaError_t launch_router(const RouterParams& p, cudaStream_t s);
 cudaError_t launch_select(const SelectParams& p, cudaStream_t s);
 cudaError_t launch_attention(const AttnParams& p, int n_sm, cudaStream_t s);
-cudaError_t launch_ffn_plan(const FfnParams& p, cudaStream_t s);
+cudaError_t launch_ffn_plan(const FfnParams& p, int n_sm, cudaStream_t s);
 cudaError_t launch_ffn(const FfnParams& p, int n_ctas, cudaStream_t s);  // n_ctas: grid size, at most ffn_grid_ctas(SM count)
 int ffn_grid_ctas(int n_sm);  // CTAs of one streaming-kernel launch (each adds one to the zero counter)
 cudaError_t launch_ffn_tc(const TcParams& p, const TcMaps& m, int n_sm, cudaStream_t s);
-bool tc_make_weight_map(void* out, const void* base, int d, int I, size_t n_slots, size_t slot_bytes, int box_rows);
-bool tc_make_rows_map(void* out, const void* base, int cols, size_t rows, size_t stride_elems);
-bool tc_make_store_maps(int fmt, void* gateup, void* down, void* sc_gateup, void* sc_down, const void* base, int d, int I, size_t n_slots,
-                        size_t slot_bytes);   // weight maps of one store in storage format fmt
-bool tc_shape_supported(int d, int I, int I_shared, int fmt);
+bool tc_make_activation_maps(TcMaps* m, const void* xb, int d, int max_batch, const void* act, size_t act_rows, int act_stride);
+bool tc_make_store_maps(int fmt, void* weights, void* scales, const void* base, int d, int I, size_t n_slots, size_t slot_bytes);  // one store, in storage format fmt
 bool ffn_shape_supported(int d);
 bool ffn_quantised_shape_supported(int d);   // widths the e4m3 / e2m1 kernels were built for
 size_t ffn_row_bytes(int fmt, int d);        // bytes of one intermediate index (three vectors and their scales)
@@ -288,16 +287,16 @@ struct apex_ctx {
   int32_t *d_pi = nullptr, *d_ncand = nullptr;              // [maxB][N], [maxB]
   apex::DevStats* d_stats = nullptr;                        // [L]
   unsigned long long* d_counters = nullptr;                 // [2]: select done, zero
-  int32_t *d_plan_exec_idx = nullptr, *d_pair_tok = nullptr, *d_pair_expert = nullptr, *d_n_pairs = nullptr;
-  float *d_plan_exec_gate = nullptr, *d_pair_gate = nullptr;
-  // batched tensor-core path
-  bool tc_ok = false;
-  int32_t* d_grp = nullptr;
-  __nv_bfloat16 *d_xg = nullptr, *d_act = nullptr;
-  int act_stride = 0;
+  // batched path (max_batch > 1)
+  int32_t *d_pair_tok = nullptr, *d_grp = nullptr;
+  float* d_pair_gate = nullptr;
+  unsigned* d_tc_sync = nullptr;
+  unsigned long long* d_plan_masks = nullptr;
+  __nv_bfloat16 *d_xb = nullptr, *d_act = nullptr;
+  int act_stride = 0, act_rows = 0;
   size_t act_plane = 0;
   apex::TcMaps tc_maps{};
-  std::vector<apex::TcMaps> tc_shared_maps;  // per layer: ws_gateup / ws_down filled
+  std::vector<apex::TcMaps> tc_shared_maps;  // per layer: ws / ssc filled
   uint8_t* d_attn = nullptr;
   size_t attn_bytes = 0, attn_layers = 1;
   float* d_attn_sink = nullptr;

@@ -394,32 +394,25 @@ cudaError_t launch_stream(apex_ctx* ctx, FfnParams p, cudaStream_t cs) {
 }
 
 
-// B > 1: plan kernel, then either the tensor-core grouped GEMM or the streaming kernel per pair.
+// B > 1: plan kernel, then the tensor-core grouped GEMM.
 int launch_batched(apex_ctx* ctx, int layer, const FfnParams& p, cudaStream_t cs) {
-  CU_TRY(ctx, launch_ffn_plan(p, cs));
-  ctx->last_was_ffn = false;
+  CU_TRY(ctx, launch_ffn_plan(p, ctx->n_sm, cs));
+  TcParams t{};
+  t.f = p;
+  t.sync = ctx->d_tc_sync;
+  t.plan_masks = ctx->d_plan_masks;
+  t.act = ctx->d_act;
+  t.act_rows = ctx->act_rows;
+  t.act_stride = ctx->act_stride;
+  t.act_plane = (size_t)ctx->act_rows * ctx->act_stride;
+  t.layer_slot0 = layer * ctx->cfg.C;
+  CU_TRY(ctx, launch_ffn_tc(t, ctx->tc_shared_maps[layer], ctx->n_sm, cs));
+  ctx->last_was_ffn = true;
+  ctx->last_ffn_y_lo = (uintptr_t)p.y;
+  ctx->last_ffn_y_hi = (uintptr_t)p.y + (size_t)p.B * p.d * sizeof(float);
   ctx->last_pred_layer = -1;
   ctx->last_stream = cs;
-  ++ctx->launches;
-  if (ctx->tc_ok && p.B >= kTcMinBatch) {
-    TcParams t{};
-    t.f = p;
-    t.grp = ctx->d_grp;
-    t.xg = ctx->d_xg;
-    t.act = ctx->d_act;
-    t.act_stride = ctx->act_stride;
-    t.act_plane = ctx->act_plane;
-    t.layer_slot0 = layer * ctx->cfg.C;
-    CU_TRY(ctx, launch_ffn_tc(t, ctx->tc_shared_maps[layer], ctx->n_sm, cs));
-    ctx->last_was_ffn = true;
-    ctx->last_ffn_y_lo = (uintptr_t)p.y;
-    ctx->last_ffn_y_hi = (uintptr_t)p.y + (size_t)p.B * p.d * sizeof(float);
-    ctx->last_pred_layer = -1;
-    ctx->launches += 3;
-  } else {
-    CU_TRY(ctx, launch_stream(ctx, p, cs));
-    ++ctx->launches;
-  }
+  ctx->launches += 2;
   return APEX_OK;
 }
 
@@ -447,17 +440,13 @@ int ffn_launch(apex_ctx* ctx, int layer, int mode, const float* hpost_dev, int B
   p.shared_w = ctx->shared_dev[layer];
   p.shared_gate = ctx->shared_gate_on[layer] ? ctx->shared_gate_dev[layer] : nullptr;
   p.slot_ready = ctx->d_slot_ready + (size_t)layer * C;
-  p.plan_exec_idx = ctx->d_plan_exec_idx;
-  p.plan_exec_gate = ctx->d_plan_exec_gate;
   p.pair_tok = ctx->d_pair_tok;
   p.pair_gate = ctx->d_pair_gate;
-  p.pair_expert = ctx->d_pair_expert;
-  p.n_pairs = ctx->d_n_pairs;
   p.grp = ctx->d_grp;
-  p.mbox_exec = mbox_exec(ctx, layer);
-  p.mbox_kr = mbox_kr(ctx, layer);
+  p.tc_sync = ctx->d_tc_sync;
+  p.plan_masks = ctx->d_plan_masks;
+  p.xb = ctx->d_xb;
   p.mbox_rec = const_cast<uint32_t*>(mbox_exec_rec(ctx, layer));
-  p.mbox_seq = mbox_exec_seq(ctx, layer);
   p.mbox_status = &mhdr(ctx)->status;
   p.seq_value = ++ctx->exec_seq[layer];
   p.stats = ctx->d_stats + layer;
@@ -502,35 +491,20 @@ int ffn_finalize(apex_ctx* ctx, int layer) {
   auto& st = ctx->step[layer];
   if (!st.pending) return APEX_OK;
   st.pending = false;
-  const int B = st.B, N = ctx->cfg.N, k = ctx->cfg.k;
+  const int B = st.B, N = ctx->cfg.N;
   cudaStream_t cs = st.pend_stream;
   auto& tab = ctx->tables[layer];
   const FfnParams& p = ctx->ffn_params[layer];
-  // the FFN's plan step posts the routed and the execution sets of this layer-step
-  std::vector<int32_t> kr_one, ex_one;  // B = 1: the sets arrive as masks, each with its sequence number in one 16-byte record
-  const int32_t* K_r = mbox_kr(ctx, layer);
-  const int32_t* ex_list = mbox_exec(ctx, layer);
-  if (B == 1) {
-    volatile uint32_t* rec = mbox_exec_rec(ctx, layer);
-    if (!host_wait_seq(ctx, rec + 2, ctx->exec_seq[layer]) || !host_wait_seq(ctx, rec + 6, ctx->exec_seq[layer]))
-      return fail(ctx, APEX_ETIMEOUT, "apex_moe_ffn: K_r did not arrive");
-    const uint64_t kr_mask = ((uint64_t)rec[1] << 32) | rec[0], ex_mask = ((uint64_t)rec[5] << 32) | rec[4];
-    for (int e = 0; e < N; ++e) {
-      if ((kr_mask >> e) & 1) kr_one.push_back(e);
-      if ((ex_mask >> e) & 1) ex_one.push_back(e);
-    }
-    kr_one.resize(k, -1);
-    ex_one.resize(k, -1);
-    K_r = kr_one.data();
-    ex_list = ex_one.data();
-  } else if (!host_wait_seq(ctx, mbox_exec_seq(ctx, layer), ctx->exec_seq[layer])) {
+  // the FFN posts the routed and the execution set of the layer-step as masks (B > 1: the unions over the tokens), each
+  // with its sequence number in one 16-byte record
+  volatile uint32_t* rec = mbox_exec_rec(ctx, layer);
+  if (!host_wait_seq(ctx, rec + 2, ctx->exec_seq[layer]) || !host_wait_seq(ctx, rec + 6, ctx->exec_seq[layer]))
     return fail(ctx, APEX_ETIMEOUT, "apex_moe_ffn: K_r did not arrive");
-  }
+  const uint64_t need = ((uint64_t)rec[1] << 32) | rec[0], ex_mask = ((uint64_t)rec[5] << 32) | rec[4];
   if (st.pend_mode == APEX_MODE_EXACT) {
     std::vector<SlotCopy> copies;
-    uint64_t need = 0;
     const std::vector<int32_t> slot_expert_before = tab.slot_expert();
-    if (!tab.plan_demand(K_r, B, k, &copies, &need)) return fail(ctx, APEX_ESTATE, "no evictable slot");
+    if (!tab.plan_demand(need, &copies)) return fail(ctx, APEX_ESTATE, "no evictable slot");
     if (p.demand_in_kernel) {
       // the running kernel waits for these experts: copy, then publish (tag, slot)
       for (size_t i = 0; i < copies.size(); ++i) {
@@ -612,7 +586,8 @@ int ffn_finalize(apex_ctx* ctx, int layer) {
     ctx->host_stats[layer].demand_copies += (int64_t)copies.size();
     ctx->last_copies[layer].insert(ctx->last_copies[layer].end(), copies.begin(), copies.end());
   } else {
-    for (int i = 0; i < B * k; ++i) tab.touch(ex_list[i]);
+    for (int e = 0; e < N; ++e)
+      if ((ex_mask >> e) & 1) tab.touch(e);
   }
   st.routed = false;  // the layer-step is complete
   st.predicted = false;

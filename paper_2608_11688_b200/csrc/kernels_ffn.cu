@@ -6,7 +6,7 @@
 // downT_i are contiguous (downT is W_down transposed) -- so one pass suffices and every CTA reads one
 // contiguous byte range:  a_i = g_e * silu(gate_i . h') * (up_i . h'),  y += a_i * downT_i.
 //
-// Kernel: persistent, one CTA per SM.  The (pair, i) row space -- a pair is (token, expert) -- is
+// Kernel (one token; batches run kernels_ffn_tc.cu): persistent, one CTA per SM.  The (expert, i) row space is
 // cut into equal contiguous ranges, one per CTA.  Each of the eight warps streams its own rows
 // (row q of the CTA belongs to warp q mod 8) into its stages of a shared-memory ring with one bulk
 // asynchronous copy per row (TMA, mbarrier completion; issuing from eight threads instead of one
@@ -59,11 +59,10 @@ __host__ __device__ constexpr int ring_stages(uint32_t entry_bytes) {
 }
 
 // ---------------------------------------------------------------- the streaming FFN kernel
-// Row space: pair p (a (token, expert) pair; routed pairs first, then the shared-expert pairs) owns
-// I (or I_shared) consecutive rows; row r of pair p is intermediate index i = r - offset(p).
+// Row space of the step's one token: each executed routed expert owns I consecutive rows, then the shared expert its
+// I_shared; row r of an expert is intermediate index i = r - its first row.
 struct RowMap {
-  int n_routed;          // routed pairs
-  int n_pairs;           // all pairs
+  int n_routed;          // executed routed experts
   int routed_rows;       // n_routed * I (the host refuses shapes whose row count does not fit 31 bits)
   int total_rows;
 };
@@ -73,10 +72,8 @@ template <int NCH, bool H_REGS, int FMT>
 __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel(const FfnParams p) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ uint64_t s_full[kMaxStages];
-  __shared__ float s_gate[kMaxStages];
-  __shared__ int s_tok[kMaxStages];
   __shared__ int s_exp[kMaxStages];
-  __shared__ int s_pos[kConsumerWarps][APEX_MAX_TOPK];  // B == 1: expert at each position of the row space (a copy per warp)
+  __shared__ int s_pos[kConsumerWarps][APEX_MAX_TOPK];  // expert at each position of the row space (a copy per warp)
   __shared__ int s_abort;
 
   constexpr int d = NCH * 256;
@@ -91,7 +88,7 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
   static_assert(NS * entry_bytes >= kConsumerWarps * d * 4, "ring must also hold the cross-warp reduction buffer");
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int N = p.N, k = p.k, I = p.I, B = p.B;
+  const int N = p.N, k = p.k, I = p.I;
   const int G = gridDim.x, cta = blockIdx.x;
 
   // ---- work that does not depend on the preceding kernel
@@ -106,9 +103,7 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   __syncthreads();  // barriers initialised
   float hreg[H_REGS ? NCH * 8 : 1];
-  int cur_tok = -1;
-  if (H_REGS && B == 1) {  // h' is an input of the gate kernel as well: complete long before this kernel
-    cur_tok = 0;
+  if (H_REGS) {  // h' is an input of the gate kernel as well: complete long before this kernel
 #pragma unroll
     for (int c = 0; c < NCH; ++c) {
       const float4 a = __ldg(reinterpret_cast<const float4*>(p.hpost) + (c * 32 + lane) * 2);
@@ -122,7 +117,7 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
   // usual case: the gate kernel), after it otherwise.
   auto zero_slice = [&]() {
     if (p.accumulate) return;
-    const size_t n4 = (size_t)B * d / 4;
+    const size_t n4 = (size_t)d / 4;
     const size_t per = (n4 + G - 1) / G;
     const size_t lo = per * cta, hi = lo + per < n4 ? lo + per : n4;
     float4* y4 = reinterpret_cast<float4*>(p.y);
@@ -158,11 +153,10 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
   bool dynamic = false;
   int S = 0, chunk = 1, n_static = 0;
   int static_base = 0, dyn_begin = 0, dyn_rows = 0;
-  auto set_geometry = [&](int n_routed, int n_pairs) {
+  auto set_geometry = [&](int n_routed) {
     rm.n_routed = n_routed;
-    rm.n_pairs = n_pairs;
     rm.routed_rows = n_routed * I;
-    rm.total_rows = rm.routed_rows + (n_pairs - n_routed) * p.I_shared;
+    rm.total_rows = rm.routed_rows + (p.run_shared ? p.I_shared : 0);
     const int per_cta = rm.total_rows / G, extra = rm.total_rows - per_cta * G;  // the first `extra` CTAs take one row more
     dynamic = per_cta >= 2 * NS;
     const int range_lo = cta * per_cta + (cta < extra ? cta : extra), range_hi = range_lo + per_cta + (cta < extra ? 1 : 0);
@@ -180,17 +174,17 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
       *pidx = (int)(r / I);
       *i = r - *pidx * I;
     } else {
-      *pidx = rm.n_routed + (int)((r - rm.routed_rows) / p.I_shared);
-      *i = r - rm.routed_rows - (*pidx - rm.n_routed) * p.I_shared;
+      *pidx = rm.n_routed;
+      *i = r - rm.routed_rows;
     }
   };
 
-  // ---- speculative first fill (B == 1).  The prefetch router ranked this step's experts long ago;
+  // ---- speculative first fill.  The prefetch router ranked this step's experts long ago;
   // its first k are the best guess of the routed set.  Their rows are requested now, while the gate
   // kernel is still running; after the dependency wait each guess is either confirmed (the copy is
   // already in flight or has landed) or dropped and its stage refilled.  Positions of the row space
   // that hold a confirmed guess keep it, so confirmed rows stay with the CTA that requested them.
-  bool spec_on = B == 1 && p.spec != nullptr;
+  bool spec_on = p.spec != nullptr;
   int spec_e = -1;
   bool spec_issued = false;  // this lane started a speculative copy into its stage (stage index = lane)
   if (spec_on) {
@@ -210,7 +204,7 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
       const unsigned long long t0 = globaltimer_ns();
       while ((long long)(globaltimer_ns() - t0) < p.spec_delay_ns) __nanosleep(200);
     }
-    set_geometry(k, k + (p.run_shared ? 1 : 0));
+    set_geometry(k);
     const int fill = n_static < NSW ? n_static : NSW;
     if (lane < fill) {
       int pidx;
@@ -225,8 +219,6 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
       }
       if (base) {
         const int s = warp + kConsumerWarps * lane;
-        s_gate[s] = 0.f;
-        s_tok[s] = 0;
         s_exp[s] = e;
         mbar_expect_tx(&s_full[s], entry_bytes);
         bulk_g2s(smem + (size_t)s * entry_bytes, base + (size_t)i * entry_bytes, entry_bytes, &s_full[s]);
@@ -242,23 +234,15 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
   if (!p.zero_early) zero_slice();  // a preceding launch of this library may still be adding to the same y
 
   // ---- every global load of the prologue is issued before the first use, so the latencies overlap.
-  TokenLoads tl1;
-  if (B == 1) tl1 = load_token(p.idx, p.z_r, p.alpha, N, k, p.mode, lane);
+  const TokenLoads tl1 = load_token(p.idx, p.z_r, p.alpha, N, k, p.mode, lane);
   if (tid == 0) TL(10);
 
-  // ---- plan: B == 1 every warp derives the execution set itself; B > 1 the plan kernel wrote it
-  unsigned long long run = 0;
-  float g0 = 0.f, g1 = 0.f;
-  TokenPlan tp1;
-  tp1.exec_mask = tp1.kr_mask = 0ull;
-  tp1.g0 = tp1.g1 = 0.f;
+  // ---- plan: every warp derives the execution set itself
+  const TokenPlan tp1 = plan_token(tl1, p.mode, p.norm_topk, p.snap.resident_mask, lane);
+  const float g0 = tp1.g0, g1 = tp1.g1;
+  const unsigned long long run = tp1.exec_mask & p.run_mask;
   bool spec_geometry = false;  // the speculative row space is the final one
-  if (B == 1) {
-    const TokenPlan tp = plan_token(tl1, p.mode, p.norm_topk, p.snap.resident_mask, lane);
-    g0 = tp.g0;
-    g1 = tp.g1;
-    tp1 = tp;
-    run = tp.exec_mask & p.run_mask;
+  {
     const int n_routed = __popcll(run);
     spec_geometry = spec_on && n_routed == k;
     int pos_e = -1;
@@ -273,20 +257,16 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
       if (lane < k) pos_e = keep ? spec_e : nth_set_bit64(rest, __popc(gaps & ((1u << lane) - 1u)));
     } else {
       if (lane < n_routed) pos_e = nth_set_bit64(run, lane);
-      set_geometry(n_routed, n_routed + (p.run_shared ? 1 : 0));
+      set_geometry(n_routed);
     }
     if (lane < APEX_MAX_TOPK) s_pos[warp][lane] = pos_e;
     __syncwarp();
-  } else {
-    const int n_pairs = p.n_pairs[0];
-    set_geometry(n_pairs - (p.run_shared ? B : 0), n_pairs);
   }
   if (tid == 0) TL(2);  // plan done
 
   float acc[NCH * 8];
 #pragma unroll
   for (int i = 0; i < NCH * 8; ++i) acc[i] = 0.f;
-  const float* hrow = p.hpost;
   bool zero_seen = p.accumulate != 0;
   bool ok = true;
   unsigned long long waited = 0;
@@ -312,17 +292,9 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
 
   // Starts the copy of row r as this warp's n-th row, into stage (n mod NSW) of the warp.
   auto issue = [&](int r, int n) {
-    int pidx, e, tok, i;
-    float gate = 0.f;
+    int pidx, i;
     locate(r, &pidx, &i);
-    if (B == 1) {
-      e = pidx < rm.n_routed ? s_pos[warp][pidx] : N;
-      tok = 0;
-    } else {
-      e = p.pair_expert[pidx];
-      tok = p.pair_tok[pidx];
-      gate = p.pair_gate[pidx];
-    }
+    const int e = pidx < rm.n_routed ? s_pos[warp][pidx] : N;
     const uint8_t* base;
     if (e < N) {
       int slot = p.snap.expert_slot[e];
@@ -380,8 +352,6 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
       base = p.shared_w;
     }
     const int s = warp + kConsumerWarps * (n % NSW);
-    s_gate[s] = gate;
-    s_tok[s] = tok;
     s_exp[s] = e;
     mbar_expect_tx(&s_full[s], entry_bytes);
     bulk_g2s(smem + (size_t)s * entry_bytes, base + (size_t)i * entry_bytes, entry_bytes, &s_full[s]);
@@ -406,7 +376,7 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
                    : "memory");
     }
   };
-  const bool poster = B == 1 && cta == 0 && warp == 0 && p.post_exec;
+  const bool poster = cta == 0 && warp == 0 && p.post_exec;
   // If an expert of this launch still has to be fetched, the host cannot start before it has seen
   // K_r: post first.  Otherwise post while the first rows are in flight.
   const bool will_wait_for_host = p.demand_in_kernel && (run & ~p.snap.resident_mask) != 0ull;
@@ -480,7 +450,7 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
     ++tail;
   }
   bool polled = false;
-  float sgate = -1.f;  // B == 1: value of the shared expert's gate, once computed
+  float sgate = -1.f;  // value of the shared expert's gate, once computed
   for (int head = 0; head < tail; ++head) {
     if (__any_sync(0xffffffffu, *(volatile int*)&s_abort != 0)) break;
     const int s = warp + kConsumerWarps * (head % NSW);
@@ -492,43 +462,10 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
     if (lane == 0 && warp == 0 && head == 0) TL(5);
     if (lane == 0 && warp == 0) TL(6);
     const int e = s_exp[s];
-    const int tok = s_tok[s];
-    float gate;
-    if (B == 1) {
-      gate = __shfl_sync(0xffffffffu, e < 32 ? g0 : g1, e & 31);
-      if (e >= N) {  // the shared expert: weight 1, or its gate's value (computed when the warp meets its first shared row)
-        if (p.shared_gate && sgate < 0.f) sgate = shared_gate_weight(p.shared_gate, p.hpost, d, lane);
-        gate = p.shared_gate ? sgate : 1.f;
-      }
-    } else {
-      gate = s_gate[s];
-    }
-    if (tok != cur_tok) {
-      if (cur_tok >= 0) {
-        // batched case: this warp moves to another token, flush its partial sums
-        if (lane == 0) poll_zeroed(true);
-        __syncwarp();
-        float4* y4 = reinterpret_cast<float4*>(p.y + (size_t)cur_tok * d);
-#pragma unroll
-        for (int c = 0; c < NCH; ++c) {
-          const int col4 = (c * 32 + lane) * 2;
-          atomicAdd(y4 + col4, make_float4(acc[c * 8 + 0], acc[c * 8 + 1], acc[c * 8 + 2], acc[c * 8 + 3]));
-          atomicAdd(y4 + col4 + 1, make_float4(acc[c * 8 + 4], acc[c * 8 + 5], acc[c * 8 + 6], acc[c * 8 + 7]));
-        }
-#pragma unroll
-        for (int i2 = 0; i2 < NCH * 8; ++i2) acc[i2] = 0.f;
-      }
-      cur_tok = tok;
-      hrow = p.hpost + (size_t)tok * d;
-      if (H_REGS) {
-#pragma unroll
-        for (int c = 0; c < NCH; ++c) {
-          const float4 a = __ldg(reinterpret_cast<const float4*>(hrow) + (c * 32 + lane) * 2);
-          const float4 b2 = __ldg(reinterpret_cast<const float4*>(hrow) + (c * 32 + lane) * 2 + 1);
-          hreg[c * 8 + 0] = a.x; hreg[c * 8 + 1] = a.y; hreg[c * 8 + 2] = a.z; hreg[c * 8 + 3] = a.w;
-          hreg[c * 8 + 4] = b2.x; hreg[c * 8 + 5] = b2.y; hreg[c * 8 + 6] = b2.z; hreg[c * 8 + 7] = b2.w;
-        }
-      }
+    float gate = __shfl_sync(0xffffffffu, e < 32 ? g0 : g1, e & 31);
+    if (e >= N) {  // the shared expert: weight 1, or its gate's value (computed when the warp meets its first shared row)
+      if (p.shared_gate && sgate < 0.f) sgate = shared_gate_weight(p.shared_gate, p.hpost, d, lane);
+      gate = p.shared_gate ? sgate : 1.f;
     }
     const uint8_t* gs = smem + (size_t)s * entry_bytes;
     const uint8_t* us = gs + row_bytes;
@@ -543,8 +480,8 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
 #pragma unroll
         for (int m = 0; m < 8; ++m) hh[m] = hreg[c * 8 + m];
       } else {
-        const float4 a = __ldg(reinterpret_cast<const float4*>(hrow) + (c * 32 + lane) * 2);
-        const float4 b2 = __ldg(reinterpret_cast<const float4*>(hrow) + (c * 32 + lane) * 2 + 1);
+        const float4 a = __ldg(reinterpret_cast<const float4*>(p.hpost) + (c * 32 + lane) * 2);
+        const float4 b2 = __ldg(reinterpret_cast<const float4*>(p.hpost) + (c * 32 + lane) * 2 + 1);
         hh[0] = a.x; hh[1] = a.y; hh[2] = a.z; hh[3] = a.w; hh[4] = b2.x; hh[5] = b2.y; hh[6] = b2.z; hh[7] = b2.w;
       }
       if (FMT == kFmtMxfp4) {  // the lane's eight elements share one block scale
@@ -620,22 +557,7 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
     }
   }
 
-  if (B > 1) {
-    if (cur_tok >= 0 && !aborted) {
-      if (lane == 0) poll_zeroed(true);
-      __syncwarp();
-      float4* y4 = reinterpret_cast<float4*>(p.y + (size_t)cur_tok * d);
-#pragma unroll
-      for (int c = 0; c < NCH; ++c) {
-        const int col4 = (c * 32 + lane) * 2;
-        atomicAdd(y4 + col4, make_float4(acc[c * 8 + 0], acc[c * 8 + 1], acc[c * 8 + 2], acc[c * 8 + 3]));
-        atomicAdd(y4 + col4 + 1, make_float4(acc[c * 8 + 4], acc[c * 8 + 5], acc[c * 8 + 6], acc[c * 8 + 7]));
-      }
-    }
-    return;
-  }
-
-  // ---- B == 1: reduce the eight partial vectors in shared memory, then one vector atomic per float4
+  // ---- reduce the eight partial vectors in shared memory, then one vector atomic per float4
   __syncthreads();  // every ring entry has been consumed; the ring is free
   if (tid == 0) TL(7);
   float* red = reinterpret_cast<float*>(smem);

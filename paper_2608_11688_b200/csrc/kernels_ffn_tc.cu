@@ -3,42 +3,44 @@
 //
 // With B tokens per step an expert serves several tokens, so its weights should be read once and
 // applied to all of them: a grouped GEMM, one group per executed expert (plus the shared expert).
-// The step is still HBM-bound (a few tens of flop per weight byte at most), so the kernels are
+// The step is still HBM-bound (a few tens of flop per weight byte at most), so the kernel is
 // organised around streaming the weights once; the tensor cores only keep arithmetic off the
-// critical path.  "Swap-AB": the weight rows are the MMA's M dimension (128 per tile), the group's
-// tokens are N (16..256), so a small token count does not waste a 128-row tile.
+// critical path.  "Swap-AB": the weight rows are the MMA's M dimension, the group's tokens are N (16..128),
+// so a small token count does not waste a 128-row tile.
 //
-//   gather     X_g[pair][d] (bf16) = h'[token of pair]   (pairs are sorted by expert); zero y
-//   gate/up    G, U [128 x n] = W_gate/up[128 rows of I x d] . X_g^T       accumulators in TMEM
-//              a = g_pair * silu(G) * U  (fp32) is kept as TWO bf16 planes, a_hi = bf16(a) and
-//              a_lo = bf16(a - a_hi), so feeding it back to the tensor cores loses 2^-17, not 2^-9
-//                                                                            -> global scratch (L2)
-//   down       D [128 cols of d x 2n] = downT[I x 128]^T . [a_hi ; a_lo]^T   (downT is MN-major; both planes
-//              y[token][col] += D[:, j] + D[:, n + j]          fp32 atomics      in one MMA: N = 2n)
-//              (at most 64 tokens per unit here; larger groups are split; the shared expert's longer K is cut
-//              into chunks of I rows so that all units are about equally long)
+//   gate/up    G, U [128 x n] = W_gate/up[128 rows of I x d] . X^T       accumulators in TMEM; the rows of X (h' in bf16)
+//              a = g_pair * silu(G) * U  (fp32) is kept as TWO bf16        are gathered by token index by the TMA loads
+//              planes, a_hi = bf16(a) and a_lo = bf16(a - a_hi), so feeding it back to the tensor cores loses 2^-17,
+//              not 2^-9                                                    -> global scratch (L2)
+//   down       D [256 cols of d x 2n] = downT[K x 256]^T . [a_hi ; a_lo]^T  (downT is MN-major, two M = 128 halves; both
+//              y[token][col] += D[:, j] + D[:, n + j]      fp32 atomics       planes in one MMA: N = 2n)
 //
-// Measured on B200: an MMA with M = 128, K = 16 costs about 35-40 ns to issue whatever N is (it streams a
-// 128 x 16 slice of A), so small-N "swap-AB" MMAs are bound by their count, not by their flops: eight per
-// 64-wide K tile was the pace of both kernels until the two planes of the down projection were merged into
-// one instruction.  Accumulators are double-buffered in TMEM (2 x 256 columns), so the epilogue of one unit
-// overlaps the MMAs of the next.
+// ONE persistent kernel runs both: the units of both projections form one list, gate/up first, and the CTAs take
+// tickets.  A down unit needs its group's intermediate, so its activations are loaded once the group's gate/up units have
+// been counted in (its weights, which wait for nothing, are already on their way); the tickets are handed out in list
+// order, so whatever a unit waits for is already running somewhere and no co-residency is assumed.  As two kernels the
+// step lost a partial round of units at the end of each (748 units of 1 MB on 148 SMs: 5.05 rounds) and a pipeline
+// refill in between: 245 us against 187 at B = 256 (60 experts of 17 MB and a shared one of 69 MB: 1.16 GB), 107 against
+// 75 at B = 8.
+//
+// A pipeline stage is 64 K values of two 128-row weight tiles (gate and up | the two column halves of downT: 32 KB) and
+// of the group's activations.  Roles: a warp loads weights and takes the tickets, a warp loads activations, a thread
+// issues MMAs, four warps run the epilogue out of TMEM.  Accumulators are double-buffered in TMEM (2 x 256 columns), so
+// the epilogue of one unit overlaps the MMAs of the next.  An MMA with M = 128, K = 16 takes 47 cycles up to N = 48 and
+// 67 at N = 128 (measured), eight per stage, against 1400 cycles of an SM's share of HBM per 32 KB: the streaming bounds
+// the bf16 step at every batch size.  Every wait is bounded.
 //
 // Operands reach shared memory through TMA tensor maps with the 128-byte swizzle and are consumed
 // by tcgen05.mma through shared-memory descriptors (K-major for gate, up, X, A; MN-major for downT).
-// One CTA per SM, three roles: two warps issue TMA loads (alternating K tiles; a single issuing
-// thread cannot keep up with 16 KB tiles), one thread issues MMAs, four warps run the epilogue out
-// of TMEM.  Every wait is bounded.
 //
 // Quantised stores (e4m3 codes with a scale per row vector, e2m1 codes with a power-of-two scale per 32
-// elements) take the same path with one more role: the producers bring the raw code bytes (and, for e2m1,
-// the scale bytes) of a K tile into a staging area of the stage, eight converter warps expand them to bf16
-// in the swizzled operand layout the MMA descriptors expect, and the MMAs run as for a bf16 store.  Both code
-// sets are exact in bf16 (3 and 1 mantissa bits), and so is an e2m1 value times its power-of-two scale, so
-// the tensor cores see the dequantised weights exactly; the per-vector fp32 scales of an e4m3 row are not
-// exact in bf16 and are applied in fp32 instead: gate and up scales to the accumulators, the down scale
-// folded into the intermediate before it is split into its two bf16 planes.  HBM sees 1 or 0.53 bytes per
-// weight; the expansion costs shared-memory bandwidth and ALU work that the streaming leaves idle.
+// elements) take the same path with one more role: the weights arrive as raw code bytes in a ring of their own, in tiles
+// of 128 bytes per row (two or four stages' worth; boxes of one stage, 64 or 32 bytes wide, had the TMA requests of
+// short rows and eight-fold re-read scale bytes as the pace), and sixteen converter warps expand them to bf16 in
+// the swizzled operand layout the MMA descriptors expect.  Both code sets are exact in bf16 (3 and 1 mantissa bits), and
+// so is an e2m1 value times its power-of-two scale, so the tensor cores see the dequantised weights exactly; the
+// per-vector fp32 scales of an e4m3 row are not exact in bf16 and are applied in fp32 instead: gate and up scales to the
+// accumulators, the down scale folded into the intermediate before it is split into its two bf16 planes.
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_bf16.h>
@@ -50,19 +52,24 @@ namespace apex {
 
 namespace {
 
-constexpr int kProducerWarps = 2;  // TMA producers: K tile t is loaded by warp t mod 2
-constexpr int kMmaWarp = kProducerWarps;
-constexpr int kCvWarp0 = kProducerWarps + 1 + 4;  // first of the converter warps (quantised stores only)
-constexpr int kCvThreads = 256;   // eight warps: two per scheduler, so one warp's shared-memory latency hides behind the other's arithmetic
-// producers, MMA + TMEM owner, four epilogue warps; for a quantised store the converter warps as well
-__host__ __device__ constexpr int tc_threads(int qf) { return (kProducerWarps + 1 + 4) * 32 + (qf ? kCvThreads : 0); }
-__host__ __device__ constexpr int tc_tiles_per_stage(int phase, int qf) { return (phase == 2 && qf == 0) ? 2 : 1; }
-// bytes of raw codes (and e2m1 scale bytes: 16 per row) a pipeline stage stages for the converters
-__host__ __device__ constexpr int tc_raw_bytes(int phase, int qf) {
-  return qf == 1 ? (phase == 1 ? 2 * 128 * 64 : 64 * 128) : qf == 2 ? (phase == 1 ? 2 * 128 * 32 + 2 * 128 * 16 : 64 * 64 + 64 * 16) : 0;
-}
-constexpr int kKTile = 64;       // K elements per pipeline stage (128 bytes: one swizzle span)
-constexpr int kXRowsPerLoad = 8;    // rows per B-tile box: one 8-row swizzle atom, so a small group does not fetch rows it has no token for
+constexpr int kWWarp = 0;      // weight loads, tickets
+constexpr int kBWarp = 1;      // activation loads
+constexpr int kMmaWarp = 2;    // MMA issue, TMEM owner
+constexpr int kEpiWarp0 = 3;   // four epilogue warps
+constexpr int kCvWarp0 = 7;    // sixteen converter warps (quantised stores only): four per scheduler hide the latency of shared memory and ALU
+constexpr int kCvThreads = 512;
+__host__ __device__ constexpr int tc_threads(int qf) { return kCvWarp0 * 32 + (qf ? kCvThreads : 0); }
+constexpr int kKTile = 64;           // K values per stage (128 bytes of bf16: one swizzle span)
+constexpr int kABytes = 2 * 128 * 128;  // the two weight tiles of a stage
+constexpr int kMaxStages = 8, kMaxRaw = 4;
+constexpr int kARowsPerLoad = 16;    // rows per box of the intermediate, and of X where the tokens follow one another: the granularity of N
+constexpr int kUnitRing = 4;         // unit descriptors between the ticket taker and the other roles
+// quantised stores: stages fed by one raw tile, and its bytes (codes, e2m1 block scales)
+__host__ __device__ constexpr int tc_sub(int qf) { return qf == 2 ? 4 : qf == 1 ? 2 : 1; }
+__host__ __device__ constexpr int tc_raw_bytes(int qf) { return qf == 2 ? 32768 + 4096 : qf == 1 ? 32768 : 0; }
+// K tiles per down unit, at most: small enough for an even end of the launch, large enough that a unit's epilogue and
+// ticket stay small beside it
+constexpr int kDownTiles = 16, kDownTilesQ = 8;  // bf16 | quantised
 
 __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, int c0, int c1, int c2, int c3, uint64_t* bar) {
   asm volatile(
@@ -80,57 +87,86 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, i
                "l"(map), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2)
                : "memory");
 }
-// Expanding codes to bf16 with conversion instructions runs at a quarter of the plain ALU rate and was the pace of the
-// whole kernel; the converters therefore build the bf16 bit patterns with integer operations and one bf16 multiply:
-// a code's exponent and mantissa bits, placed at the top of a bf16's mantissa and the bottom of its exponent field,
-// read as the code's value times 2^(code bias - 127), subnormal codes included (they become bf16 subnormals, which
-// the multiply does not flush); the multiply by a power of two puts the exponent right and is exact.
+// four rows of a [rows][cols] map (box one row high), 64 columns each, to four consecutive 128-byte rows
+__device__ __forceinline__ void tma_gather4(void* dst, const CUtensorMap* map, int c0, int r0, int r1, int r2, int r3, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile::gather4.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6, %7}], [%2];" ::"r"(
+          smem_u32(dst)),
+      "l"(map), "r"(smem_u32(bar)), "r"(c0), "r"(r0), "r"(r1), "r"(r2), "r"(r3)
+      : "memory");
+}
+// Expanding codes to bf16.  A code's exponent and mantissa bits, placed at the top of a bf16's mantissa and the bottom of
+// its exponent field, read as the code's value times 2^(code bias - 127), subnormal codes included (they become bf16
+// subnormals, which the multiply does not flush); a multiply by a power of two puts the exponent right and is exact.
+// The integer pipe (16 lanes per scheduler and cycle) is the converters' bound, so the fields are masked there and moved by
+// multiply-adds, which run beside it (by kernel parameters: multiplications by constants the compiler knows would be
+// turned back into shifts): two masks per pair of codes instead of five integer operations.  A pair is made of
+// the codes that lie 16 bits apart in their word, so the values come out in the order 0 2 1 3 (e4m3: within four) and
+// 0 4 1 5 2 6 3 7 (e2m1: within eight): the activations a gate/up tile meets are stored in that order (by the plan kernel), and for a
+// down tile, whose codes run along the output columns, the epilogue undoes it.
+__host__ __device__ constexpr int tc_column_of(int qf, int j) {  // value at position j
+  return qf == 2 ? (j & ~7) | ((j & 1) << 2) | ((j >> 1) & 3) : qf == 1 ? (j & ~3) | ((j & 1) << 1) | ((j >> 1) & 1) : j;
+}
 __device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b) {
   uint32_t o;
   asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(o) : "r"(a), "r"(b));
   return o;
 }
-// four e4m3 codes (s eeee mmm, bias 7) -> four bf16 values
-__device__ __forceinline__ void e4m3x4_to_bf16(uint32_t c, uint32_t& o0, uint32_t& o1) {
-  const uint32_t k = 0x7B807B80u;                       // 2^120, twice
-  const uint32_t r0 = __byte_perm(c, 0u, 0x1404u);      // codes 0, 1 in the high byte of each half
-  const uint32_t r1 = __byte_perm(c, 0u, 0x3424u);      // codes 2, 3
-  o0 = mul_bf16x2((r0 & 0x80008000u) | ((r0 >> 4) & 0x07f007f0u), k);
-  o1 = mul_bf16x2((r1 & 0x80008000u) | ((r1 >> 4) & 0x07f007f0u), k);
+// (c & sign) * up_s + (c & rest) * up_r: fields that do not meet
+__device__ __forceinline__ uint32_t place(uint32_t c, uint32_t sign, uint32_t up_s, uint32_t rest, uint32_t up_r) {
+  const uint32_t o = (c & sign) * up_s + (c & rest) * up_r;
+  return o;
 }
-// eight e2m1 codes (s ee m, bias 1; the even element in the low nibble of its byte) times the block scale
-// 2^(sb - 127) (sb = 0: zero) -> eight bf16 values
-__device__ __forceinline__ uint4 e2m1x8_to_bf16(uint32_t c, uint32_t sb) {
-  uint32_t o[4];
-  if (sb <= 128u) {
-    // code bits as a bf16 read as value * 2^-126; times 2^126 * 2^(sb - 127) = 2^(sb - 1): one multiply
-    const uint32_t m1 = sb ? (sb + 126u) << 7 : 0u;
-    const uint32_t m = m1 | (m1 << 16);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint32_t t = __byte_perm(c, 0u, 0x4440u + j) * 4097u;   // low nibble at bits 0..3, high nibble at bits 16..19
-      o[j] = mul_bf16x2(((t & 0x00080008u) << 12) | ((t & 0x00070007u) << 6), m);
-    }
-  } else {
-    // scales above 2 (never produced for weights of ordinary size): through the conversion instructions
-    const float scale = __uint_as_float(sb << 23);
-    uint32_t h[4];
-    asm("{\n.reg .b8 b0, b1, b2, b3;\n"
-        "mov.b32 {b0, b1, b2, b3}, %4;\n"
-        "cvt.rn.f16x2.e2m1x2 %0, b0;\n"
-        "cvt.rn.f16x2.e2m1x2 %1, b1;\n"
-        "cvt.rn.f16x2.e2m1x2 %2, b2;\n"
-        "cvt.rn.f16x2.e2m1x2 %3, b3;\n}"
-        : "=r"(h[0]), "=r"(h[1]), "=r"(h[2]), "=r"(h[3])
-        : "r"(c));
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&h[j]));
-      const __nv_bfloat162 b = __floats2bfloat162_rn(f.x * scale, f.y * scale);
-      o[j] = *reinterpret_cast<const uint32_t*>(&b);
-    }
+// four e4m3 codes (s eeee mmm, bias 7) -> bf16 pairs (0, 2), (1, 3)
+__device__ __forceinline__ void e4m3x4_to_bf16(const TcShifts& k, uint32_t c, uint32_t& o0, uint32_t& o1) {
+  const uint32_t e = 0x7B807B80u;  // 2^120, twice
+  o0 = mul_bf16x2(place(c, 0x00800080u, k.up8, 0x007f007fu, k.up4), e);
+  o1 = mul_bf16x2(place(c >> 8, 0x00800080u, k.up8, 0x007f007fu, k.up4), e);
+}
+// the block scale 2^(sb - 127) of e2m1 codes times 2^126, twice; for scales above 2 (never produced for weights of ordinary
+// size) that exceeds bf16: half the exponent, to be applied twice
+__device__ __forceinline__ uint32_t e2m1_scale(uint32_t sb, uint32_t& again) {
+  uint32_t m = sb ? (sb + 126u) << 7 : 0u;
+  again = 0x3F803F80u;
+  if (sb > 128u) {
+    m = 253u << 7;  // 2^126
+    again = sb << 7;
+    again |= again << 16;
   }
-  return make_uint4(o[0], o[1], o[2], o[3]);
+  return m | (m << 16);
+}
+// eight e2m1 codes (s ee m, bias 1; the even element in the low nibble of its byte) -> bf16 pairs (0, 4), (1, 5), (2, 6), (3, 7)
+template <bool TWICE>
+__device__ __forceinline__ uint4 e2m1x8_to_bf16(const TcShifts& k, uint32_t c, uint32_t m, uint32_t again) {
+  const uint32_t c2 = c >> 8;
+  uint4 o;
+  o.x = mul_bf16x2(place(c, 0x00080008u, k.up12, 0x00070007u, k.up6), m);
+  o.y = mul_bf16x2(place(c, 0x00800080u, k.up8, 0x00700070u, k.up2), m);
+  o.z = mul_bf16x2(place(c2, 0x00080008u, k.up12, 0x00070007u, k.up6), m);
+  o.w = mul_bf16x2(place(c2, 0x00800080u, k.up8, 0x00700070u, k.up2), m);
+  if (TWICE) {
+    o.x = mul_bf16x2(o.x, again);
+    o.y = mul_bf16x2(o.y, again);
+    o.z = mul_bf16x2(o.z, again);
+    o.w = mul_bf16x2(o.w, again);
+  }
+  return o;
+}
+// the 32 codes of one block
+__device__ __forceinline__ void e2m1x32_to_bf16(const TcShifts& k, const uint4& v, uint32_t sb, uint4 (&o)[4]) {
+  uint32_t again;
+  const uint32_t m = e2m1_scale(sb, again);
+  if (__any_sync(0xffffffffu, sb > 128u)) {
+    o[0] = e2m1x8_to_bf16<true>(k, v.x, m, again);
+    o[1] = e2m1x8_to_bf16<true>(k, v.y, m, again);
+    o[2] = e2m1x8_to_bf16<true>(k, v.z, m, again);
+    o[3] = e2m1x8_to_bf16<true>(k, v.w, m, again);
+  } else {
+    o[0] = e2m1x8_to_bf16<false>(k, v.x, m, again);
+    o[1] = e2m1x8_to_bf16<false>(k, v.y, m, again);
+    o[2] = e2m1x8_to_bf16<false>(k, v.z, m, again);
+    o[3] = e2m1x8_to_bf16<false>(k, v.w, m, again);
+  }
 }
 // shared-memory matrix descriptor, 128-byte swizzle (layout type 2), version 1
 __device__ __forceinline__ uint64_t umma_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
@@ -158,141 +194,129 @@ __device__ __forceinline__ void umma(uint32_t tmem_d, uint64_t adesc, uint64_t b
                "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
                : "memory");
 }
+// A from TMEM (lane = row, a 32-bit column holds two consecutive K values)
+__device__ __forceinline__ void umma_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(tmem_d),
+               "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
+               : "memory");
+}
+// One lane of a converged warp.  MMAs are issued under this predicate in warp-uniform code, so descriptors stay in uniform
+// registers; issued from `if (lane == 0)` an MMA cost 47 cycles of moves whatever its size, and three times that beside
+// busy converter warps.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n.reg .pred e;\nelect.sync _|e, 0xffffffff;\nselp.u32 %0, 1, 0, e;\n}" : "=r"(r));
+  return r != 0;
+}
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
-        "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
-        "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
-        "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15};" ::"r"(r[0]), "r"(r[1]),
+      "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]),
+      "r"(r[14]), "r"(r[15]), "r"(taddr)
       : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 #ifdef APEX_TIMELINE
-__device__ unsigned long long g_tc_tl[2][148][128];
-#define TCTL(ph, i) do { if ((i) < 128) g_tc_tl[(ph) - 1][blockIdx.x][(i)] = globaltimer_ns(); } while (0)
-// per K tile (the first 96 of a CTA): loads issued, raw bytes landed, operand buffer free, tiles converted; stage free
-// (producer), operands complete (MMA thread), MMAs issued
-__device__ unsigned long long g_cv_tl[2][148][96][8];
-#define CVTL(ph, it, i) do { if ((it) < 96u) g_cv_tl[(ph) - 1][blockIdx.x][(it)][(i)] = globaltimer_ns(); } while (0)
+// per CTA and unit: 0 ticket taken, 1 first weights landed (MMA thread), 2 MMAs issued, 3 accumulators complete, 4 epilogue done
+__device__ unsigned long long g_tc_tl[148][64][8];
+#define TCTL(u, i) do { if ((u) < 64u && blockIdx.x < 148) g_tc_tl[blockIdx.x][(u)][(i)] = globaltimer_ns(); } while (0)
 #else
-#define TCTL(ph, i) do { } while (0)
-#define CVTL(ph, it, i) do { } while (0)
+#define TCTL(u, i) do { } while (0)
 #endif
 
-struct Group {
-  int expert, pair_off, n_tok;
-};
-// One unit of work of a GEMM CTA: the (part of a) group, the M block and the K-tile range.
+// One unit of work: the (part of a) group, the M block and the K-tile range of one of the projections (phase 1: gate/up,
+// 2: down; 0: the list is at its end).
 struct UnitDesc {
-  int expert, pair_off, n_tok, blk, kt_begin, kt_end;
+  int phase, group, expert, pair_off, n_tok, blk, kt_begin, kt_end;
 };
-constexpr int kUnitChunk = 32;  // unit descriptors held in shared memory at a time
-__device__ __forceinline__ Group load_group(const int32_t* grp, int g) {
-  Group r;
-  r.expert = grp[4 + 3 * g];
-  r.pair_off = grp[5 + 3 * g];
-  r.n_tok = grp[6 + 3 * g];
-  return r;
-}
+// TMEM.  bf16 stores: two accumulator buffers of 256 columns.  Quantised stores: two of 128 columns, which a unit with more
+// than 64 (gate/up) or 32 (down) tokens takes together, and above them the gate/up weight tiles of the operand stages
+// (64 columns each).  The MMA thread and the epilogue walk the units with the same bookkeeping.
+__host__ __device__ constexpr uint32_t tc_acc_cols(int qf) { return qf ? 128u : 256u; }
+constexpr uint32_t kTmemA = 256;
+// Position in a ring: slot, and the parity of its current round (a "full" barrier is waited for with it, an "empty" barrier
+// with the other, which passes at once in the first round).  Counters, not divisions by the run-time depth: those were a
+// third of the converters' instructions.
+struct RingPos {
+  uint32_t s = 0, parity = 0;
+  __device__ __forceinline__ void next(uint32_t depth) {
+    if (++s == depth) {
+      s = 0;
+      parity ^= 1u;
+    }
+  }
+};
+struct AccBuffers {
+  uint32_t next = 0, uses[2] = {0, 0};  // buffer of the next unit that needs one; units that have used each
+};
+template <int QF>
+__device__ __forceinline__ bool unit_is_wide(const UnitDesc& ud) { return QF != 0 && ud.n_tok > (ud.phase == 1 ? 64 : 32); }
 
 }  // namespace
 
-// ---------------------------------------------------------------- gather + zero
-__global__ void __launch_bounds__(256) ffn_tc_gather_kernel(const TcParams p) {
-  SPAN_BEGIN();
-  pdl_wait();               // the plan kernel's pair list is complete from here on
-  pdl_launch_dependents();  // the next kernel may start its prologue
-  const int n_pairs = p.f.n_pairs[0];
-  const int d = p.f.d;
-  if (!p.f.accumulate) {
-    float4* y4 = reinterpret_cast<float4*>(p.f.y);
-    const size_t n4 = (size_t)p.f.B * d / 4;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x)
-      y4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-  for (int pr = blockIdx.x; pr < n_pairs; pr += gridDim.x) {
-    const int t = p.f.pair_tok[pr];
-    const float4* src = reinterpret_cast<const float4*>(p.f.hpost + (size_t)t * d);
-    uint2* dst = reinterpret_cast<uint2*>(p.xg + (size_t)pr * d);
-    for (int c = threadIdx.x; c < d / 4; c += blockDim.x) {
-      const float4 v = __ldg(src + c);
-      __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
-      uint2 o;
-      o.x = *reinterpret_cast<uint32_t*>(&lo);
-      o.y = *reinterpret_cast<uint32_t*>(&hi);
-      dst[c] = o;
-    }
-  }
-  SPAN_END(7);
-}
-
-// ---------------------------------------------------------------- the two GEMM kernels
-// PHASE 1: gate/up.  A tiles: gate and up rows [128 x 64] (K-major), B tile: X_g rows [<=256 x 64].
-// PHASE 2: down.     A tile: downT [64 k-rows x 128 cols] as two 64-column atoms (MN-major), B tile: the group's rows of
-//                    a_hi, then of a_lo [2 x <=64 x 64].
-//
-// QF: storage format of the weights (0 bf16, 1 e4m3, 2 e2m1).  For QF != 0, tm_w / tm_ws cover the raw row bytes of
-// the slots / the shared expert (boxes of one K tile's code bytes) and tm_sc / tm_ssc the same bytes with 16-byte boxes
-// (the e2m1 scale bytes); a stage is [A tiles, bf16, written by the converters][B planes][raw bytes, written by TMA].
-template <int PHASE, int QF>
+// tm_w, tm_ws: weights of the slots / of the shared expert.  bf16: boxes of 64 columns x 64 rows; quantised: the raw row
+// bytes, boxes of 128 bytes x 128 rows.  tm_sc, tm_ssc: the same bytes in boxes of 16 bytes x 128 rows (e2m1 block scales).
+// tm_x, tm_xc: h' in bf16, boxes of one row (gathered) and of kARowsPerLoad.  tm_act: the intermediate, plane a_lo below plane a_hi.
+template <int QF>
 __global__ void __launch_bounds__(tc_threads(QF), 1)
-ffn_tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_ws,
-                   const __grid_constant__ CUtensorMap tm_sc, const __grid_constant__ CUtensorMap tm_ssc,
-                   const __grid_constant__ CUtensorMap tm_b, const __grid_constant__ CUtensorMap tm_b2, const TcParams p) {
+ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_ws,
+              const __grid_constant__ CUtensorMap tm_sc, const __grid_constant__ CUtensorMap tm_ssc,
+              const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_xc, const __grid_constant__ CUtensorMap tm_act, const TcParams p) {
   SPAN_BEGIN();
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  constexpr int A_BYTES = PHASE == 1 ? 2 * 128 * 128 : 2 * 64 * 128;  // gate+up tiles | two downT atoms
-  constexpr int PLANES = PHASE == 1 ? 1 : 2;                          // X | a_hi and a_lo
-  constexpr int MAX_STAGES = 8;
-  // Tokens per unit (NMAX), hence the size of a B tile and the pipeline depth, are chosen per launch:
-  // small batches get deep pipelines (more weight bytes in flight), large groups are cut into parts.
-  const int NMAX = PHASE == 1 ? p.nmax1 : p.nmax2;
-  const int B_PLANE = NMAX * 128;
-  constexpr int RAW_BYTES = tc_raw_bytes(PHASE, QF);
-  // K tiles per stage.  The down projection of a bf16 store puts two in a stage (each laid out as a stage of one): its
-  // tiles are small (16 KB of weights) and cheap in MMAs (four), so the fixed cost of a stage -- a barrier round trip,
-  // a commit, the producer's turn -- weighed as much as the tile itself (672 ns per tile, 3.5 TB/s while it streamed).
-  constexpr int KPS = tc_tiles_per_stage(PHASE, QF);
-  const int HALF_BYTES = A_BYTES + PLANES * B_PLANE;
-  const int STAGE_BYTES = KPS * HALF_BYTES + RAW_BYTES;
-  const int NSTAGE = PHASE == 1 ? p.nstage1 : p.nstage2;
-  __shared__ uint64_t full[MAX_STAGES], empty[MAX_STAGES], rawfull[MAX_STAGES], tmem_full[2], tmem_empty[2];
+  constexpr int SUB = tc_sub(QF);
+  constexpr int RAW_BYTES = tc_raw_bytes(QF);
+  const int STAGE_BYTES = p.stage_bytes, NS = p.nstage, NR = p.nraw;
+  uint8_t* raw_ring = smem + (size_t)NS * STAGE_BYTES;
+  __shared__ uint64_t full[kMaxStages], empty[kMaxStages], rawfull[kMaxRaw], rawempty[kMaxRaw], tmem_full[2], tmem_empty[2];
+  __shared__ uint64_t unit_full[kUnitRing], unit_empty[kUnitRing];
+  __shared__ UnitDesc s_unit[kUnitRing];
   __shared__ uint32_t tmem_base_s;
   __shared__ int s_abort;
-  __shared__ UnitDesc s_unit[kUnitChunk];
-  __shared__ unsigned long long s_ready_mask;  // experts whose slot was seen ready in the prologue
-  __shared__ int s_ustart[APEX_MAX_EXPERTS + 3];  // first unit of each group
+  __shared__ int s_u1[APEX_MAX_EXPERTS + 2], s_u2[APEX_MAX_EXPERTS + 2];  // first unit of each group, in list order, per projection
   __shared__ int32_t s_grp[4 + 3 * (APEX_MAX_EXPERTS + 1)];
+  __shared__ uint8_t s_tok[APEX_MAX_BATCH * (APEX_MAX_TOPK + 1)];  // token of each pair
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int N = p.f.N, d = p.f.d, I = p.f.I, I_s = p.f.I_shared;
-  const int32_t* grp = p.grp;
 
   if (tid == 0) {
     s_abort = 0;
-    for (int s = 0; s < MAX_STAGES; ++s) {
-      mbar_init(&full[s], QF ? 1 + kCvThreads / 32 : 1);  // the producer's arrival (B tile bytes) and one per converter warp
+    for (int s = 0; s < kMaxStages; ++s) {
+      mbar_init(&full[s], QF ? 1 + kCvThreads / 32 : 2);  // the activations' bytes, and the weights' (bytes, or the converter warps)
       mbar_init(&empty[s], 1);
-      mbar_init(&rawfull[s], 1);
+    }
+    for (int r = 0; r < kMaxRaw; ++r) {
+      mbar_init(&rawfull[r], 1);
+      mbar_init(&rawempty[r], kCvThreads / 32);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&tmem_full[b], 1);
       mbar_init(&tmem_empty[b], 128);
     }
+    for (int u = 0; u < kUnitRing; ++u) {
+      mbar_init(&unit_full[u], 1);
+      mbar_init(&unit_empty[u], 6 + (QF ? kCvThreads / 32 : 0));  // every warp that reads the descriptor
+    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_w) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_ws) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_b) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_b2) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_x) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_act) : "memory");
     if (QF == 2) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_sc) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_ssc) : "memory");
@@ -303,9 +327,10 @@ ffn_tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   // Slot-ready flags of all resident experts in one round of loads (neither the flags nor the snapshot come from the
-  // preceding kernel): the producers then skip the per-unit check, a system-scope load and a proxy fence on their path
+  // preceding kernel): the weight warp then skips the per-unit check, a system-scope load and a proxy fence on its path
   // at every unit boundary, for every expert already seen ready here.
-  if (warp == 0) {
+  unsigned long long ready_mask = 0;
+  if (warp == kWWarp) {
     bool r0 = false, r1 = false;
     const int e0 = lane, e1 = lane + 32;
     if (e0 < N) {
@@ -316,375 +341,520 @@ ffn_tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
       const int sl = p.f.snap.expert_slot[e1];
       if (sl >= 0) r1 = (int32_t)(ld_acquire_sys(p.f.slot_ready + sl) - p.f.snap.need_gen[e1]) >= 0;
     }
-    const unsigned m0 = __ballot_sync(0xffffffffu, r0), m1 = __ballot_sync(0xffffffffu, r1);
-    if (lane == 0) s_ready_mask = ((unsigned long long)m1 << 32) | m0;
-    asm volatile("fence.proxy.async;" ::: "memory");  // the tensor-map loads that follow the barrier read what the flags cover
+    ready_mask = ((unsigned long long)__ballot_sync(0xffffffffu, r1) << 32) | __ballot_sync(0xffffffffu, r0);
+    asm volatile("fence.proxy.async;" ::: "memory");  // the tensor-map loads below read what the flags cover
   }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = tmem_base_s;
   // everything above (barriers, TMEM, tensor-map prefetch, flags) is independent of the preceding kernel
   pdl_wait();
   pdl_launch_dependents();
 
-  // the group table goes to shared memory once: a global load per unit would sit on every role's path
-  for (int i = tid; i < 4 + 3 * (N + 1); i += (int)blockDim.x) s_grp[i] = grp[i];
+  // the group table and the pairs' tokens go to shared memory once: a global load per unit (1 to 2 us while the GPU
+  // streams) would sit on every role's path
+  for (int i = tid; i < 4 + 3 * (N + 1); i += (int)blockDim.x) s_grp[i] = p.f.grp[i];
+  for (int i = tid; i < p.f.B * (p.f.k + 1); i += (int)blockDim.x) s_tok[i] = (uint8_t)p.f.pair_tok[i];  // (past the last pair: unused)
+  tc_fence_before();
   __syncthreads();
-  const int n_rg = s_grp[0], n_g = s_grp[1];
-  const int blocks_r = PHASE == 1 ? I / 128 : d / 128;                       // M blocks of a routed group
-  const int blocks_s = PHASE == 1 ? (I_s > 0 ? I_s / 128 : 0) : d / 128;     // ... of the shared group
-  const int kdim_r = PHASE == 1 ? d : I, kdim_s = PHASE == 1 ? d : I_s;
-  // A group of n tokens is cut into ceil(n / NMAX) parts; a unit is (group, M block, part), parts
-  // fastest so that the CTAs that share a weight block run at the same time (second reader hits L2).
-  // The shared expert's down projection has a longer K (I_s) than a routed expert's (I): it is cut into
-  // chunks of I rows, each a unit of its own (partial sums meet in y through the atomics), so that all
-  // units of a launch are about equally long and the round-robin assignment stays balanced.
-  const int kchunks_s = (PHASE == 2 && I_s > I) ? (I_s + I - 1) / I : 1;
-  if (tid == 0) {
-    int acc = 0;
-    for (int g = 0; g < n_g; ++g) {
-      s_ustart[g] = acc;
-      const int parts = (s_grp[6 + 3 * g] + NMAX - 1) / NMAX;
-      acc += (g < n_rg ? blocks_r : blocks_s * kchunks_s) * parts;
+  tc_fence_after();
+  const uint32_t tmem_base = tmem_base_s;
+  const int n_g = s_grp[1];
+  // Unit list: both projections take the groups from the end of the table -- the shared expert (the widest token tiles,
+  // the longest epilogues) first, so that its epilogues overlap later units.  A group of n tokens is cut into
+  // ceil(n / nmax) parts; parts fastest, so the CTAs that share a weight block run at the same time and the second
+  // reader hits L2.  The K of a down unit is cut into equal chunks of at most kDownTiles tiles (partial sums meet in y).
+  auto k_tiles = [&](int expert) { return ((expert >= N ? I_s : I) + kKTile - 1) / kKTile; };
+  auto down_chunk = [&](int tiles) {  // K tiles per down unit; whole raw tiles
+    const int n = (tiles + (QF ? kDownTilesQ : kDownTiles) - 1) / (QF ? kDownTilesQ : kDownTiles);
+    return ((tiles + n - 1) / n + SUB - 1) / SUB * SUB;
+  };
+  if (warp == 0) {  // two prefix sums over up to 65 groups: lanes own groups 2 lane, 2 lane + 1 (and lane 0 group 64)
+    auto units = [&](int o, int phase) -> int {
+      if (o >= n_g) return 0;
+      const int g = n_g - 1 - o, e = s_grp[4 + 3 * g], n = s_grp[6 + 3 * g];
+      if (phase == 1) return ((e >= N ? I_s : I) + 127) / 128 * ((n + p.nmax1 - 1) / p.nmax1);
+      const int t = k_tiles(e), c = down_chunk(t);
+      return d / 256 * ((t + c - 1) / c) * ((n + p.nmax2 - 1) / p.nmax2);
+    };
+    for (int phase = 1; phase <= 2; ++phase) {
+      int* su = phase == 1 ? s_u1 : s_u2;
+      const int a = units(2 * lane, phase), b = units(2 * lane + 1, phase);
+      int v = a + b;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int w = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += w;
+      }
+      su[2 * lane] = v - a - b;
+      su[2 * lane + 1] = v - b;
+      if (lane == 31) {
+        su[64] = v;
+        su[65] = v + units(64, phase);
+      }
     }
-    s_ustart[n_g] = acc;
   }
   __syncthreads();
-  const int n_units = s_ustart[n_g];
+  const int n1 = s_u1[APEX_MAX_EXPERTS + 1], n2 = s_u2[APEX_MAX_EXPERTS + 1];
 
-  uint32_t it_load = 0, it_mma = 0, it_cv = 0;  // running K-tile counters of the producers, the MMA thread and the converters
-  uint32_t unit_no = 0;              // units done by this CTA (phase of the TMEM barriers)
-  // The units of this CTA (uu = blockIdx.x, + gridDim.x, ...) are described once, kUnitChunk at a time and a thread
-  // per unit: group lookup and index arithmetic are then off every role's path at the unit boundaries, where that
-  // cold code cost each role more than a microsecond per unit.
-  for (int chunk0 = blockIdx.x; chunk0 < n_units; chunk0 += (int)gridDim.x * kUnitChunk) {
-    if (tid < kUnitChunk) {
-      // units are taken from the end of the list: the shared expert's (the widest token tiles, the longest epilogues)
-      // come first, so that their epilogues overlap later units instead of forming the tail of the launch
-      const int uf = chunk0 + tid * (int)gridDim.x;
-      const int uu = n_units - 1 - uf;
-      UnitDesc ud = {};
-      if (uf < n_units) {
-        int g = 0;
-        while (uu >= s_ustart[g + 1]) ++g;
-        Group gr = load_group(s_grp, g);
-        const int parts = (gr.n_tok + NMAX - 1) / NMAX;
-        const int local = uu - s_ustart[g];
-        const bool shared = gr.expert >= N;
-        const int kch = shared ? kchunks_s : 1;
-        const int blk = local / (parts * kch), kc = (local / parts) % kch, sub = local % parts;
-        const int kdim = shared ? kdim_s : kdim_r;
-        ud.expert = gr.expert;
-        ud.pair_off = gr.pair_off + sub * NMAX;
-        ud.n_tok = gr.n_tok - sub * NMAX < NMAX ? gr.n_tok - sub * NMAX : NMAX;
-        ud.blk = blk;
-        ud.kt_begin = kch > 1 ? kc * (I / kKTile) : 0;  // K tiles of this unit
-        ud.kt_end = kch > 1 ? (ud.kt_begin + I / kKTile < kdim / kKTile ? ud.kt_begin + I / kKTile : kdim / kKTile) : kdim / kKTile;
-      }
-      s_unit[tid] = ud;
+  bool ok = true;
+  auto give_up = [&]() {  // a wait ran out: tell the CTA, the other CTAs and the host
+    atomicExch(&s_abort, 1);
+    atomicExch(p.sync + kTcAbort, 1u);
+    *p.f.mbox_status = 1u;
+    if (p.f.stats) atomicAdd(&p.f.stats->timeouts, 1ull);
+  };
+  // the descriptor of this role's n-th unit; phase 0 at the end of the list and after an abort
+  auto next_unit = [&](uint32_t n) -> UnitDesc {
+    UnitDesc ud = {};
+    const uint32_t s = n % kUnitRing;
+    if (__all_sync(0xffffffffu, mbar_wait(&unit_full[s], (n / kUnitRing) & 1, &s_abort, p.f.wait_limit_ns))) {
+      ud = s_unit[s];
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&unit_empty[s]);
     }
-    __syncthreads();
-  for (int uj = 0; uj < kUnitChunk && chunk0 + uj * (int)gridDim.x < n_units && !*(volatile int*)&s_abort; ++uj) {
-    const UnitDesc ud = s_unit[uj];
-    Group gr;
-    gr.expert = ud.expert;
-    gr.pair_off = ud.pair_off;
-    gr.n_tok = ud.n_tok;
-    const bool shared = gr.expert >= N;
-    const int blk = ud.blk, kt_begin = ud.kt_begin, kt_end = ud.kt_end;
-    const int n_pad = (gr.n_tok + 15) & ~15;                                  // MMA N
-    const int n_loads = (gr.n_tok + kXRowsPerLoad - 1) / kXRowsPerLoad;       // 32-row boxes of the B tile
+    return ud;
+  };
 
-    if (warp < kProducerWarps) {
-      // ================= TMA producers: the whole warp walks the K tiles; lane 0 owns the barriers and
-      // each load of a stage is issued by a different lane (one thread sustains only about one bulk
-      // copy per 570 cycles)
+  if (warp == kWWarp) {
+    // ================= tickets and weight loads.  Each load of a stage is issued by a different lane (one thread
+    // sustains only about one bulk copy per 570 cycles).
+    RingPos rp;  // over the stages (bf16) or the raw tiles (quantised)
+    // The next ticket is taken a ring's depth before the end of a unit: the answer is there when the unit's last load has
+    // been issued (taken only then, it left the ring empty for 1.5 us per unit), and no unit waits long for its CTA.
+    const int ahead = (QF ? NR : NS) * SUB;
+    int ticket = lane == 0 ? (int)atomicAdd(p.sync + kTcTicket, 1u) : 0;
+    for (uint32_t n = 0; ok; ++n) {
+      const int t = __shfl_sync(0xffffffffu, ticket, 0);
+      bool taken = false;
+      UnitDesc ud = {};
+      if (t < n1 + n2) {
+        const bool down = t >= n1;
+        const int u = down ? t - n1 : t;
+        const int* su = down ? s_u2 : s_u1;
+        // order index of the group: the number of groups that end at or before u
+        const int o = __popc(__ballot_sync(0xffffffffu, su[lane + 1] <= u)) + __popc(__ballot_sync(0xffffffffu, su[lane + 33] <= u)) +
+                      (su[65] <= u ? 1 : 0);
+        const int g = n_g - 1 - o, nt = s_grp[6 + 3 * g], nmax = down ? p.nmax2 : p.nmax1;
+        const int parts = (nt + nmax - 1) / nmax;
+        int local = u - su[o];
+        const int part = local % parts;
+        local /= parts;
+        ud.phase = down ? 2 : 1;
+        ud.group = g;
+        ud.expert = s_grp[4 + 3 * g];
+        ud.pair_off = s_grp[5 + 3 * g] + part * nmax;
+        ud.n_tok = nt - part * nmax < nmax ? nt - part * nmax : nmax;
+        if (down) {
+          const int tiles = k_tiles(ud.expert), c = down_chunk(tiles), kch = (tiles + c - 1) / c;
+          ud.blk = local / kch;
+          ud.kt_begin = local % kch * c;
+          ud.kt_end = ud.kt_begin + c < tiles ? ud.kt_begin + c : tiles;
+        } else {
+          ud.blk = local;
+          ud.kt_end = d / kKTile;
+        }
+      }
+      if (lane == 0) {
+        const uint32_t s = n % kUnitRing;
+        if (n >= kUnitRing && !mbar_wait(&unit_empty[s], (n / kUnitRing - 1) & 1, &s_abort, p.f.wait_limit_ns)) ok = false;
+        s_unit[s] = ud;
+        mbar_arrive(&unit_full[s]);
+        TCTL(n, 0);
+      }
+      ok = __all_sync(0xffffffffu, ok);
+      if (ud.phase == 0 || !ok) break;
+      const bool shared = ud.expert >= N;
       int slot = 0;
-      bool ok = true;
       if (!shared) {
-        slot = p.f.snap.expert_slot[gr.expert];
+        slot = p.f.snap.expert_slot[ud.expert];
         if (slot < 0) ok = false;
-        if (ok && lane == 0 && !((s_ready_mask >> gr.expert) & 1ull)) {
-          const uint32_t need = p.f.snap.need_gen[gr.expert];
-          const uint32_t* flag = p.f.slot_ready + slot;
-          if ((int32_t)(ld_acquire_sys(flag) - need) < 0) {
+        if (ok && !((ready_mask >> ud.expert) & 1ull)) {
+          if (lane == 0) {
+            const uint32_t need = p.f.snap.need_gen[ud.expert];
+            const uint32_t* flag = p.f.slot_ready + slot;
             const unsigned long long t0 = globaltimer_ns();
-            while ((int32_t)(ld_acquire_sys(flag) - need) < 0) {
-              if ((long long)(globaltimer_ns() - t0) > p.f.wait_limit_ns) {
+            for (uint32_t n_poll = 1; (int32_t)(ld_acquire_sys(flag) - need) < 0; ++n_poll) {
+              if ((long long)(globaltimer_ns() - t0) > p.f.wait_limit_ns || ((n_poll & 7u) == 0u && *(volatile unsigned*)(p.sync + kTcAbort))) {
                 ok = false;
                 break;
               }
               __nanosleep(64);
             }
-            if (p.f.stats) atomicAdd(&p.f.stats->stall_ns, (globaltimer_ns() - t0) * (unsigned long long)gridDim.x / 4ull);
+            if (p.f.stats) atomicAdd(&p.f.stats->stall_ns, globaltimer_ns() - t0);
           }
+          ready_mask |= 1ull << ud.expert;
           asm volatile("fence.proxy.async;" ::: "memory");
         }
         ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
         slot += p.layer_slot0;  // the tensor map covers the slots of all layers
       }
       const CUtensorMap* wmap = shared ? &tm_ws : &tm_w;
-      constexpr int planes = PLANES;
-      for (int kt = kt_begin; kt < kt_end && ok; kt += KPS, ++it_load) {
-        if ((int)(it_load % kProducerWarps) != warp) continue;  // the other producer warp's stage
-        const int s = it_load % NSTAGE;
-        if (lane == 0) {
-          if (it_load >= (uint32_t)NSTAGE && !mbar_wait(&empty[s], ((it_load / NSTAGE) - 1) & 1, &s_abort, p.f.wait_limit_ns)) ok = false;
-          CVTL(PHASE, it_load, 4);
-          if (ok) {
-            mbar_expect_tx(&full[s], KPS * ((QF ? 0 : A_BYTES) + planes * n_loads * kXRowsPerLoad * 128));
-            if (QF) mbar_expect_tx(&rawfull[s], RAW_BYTES);
-          }
+      for (int kt = ud.kt_begin; kt < ud.kt_end; kt += SUB, rp.next(QF ? NR : NS)) {
+        uint64_t* bar;
+        uint8_t* dst;
+        if (QF == 0) {
+          if (lane == 0 && !mbar_wait(&empty[rp.s], rp.parity ^ 1, &s_abort, p.f.wait_limit_ns)) ok = false;
+          bar = &full[rp.s];
+          dst = smem + rp.s * STAGE_BYTES;
+        } else {
+          if (lane == 0 && !mbar_wait(&rawempty[rp.s], rp.parity ^ 1, &s_abort, p.f.wait_limit_ns)) ok = false;
+          bar = &rawfull[rp.s];
+          dst = raw_ring + rp.s * RAW_BYTES;
         }
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
-        uint8_t* st0 = smem + (size_t)s * STAGE_BYTES;
-        // the weight loads first; then op n_wops + r*planes + pl: 8-row box r of B plane pl
-        constexpr int n_wops = QF == 0 ? 2 : QF == 1 ? (PHASE == 1 ? 2 : 1) : (PHASE == 1 ? 4 : 2);
-        const int n_ops = n_wops + planes * n_loads;
-        uint8_t* raw = st0 + A_BYTES + planes * B_PLANE;
-        const int kt0 = kt;
-        for (int opx = lane; opx < KPS * n_ops; opx += 32) {
-          const int half = KPS > 1 ? opx / n_ops : 0, op = KPS > 1 ? opx - half * n_ops : opx;
-          const int kt = kt0 + half;                      // (shadows the stage's first tile)
-          uint8_t* st = st0 + (size_t)half * HALF_BYTES;
-          if (op < n_wops) {
-            if (QF == 0) {
-              if (PHASE == 1) tma_load_4d(st + op * 128 * 128, wmap, kt * kKTile, op, blk * 128, slot, &full[s]);   // gate | up rows
-              else tma_load_4d(st + op * 64 * 128, wmap, blk * 128 + op * 64, 2, kt * kKTile, slot, &full[s]);      // downT, 64 columns
-            } else if (QF == 1) {  // row: gate | up | downT codes (d bytes each), then the scales
-              if (PHASE == 1) tma_load_3d(raw + op * 128 * 64, wmap, op * d + kt * kKTile, blk * 128, slot, &rawfull[s]);
-              else tma_load_3d(raw, wmap, 2 * d + blk * 128, kt * kKTile, slot, &rawfull[s]);
-            } else {  // row: gate | up | downT codes (d/2 bytes each), then their scale bytes (d/32 each)
-              const CUtensorMap* smap = shared ? &tm_ssc : &tm_sc;
-              if (PHASE == 1) {
-                if (op < 2) tma_load_3d(raw + op * 128 * 32, wmap, op * (d / 2) + kt * (kKTile / 2), blk * 128, slot, &rawfull[s]);
-                else tma_load_3d(raw + 2 * 128 * 32 + (op - 2) * 128 * 16, smap, 3 * (d / 2) + (op - 2) * (d / 32) + ((kt * 2) & ~15), blk * 128,
-                                 slot, &rawfull[s]);
-              } else {
-                if (op == 0) tma_load_3d(raw, wmap, d + blk * 64, kt * kKTile, slot, &rawfull[s]);
-                else tma_load_3d(raw + 64 * 64, smap, 3 * (d / 2) + 2 * (d / 32) + ((blk * 4) & ~15), kt * kKTile, slot, &rawfull[s]);
-              }
-            }
-          } else {
-            // B rows of this stage: the tokens' rows of plane 0, padded to n_pad, then those of plane 1
-            const int r = (op - n_wops) / planes, pl = (op - n_wops) % planes;
-            tma_load_2d(st + A_BYTES + pl * n_pad * 128 + r * kXRowsPerLoad * 128, pl ? &tm_b2 : &tm_b, kt * kKTile,
-                        gr.pair_off + r * kXRowsPerLoad, &full[s]);
+        if (!taken && kt + ahead >= ud.kt_end) {
+          taken = true;
+          if (lane == 0) ticket = (int)atomicAdd(p.sync + kTcTicket, 1u);
+        }
+        if (lane == 0) mbar_expect_tx(bar, QF ? RAW_BYTES : kABytes);
+        __syncwarp();
+        if (QF == 0) {
+          if (lane < 4) {
+            if (ud.phase == 1) tma_load_4d(dst + lane * 8192, wmap, kt * kKTile, lane >> 1, ud.blk * 128 + (lane & 1) * 64, slot, bar);  // gate | up, two row halves each
+            else tma_load_4d(dst + lane * 8192, wmap, ud.blk * 256 + lane * 64, 2, kt * kKTile, slot, bar);                               // downT, 64 columns each
+          }
+        } else if (QF == 1) {  // row: gate | up | downT codes (d bytes each), then the scales
+          if (lane < 2) {
+            if (ud.phase == 1) tma_load_3d(dst + lane * 16384, wmap, lane * d + kt * kKTile, ud.blk * 128, slot, bar);
+            else tma_load_3d(dst + lane * 16384, wmap, 2 * d + ud.blk * 256 + lane * 128, kt * kKTile, slot, bar);
+          }
+        } else {  // row: gate | up | downT codes (d/2 bytes each), then their scale bytes (d/32 each)
+          const CUtensorMap* smap = shared ? &tm_ssc : &tm_sc;
+          if (lane < 2) {
+            if (ud.phase == 1) tma_load_3d(dst + lane * 16384, wmap, lane * (d / 2) + kt * (kKTile / 2), ud.blk * 128, slot, bar);
+            else tma_load_3d(dst + lane * 16384, wmap, d + ud.blk * 128, kt * kKTile + lane * 128, slot, bar);
+          } else if (lane < 4) {
+            const int h = lane - 2;
+            if (ud.phase == 1) tma_load_3d(dst + 32768 + h * 2048, smap, 3 * (d / 2) + h * (d / 32) + ((kt * 2) & ~15), ud.blk * 128, slot, bar);
+            else tma_load_3d(dst + 32768 + h * 2048, smap, 3 * (d / 2) + 2 * (d / 32) + ((ud.blk * 8) & ~15), kt * kKTile + h * 128, slot, bar);
           }
         }
         __syncwarp();
-        if (lane == 0) CVTL(PHASE, it_load, 0);
       }
-      if (!ok && lane == 0) {
-        atomicExch(&s_abort, 1);
-        *p.f.mbox_status = 1u;
-        if (p.f.stats) atomicAdd(&p.f.stats->timeouts, 1ull);
-      }
-    } else if (warp == kMmaWarp) {
-      // ================= MMA issuer
-      if (lane == 0) {
-        bool ok = true;
-        // two accumulator buffers of 256 TMEM columns: this unit's MMAs run while the epilogue warps
-        // still read the previous unit's
-        const uint32_t buf = unit_no & 1u;
-        TCTL(PHASE, unit_no * 16 + 15);
-        if (unit_no >= 2) ok = mbar_wait(&tmem_empty[buf], ((unit_no >> 1) - 1) & 1, &s_abort, p.f.wait_limit_ns);
-        tc_fence_after();
-        TCTL(PHASE, unit_no * 16);
-        const uint32_t tacc = tmem_base + buf * 256u;
-        // An MMA costs about 128 cycles whatever N is (it streams a 128 x 16 slice of A), so the down
-        // projection multiplies both planes of the intermediate in one instruction: N = 2 * n_pad.
-        const uint32_t idesc = umma_idesc(128, PHASE == 2 ? 2 * n_pad : n_pad, PHASE == 2 ? 1 : 0);
-        const uint64_t desc_a0 = PHASE == 1 ? umma_desc(smem_u32(smem), 16, 1024) : umma_desc(smem_u32(smem), 64 * 128, 1024);
-        const uint64_t desc_b0 = umma_desc(smem_u32(smem) + A_BYTES, 16, 1024);
-        for (int kt = kt_begin; kt < kt_end && ok; kt += KPS, ++it_mma) {
-          const int s = it_mma % NSTAGE;
-          if (!mbar_wait(&full[s], (it_mma / NSTAGE) & 1, &s_abort, p.f.wait_limit_ns)) {
-            ok = false;
-            break;
-          }
-          if (kt - kt_begin < 10) TCTL(PHASE, unit_no * 16 + 1 + kt - kt_begin);
-          CVTL(PHASE, it_mma, 5);
-          tc_fence_after();
-          // descriptors differ from the stage-0, k-step-0 ones only in the start-address field (address >> 4, the low
-          // 14 bits; the sums below stay inside the CTA's shared memory, so nothing carries into the next field)
-          const uint64_t soff = (uint64_t)((uint32_t)s * (uint32_t)STAGE_BYTES >> 4);
+    }
+    if (!ok && lane == 0) give_up();
+  } else if (warp == kBWarp) {
+    // ================= activation loads: rows of X gathered by token index, or the group's rows of a_hi and a_lo
+    RingPos rp;
+    for (uint32_t n = 0; ok; ++n) {
+      const UnitDesc ud = next_unit(n);
+      if (ud.phase == 0) break;
+      const int n_pad = (ud.n_tok + 15) & ~15;
+      int tok[4] = {0, 0, 0, 0};
+      if (ud.phase == 1) {  // lane j: rows 4 j .. 4 j + 3 (past the last token: any row, the result is not used)
 #pragma unroll
-          for (int half = 0; half < KPS; ++half) {
-          const uint64_t hoff = soff + (uint64_t)((uint32_t)half * (uint32_t)HALF_BYTES >> 4);
-          const uint64_t da = desc_a0 + hoff, db = desc_b0 + hoff;
-#pragma unroll
-          for (int ks = 0; ks < kKTile / 16; ++ks) {
-            const uint32_t acc = (kt > kt_begin || half > 0 || ks > 0) ? 1u : 0u;
-            const uint64_t bdesc = db + (uint64_t)(ks * 2);   // 32 bytes per k-step
-            if (PHASE == 1) {
-              umma(tacc, da + (uint64_t)(ks * 2), bdesc, idesc, acc);                           // G
-              umma(tacc + 128, da + (uint64_t)(128 * 128 / 16 + ks * 2), bdesc, idesc, acc);    // U
-            } else {
-              umma(tacc, da + (uint64_t)(ks * 128), bdesc, idesc, acc);  // 2 KB per k-step; columns [0, n_pad): a_hi, [n_pad, 2 n_pad): a_lo
+        for (int i = 0; i < 4; ++i) tok[i] = s_tok[ud.pair_off + min(4 * lane + i, ud.n_tok - 1)];
+      } else {
+        // the group's intermediate must be complete: every gate/up unit of the group has been counted in
+        if (lane == 0) {
+          const unsigned want = (unsigned)(((ud.expert >= N ? I_s : I) + 127) / 128 * ((s_grp[6 + 3 * ud.group] + p.nmax1 - 1) / p.nmax1));
+          const unsigned* done = p.sync + kTcDone + ud.group;
+          unsigned v;
+          asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(done) : "memory");
+          if (v < want) {
+            const unsigned long long t0 = globaltimer_ns();
+            for (uint32_t n_poll = 1; v < want; ++n_poll) {
+              if ((n_poll & 31u) == 0u && (*(volatile int*)&s_abort || *(volatile unsigned*)(p.sync + kTcAbort) ||
+                                           (long long)(globaltimer_ns() - t0) > p.f.wait_limit_ns)) {
+                ok = false;
+                break;
+              }
+              __nanosleep(40);
+              asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(done) : "memory");
             }
           }
+          asm volatile("fence.proxy.async;" ::: "memory");  // the bulk loads below read what other CTAs' threads have stored
+        }
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+      }
+      // The shared expert runs all tokens in order: plain boxes (32 gathers per stage were its pace, 1.3 us at 128 tokens)
+      const bool gather = ud.phase == 1 && ud.expert < N;
+      const int n_loads = gather ? (ud.n_tok + 3) / 4 : n_pad / kARowsPerLoad;
+      const uint32_t bytes = gather ? n_loads * 512u : (uint32_t)(ud.phase * n_pad * 128);
+      for (int kt = ud.kt_begin; kt < ud.kt_end; ++kt, rp.next(NS)) {
+        const uint32_t s = rp.s;
+        if (lane == 0 && !mbar_wait(&empty[s], rp.parity ^ 1, &s_abort, p.f.wait_limit_ns)) ok = false;
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        if (lane == 0) mbar_expect_tx(&full[s], bytes);
+        __syncwarp();
+        uint8_t* dst = smem + s * STAGE_BYTES + kABytes;
+        if (ud.phase == 1 && !gather) {
+          if (lane < n_loads)
+            tma_load_2d(dst + lane * kARowsPerLoad * 128, &tm_xc, kt * kKTile, s_tok[ud.pair_off] + lane * kARowsPerLoad, &full[s]);
+        } else if (ud.phase == 1) {
+          if (lane < n_loads) tma_gather4(dst + lane * 512, &tm_x, kt * kKTile, tok[0], tok[1], tok[2], tok[3], &full[s]);
+        } else if (lane < 2 * n_loads) {  // (at most 64 tokens: 4 boxes per plane)
+          const int pl = lane >= n_loads ? 1 : 0, r = lane - pl * n_loads;
+          tma_load_2d(dst + (pl * n_pad + r * kARowsPerLoad) * 128, &tm_act, kt * kKTile, pl * p.act_rows + ud.pair_off + r * kARowsPerLoad, &full[s]);
+        }
+        __syncwarp();
+      }
+    }
+    if (!ok && lane == 0) give_up();
+  } else if (warp == kMmaWarp) {
+    // ================= MMA issuer: the whole warp walks the stages, one elected lane issues
+    RingPos rp;
+    AccBuffers acc;
+    const uint64_t desc_a1 = umma_desc(smem_u32(smem), 16, 1024), desc_a2 = umma_desc(smem_u32(smem), 64 * 128, 1024);
+    const uint64_t desc_b = umma_desc(smem_u32(smem) + kABytes, 16, 1024);
+    const uint32_t tbase = __shfl_sync(0xffffffffu, tmem_base, 0);
+    for (uint32_t n = 0; ok; ++n) {
+      const UnitDesc ud = next_unit(n);
+      // (shuffles: the compiler keeps what comes out of them in uniform registers)
+      const int phase = __shfl_sync(0xffffffffu, ud.phase, 0), n_tok = __shfl_sync(0xffffffffu, ud.n_tok, 0);
+      if (phase == 0) break;
+      const int kt_begin = __shfl_sync(0xffffffffu, ud.kt_begin, 0), kt_end = __shfl_sync(0xffffffffu, ud.kt_end, 0);
+      // this unit's MMAs run while the epilogue warps still read the previous unit's accumulators
+      const bool wide = unit_is_wide<QF>(ud);
+      const uint32_t b0 = wide ? 0u : acc.next, b1 = wide ? 1u : acc.next;
+      for (uint32_t b = b0; b <= b1; ++b)
+        if (acc.uses[b]++ > 0) ok = ok && mbar_wait(&tmem_empty[b], acc.uses[b] & 1, &s_abort, p.f.wait_limit_ns);
+      if (!wide) acc.next ^= 1u;
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      tc_fence_after();
+      const bool down = phase == 2;
+      const int n_pad = (n_tok + 15) & ~15;
+      const uint32_t tacc = tbase + b0 * tc_acc_cols(QF);
+      const uint32_t second = QF != 0 && !wide ? 64u : 128u;   // columns of U | of the upper 128 output columns
+      const uint32_t idesc = umma_idesc(128, down ? 2 * n_pad : n_pad, down ? 1 : 0);
+      const uint64_t desc_a = down ? desc_a2 : desc_a1;
+      const uint64_t a_step = down ? 128 : 2;   // per 16 K values: 16 rows of 128 bytes (MN-major) | 32 bytes of a row
+      for (int kt = kt_begin; kt < kt_end; ++kt, rp.next(NS)) {
+        const uint32_t s = rp.s;
+        ok = __all_sync(0xffffffffu, mbar_wait(&full[s], rp.parity, &s_abort, p.f.wait_limit_ns));
+        if (!ok) break;
+        if (lane == 0 && kt == kt_begin) TCTL(n, 1);
+        tc_fence_after();
+        // descriptors differ from the stage-0, k-step-0 ones only in the start-address field (address >> 4, the low
+        // 14 bits; the sums below stay inside the CTA's shared memory, so nothing carries into the next field)
+        const uint64_t soff = (uint64_t)(s * (uint32_t)STAGE_BYTES >> 4);
+        const uint64_t da = desc_a + soff, db = desc_b + soff;
+        if (elect_one()) {
+          if (QF != 0 && !down) {
+            const uint32_t ta = tbase + kTmemA + s * 64u;  // gate, then up: 32 columns each
+#pragma unroll
+            for (int ks = 0; ks < kKTile / 16; ++ks) {
+              const uint32_t a = (kt > kt_begin || ks > 0) ? 1u : 0u;
+              umma_ts(tacc, ta + ks * 8, db + (uint64_t)(ks * 2), idesc, a);                 // G
+              umma_ts(tacc + second, ta + 32 + ks * 8, db + (uint64_t)(ks * 2), idesc, a);   // U
+            }
+          } else {
+#pragma unroll
+            for (int ks = 0; ks < kKTile / 16; ++ks) {
+              const uint32_t a = (kt > kt_begin || ks > 0) ? 1u : 0u;
+              umma(tacc, da + a_step * ks, db + (uint64_t)(ks * 2), idesc, a);                                     // G | columns 0 .. 127
+              umma(tacc + second, da + (uint64_t)(128 * 128 / 16) + a_step * ks, db + (uint64_t)(ks * 2), idesc, a);  // U | columns 128 .. 255
+            }
           }
           umma_commit(&empty[s]);  // the stage is free once these MMAs have read it
-          CVTL(PHASE, it_mma, 6);
-        }
-        TCTL(PHASE, unit_no * 16 + 11);
-        if (ok) umma_commit(&tmem_full[buf]);
-        else atomicExch(&s_abort, 1);
-        TCTL(PHASE, unit_no * 16 + 14);
-      }
-    } else if (QF != 0 && warp >= kCvWarp0) {
-      // ================= converters: raw codes of a stage -> bf16 operand tiles in the 128-byte-swizzled layout
-      // (a tile row is 128 bytes = 64 values; its 16-byte chunk j sits at chunk j ^ (row mod 8))
-      const int ct = tid - kCvWarp0 * 32;
-      bool ok = true;
-      for (int kt = kt_begin; kt < kt_end && ok; kt += KPS, ++it_cv) {
-        const int s = it_cv % NSTAGE;
-        ok = __all_sync(0xffffffffu, mbar_wait(&rawfull[s], (it_cv / NSTAGE) & 1, &s_abort, p.f.wait_limit_ns));
-        if (ct == 0) CVTL(PHASE, it_cv, 1);
-        if (!ok) break;
-        uint8_t* st = smem + (size_t)s * STAGE_BYTES;
-        const uint8_t* raw = st + A_BYTES + PLANES * B_PLANE;
-        if (QF == 1 && PHASE == 1) {
-          // two tiles [128 rows][64 codes]: chunk q of 16 codes -> two chunks of 8 bf16
-#pragma unroll
-          for (int q = ct; q < 1024; q += kCvThreads) {
-            const int tile = q >> 9, row = (q & 511) >> 2, c = q & 3;
-            const uint4 v = *reinterpret_cast<const uint4*>(raw + q * 16);
-            uint4 o0, o1;
-            e4m3x4_to_bf16(v.x, o0.x, o0.y);
-            e4m3x4_to_bf16(v.y, o0.z, o0.w);
-            e4m3x4_to_bf16(v.z, o1.x, o1.y);
-            e4m3x4_to_bf16(v.w, o1.z, o1.w);
-            uint8_t* dst = st + tile * (128 * 128) + row * 128;
-            *reinterpret_cast<uint4*>(dst + (((2 * c) ^ (row & 7)) << 4)) = o0;
-            *reinterpret_cast<uint4*>(dst + (((2 * c + 1) ^ (row & 7)) << 4)) = o1;
-          }
-        } else if (QF == 1) {
-          // [64 k-rows][128 codes] -> two 64-column atoms, MN-major
-#pragma unroll
-          for (int q = ct; q < 512; q += kCvThreads) {
-            const int kk = q >> 3, cc = q & 7;
-            const uint4 v = *reinterpret_cast<const uint4*>(raw + q * 16);
-            uint4 o0, o1;
-            e4m3x4_to_bf16(v.x, o0.x, o0.y);
-            e4m3x4_to_bf16(v.y, o0.z, o0.w);
-            e4m3x4_to_bf16(v.z, o1.x, o1.y);
-            e4m3x4_to_bf16(v.w, o1.z, o1.w);
-            uint8_t* dst = st + (cc >> 2) * (64 * 128) + kk * 128;
-            const int jc = (cc & 3) * 2;
-            *reinterpret_cast<uint4*>(dst + ((jc ^ (kk & 7)) << 4)) = o0;
-            *reinterpret_cast<uint4*>(dst + (((jc + 1) ^ (kk & 7)) << 4)) = o1;
-          }
-        } else if (PHASE == 1) {
-          // two tiles [128 rows][32 bytes = 64 codes]: a 16-byte chunk is one 32-element scale block
-          const uint8_t* rsc = raw + 2 * 128 * 32;
-#pragma unroll
-          for (int q = ct; q < 512; q += kCvThreads) {
-            const int tile = q >> 8, row = (q & 255) >> 1, half = q & 1;
-            const uint4 v = *reinterpret_cast<const uint4*>(raw + q * 16);
-            const uint32_t sc = rsc[tile * (128 * 16) + row * 16 + ((kt * 2) & 15) + half];
-            uint8_t* dst = st + tile * (128 * 128) + row * 128;
-            const int jc = half * 4;
-            *reinterpret_cast<uint4*>(dst + (((jc + 0) ^ (row & 7)) << 4)) = e2m1x8_to_bf16(v.x, sc);
-            *reinterpret_cast<uint4*>(dst + (((jc + 1) ^ (row & 7)) << 4)) = e2m1x8_to_bf16(v.y, sc);
-            *reinterpret_cast<uint4*>(dst + (((jc + 2) ^ (row & 7)) << 4)) = e2m1x8_to_bf16(v.z, sc);
-            *reinterpret_cast<uint4*>(dst + (((jc + 3) ^ (row & 7)) << 4)) = e2m1x8_to_bf16(v.w, sc);
-          }
-        } else {
-          // [64 k-rows][64 bytes = 128 codes]: chunk cb of a row is the scale block of columns 32 cb .. 32 cb + 31
-          const uint8_t* rsc = raw + 64 * 64;
-#pragma unroll
-          for (int q = ct; q < 256; q += kCvThreads) {
-            const int kk = q >> 2, cb = q & 3;
-            const uint4 v = *reinterpret_cast<const uint4*>(raw + q * 16);
-            const uint32_t sc = rsc[kk * 16 + ((blk * 4) & 15) + cb];
-            uint8_t* dst = st + (cb >> 1) * (64 * 128) + kk * 128;
-            const int jc = (cb & 1) * 4;
-            *reinterpret_cast<uint4*>(dst + (((jc + 0) ^ (kk & 7)) << 4)) = e2m1x8_to_bf16(v.x, sc);
-            *reinterpret_cast<uint4*>(dst + (((jc + 1) ^ (kk & 7)) << 4)) = e2m1x8_to_bf16(v.y, sc);
-            *reinterpret_cast<uint4*>(dst + (((jc + 2) ^ (kk & 7)) << 4)) = e2m1x8_to_bf16(v.z, sc);
-            *reinterpret_cast<uint4*>(dst + (((jc + 3) ^ (kk & 7)) << 4)) = e2m1x8_to_bf16(v.w, sc);
+          if (kt + 1 == kt_end) {
+            umma_commit(&tmem_full[b0]);
+            if (wide) umma_commit(&tmem_full[1]);
           }
         }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the MMAs read these tiles through the async proxy
         __syncwarp();
-        if (lane == 0) mbar_arrive(&full[s]);
-        if (ct == 0) CVTL(PHASE, it_cv, 3);
       }
-      if (!ok && lane == 0) atomicExch(&s_abort, 1);
-    } else {
-      // ================= epilogue: warp w owns TMEM lanes 32*(w%4) .. +31
-      const int quad = warp & 3;
-      const int row = quad * 32 + lane;  // row of the 128-row tile
-      const uint32_t buf = unit_no & 1u;
-      if (__all_sync(0xffffffffu, mbar_wait(&tmem_full[buf], (unit_no >> 1) & 1, &s_abort, p.f.wait_limit_ns))) {
-        tc_fence_after();
-        if (warp == kMmaWarp + 1 && lane == 0) TCTL(PHASE, unit_no * 16 + 12);
-        for (int c0 = 0; c0 < gr.n_tok; c0 += 32) {
-          uint32_t a[32];
-          const uint32_t taddr = tmem_base + buf * 256u + ((uint32_t)(quad * 32) << 16) + (uint32_t)c0;
-          tmem_ld32(taddr, a);
-          uint32_t b2[32];
-          tmem_ld32(taddr + (PHASE == 1 ? 128 : n_pad), b2);   // U | the a_lo half of the down product
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          if (PHASE == 1) {
-            const int i = blk * 128 + row;
-            float sg = 1.f, su = 1.f, sd = 1.f;
-            if (QF == 1) {  // the row's three fp32 scales follow its 3 d code bytes
-              const uint8_t* wb = shared ? p.f.shared_w : p.f.cache + (size_t)p.f.snap.expert_slot[gr.expert] * p.f.slot_stride;
-              const float* sc = reinterpret_cast<const float*>(wb + (size_t)i * (3u * d + 16u) + 3u * d);
-              sg = __ldg(sc);
-              su = __ldg(sc + 1);
-              sd = __ldg(sc + 2);
-            }
+      if (lane == 0) TCTL(n, 2);
+    }
+    if (!ok && lane == 0) atomicExch(&s_abort, 1);
+  } else if (QF != 0 && warp >= kCvWarp0) {
+    // ================= converters: the codes of a raw tile -> bf16 operand tiles of its SUB stages.  Gate and up go to
+    // TMEM (lane = row, as the codes lie): a shared-memory tile is written once and read by its MMAs once at 128 bytes per
+    // cycle, 500 cycles of a stage, and an MMA with A in TMEM takes N / 2 cycles where one from shared memory takes 40 at
+    // least.  downT, whose rows are K, goes to shared memory in the 128-byte-swizzled layout (a tile row is 128 bytes = 64
+    // values; its 16-byte chunk j sits at chunk j ^ (row mod 8)).  The raw tile has the same swizzle.  A lane owns a row, so
+    // the eight lanes of an access phase touch eight different chunks.
+    const int ct = tid - kCvWarp0 * 32;
+    RingPos rp, rr;  // stages, raw tiles
+    for (uint32_t n = 0; ok; ++n) {
+      const UnitDesc ud = next_unit(n);
+      if (ud.phase == 0) break;
+      for (int kt = ud.kt_begin; kt < ud.kt_end && ok; kt += SUB, rr.next(NR)) {
+        const uint32_t r = rr.s;
+        ok = __all_sync(0xffffffffu, mbar_wait(&rawfull[r], rr.parity, &s_abort, p.f.wait_limit_ns));
+        if (!ok) break;
+        const uint8_t* raw = raw_ring + r * RAW_BYTES;
+        // gate/up: tile (gate, up), row and 32-value half of the stage; down: K row of the stage and group of 32 columns
+        // (a warp reaches the TMEM lanes of its quarter only: warp mod 4)
+        const int t1 = (ct >> 7) & 1, row1 = (warp & 3) * 32 + lane, hf = ct >> 8, kk = ct & 63, og = ct >> 6;
+        uint2 sc1 = make_uint2(0u, 0u);
+        if (QF == 2 && ud.phase == 1) sc1 = *reinterpret_cast<const uint2*>(raw + 32768 + t1 * 2048 + row1 * 16 + ((kt * 2) & 15));
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              if (c0 + j < gr.n_tok) {
-                const float gq = sg * __uint_as_float(a[j]), uq = su * __uint_as_float(b2[j]);
-                const float w = __ldg(p.f.pair_gate + gr.pair_off + c0 + j);
-                const float v = w * (gq / (1.f + expf(-gq))) * uq * sd;
-                const __nv_bfloat16 hi = __float2bfloat16(v);
-                const size_t at = (size_t)(gr.pair_off + c0 + j) * p.act_stride + i;
-                p.act[at] = hi;
-                p.act[p.act_plane + at] = __float2bfloat16(v - __bfloat162float(hi));
+        for (int sub = 0; sub < SUB; ++sub) {
+          if (kt + sub >= ud.kt_end) break;
+          const uint32_t s = rp.s;
+          ok = __all_sync(0xffffffffu, mbar_wait(&empty[s], rp.parity ^ 1, &s_abort, p.f.wait_limit_ns));
+          if (!ok) break;
+          tc_fence_after();  // (the MMAs that read this stage's tiles before have completed)
+          uint8_t* st = smem + s * STAGE_BYTES;
+          if (ud.phase == 1) {
+            const uint8_t* src = raw + t1 * 16384 + row1 * 128;
+            const int x = row1 & 7;
+            uint4 o[4];
+            if (QF == 1) {
+#pragma unroll
+              for (int cc = 0; cc < 2; ++cc) {
+                const uint4 v = *reinterpret_cast<const uint4*>(src + (((4 * sub + 2 * hf + cc) ^ x) << 4));
+                e4m3x4_to_bf16(p.shifts, v.x, o[2 * cc].x, o[2 * cc].y);
+                e4m3x4_to_bf16(p.shifts, v.y, o[2 * cc].z, o[2 * cc].w);
+                e4m3x4_to_bf16(p.shifts, v.z, o[2 * cc + 1].x, o[2 * cc + 1].y);
+                e4m3x4_to_bf16(p.shifts, v.w, o[2 * cc + 1].z, o[2 * cc + 1].w);
               }
+            } else {
+              const uint4 v = *reinterpret_cast<const uint4*>(src + (((2 * sub + hf) ^ x) << 4));  // 32 codes: one scale block
+              e2m1x32_to_bf16(p.shifts, v, ((sub < 2 ? sc1.x : sc1.y) >> (8 * (2 * (sub & 1) + hf))) & 0xffu, o);
             }
+            tmem_st16(tmem_base + kTmemA + s * 64u + t1 * 32 + hf * 16 + ((uint32_t)((warp & 3) * 32) << 16), reinterpret_cast<const uint32_t*>(o));
+            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+            tc_fence_before();
           } else {
-            const int col = blk * 128 + row;
+            const int x = kk & 7;
+            uint8_t* dst = st + (og >> 1) * (64 * 128) + kk * 128;
+            if (QF == 1) {
+              const uint8_t* src = raw + (og >> 2) * 16384 + (sub * 64 + kk) * 128;
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              if (c0 + j < gr.n_tok) {
-                const int t = __ldg(p.f.pair_tok + gr.pair_off + c0 + j);
-                atomicAdd(p.f.y + (size_t)t * d + col, __uint_as_float(a[j]) + __uint_as_float(b2[j]));
+              for (int cc = 0; cc < 2; ++cc) {
+                const int c = (og & 1) * 2 + cc;
+                const uint4 v = *reinterpret_cast<const uint4*>(src + (((((og >> 1) & 1) * 4 + c) ^ x) << 4));
+                uint4 o0, o1;
+                e4m3x4_to_bf16(p.shifts, v.x, o0.x, o0.y);
+                e4m3x4_to_bf16(p.shifts, v.y, o0.z, o0.w);
+                e4m3x4_to_bf16(p.shifts, v.z, o1.x, o1.y);
+                e4m3x4_to_bf16(p.shifts, v.w, o1.z, o1.w);
+                *reinterpret_cast<uint4*>(dst + (((2 * c) ^ x) << 4)) = o0;
+                *reinterpret_cast<uint4*>(dst + (((2 * c + 1) ^ x) << 4)) = o1;
+              }
+            } else {
+              const uint8_t* src = raw + (sub * 64 + kk) * 128;
+              const uint4 v = *reinterpret_cast<const uint4*>(src + ((og ^ x) << 4));
+              const int c = og & 1;
+              uint4 o[4];
+              e2m1x32_to_bf16(p.shifts, v, raw[32768 + (sub * 64 + kk) * 16 + ((ud.blk * 8) & 15) + og], o);
+#pragma unroll
+              for (int j = 0; j < 4; ++j) *reinterpret_cast<uint4*>(dst + (((4 * c + j) ^ x) << 4)) = o[j];
+            }
+          }
+          if (ud.phase == 2) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the MMAs read these tiles through the async proxy
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&full[s]);
+          rp.next(NS);
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&rawempty[r]);
+      }
+    }
+    if (!ok && lane == 0) atomicExch(&s_abort, 1);
+  } else {
+    // ================= epilogue: warp w owns TMEM lanes 32*(w%4) .. +31
+    if (warp == kEpiWarp0 && blockIdx.x == 0 && lane == 0 && p.f.post_exec) {
+      // the unions of the routed and of the execution sets for the host: one 16-byte store each, with the sequence number
+      const unsigned long long kr = p.plan_masks[0], ex = p.plan_masks[1];
+      asm volatile("st.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p.f.mbox_rec), "r"((uint32_t)kr), "r"((uint32_t)(kr >> 32)), "r"(p.f.seq_value), "r"(0u) : "memory");
+      asm volatile("st.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p.f.mbox_rec + 4), "r"((uint32_t)ex), "r"((uint32_t)(ex >> 32)), "r"(p.f.seq_value), "r"(0u) : "memory");
+    }
+    const int quad = warp & 3;
+    const int row = quad * 32 + lane;  // row of the 128-row tile
+    AccBuffers acc;
+    for (uint32_t n = 0;; ++n) {
+      const UnitDesc ud = next_unit(n);
+      if (ud.phase == 0) break;
+      const bool shared = ud.expert >= N;
+      const bool wide = unit_is_wide<QF>(ud);
+      const uint32_t b0 = wide ? 0u : acc.next, b1 = wide ? 1u : acc.next;
+      // the pairs' weights, sixteen at a time, asked for before the wait and then one batch ahead
+      auto load_gates = [&](int c0) { return ud.phase == 1 && c0 + (lane & 15) < ud.n_tok ? __ldg(p.f.pair_gate + ud.pair_off + c0 + (lane & 15)) : 0.f; };
+      float gates_next = load_gates(0);
+      bool landed = true;
+      for (uint32_t b = b0; b <= b1; ++b) landed = landed && mbar_wait(&tmem_full[b], acc.uses[b]++ & 1, &s_abort, p.f.wait_limit_ns);
+      if (!wide) acc.next ^= 1u;
+      if (!__all_sync(0xffffffffu, landed)) break;
+      auto release = [&]() {
+        tc_fence_before();
+        for (uint32_t b = b0; b <= b1; ++b) mbar_arrive(&tmem_empty[b]);
+      };
+      const uint32_t second = QF != 0 && !wide ? 64u : 128u;
+      tc_fence_after();
+      if (warp == kEpiWarp0 && lane == 0) TCTL(n, 3);
+      const uint32_t tacc = tmem_base + b0 * tc_acc_cols(QF) + ((uint32_t)(quad * 32) << 16);
+      if (ud.phase == 1) {
+        const int i = ud.blk * 128 + row;
+        const bool row_ok = i < (shared ? I_s : I);
+        float sg = 1.f, su = 1.f, sd = 1.f;
+        if (QF == 1 && row_ok) {  // the row's three fp32 scales follow its 3 d code bytes
+          const uint8_t* wb = shared ? p.f.shared_w : p.f.cache + (size_t)p.f.snap.expert_slot[ud.expert] * p.f.slot_stride;
+          const float* sc = reinterpret_cast<const float*>(wb + (size_t)i * (3u * d + 16u) + 3u * d);
+          sg = __ldg(sc);
+          su = __ldg(sc + 1);
+          sd = __ldg(sc + 2);
+        }
+        for (int c0 = 0; c0 < ud.n_tok; c0 += 16) {
+          uint32_t a[16], b2[16];
+          tmem_ld16(tacc + (uint32_t)c0, a);
+          tmem_ld16(tacc + second + (uint32_t)c0, b2);
+          const float gates = gates_next;
+          gates_next = load_gates(c0 + 16);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          __nv_bfloat16* dst = p.act + (size_t)(ud.pair_off + c0) * p.act_stride + i;
+          float v[16];
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {  // (no branches: sixteen independent chains; columns past the last token are not stored)
+            const float gq = sg * __uint_as_float(a[j]), uq = su * __uint_as_float(b2[j]);
+            v[j] = __shfl_sync(0xffffffffu, gates, j) * (gq / (1.f + expf(-gq))) * uq * sd;
+          }
+          if (row_ok) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              if (c0 + j < ud.n_tok) {
+                const __nv_bfloat16 hi = __float2bfloat16(v[j]);
+                dst[(size_t)j * p.act_stride] = hi;
+                dst[(size_t)j * p.act_stride + p.act_plane] = __float2bfloat16(v[j] - __bfloat162float(hi));
               }
             }
           }
         }
+        release();
+        // count the unit in: the stores of the four warps, ordered before another CTA's bulk loads of the intermediate
+        // (the proxy fence stands on the reading side, behind the acquire)
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        if (warp == kEpiWarp0 && lane == 0)
+          asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p.sync + kTcDone + ud.group), "r"(1u) : "memory");
+      } else {
+        const int n_pad = (ud.n_tok + 15) & ~15;
+        for (int half = 0; half < 2; ++half) {
+          float* ycol = p.f.y + ud.blk * 256 + half * 128 + tc_column_of(QF, row);
+          for (int c0 = 0; c0 < ud.n_tok; c0 += 16) {
+            uint32_t a[16], b2[16];
+            tmem_ld16(tacc + half * second + (uint32_t)c0, a);
+            tmem_ld16(tacc + half * second + (uint32_t)(n_pad + c0), b2);   // the a_lo half of the product
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+              if (c0 + j < ud.n_tok) atomicAdd(ycol + (size_t)s_tok[ud.pair_off + c0 + j] * d, __uint_as_float(a[j]) + __uint_as_float(b2[j]));
+          }
+        }
+        release();
       }
-      tc_fence_before();
-      if (warp == kMmaWarp + 1 && lane == 0) TCTL(PHASE, unit_no * 16 + 13);
-      mbar_arrive(&tmem_empty[unit_no & 1u]);
+      if (warp == kEpiWarp0 && lane == 0) TCTL(n, 4);
     }
-    ++unit_no;
-    if (*(volatile int*)&s_abort) break;
-  }
-    __syncthreads();  // every role is done with this chunk's descriptors (after an abort the later chunks fall through)
   }
   tc_fence_before();
   __syncthreads();
+  if (*(volatile int*)&s_abort) {
+    // after an abort copies and MMAs may still be under way (everything they touch is this GPU's own memory: microseconds)
+    const unsigned long long t0 = globaltimer_ns();
+    while (globaltimer_ns() - t0 < 1000000ull) __nanosleep(1000);
+    __syncthreads();
+  }
   if (warp == kMmaWarp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
-  SPAN_END(PHASE == 1 ? 8 : 9);
+  SPAN_END(8);
 }
 
 #ifdef APEX_TIMELINE
 extern "C" int apex_debug_read_tc_timeline(unsigned long long* host) {
   return (int)cudaMemcpyFromSymbol(host, g_tc_tl, sizeof(g_tc_tl));
-}
-extern "C" int apex_debug_read_tc_converter_timeline(unsigned long long* host) {
-  return (int)cudaMemcpyFromSymbol(host, g_cv_tl, sizeof(g_cv_tl));
 }
 #endif
 
@@ -705,134 +875,98 @@ static EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// Weights of n_slots consecutive slots, each [I][3][d] bf16: dims (d, 3, I, n_slots); box (64, 1, box_rows, 1).
-bool tc_make_weight_map(void* out, const void* base, int d, int I, size_t n_slots, size_t slot_bytes, int box_rows) {
+static bool encode(void* out, CUtensorMapDataType type, int rank, const void* base, const cuuint64_t* dims, const cuuint64_t* strides,
+                   const cuuint32_t* box, CUtensorMapSwizzle swizzle) {
   EncodeTiledFn fn = encode_fn();
-  if (!fn) return false;
-  cuuint64_t dims[4] = {(cuuint64_t)d, 3, (cuuint64_t)I, (cuuint64_t)n_slots};
-  cuuint64_t strides[3] = {(cuuint64_t)d * 2, (cuuint64_t)d * 6, (cuuint64_t)slot_bytes};
-  cuuint32_t box[4] = {64, 1, (cuuint32_t)box_rows, 1};
-  cuuint32_t es[4] = {1, 1, 1, 1};
-  return fn(reinterpret_cast<CUtensorMap*>(out), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, es,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  const cuuint32_t es[4] = {1, 1, 1, 1};
+  return fn && fn(reinterpret_cast<CUtensorMap*>(out), type, rank, const_cast<void*>(base), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Row-major bf16 matrix [rows][cols] with row stride `stride_elems`: dims (cols, rows); box (64, 32).
-bool tc_make_rows_map(void* out, const void* base, int cols, size_t rows, size_t stride_elems) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn) return false;
-  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)stride_elems * 2};
-  cuuint32_t box[2] = {64, kXRowsPerLoad};
-  cuuint32_t es[2] = {1, 1};
-  return fn(reinterpret_cast<CUtensorMap*>(out), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, es,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+// Row-major bf16 matrix [rows][cols] with row stride `stride_elems`; boxes of 64 columns and `box_rows` rows.
+static bool rows_map(void* out, const void* base, int cols, size_t rows, size_t stride_elems, int box_rows) {
+  const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows}, strides[1] = {(cuuint64_t)stride_elems * 2};
+  const cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
+  return encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
-// Raw bytes of n_slots consecutive slots of a quantised store, each [I][row_bytes]: dims (row_bytes, I, n_slots);
-// box (box_bytes, box_rows, 1), no swizzle (the converters read the staging area with plain loads).
-bool tc_make_raw_map(void* out, const void* base, size_t row_bytes, int I, size_t n_slots, size_t slot_bytes, int box_bytes, int box_rows) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn) return false;
-  cuuint64_t dims[3] = {(cuuint64_t)row_bytes, (cuuint64_t)I, (cuuint64_t)n_slots};
-  cuuint64_t strides[2] = {(cuuint64_t)row_bytes, (cuuint64_t)slot_bytes};
-  cuuint32_t box[3] = {(cuuint32_t)box_bytes, (cuuint32_t)box_rows, 1};
-  cuuint32_t es[3] = {1, 1, 1};
-  return fn(reinterpret_cast<CUtensorMap*>(out), CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<void*>(base), dims, strides, box, es,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+bool tc_make_activation_maps(TcMaps* m, const void* xb, int d, int max_batch, const void* act, size_t act_rows, int act_stride) {
+  return rows_map(m->x, xb, d, max_batch, d, 1) && rows_map(m->xc, xb, d, max_batch, d, kARowsPerLoad) && rows_map(m->act, act, act_stride, 2 * act_rows, act_stride, kARowsPerLoad);
 }
 
-// The weight maps of one store (the slots of all layers, or one shared expert) for the storage format.
-bool tc_make_store_maps(int fmt, void* gateup, void* down, void* sc_gateup, void* sc_down, const void* base, int d, int I, size_t n_slots,
-                        size_t slot_bytes) {
-  if (fmt == 0)
-    return tc_make_weight_map(gateup, base, d, I, n_slots, slot_bytes, 128) && tc_make_weight_map(down, base, d, I, n_slots, slot_bytes, 64);
-  const size_t rb = ffn_row_bytes(fmt, d);
-  if (fmt == 1)  // a K tile of 64 codes is 64 bytes of a gate / up row; 128 columns of a downT row are 128 bytes
-    return tc_make_raw_map(gateup, base, rb, I, n_slots, slot_bytes, 64, 128) && tc_make_raw_map(down, base, rb, I, n_slots, slot_bytes, 128, 64);
-  return tc_make_raw_map(gateup, base, rb, I, n_slots, slot_bytes, 32, 128) && tc_make_raw_map(down, base, rb, I, n_slots, slot_bytes, 64, 64) &&
-         tc_make_raw_map(sc_gateup, base, rb, I, n_slots, slot_bytes, 16, 128) && tc_make_raw_map(sc_down, base, rb, I, n_slots, slot_bytes, 16, 64);
-}
-
-bool tc_shape_supported(int d, int I, int I_shared, int fmt) {
-  if (d % 128 != 0 || I % 128 != 0 || I_shared % 128 != 0) return false;
-  if (fmt == 1) return d % 256 == 0;   // code offsets of a row stay 16-byte aligned
-  if (fmt == 2) return d % 512 == 0;   // ... and so do the scale bytes of each vector (d / 32 of them)
-  return true;
+// The weight maps of one store (the slots of all layers, or one shared expert): n_slots consecutive slots of I rows.  Rows
+// past I (the last tile of an I that is not a multiple of the tile) read as zero.
+bool tc_make_store_maps(int fmt, void* weights, void* scales, const void* base, int d, int I, size_t n_slots, size_t slot_bytes) {
+  if (fmt == 0) {  // [I][3][d] bf16
+    const cuuint64_t dims[4] = {(cuuint64_t)d, 3, (cuuint64_t)I, (cuuint64_t)n_slots};
+    const cuuint64_t strides[3] = {(cuuint64_t)d * 2, (cuuint64_t)d * 6, (cuuint64_t)slot_bytes};
+    const cuuint32_t box[4] = {64, 1, 64, 1};
+    return encode(weights, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
+  }
+  const size_t rb = ffn_row_bytes(fmt, d);  // raw bytes [I][row bytes]
+  const cuuint64_t dims[3] = {(cuuint64_t)rb, (cuuint64_t)I, (cuuint64_t)n_slots};
+  const cuuint64_t strides[2] = {(cuuint64_t)rb, (cuuint64_t)slot_bytes};
+  const cuuint32_t box[3] = {128, 128, 1}, sbox[3] = {16, 128, 1};
+  return encode(weights, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B) &&
+         encode(scales, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, base, dims, strides, sbox, CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
 namespace {
+constexpr int kTcSmemBudget = 216 * 1024;  // rings of a CTA, 1 KB of alignment included
+
 template <int QF>
-cudaError_t launch_tc_gemms(const TcParams& p, const TcMaps& m, cudaLaunchConfig_t& cfg, size_t ring1, size_t ring2, size_t st1, size_t st2) {
-  const CUtensorMap* w1 = reinterpret_cast<const CUtensorMap*>(m.w_gateup);
-  const CUtensorMap* ws1 = reinterpret_cast<const CUtensorMap*>(p.f.shared_w ? m.ws_gateup : m.w_gateup);
-  const CUtensorMap* w2 = reinterpret_cast<const CUtensorMap*>(m.w_down);
-  const CUtensorMap* ws2 = reinterpret_cast<const CUtensorMap*>(p.f.shared_w ? m.ws_down : m.w_down);
-  // the 16-byte-box maps exist for the e2m1 store only; the other formats pass the weight maps again (never used)
-  const CUtensorMap* c1 = QF == 2 ? reinterpret_cast<const CUtensorMap*>(m.sc_gateup) : w1;
-  const CUtensorMap* cs1 = QF == 2 ? reinterpret_cast<const CUtensorMap*>(p.f.shared_w ? m.ssc_gateup : m.sc_gateup) : w1;
-  const CUtensorMap* c2 = QF == 2 ? reinterpret_cast<const CUtensorMap*>(m.sc_down) : w2;
-  const CUtensorMap* cs2 = QF == 2 ? reinterpret_cast<const CUtensorMap*>(p.f.shared_w ? m.ssc_down : m.sc_down) : w2;
-  const CUtensorMap* xg = reinterpret_cast<const CUtensorMap*>(m.xg);
+cudaError_t launch_tc(const TcParams& p, const TcMaps& m, cudaLaunchConfig_t& cfg) {
+  static bool configured[kMaxDevices] = {};  // the attribute is per device
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev < 0 || dev >= kMaxDevices || !configured[dev]) {
+    cudaError_t e = cudaFuncSetAttribute(ffn_tc_kernel<QF>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemBudget);
+    if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < kMaxDevices) configured[dev] = true;
+  }
+  const CUtensorMap* w = reinterpret_cast<const CUtensorMap*>(m.w);
+  const CUtensorMap* ws = reinterpret_cast<const CUtensorMap*>(p.f.shared_w ? m.ws : m.w);
+  // the 16-byte-box maps are used for the e2m1 store only; bf16 passes the weight maps again
+  const CUtensorMap* sc = QF ? reinterpret_cast<const CUtensorMap*>(m.sc) : w;
+  const CUtensorMap* ssc = QF ? reinterpret_cast<const CUtensorMap*>(p.f.shared_w ? m.ssc : m.sc) : w;
   cfg.blockDim = dim3(tc_threads(QF), 1, 1);
-  // Each CTA allocates all 512 TMEM columns, so two CTAs must never share an SM (the second would sit in
-  // tcgen05.alloc until the first has finished): ask for more than half an SM's shared memory in any case.
-  const size_t one_per_sm = 120 * 1024;
-  cfg.dynamicSmemBytes = ring1 + p.nstage1 * st1 + 1024 > one_per_sm ? ring1 + p.nstage1 * st1 + 1024 : one_per_sm;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, ffn_tc_gemm_kernel<1, QF>, *w1, *ws1, *c1, *cs1, *xg, *xg, p);
-  if (e != cudaSuccess) return e;
-  cfg.dynamicSmemBytes = ring2 + p.nstage2 * st2 + 1024 > one_per_sm ? ring2 + p.nstage2 * st2 + 1024 : one_per_sm;
-  return cudaLaunchKernelEx(&cfg, ffn_tc_gemm_kernel<2, QF>, *w2, *ws2, *c2, *cs2, *reinterpret_cast<const CUtensorMap*>(m.act),
-                            *reinterpret_cast<const CUtensorMap*>(m.act_lo), p);
-}
-template <int QF>
-cudaError_t configure_tc(int budget) {
-  cudaError_t e = cudaFuncSetAttribute(ffn_tc_gemm_kernel<1, QF>, cudaFuncAttributeMaxDynamicSharedMemorySize, budget);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(ffn_tc_gemm_kernel<2, QF>, cudaFuncAttributeMaxDynamicSharedMemorySize, budget);
+  return cudaLaunchKernelEx(&cfg, ffn_tc_kernel<QF>, *w, *ws, *sc, *ssc, *reinterpret_cast<const CUtensorMap*>(m.x), *reinterpret_cast<const CUtensorMap*>(m.xc),
+                            *reinterpret_cast<const CUtensorMap*>(m.act), p);
 }
 }  // namespace
 
 cudaError_t launch_ffn_tc(const TcParams& p_in, const TcMaps& m, int n_sm, cudaStream_t s) {
-  static bool configured[kMaxDevices] = {};  // the attribute is per device
-  const size_t budget = 196 * 1024;  // ring bytes per CTA
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev < 0 || dev >= kMaxDevices || !configured[dev]) {
-    cudaError_t e = configure_tc<0>((int)budget + 1024);
-    if (e == cudaSuccess) e = configure_tc<1>((int)budget + 1024);
-    if (e == cudaSuccess) e = configure_tc<2>((int)budget + 1024);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < kMaxDevices) configured[dev] = true;
-  }
   TcParams p = p_in;
+  p.shifts = TcShifts{1u << 2, 1u << 4, 1u << 6, 1u << 8, 1u << 12};
   const int qf = p.f.fmt;
-  const int b32 = (p.f.B + 31) & ~31;
-  p.nmax1 = b32 < 128 ? b32 : 128;
-  p.nmax2 = b32 < 64 ? b32 : 64;
-  const size_t ring1 = 0, ring2 = 0;
-  const size_t st1 = 2 * 128 * 128 + (size_t)p.nmax1 * 128 + tc_raw_bytes(1, qf);
-  const size_t st2 = tc_tiles_per_stage(2, qf) * (2 * 64 * 128 + 2 * (size_t)p.nmax2 * 128) + tc_raw_bytes(2, qf);
-  p.nstage1 = (int)(budget / st1) < 4 ? (int)(budget / st1) : 4;
-  p.nstage2 = (int)(budget / st2) < 4 ? (int)(budget / st2) : 4;
+  // Tokens per unit: up to 128 (gate/up), 64 (down: both planes of the intermediate share an MMA).  Small batches leave
+  // the activations' share of a stage small and get deeper rings.
+  const int b16 = (p.f.B + 15) & ~15;
+  p.nmax1 = b16 < 128 ? b16 : 128;
+  p.nmax2 = b16 < 64 ? b16 : 64;
+  const int b_bytes = p.nmax1 * 128 > 2 * p.nmax2 * 128 ? p.nmax1 * 128 : 2 * p.nmax2 * 128;
+  p.stage_bytes = kABytes + ((b_bytes + 1023) & ~1023);
+  const int budget = kTcSmemBudget - 1024;
+  if (qf == 0) {
+    p.nraw = 0;
+    p.nstage = budget / p.stage_bytes < kMaxStages ? budget / p.stage_bytes : kMaxStages;
+  } else {  // two operand stages; the raw ring, which covers the HBM latency, gets the rest
+    p.nstage = 2;
+    const int left = (budget - p.nstage * p.stage_bytes) / tc_raw_bytes(qf);
+    p.nraw = left < kMaxRaw ? left : kMaxRaw;
+  }
   cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // prologues overlap the preceding kernel's tail
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // the prologue overlaps the preceding kernel's tail
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cfg.gridDim = dim3(n_sm * 2, 1, 1);
-  cfg.blockDim = dim3(256, 1, 1);
-  cfg.dynamicSmemBytes = 0;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, ffn_tc_gather_kernel, p);
-  if (e != cudaSuccess) return e;
   cfg.gridDim = dim3(n_sm, 1, 1);
-  return qf == 1 ? launch_tc_gemms<1>(p, m, cfg, ring1, ring2, st1, st2)
-                 : qf == 2 ? launch_tc_gemms<2>(p, m, cfg, ring1, ring2, st1, st2) : launch_tc_gemms<0>(p, m, cfg, ring1, ring2, st1, st2);
+  // Each CTA allocates all 512 TMEM columns, so two CTAs must never share an SM (the second would sit in
+  // tcgen05.alloc until the first has finished): the rings take more than half an SM's shared memory in any case.
+  cfg.dynamicSmemBytes = (size_t)p.nstage * p.stage_bytes + (size_t)p.nraw * tc_raw_bytes(qf) + 1024;
+  return qf == 1 ? launch_tc<1>(p, m, cfg) : qf == 2 ? launch_tc<2>(p, m, cfg) : launch_tc<0>(p, m, cfg);
 }
 
 }  // namespace apex

@@ -1,114 +1,111 @@
-// ffn_plan_kernel: the execution sets of a batched step (B > 1) and the (expert, token) pair list sorted by expert,
-// for the tensor-core grouped GEMMs and for the per-pair streaming kernel.
+// ffn_plan_kernel: the execution sets of a batched step (B > 1), the (expert, token) pair list sorted by expert for the
+// tensor-core grouped GEMM, and the rest of that kernel's preparation.
 #include <cooperative_groups.h>
 
 #include "apex_internal.hpp"
 #include "ptx.cuh"
-#include "timeline.cuh"
 #include "token_plan.cuh"
 
 namespace cg = cooperative_groups;
 
 namespace apex {
 
-// ---------------------------------------------------------------- batched plan (B > 1)
-// A cluster of ceil(B / 32) CTAs (at most 8) of 32 warps.  Phase A: every warp of the cluster plans one token (planning
-// a token costs a warp 2-3 us of dependent latency, so eight tokens per warp on one SM were 16 us at B = 256) and puts
-// its execution mask and gates into the leader CTA's shared memory through distributed shared memory.  Phase B, leader
+// Clusters of ceil(B / 32) CTAs (at most 8) of 32 warps.  The first cluster plans.  Phase A: a warp per token (planning
+// a token costs a warp 2-3 us of dependent latency, so eight tokens per warp on one SM were 16 us at B = 256); its
+// execution mask and gates go into the leader CTA's shared memory through distributed shared memory.  Phase B, leader
 // CTA only: warp w owns experts w and w+32 and gathers the tokens that execute them with ballots, so the pair list is
 // sorted by (expert, token).  Shared-expert pairs (expert id N) follow.
+// The other clusters zero y and round h' to bf16 (the rows the GEMM gathers by token), so no kernel of its own does that.
+// Nothing here waits for the host link: the sets the host needs leave from the GEMM kernel (a system-scope fence at
+// this kernel's end was 2 us on the path of everything behind it).
 constexpr int kPlanMaxCtas = APEX_MAX_BATCH / 32;
 static_assert(kPlanMaxCtas <= 8, "one token per warp needs a cluster of at most 8 CTAs");
 
-#ifdef APEX_TIMELINE
-#define PTL(i) do { if (threadIdx.x == 0) g_timeline[1000 * 16 + (i)] = globaltimer_ns_raw(); } while (0)
-#else
-#define PTL(i) do { } while (0)
-#endif
-
 __global__ void __launch_bounds__(1024) ffn_plan_kernel(const FfnParams p) {
-  constexpr int TOK_PER_WARP = 1;
   cg::cluster_group cluster = cg::this_cluster();
   const unsigned crank = cluster.block_rank();
-  __shared__ unsigned long long s_exec[APEX_MAX_BATCH];
+  __shared__ unsigned long long s_exec[APEX_MAX_BATCH], s_kr[APEX_MAX_BATCH];
   __shared__ float s_pgate[APEX_MAX_BATCH][APEX_MAX_TOPK];  // gate of the j-th executed expert of each token
   __shared__ float s_sgate[APEX_MAX_BATCH];                 // weight of the shared expert for each token (gated variant)
   __shared__ int s_count[APEX_MAX_EXPERTS + 1];
   __shared__ int s_off[APEX_MAX_EXPERTS + 2];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
   const int N = p.N, k = p.k, B = p.B;
-  int my_subst = 0, my_hits = 0;
+  SPAN_BEGIN();
+  pdl_wait();               // the gate's outputs are complete, and nobody reads the previous step's plan any more
+  pdl_launch_dependents();
+  if (blockIdx.x >= cluster.num_blocks()) {  // helpers
+    const size_t n8 = (size_t)B * p.d / 8, stride = (size_t)(gridDim.x - cluster.num_blocks()) * blockDim.x;
+    float4* y4 = reinterpret_cast<float4*>(p.y);
+    const float4* h4 = reinterpret_cast<const float4*>(p.hpost);
+    auto pack = [](float a, float b) {
+      const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+      return *reinterpret_cast<const uint32_t*>(&v);
+    };
+    for (size_t i = (size_t)(blockIdx.x - cluster.num_blocks()) * blockDim.x + threadIdx.x; i < n8; i += stride) {
+      const float4 a = __ldg(h4 + 2 * i), b = __ldg(h4 + 2 * i + 1);
+      // in the order in which the GEMM's converters leave the weights (kernels_ffn_tc.cu)
+      uint4 o;
+      if (p.fmt == 2) o = make_uint4(pack(a.x, b.x), pack(a.y, b.y), pack(a.z, b.z), pack(a.w, b.w));
+      else if (p.fmt == 1) o = make_uint4(pack(a.x, a.z), pack(a.y, a.w), pack(b.x, b.z), pack(b.y, b.w));
+      else o = make_uint4(pack(a.x, a.y), pack(a.z, a.w), pack(b.x, b.y), pack(b.z, b.w));
+      reinterpret_cast<uint4*>(p.xb)[i] = o;
+      if (!p.accumulate) y4[2 * i] = y4[2 * i + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    return;
+  }
   // the leader's copies of the per-token results
   unsigned long long* l_exec = cluster.map_shared_rank(&s_exec[0], 0);
+  unsigned long long* l_kr = cluster.map_shared_rank(&s_kr[0], 0);
   float* l_pgate = cluster.map_shared_rank(&s_pgate[0][0], 0);
   float* l_sgate = cluster.map_shared_rank(&s_sgate[0], 0);
-  SPAN_BEGIN();
-  PTL(0);
-  TokenLoads tls[TOK_PER_WARP];
-#pragma unroll
-  for (int j = 0; j < TOK_PER_WARP; ++j) {
-    const int b = (int)crank * nwarp + warp + j * nwarp * (int)cluster.num_blocks();
-    if (b < B) tls[j] = load_token(p.idx + (size_t)b * k, p.z_r + (size_t)b * N, p.alpha + (size_t)b * N, N, k, p.mode, lane);
-  }
-#pragma unroll
-  for (int j = 0; j < TOK_PER_WARP; ++j) {
-    const int b = (int)crank * nwarp + warp + j * nwarp * (int)cluster.num_blocks();
-    if (b >= B) break;
-    const TokenLoads& tl = tls[j];
+  if (crank == 0)
+    for (int i = threadIdx.x; i < kTcSyncWords; i += (int)blockDim.x) p.tc_sync[i] = 0u;
+  const int b = (int)crank * nwarp + warp;
+  if (b < B) {
+    const TokenLoads tl = load_token(p.idx + (size_t)b * k, p.z_r + (size_t)b * N, p.alpha + (size_t)b * N, N, k, p.mode, lane);
     const TokenPlan tp = plan_token(tl, p.mode, p.norm_topk, p.snap.resident_mask, lane);
-    store_token_plan(tp, lane, k, p.plan_exec_idx + (size_t)b * k, p.plan_exec_gate + (size_t)b * k, nullptr);
-    if (p.post_exec) {
-      const int e0 = lane, e1 = lane + 32;
-      if ((tp.exec_mask >> e0) & 1) {
-        const int pos = __popcll(tp.exec_mask & ((1ull << e0) - 1ull));
-        if (p.exec_idx) p.exec_idx[(size_t)b * k + pos] = e0;
-        if (p.exec_gate) p.exec_gate[(size_t)b * k + pos] = tp.g0;
-      }
-      if ((tp.exec_mask >> e1) & 1) {
-        const int pos = __popcll(tp.exec_mask & ((1ull << e1) - 1ull));
-        if (p.exec_idx) p.exec_idx[(size_t)b * k + pos] = e1;
-        if (p.exec_gate) p.exec_gate[(size_t)b * k + pos] = tp.g1;
-      }
-      my_subst += __popcll(tp.exec_mask & ~tp.kr_mask);
-      my_hits += __popcll(tp.kr_mask & p.snap.resident_mask);
+    if (lane == 0) {
+      l_exec[b] = tp.exec_mask;
+      l_kr[b] = tp.kr_mask;
     }
-    if (lane == 0) l_exec[b] = tp.exec_mask;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int e = lane + 32 * h;
+      if ((tp.exec_mask >> e) & 1) {
+        const int pos = __popcll(tp.exec_mask & ((1ull << e) - 1ull));
+        const float g = h ? tp.g1 : tp.g0;
+        if (pos < APEX_MAX_TOPK) l_pgate[b * APEX_MAX_TOPK + pos] = g;
+        if (p.post_exec && p.exec_idx) p.exec_idx[(size_t)b * k + pos] = e;
+        if (p.post_exec && p.exec_gate) p.exec_gate[(size_t)b * k + pos] = g;
+      }
+    }
     if (p.run_shared && p.shared_gate) {
       const float sg = shared_gate_weight(p.shared_gate, p.hpost + (size_t)b * p.d, p.d, lane);
       if (lane == 0) l_sgate[b] = sg;
     }
-    {
-      const int e0 = lane, e1 = lane + 32;
-      if ((tp.exec_mask >> e0) & 1) {
-        const int pos = __popcll(tp.exec_mask & ((1ull << e0) - 1ull));
-        if (pos < APEX_MAX_TOPK) l_pgate[b * APEX_MAX_TOPK + pos] = tp.g0;
-      }
-      if ((tp.exec_mask >> e1) & 1) {
-        const int pos = __popcll(tp.exec_mask & ((1ull << e1) - 1ull));
-        if (pos < APEX_MAX_TOPK) l_pgate[b * APEX_MAX_TOPK + pos] = tp.g1;
-      }
+    if (p.post_exec && lane == 0 && p.stats) {
+      const int subst = __popcll(tp.exec_mask & ~tp.kr_mask), hits = __popcll(tp.kr_mask & p.snap.resident_mask);
+      if (subst) atomicAdd(&p.stats->substitutions, (unsigned long long)subst);
+      if (hits) atomicAdd(&p.stats->hits_R, (unsigned long long)hits);
     }
   }
-  if (p.post_exec && lane == 0 && my_subst && p.stats) atomicAdd(&p.stats->substitutions, (unsigned long long)my_subst);
-  if (p.post_exec && lane == 0 && my_hits && p.stats) atomicAdd(&p.stats->hits_R, (unsigned long long)my_hits);
   cluster.sync();  // every token's mask and gates are in the leader's shared memory
   if (crank != 0) return;
-  PTL(1);
   // ---- phase B, counts: warp w counts the tokens of experts w and w + 32
   for (int e = warp; e < N; e += nwarp) {
     int c = 0;
     if ((p.run_mask >> e) & 1)
       for (int b0 = 0; b0 < B; b0 += 32) {
-        const int b = b0 + lane;
-        c += __popc(__ballot_sync(0xffffffffu, b < B && ((s_exec[b] >> e) & 1)));
+        const int t = b0 + lane;
+        c += __popc(__ballot_sync(0xffffffffu, t < B && ((s_exec[t] >> e) & 1)));
       }
     if (lane == 0) s_count[e] = c;
   }
   __syncthreads();
-  PTL(2);
   if (warp == 0) {
-    // exclusive prefix over the experts (lane owns experts lane and lane + 32), then the group table
-    // of the tensor-core path: one group per executed expert, then the shared expert
+    // exclusive prefix over the experts (lane owns experts lane and lane + 32), then the group table: one group per
+    // executed expert, then the shared expert
     const int c0 = lane < N ? s_count[lane] : 0, c1 = lane + 32 < N ? s_count[lane + 32] : 0;
     int i0 = c0, i1 = c1;
 #pragma unroll
@@ -139,7 +136,6 @@ __global__ void __launch_bounds__(1024) ffn_plan_kernel(const FfnParams p) {
     }
     if (lane == 0) {
       s_off[N] = acc;  // routed pairs
-      p.n_pairs[0] = acc + (p.run_shared ? B : 0);
       p.grp[0] = ng_routed;
       if (p.run_shared) {
         p.grp[4 + 3 * ng_routed] = N;
@@ -148,74 +144,67 @@ __global__ void __launch_bounds__(1024) ffn_plan_kernel(const FfnParams p) {
       }
       p.grp[1] = ng_routed + (p.run_shared ? 1 : 0);
     }
+  } else if (warp == 1) {  // unions over the tokens
+    unsigned long long kr = 0ull, ex = 0ull;
+    for (int t = lane; t < B; t += 32) {
+      kr |= s_kr[t];
+      ex |= s_exec[t];
+    }
+    const unsigned kl = __reduce_or_sync(0xffffffffu, (unsigned)kr), kh = __reduce_or_sync(0xffffffffu, (unsigned)(kr >> 32));
+    const unsigned el = __reduce_or_sync(0xffffffffu, (unsigned)ex), eh = __reduce_or_sync(0xffffffffu, (unsigned)(ex >> 32));
+    if (lane == 0) {
+      p.plan_masks[0] = ((unsigned long long)kh << 32) | kl;
+      p.plan_masks[1] = ((unsigned long long)eh << 32) | el;
+    }
   }
   __syncthreads();
-  PTL(3);
   // ---- phase B, placement: token b of expert e goes to s_off[e] + (number of earlier tokens of e)
   for (int e = warp; e < N; e += nwarp) {
     if (s_count[e] == 0) continue;
     int o = s_off[e];
     for (int b0 = 0; b0 < B; b0 += 32) {
-      const int b = b0 + lane;
-      const bool has = b < B && ((s_exec[b] >> e) & 1);
+      const int t = b0 + lane;
+      const bool has = t < B && ((s_exec[t] >> e) & 1);
       const unsigned m = __ballot_sync(0xffffffffu, has);
       if (has) {
         const int at = o + __popc(m & ((1u << lane) - 1u));
-        const int pos = __popcll(s_exec[b] & ((1ull << e) - 1ull));
-        p.pair_tok[at] = b;
-        p.pair_expert[at] = e;
-        p.pair_gate[at] = s_pgate[b][pos];
+        p.pair_tok[at] = t;
+        p.pair_gate[at] = s_pgate[t][__popcll(s_exec[t] & ((1ull << e) - 1ull))];
       }
       o += __popc(m);
     }
   }
   if (p.run_shared) {
     const int base = s_off[N];
-    for (int b = threadIdx.x; b < B; b += blockDim.x) {
-      p.pair_tok[base + b] = b;
-      p.pair_expert[base + b] = N;
-      p.pair_gate[base + b] = p.shared_gate ? s_sgate[b] : 1.f;
+    for (int t = threadIdx.x; t < B; t += blockDim.x) {
+      p.pair_tok[base + t] = t;
+      p.pair_gate[base + t] = p.shared_gate ? s_sgate[t] : 1.f;
     }
   }
-  PTL(4);
-  // The routed and the execution sets go to the host mailbox last, as whole lines from consecutive
-  // threads (a 4-byte store per lane and token from inside the planning loop cost 2 us per token).
-  if (p.post_exec) {
-    for (int t = threadIdx.x; t < B * k; t += blockDim.x) {
-      const int b = t / k, j = t - b * k;
-      const unsigned long long m = s_exec[b];
-      p.mbox_exec[t] = j < __popcll(m) ? nth_set_bit64(m, j) : -1;
-      p.mbox_kr[t] = p.idx[t];
-    }
-  }
-  if (p.post_exec) {
-    // the barrier orders every thread's mailbox stores before thread 0's system-scope fence
-    // (fences are cumulative), which orders them before the sequence number
-    __syncthreads();
-    PTL(5);
-    if (threadIdx.x == 0) {
-      __threadfence_system();
-      *p.mbox_seq = p.seq_value;
-    }
-  }
-  PTL(6);
   SPAN_END(6);
 }
 
-cudaError_t launch_ffn_plan(const FfnParams& p, cudaStream_t s) {
+cudaError_t launch_ffn_plan(const FfnParams& p, int n_sm, cudaStream_t s) {
   int n_cta = (p.B + 31) / 32;
   n_cta = n_cta < 1 ? 1 : (n_cta > kPlanMaxCtas ? kPlanMaxCtas : n_cta);
+  // helpers: eight values per thread while the GPU has SMs for it
+  int helpers = ((int)((size_t)p.B * p.d / 8 + 1023) / 1024 + n_cta - 1) / n_cta;
+  const int most = n_sm / n_cta - 1;
+  helpers = helpers > most ? most : helpers;
+  helpers = helpers < 1 ? 1 : helpers;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(n_cta, 1, 1);
+  cfg.gridDim = dim3(n_cta * (1 + helpers), 1, 1);
   cfg.blockDim = dim3(1024, 1, 1);
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = n_cta;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, ffn_plan_kernel, p);
 }
 

@@ -73,6 +73,10 @@ class SlotTable {
         int e = cand[(size_t)b * stride + j];
         if (e >= 0 && e < N_) ++count[e];
       }
+    return plan_prefetch(count, copies, U_mask_out);
+  }
+  // The same from the number of tokens that want each expert.
+  bool plan_prefetch(const int* count, std::vector<SlotCopy>* copies, uint64_t* U_mask_out = nullptr) {
     std::vector<int> wanted;
     for (int e = 0; e < N_; ++e)
       if (count[e] > 0) wanted.push_back(e);
@@ -96,6 +100,10 @@ class SlotTable {
     for (int i = 0; i < B * k; ++i)
       if (K_r[i] >= 0 && K_r[i] < N_) need |= (1ull << K_r[i]);
     if (need_mask_out) *need_mask_out = need;
+    return plan_demand(need, copies);
+  }
+  // The same from the union of the routed sets.
+  bool plan_demand(uint64_t need, std::vector<SlotCopy>* copies) {
     std::vector<int> missing;
     for (int e = 0; e < N_; ++e) {
       if (!((need >> e) & 1)) continue;

@@ -239,6 +239,32 @@ def test_fp8_store_of_subnormal_codes(B):
     assert rep.ffn_checked == 2 * B and rep.near_ties == 0
 
 
+@pytest.mark.parametrize("fmt", ["bf16", "fp8", "fp4"])
+@pytest.mark.parametrize("N,k,I,I_shared,B", [(4, 2, 72, 200, 2), (5, 2, 200, 0, 31), (3, 1, 130, 72, 130), (2, 2, 1100, 64, 256)])
+def test_grouped_gemm_tile_edges(fmt, N, k, I, I_shared, B):
+    """Intermediate sizes off the 64- and 128-row tiles (the rest reads as zero), one and several chunks of K in the down
+    projection, and groups of 2 to 256 tokens: one part or several, and on the quantised stores both accumulator layouts."""
+    cfg = synth.tiny_config(d=512, N=N, k=k, I=I, C=N, T=2, I_shared=I_shared, sigma_p=1.0, cfg_id=279)
+    run = {"bf16": _run, "fp8": _run_fp8, "fp4": _run_fp4}[fmt]
+    rep, stats = run(cfg, mode="exact", tau=0.8, T=2, B=B, ffn_token_stride=max(1, B // 16))
+    assert stats["tokens"] == 2 * B and rep.near_ties == 0
+
+
+def test_fp4_store_of_large_block_scales():
+    # block scales above 2 (up) and tiny ones (down), which the converters apply in two multiplications: the factors cancel
+    hz = _harness()
+    cfg = synth.tiny_config(d=512, N=6, k=2, I=128, C=6, T=2, sigma_p=1.0, cfg_id=281)
+    prob = hz.Problem(cfg, fp4=True)
+    o = 3 * (cfg.d // 2)
+    for st in prob.stores:
+        up, down = st[..., o + cfg.d // 32:o + 2 * (cfg.d // 32)], st[..., o + 2 * (cfg.d // 32):o + 3 * (cfg.d // 32)]
+        up[up > 0] += 14
+        down[down > 0] -= 14
+        assert int(up.max()) > 128
+    rep, stats = _run(cfg, mode="exact", tau=0.8, T=2, B=24, prob=prob)
+    assert rep.ffn_checked == 48 and rep.near_ties == 0
+
+
 @pytest.mark.parametrize("fmt", ["fp8", "fp4"])
 def test_quantised_store_tensor_core_path_wide(fmt):
     # d = 1024: sixteen K tiles, so the e2m1 scale bytes of a gate / up row span two 16-byte groups; 8 column blocks in
