@@ -148,10 +148,9 @@ int apex_create(const apex_config* cfg, apex_ctx** out) {
   MailboxLayout& ml = ctx->ml;
   size_t off = sizeof(MailboxHeader);
   off = (off + 15) & ~(size_t)15;
-  ml.off_sel_rec = off;   off += 16;
+  ml.off_sel_rec = off;   off += 16 * MB;   // a record per token
   ml.off_exec_rec = off;  off += L * 32;   // per layer: routed-set record, execution-set record
-  ml.off_ncand = off; off += MB * sizeof(int32_t);
-  ml.off_cand = off;  off += MB * C * sizeof(int32_t);
+  ml.off_cand = off;  off += C * sizeof(int32_t);
   ml.bytes = off;
   ctx->exec_seq.assign(L, 0u);
   CR(cudaHostAlloc(reinterpret_cast<void**>(&ctx->mbox), ml.bytes, cudaHostAllocMapped | cudaHostAllocPortable));

@@ -42,15 +42,14 @@ __device__ __forceinline__ unsigned long long span_now() {
 // ---- mapped host mailbox: the kernels post small decision records here so that the host can
 // plan copies without a stream synchronisation.  One per context; sequence numbers only grow.
 struct MailboxHeader {
-  volatile uint32_t sel_seq;  // written by the candidate-selection kernel, after the lists
   volatile uint32_t status;   // sticky device status (0 ok, 1 a bounded wait ran out)
-  uint32_t pad[2];
+  uint32_t pad[3];
 };
 
 // Byte offsets inside the mailbox.  Per layer: two records of the FFN step, routed and execution set (B > 1: their
 // unions over the tokens), each with its sequence number.
 struct MailboxLayout {
-  size_t off_sel_rec, off_exec_rec, off_ncand, off_cand, bytes;
+  size_t off_sel_rec, off_exec_rec, off_cand, bytes;
 };
 
 // Device-side counters of one layer (S9), accumulated with 64-bit atomics.
@@ -74,13 +73,9 @@ struct SelectParams {
   int32_t* cand_out;    // [B][C] device, caller's
   int32_t* ncand_out;   // [B]
   int32_t* ncand_keep;  // [B] context-owned copy for the metrics
-  int32_t* mbox_cand;   // mapped host [B][C]
-  int32_t* mbox_ncand;  // mapped host [B]
-  volatile uint32_t* mbox_seq;
-  uint32_t* mbox_rec;   // mapped host, 16-byte aligned: {mask lo, mask hi, ncand, seq} for B == 1
+  int32_t* mbox_cand;   // mapped host [C], B == 1: the ranked list (advisory)
+  uint32_t* mbox_rec;   // mapped host, 16-byte aligned, a record per token: {mask lo, mask hi, ncand, seq}
   uint32_t seq_value;
-  unsigned long long* done_counter;
-  unsigned long long done_target;
   DevStats* stats;
   float t_tau;
   int force;  // 0: threshold test, 1: delta_hat = 0, 2: delta_hat = N-k
@@ -97,7 +92,6 @@ struct RouterParams {
   int32_t* topk_out;  // [B][k] or null
   int N, d, B, k;
   int warps_per_cta;
-  int tok_per_group;  // batched kernel: tokens a cluster handles per pass (set by the launcher)
   // gate-kernel epilogue (S9 metrics + mailbox); all null/0 for the prefetch router
   const int32_t* pi_pred;     // [B][N] ranking of the prefetch router for this step, or null
   const int32_t* ncand_pred;  // [B]
@@ -286,7 +280,7 @@ struct apex_ctx {
   uint32_t* d_demand = nullptr;            // [L][N]
   int32_t *d_pi = nullptr, *d_ncand = nullptr;              // [maxB][N], [maxB]
   apex::DevStats* d_stats = nullptr;                        // [L]
-  unsigned long long* d_counters = nullptr;                 // [2]: select done, zero
+  unsigned long long* d_counters = nullptr;                 // [2]: -, zero
   // batched path (max_batch > 1)
   int32_t *d_pair_tok = nullptr, *d_grp = nullptr;
   float* d_pair_gate = nullptr;
@@ -312,7 +306,7 @@ struct apex_ctx {
   apex::MailboxLayout ml{};
   uint32_t sel_seq = 0;
   std::vector<uint32_t> exec_seq;                 // per layer, last value asked for
-  unsigned long long sel_done = 0, zero_done = 0;
+  unsigned long long zero_done = 0;
   unsigned int* d_tickets = nullptr;  // [64] ring of row-ticket counters
   int32_t* d_spec = nullptr;          // [L][APEX_MAX_TOPK]: top-k of the prefetch router (B = 1), the FFN's speculative first fill
   uint32_t ffn_launch_id = 0;

@@ -162,13 +162,8 @@ int fill_select(apex_ctx* ctx, int layer, int B, float tau, int32_t* cand_dev, i
   p->ncand_out = ncand_dev;
   p->ncand_keep = ctx->d_ncand;
   p->mbox_cand = mbox_i32(ctx, ctx->ml.off_cand);
-  p->mbox_ncand = mbox_i32(ctx, ctx->ml.off_ncand);
-  p->mbox_seq = &mhdr(ctx)->sel_seq;
   p->mbox_rec = const_cast<uint32_t*>(mbox_sel_rec(ctx));
   p->seq_value = ++ctx->sel_seq;
-  if (B > 1) ctx->sel_done += (unsigned long long)B;
-  p->done_counter = ctx->d_counters + 0;
-  p->done_target = ctx->sel_done;
   p->stats = ctx->d_stats + layer;
   p->force = tau <= 0.f ? 1 : (tau >= 1.f ? 2 : 0);
   p->t_tau = p->force ? 0.f : (float)std::log((double)tau / (1.0 - (double)tau));
@@ -244,7 +239,6 @@ int apex_prefetch(apex_ctx* ctx, int layer, int B, void* copy_stream) {
   for (int i = 0; i < ctx->n_copy_streams; ++i)
     ctx->cur_copy_streams[i] = copy_stream ? (cudaStream_t)copy_stream : ctx->copy_streams[i];
   const int C = ctx->cfg.C;
-  const int32_t* ncand = mbox_i32(ctx, ctx->ml.off_ncand);
   const int32_t* cand = mbox_i32(ctx, ctx->ml.off_cand);
   std::vector<SlotCopy> copies;
   std::vector<SlotCopy> ordered;
@@ -275,9 +269,24 @@ int apex_prefetch(apex_ctx* ctx, int layer, int B, void* copy_stream) {
     if (valid && copies.size() > 1)
       std::stable_sort(ordered.begin(), ordered.end(), [&](const SlotCopy& a, const SlotCopy& b) { return pos[a.expert] < pos[b.expert]; });
   } else {
-    if (!host_wait_seq(ctx, &mhdr(ctx)->sel_seq, ctx->sel_seq))
-      return fail(ctx, APEX_ETIMEOUT, "apex_prefetch: candidate lists did not arrive");
-    if (!ctx->tables[layer].plan_prefetch(cand, ncand, B, C, &copies)) return fail(ctx, APEX_ESTATE, "no evictable slot");
+    // tokens that want each expert, from the tokens' masks: bit-sliced counters (plane j holds bit j of all 64 counts)
+    uint64_t plane[9] = {};  // counts up to APEX_MAX_BATCH
+    volatile uint32_t* rec = mbox_sel_rec(ctx);
+    for (int b = 0; b < B; ++b) {
+      if (!host_wait_seq(ctx, rec + 4 * b + 3, ctx->sel_seq)) return fail(ctx, APEX_ETIMEOUT, "apex_prefetch: a candidate set did not arrive");
+      uint64_t carry = ((uint64_t)rec[4 * b + 1] << 32) | rec[4 * b];
+      for (int j = 0; carry; ++j) {
+        const uint64_t c = plane[j] & carry;
+        plane[j] ^= carry;
+        carry = c;
+      }
+    }
+    int count[APEX_MAX_EXPERTS];
+    for (int e = 0; e < APEX_MAX_EXPERTS; ++e) {
+      count[e] = 0;
+      for (int j = 0; j < 9; ++j) count[e] |= (int)((plane[j] >> e) & 1) << j;
+    }
+    if (!ctx->tables[layer].plan_prefetch(count, &copies)) return fail(ctx, APEX_ESTATE, "no evictable slot");
     ordered = copies;
   }
   for (size_t i = 0; i < ordered.size(); ++i) {

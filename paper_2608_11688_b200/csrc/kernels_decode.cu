@@ -456,14 +456,15 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_token_kernel(const Deco
       sp.ncand_out = p.ncand_dev;
       sp.ncand_keep = p.ncand_keep;
       sp.mbox_cand = p.mbox[l].cand;
-      sp.mbox_ncand = reinterpret_cast<int32_t*>(&p.mbox[l].pad[0]);
       sp.mbox_rec = p.mbox[l].sel_rec;
       sp.seq_value = p.seq;
       sp.stats = p.stats + l;
       sp.t_tau = p.t_tau;
       sp.force = p.force;
       sp.N = N; sp.k = k; sp.C = p.C; sp.B = 1;
-      select_token(sp, 0, lane, pj0, pj1, x0, x1);
+      SelectVals sv;
+      sv.w0 = cw0; sv.w1 = cw1; sv.th0 = cth0; sv.th1 = cth1;
+      select_token(sp, sv, 0, lane, pj0, pj1, x0, x1);
       DTL(10);
       pref_done = true;
 

@@ -60,10 +60,13 @@ __global__ void __launch_bounds__(256) router_kernel(const RouterParams p) {
     }
     if (p.bias) bias_e = __ldg(p.bias + e);
   }
+  EpilogueVals ev;
+  if (p.fuse_select && crank == 0 && warp == 0) ev.sel = load_select_vals(p.sel, lane);
   RTL(0);
   pdl_wait();               // everything queued before this kernel is complete: x may be read
   pdl_launch_dependents();  // the next kernel may begin its own prologue
   RTL(1);
+  if (crank == 0 && warp == 0) load_prediction(p, b, lane, &ev);
 
   // x is staged in shared memory by the whole CTA in one round of loads
   {
@@ -97,129 +100,180 @@ __global__ void __launch_bounds__(256) router_kernel(const RouterParams p) {
   if (crank != 0 || warp != 0) return;
 
   // ---- leader warp
-  router_epilogue(p, b, lane, zs, qs, pis, posp);
+  router_epilogue(p, ev, b, lane, zs, qs, pis, posp);
   SPAN_END((p.fuse_select || !p.topk_out || !p.stats) ? 1 : 4);
 }
 
-// The same for a batch (B > 1).  A cluster keeps its weight rows in registers and walks over groups of
-// kRouterTok tokens: the group's hidden states (1 to kRouterTok tokens, chosen by the launcher) are staged in shared memory once, every warp takes the dot
-// products of its expert's row with all of them (per token the arithmetic and its order are those of
-// router_kernel), the logits go to the leader CTA, one cluster barrier per group, and warp t of the leader
-// CTA finishes token t of the group.  The logits are double-buffered: a buffer is written again two groups
-// later, after the barrier of the group in between, which the leader's warps reach only when they are done
-// reading it.  W_r is read once per cluster instead of once per token.
-constexpr int kRouterTok = 8;  // tokens per group = warps of a CTA
+// The same for a batch (B > 1): a cluster takes TT tokens, its CTA r the experts r * wpc .. r * wpc + wpc - 1 (wpc <= 8).
+// Rows of W and of x come into shared memory by bulk copies in chunks of kChunk columns, two buffers (the W rows are
+// parameters and are asked for before the dependency wait).  A warp takes a tile of tokens x experts with its lanes along
+// the columns: per (token, expert) every lane runs the multiply-add chain of router_kernel and the lanes are added by the
+// same xor tree -- halving the set of values a lane keeps at every level, which pairs the same partial sums -- so the
+// logits have the same bits.  Each token's logits go to one CTA of the cluster, whose warps finish the tokens.
+//
+// Bound by latency: two rounds of loads, 16 multiply-adds per lane, token and expert at d = 2048, one cluster barrier, a
+// serial epilogue.  As one token per pass over register-held rows it took 29 us at B = 256, N = 60, d = 2048.
+constexpr int kChunk = 1024;
+constexpr int kRouterWarps = 8;
 
-__global__ void __launch_bounds__(256) router_batched_kernel(const RouterParams p) {
+__host__ __device__ constexpr int router_tile_tok(int tt) { return tt < 4 ? tt : 4; }
+__host__ __device__ constexpr int router_tile_exp(int tt) { return tt <= 4 ? 1 : tt / 4; }
+
+template <int TT>
+__global__ void __launch_bounds__(kRouterWarps * 32, 2) router_batched_kernel(const RouterParams p) {
   SPAN_BEGIN();
   cg::cluster_group cluster = cg::this_cluster();
-  const unsigned crank = cluster.block_rank();
+  const unsigned crank = cluster.block_rank(), csize = cluster.num_blocks();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __shared__ float zs[2][kRouterTok][APEX_MAX_EXPERTS];
-  __shared__ float qs[kRouterTok][APEX_MAX_EXPERTS];
-  __shared__ int pis[kRouterTok][APEX_MAX_EXPERTS];
-  __shared__ int posp[kRouterTok][APEX_MAX_EXPERTS];
-  extern __shared__ float4 xs_dyn[];  // [kRouterTok][d / 4]
-
-  const int e = (int)crank * p.warps_per_cta + warp;
-  const bool active = warp < p.warps_per_cta && e < p.N;
-  const int nv = p.d >> 2;
-  float4 wreg[kRouterMaxVec];
-  float bias_e = 0.f;
-  if (active) {
-    const float4* __restrict__ Wrow = reinterpret_cast<const float4*>(p.W + (size_t)e * p.d);
-#pragma unroll
-    for (int i = 0; i < kRouterMaxVec; ++i) {
-      const int c = i * 32 + lane;
-      // volatile: under this kernel's register pressure the compiler would otherwise sink the loads into the
-      // token loop, behind the dependency wait and once per group
-      if (c < nv)
-        asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];"
-                     : "=f"(wreg[i].x), "=f"(wreg[i].y), "=f"(wreg[i].z), "=f"(wreg[i].w)
-                     : "l"(Wrow + c));
-    }
-    if (p.bias) bias_e = __ldg(p.bias + e);
+  constexpr int NT = router_tile_tok(TT), NX = router_tile_exp(TT);
+  __shared__ float zs[TT][APEX_MAX_EXPERTS];   // tokens finished here (at most all of them)
+  __shared__ float qs[kRouterWarps][APEX_MAX_EXPERTS];
+  __shared__ int pis[kRouterWarps][APEX_MAX_EXPERTS];
+  __shared__ int posp[kRouterWarps][APEX_MAX_EXPERTS];
+  __shared__ uint64_t s_bar[2];
+  extern __shared__ __align__(128) float tiles[];  // [2][TT + 8][kChunk]: x rows, W rows
+  const int b0 = blockIdx.y * TT, nt = min(TT, p.B - b0);
+  const int e0 = (int)crank * p.warps_per_cta, ne = max(0, min(p.warps_per_cta, p.N - e0));
+  const int n_chunks = (p.d + kChunk - 1) / kChunk;
+  if (threadIdx.x == 0) {
+    mbar_init(&s_bar[0], 2);
+    mbar_init(&s_bar[1], 2);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  __syncthreads();
+  auto chunk_bytes = [&](int c) { return (uint32_t)(min(kChunk, p.d - c * kChunk) * 4); };
+  auto load_w = [&](int c) {  // warp 0
+    if (lane == 0) mbar_expect_tx(&s_bar[c & 1], ne * chunk_bytes(c));
+    __syncwarp();
+    if (lane < ne) bulk_g2s(tiles + ((c & 1) * (TT + 8) + TT + lane) * kChunk, p.W + (size_t)(e0 + lane) * p.d + c * kChunk, chunk_bytes(c), &s_bar[c & 1]);
+  };
+  auto load_x = [&](int c) {
+    if (lane == 0) mbar_expect_tx(&s_bar[c & 1], nt * chunk_bytes(c));
+    __syncwarp();
+    if (lane < nt) bulk_g2s(tiles + ((c & 1) * (TT + 8) + lane) * kChunk, p.x + (size_t)(b0 + lane) * p.d + c * kChunk, chunk_bytes(c), &s_bar[c & 1]);
+  };
+  if (warp == 0)
+    for (int c = 0; c < 2 && c < n_chunks; ++c) load_w(c);
+  const int te = warp * (int)csize + (int)crank;  // the token this warp finishes
+  EpilogueVals ev;
+  if (p.fuse_select && te < nt) ev.sel = load_select_vals(p.sel, lane);
   RTL(0);
   pdl_wait();
   pdl_launch_dependents();
   RTL(1);
-
-  const int tpg = p.tok_per_group;  // tokens per group, 1..kRouterTok
-  const int n_groups = (p.B + tpg - 1) / tpg;
-  int buf = 0;
-  for (int g = blockIdx.y; g < n_groups; g += gridDim.y, buf ^= 1) {
-    const int b0 = g * tpg;
-    const int nt = p.B - b0 < tpg ? p.B - b0 : tpg;
-    {
-      // the group's rows of x are contiguous: one linear copy.  (Every warp of this CTA passed the cluster
-      // barrier of the previous group after its last read of xs.)
-      // Asynchronous 16-byte copies, all in flight at once: a loop of load-then-store would pay the memory
-      // latency once per trip (up to 32 trips per thread).
-      const float4* __restrict__ xv = reinterpret_cast<const float4*>(p.x + (size_t)b0 * p.d);
-      for (int c = threadIdx.x; c < nt * nv; c += blockDim.x)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(xs_dyn + c)), "l"(xv + c) : "memory");
-      asm volatile("cp.async.wait_all;" ::: "memory");
-    }
-    __syncthreads();
-    RTL(2);
+  if (te < nt) load_prediction(p, b0 + te, lane, &ev);
+  if (warp == 0)
+    for (int c = 0; c < 2 && c < n_chunks; ++c) load_x(c);
+  // this warp's tile: tokens t0 .. t0 + NT - 1, experts x0 .. x0 + NX - 1 of the CTA
+  constexpr int TILES_T = TT / NT;
+  const int t0 = (warp % TILES_T) * NT, x0 = (warp / TILES_T) * NX;
+  const bool active = x0 < ne && t0 < nt;
+  float acc[NT * NX];
+#pragma unroll
+  for (int v = 0; v < NT * NX; ++v) acc[v] = 0.f;
+  for (int c = 0; c < n_chunks; ++c) {
+    mbar_wait(&s_bar[c & 1], (c >> 1) & 1, nullptr, 2000000000ll);
     if (active) {
-      float acc[kRouterTok];
+      const int nv = min(kChunk, p.d - c * kChunk) >> 2;
+      const float4* xt = reinterpret_cast<const float4*>(tiles + ((c & 1) * (TT + 8) + t0) * kChunk) + lane;
+      const float4* wt = reinterpret_cast<const float4*>(tiles + ((c & 1) * (TT + 8) + TT + x0) * kChunk) + lane;
+      auto step = [&](int i) {
+        float4 xv[NT];
 #pragma unroll
-      for (int t = 0; t < kRouterTok; ++t) acc[t] = 0.f;
-      if (nt == kRouterTok) {  // full group: no per-token predicate inside the unrolled loops
+        for (int t = 0; t < NT; ++t) xv[t] = xt[t * (kChunk / 4) + i];
 #pragma unroll
-        for (int i = 0; i < kRouterMaxVec; ++i) {
-          const int c = i * 32 + lane;
-          if (c < nv) {
+        for (int x = 0; x < NX; ++x) {
+          const float4 wv = wt[x * (kChunk / 4) + i];
 #pragma unroll
-            for (int t = 0; t < kRouterTok; ++t) {
-              const float4 x = xs_dyn[t * nv + c];
-              acc[t] = fmaf(wreg[i].x, x.x, acc[t]);
-              acc[t] = fmaf(wreg[i].y, x.y, acc[t]);
-              acc[t] = fmaf(wreg[i].z, x.z, acc[t]);
-              acc[t] = fmaf(wreg[i].w, x.w, acc[t]);
-            }
+          for (int t = 0; t < NT; ++t) {
+            float a = acc[x * NT + t];
+            a = fmaf(wv.x, xv[t].x, a);
+            a = fmaf(wv.y, xv[t].y, a);
+            a = fmaf(wv.z, xv[t].z, a);
+            a = fmaf(wv.w, xv[t].w, a);
+            acc[x * NT + t] = a;
           }
         }
-      }
-      float mine = 0.f;  // lane t delivers token t
-      if (nt == kRouterTok) {
-#pragma unroll
-        for (int t = 0; t < kRouterTok; ++t) {
-          const float v = warp_sum_tree(acc[t]);
-          if (lane == t) mine = v;
-        }
-      } else {  // partial group: token by token
-        for (int t = 0; t < nt; ++t) {
-          float a = 0.f;
-#pragma unroll
-          for (int i = 0; i < kRouterMaxVec; ++i) {
-            const int c = i * 32 + lane;
-            if (c < nv) {
-              const float4 x = xs_dyn[t * nv + c];
-              a = fmaf(wreg[i].x, x.x, a);
-              a = fmaf(wreg[i].y, x.y, a);
-              a = fmaf(wreg[i].z, x.z, a);
-              a = fmaf(wreg[i].w, x.w, a);
-            }
-          }
-          a = warp_sum_tree(a);
-          if (lane == t) mine = a;
-        }
-      }
-      if (lane < nt) {
-        float* dst = cluster.map_shared_rank(&zs[0][0][0], 0);
-        dst[(buf * kRouterTok + lane) * APEX_MAX_EXPERTS + e] = mine + bias_e;
+      };
+      int i = 0;
+#pragma unroll 2
+      for (; i + 32 <= nv; i += 32) step(i);
+      if (i + lane < nv) step(i);  // (a remainder of columns: some lanes)
+    }
+    if (c + 2 < n_chunks) {
+      __syncthreads();  // everybody has read this buffer
+      if (warp == 0) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        load_w(c + 2);
+        load_x(c + 2);
       }
     }
-    RTL(3);
-    cluster.sync();
-    RTL(4);
-    if (crank == 0 && warp < nt) router_epilogue(p, b0 + warp, lane, zs[buf][warp], qs[warp], pis[warp], posp[warp]);
+  }
+  RTL(2);
+  // The xor tree over the lanes.  While more than one value is left, a lane keeps the half of the values its bit selects
+  // and hands the other half to its partner.
+  int idx = 0;  // index of the value this lane ends up with
+  {
+    int n = NT * NX;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      if (n > 1) {
+        n >>= 1;
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int v = 0; v < NT * NX / 2; ++v) {
+          if (v < n) {
+            const float give = up ? acc[v] : acc[v + n], keep = up ? acc[v + n] : acc[v];
+            acc[v] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+          }
+        }
+        idx = idx * 2 + (up ? 1 : 0);
+      } else {
+        acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
+      }
+    }
+  }
+  constexpr int DUP = 32 / (NT * NX);  // lanes that end up with the same value
+  if (active && (lane & (DUP - 1)) == 0) {
+    const int x = x0 + idx / NT, t = t0 + idx % NT;
+    if (x < ne && t < nt) {
+      const float z = acc[0] + (p.bias ? __ldg(p.bias + e0 + x) : 0.f);
+      float* dst = cluster.map_shared_rank(&zs[0][0], t % csize);
+      dst[(t / csize) * APEX_MAX_EXPERTS + e0 + x] = z;
+    }
+  }
+  RTL(3);
+  cluster.sync();
+  RTL(4);
+  if (te < nt) router_epilogue(p, ev, b0 + te, lane, zs[warp], qs[warp], pis[warp], posp[warp]);
+  for (int t = te + kRouterWarps * (int)csize; t < nt; t += kRouterWarps * (int)csize) {  // (a cluster of one CTA: more tokens than warps)
+    __syncwarp();
+    load_prediction(p, b0 + t, lane, &ev);
+    router_epilogue(p, ev, b0 + t, lane, zs[t / csize], qs[warp], pis[warp], posp[warp]);
   }
   RTL(6);
   SPAN_END((p.fuse_select || !p.topk_out || !p.stats) ? 1 : 4);
+}
+
+template <int TT>
+cudaError_t launch_router_batched(const RouterParams& p, cudaLaunchConfig_t& cfg, int csize) {
+  constexpr int smem = 2 * (TT + 8) * kChunk * (int)sizeof(float);
+  static bool configured[kMaxDevices];
+  static std::mutex setup_mutex;  // contexts of several host threads (and the context-free gate) share this set-up
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  {
+    std::lock_guard<std::mutex> lock(setup_mutex);
+    if (!configured[dev]) {
+      if ((e = cudaFuncSetAttribute(router_batched_kernel<TT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
+      configured[dev] = true;
+    }
+  }
+  cfg.gridDim = dim3(csize, (p.B + TT - 1) / TT, 1);
+  cfg.dynamicSmemBytes = smem;
+  return cudaLaunchKernelEx(&cfg, router_batched_kernel<TT>, p);
 }
 
 cudaError_t launch_router(const RouterParams& p, cudaStream_t s) {
@@ -233,40 +287,6 @@ cudaError_t launch_router(const RouterParams& p, cudaStream_t s) {
   cfg.blockDim = dim3(256, 1, 1);
   cfg.dynamicSmemBytes = 0;
   cfg.stream = s;
-  const bool batched = p.B > 1;
-  if (batched) {
-    // one cluster per group of tokens, at most as many clusters as fit the GPU at one CTA per SM (the weight
-    // rows in registers allow no more); further groups are walked by the same clusters
-    static int n_sm_of[kMaxDevices];
-    static bool configured[kMaxDevices];
-    static std::mutex setup_mutex;  // contexts of several host threads (and the context-free gate) share this set-up
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    int n_sm = 0;
-    {
-      std::lock_guard<std::mutex> lock(setup_mutex);
-      if (!configured[dev]) {
-        if ((e = cudaDeviceGetAttribute(&n_sm_of[dev], cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        if ((e = cudaFuncSetAttribute(router_batched_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      kRouterTok * kRouterMaxVec * 32 * (int)sizeof(float4))) != cudaSuccess)
-          return e;
-        configured[dev] = true;
-      }
-      n_sm = n_sm_of[dev];
-    }
-    int resident = n_sm / csize;
-    if (resident < 1) resident = 1;
-    // small batches spread over the clusters (a token per cluster while they last); large ones fill the groups,
-    // because a group costs a barrier and a round of shared-memory reads of all its tokens per warp
-    int tpg = (p.B + resident - 1) / resident;
-    tpg = tpg > kRouterTok ? kRouterTok : tpg;
-    q.tok_per_group = tpg;
-    const int n_groups = (p.B + tpg - 1) / tpg;
-    cfg.gridDim = dim3(csize, n_groups < resident ? n_groups : resident, 1);
-    cfg.dynamicSmemBytes = (size_t)tpg * p.d * sizeof(float);
-  }
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = csize;
@@ -276,7 +296,15 @@ cudaError_t launch_router(const RouterParams& p, cudaStream_t s) {
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return batched ? cudaLaunchKernelEx(&cfg, router_batched_kernel, q) : cudaLaunchKernelEx(&cfg, router_kernel, q);
+  if (p.B == 1) return cudaLaunchKernelEx(&cfg, router_kernel, q);
+  // Tokens per cluster: as few as let all clusters run at once on 148 SMs (18 clusters of eight CTAs), since a cluster's
+  // time grows with its tokens; at most 16
+  const int clusters = 144 / csize;
+  if (p.B <= clusters) return launch_router_batched<1>(q, cfg, csize);
+  if (p.B <= 2 * clusters) return launch_router_batched<2>(q, cfg, csize);
+  if (p.B <= 4 * clusters) return launch_router_batched<4>(q, cfg, csize);
+  if (p.B <= 8 * clusters) return launch_router_batched<8>(q, cfg, csize);
+  return launch_router_batched<16>(q, cfg, csize);
 }
 
 // One warp per token: x_j = q_p[pi[j]] (the prefetch distribution in descending order),
@@ -284,10 +312,11 @@ cudaError_t launch_router(const RouterParams& p, cudaStream_t s) {
 // domain), capped to C - k; K_p = first k + delta_hat experts of E (Eq. (1)).
 __global__ void __launch_bounds__(128) select_kernel(const SelectParams p) {
   SPAN_BEGIN();
-  pdl_wait();
-  pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int b = blockIdx.x * (blockDim.x >> 5) + warp;
+  const SelectVals sv = load_select_vals(p, lane);
+  pdl_wait();
+  pdl_launch_dependents();
   if (b >= p.B) return;
   const int N = p.N;
   const size_t row = (size_t)b * N;
@@ -301,7 +330,7 @@ __global__ void __launch_bounds__(128) select_kernel(const SelectParams p) {
     pj1 = __ldg(p.pi + row + lane + 32);
     x1 = __ldg(p.q + row + pj1);
   }
-  select_token(p, b, lane, pj0, pj1, x0, x1);
+  select_token(p, sv, b, lane, pj0, pj1, x0, x1);
   SPAN_END(2);
 }
 
@@ -327,13 +356,22 @@ __global__ void __launch_bounds__(512) attention_standin_kernel(const AttnParams
   pdl_launch_dependents();
   const size_t stride = (size_t)gridDim.x * blockDim.x;
   uint4 a = make_uint4(0, 0, 0, 0);
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < p.n_vec; i += stride) {
-    const uint4 v = __ldcs(p.buf + i);
+  auto take = [&](const uint4& v) {
     a.x ^= v.x;
     a.y ^= v.y;
     a.z ^= v.z;
     a.w ^= v.w;
+  };
+  // eight loads of a thread in flight: with one, 2.4 MB under way on the whole GPU were 14 us for the 42 MB of d = 2048
+  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  for (; i + 7 * stride < p.n_vec; i += 8 * stride) {
+    uint4 v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = __ldcs(p.buf + i + u * stride);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) take(v[u]);
   }
+  for (; i < p.n_vec; i += stride) take(__ldcs(p.buf + i));
   if (a.x == 0x12345678u && a.y == 0x9abcdef0u && a.z == 0x0fedcba9u && a.w == 0x87654321u) p.sink[0] = 1.f;
   // Streamed beside the preceding kernel: wait for it now, so that whoever waits for this kernel has, as
   // always, everything before it on the stream complete.

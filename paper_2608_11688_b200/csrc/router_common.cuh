@@ -56,67 +56,58 @@ __device__ __forceinline__ int select_budget_vals(float w0, float w1, float th0,
   *uncapped = d_hat;
   return min(d_hat, C - k);
 }
-__device__ __forceinline__ int select_budget(const float* __restrict__ w, const float* __restrict__ theta, float t_tau, int force,
-                                             int N, int k, int C, int lane, float x0, float x1, int* uncapped) {
-  const int nth = N - k + 1;
-  const float w0 = lane < N ? __ldg(w + lane) : 0.f, w1 = lane + 32 < N ? __ldg(w + lane + 32) : 0.f;
-  const float th0 = lane < nth ? __ldg(theta + lane) : 0.f, th1 = lane + 32 < nth ? __ldg(theta + lane + 32) : 0.f;
-  return select_budget_vals(w0, w1, th0, th1, t_tau, force, N, k, C, lane, x0, x1, uncapped);
+// The parameters of the confidence model a lane needs, loaded ahead of the token's logits
+struct SelectVals {
+  float w0 = 0.f, w1 = 0.f, th0 = 0.f, th1 = 0.f;
+};
+__device__ __forceinline__ SelectVals load_select_vals(const SelectParams& p, int lane) {
+  const int nth = p.N - p.k + 1;
+  SelectVals v;
+  if (lane < p.N) v.w0 = __ldg(p.w + lane);
+  if (lane + 32 < p.N) v.w1 = __ldg(p.w + lane + 32);
+  if (lane < nth) v.th0 = __ldg(p.theta + lane);
+  if (lane + 32 < nth) v.th1 = __ldg(p.theta + lane + 32);
+  return v;
 }
 
-__device__ __forceinline__ void select_token(const SelectParams& p, int b, int lane, int pj0, int pj1, float x0, float x1) {
+__device__ __forceinline__ void select_token(const SelectParams& p, const SelectVals& v, int b, int lane, int pj0, int pj1, float x0, float x1) {
   const int N = p.N, k = p.k, C = p.C;
   int uncapped;
-  const int d_hat = select_budget(p.w, p.theta, p.t_tau, p.force, N, k, C, lane, x0, x1, &uncapped);
+  const int d_hat = select_budget_vals(v.w0, v.w1, v.th0, v.th1, p.t_tau, p.force, N, k, C, lane, x0, x1, &uncapped);
   const int ncand = k + d_hat;
-  // candidates in rank order, padded with -1
   const bool in0 = lane < ncand, in1 = lane + 32 < ncand;
-  if (lane < C) {
-    const int v = in0 ? pj0 : -1;
-    p.cand_out[(size_t)b * C + lane] = v;
-    p.mbox_cand[(size_t)b * C + lane] = v;
-  }
-  if (lane + 32 < C) {
-    const int v = in1 ? pj1 : -1;
-    p.cand_out[(size_t)b * C + lane + 32] = v;
-    p.mbox_cand[(size_t)b * C + lane + 32] = v;
-  }
   // the candidate set as a 64-bit mask
   unsigned lo = 0, hi = 0;
   if (in0) { if (pj0 < 32) lo |= 1u << pj0; else hi |= 1u << (pj0 - 32); }
   if (in1) { if (pj1 < 32) lo |= 1u << pj1; else hi |= 1u << (pj1 - 32); }
   lo = __reduce_or_sync(0xffffffffu, lo);
   hi = __reduce_or_sync(0xffffffffu, hi);
+  // The host needs only the sets, a record per token: mask, count and sequence number travel in ONE aligned 16-byte store,
+  // so no system-scope fence and no counter over the batch sits on the kernel's path.  (The ranked list below is
+  // advisory for the host at B = 1: it is used for the issue order only if it matches the mask.)
+  if (lane == 0)
+    asm volatile("st.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p.mbox_rec + 4 * b), "r"(lo), "r"(hi), "r"((unsigned)ncand), "r"(p.seq_value)
+                 : "memory");
+  // candidates in rank order, padded with -1
+  if (lane < C) {
+    const int e = in0 ? pj0 : -1;
+    p.cand_out[(size_t)b * C + lane] = e;
+    if (p.B == 1) p.mbox_cand[lane] = e;
+  }
+  if (lane + 32 < C) {
+    const int e = in1 ? pj1 : -1;
+    p.cand_out[(size_t)b * C + lane + 32] = e;
+    if (p.B == 1) p.mbox_cand[lane + 32] = e;
+  }
   if (lane == 0) {
     p.ncand_out[b] = ncand;
     p.ncand_keep[b] = ncand;
-    p.mbox_ncand[b] = ncand;
     if (p.stats) {
       atomicAdd(&p.stats->tokens, 1ull);
       atomicAdd(&p.stats->sum_delta_hat, (unsigned long long)d_hat);
       atomicAdd(&p.stats->sum_ncand, (unsigned long long)ncand);
       atomicAdd(&p.stats->capped, (unsigned long long)(uncapped > d_hat ? 1 : 0));
       atomicAdd(&p.stats->near_full, (unsigned long long)(2 * ncand > N ? 1 : 0));
-    }
-  }
-  if (p.B == 1) {
-    // one token: the host needs only the set.  Mask, count and sequence number travel in ONE aligned
-    // 16-byte store, so no system-scope fence sits on the kernel's critical path.  (The ranked list
-    // above is advisory for the host: it is used for the issue order only if it matches the mask.)
-    if (lane == 0) {
-      asm volatile("st.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p.mbox_rec), "r"(lo), "r"(hi), "r"((unsigned)ncand),
-                   "r"(p.seq_value)
-                   : "memory");
-    }
-    return;
-  }
-  __threadfence_system();
-  __syncwarp();
-  if (lane == 0) {
-    const unsigned long long old = atomicAdd(p.done_counter, 1ull);
-    if (old + 1 == p.done_target) {
-      __threadfence_system();
-      *p.mbox_seq = p.seq_value;
     }
   }
 }
@@ -163,26 +154,42 @@ __device__ __forceinline__ RankedLogits softmax_and_rank(const float* zs, int N,
   return R;
 }
 
-__device__ __forceinline__ void router_epilogue(const RouterParams& p, int b, int lane, const float* zs, float* qs, int* pis,
-                                                int* posp) {
+// What the epilogue of a token reads from memory besides the logits, asked for before they are there: the confidence
+// model (fused selection), or the prefetch stage's ranking and budget (gate).
+struct EpilogueVals {
+  SelectVals sel;
+  int pred0 = -1, pred1 = -1, ncand = 0;
+};
+__device__ __forceinline__ void load_prediction(const RouterParams& p, int b, int lane, EpilogueVals* v) {  // after the dependency wait
+  if (!p.pi_pred || b >= p.B) return;
+  const size_t row = (size_t)b * p.N;
+  if (lane < p.N) v->pred0 = __ldg(p.pi_pred + row + lane);
+  if (lane + 32 < p.N) v->pred1 = __ldg(p.pi_pred + row + lane + 32);
+  v->ncand = __ldg(p.ncand_pred + b);
+}
+
+__device__ __forceinline__ void router_epilogue(const RouterParams& p, const EpilogueVals& v, int b, int lane, const float* zs, float* qs,
+                                                int* pis, int* posp) {
   const int N = p.N, k = p.k;
   const int e0 = lane, e1 = lane + 32;
   const RankedLogits R = softmax_and_rank(zs, N, lane);
   const float z0 = R.z0, z1 = R.z1, q0 = R.q0, q1 = R.q1;
   const int r0 = R.r0, r1 = R.r1;
-  const size_t row = (size_t)b * N;
-  if (e0 < N) {
-    p.z_out[row + e0] = z0;
-    p.q_out[row + e0] = q0;
-    if (p.pi_out) p.pi_out[row + r0] = e0;
-    if (p.topk_out && r0 < k) p.topk_out[(size_t)b * k + r0] = e0;
-  }
-  if (e1 < N) {
-    p.z_out[row + e1] = z1;
-    p.q_out[row + e1] = q1;
-    if (p.pi_out) p.pi_out[row + r1] = e1;
-    if (p.topk_out && r1 < k) p.topk_out[(size_t)b * k + r1] = e1;
-  }
+  auto outputs = [&]() {
+    const size_t row = (size_t)b * N;
+    if (e0 < N) {
+      p.z_out[row + e0] = z0;
+      p.q_out[row + e0] = q0;
+      if (p.pi_out) p.pi_out[row + r0] = e0;
+      if (p.topk_out && r0 < k) p.topk_out[(size_t)b * k + r0] = e0;
+    }
+    if (e1 < N) {
+      p.z_out[row + e1] = z1;
+      p.q_out[row + e1] = q1;
+      if (p.pi_out) p.pi_out[row + r1] = e1;
+      if (p.topk_out && r1 < k) p.topk_out[(size_t)b * k + r1] = e1;
+    }
+  };
   RTL(4);
   if (p.fuse_select) {
     // prefetch router and budget selection in one launch: the ranked list goes through shared memory
@@ -191,10 +198,12 @@ __device__ __forceinline__ void router_epilogue(const RouterParams& p, int b, in
     __syncwarp();
     const int pj0 = lane < N ? pis[lane] : -1, pj1 = lane + 32 < N ? pis[lane + 32] : -1;
     const float x0 = pj0 >= 0 ? qs[pj0] : 0.f, x1 = pj1 >= 0 ? qs[pj1] : 0.f;
-    select_token(p.sel, b, lane, pj0, pj1, x0, x1);
+    select_token(p.sel, v.sel, b, lane, pj0, pj1, x0, x1);
+    outputs();
     RTL(5);
     return;
   }
+  outputs();
   if (!p.topk_out || !p.stats) return;
 
   // ---- gate epilogue: metrics of this token against the prefetch stage (Eq. (2), (3))
@@ -203,10 +212,10 @@ __device__ __forceinline__ void router_epilogue(const RouterParams& p, int b, in
     int dstar = 0, hitsP = 0, have_pred = 0;
     if (p.pi_pred) {
       have_pred = 1;
-      if (e0 < N) posp[__ldg(p.pi_pred + row + e0)] = e0;  // position of expert pi[j] in E is j
-      if (e1 < N) posp[__ldg(p.pi_pred + row + e1)] = e1;
+      if (e0 < N) posp[v.pred0] = e0;  // position of expert pi[j] in E is j
+      if (e1 < N) posp[v.pred1] = e1;
       __syncwarp();
-      const int nc = __ldg(p.ncand_pred + b);
+      const int nc = v.ncand;
       const int pos0 = in0 ? posp[e0] : -1, pos1 = in1 ? posp[e1] : -1;
       dstar = warp_max_int(max(pos0, pos1)) + 1 - k;
       hitsP = __popc(__ballot_sync(0xffffffffu, in0 && pos0 < nc)) + __popc(__ballot_sync(0xffffffffu, in1 && pos1 < nc));
