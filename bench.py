@@ -417,7 +417,7 @@ def other_config_rooflines(dev, peak, peak_kind):
             else:
                 distinct = cfg.N * (1.0 - (1.0 - cfg.k / cfg.N) ** B)
                 bytes_ffn = distinct * cfg.expert_bytes + cfg.shared_bytes + 2 * B * cfg.d * 4
-                kernel = "ffn_plan_kernel + ffn_tc_gather_kernel + ffn_tc_gemm_kernel<1>, <2>"
+                kernel = "ffn_tc_kernel"
             ach = bytes_ffn / mean_s / 1e9
             rec = {
                 "bound": "hbm", "kernel": kernel, "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,

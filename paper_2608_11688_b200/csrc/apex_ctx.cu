@@ -117,16 +117,14 @@ int apex_create(const apex_config* cfg, apex_ctx** out) {
   CR(dev_alloc(&ctx->d_alpha, L * MB * N));
   CR(dev_alloc(&ctx->d_exec_gate, MB * k));
   CR(dev_alloc(&ctx->d_cand_ncand, MB));
-  // batched path (only for contexts that will see batches): pair list, scratch and tensor maps of the grouped GEMM
+  // batched path (only for contexts that will see batches): scratch and tensor maps of the grouped GEMM
   if (MB > 1) {
     const size_t max_pairs = MB * (k + 1);
     const size_t rows = max_pairs + 64;  // (boxes of the last group reach past its rows)
     const size_t i_max = ((size_t)(c.I > c.I_shared ? c.I : c.I_shared) + 63) / 64 * 64;
-    CR(dev_alloc(&ctx->d_pair_tok, max_pairs));
-    CR(dev_alloc(&ctx->d_pair_gate, max_pairs));
-    CR(dev_alloc(&ctx->d_grp, 4 + 3 * (N + 1)));
     CR(dev_alloc(&ctx->d_tc_sync, (size_t)kTcSyncWords));
-    CR(dev_alloc(&ctx->d_plan_masks, 2));
+    CR(cudaMemset(ctx->d_tc_sync, 0, kTcSyncWords * sizeof(unsigned)));
+    CR(dev_alloc(&ctx->d_sgate, MB));
     ctx->act_stride = (int)i_max;
     ctx->act_rows = (int)rows;
     CR(dev_alloc(&ctx->d_xb, MB * d));
@@ -210,8 +208,8 @@ int apex_destroy(apex_ctx* ctx) {
   cudaDeviceSynchronize();
   cudaGetLastError();
   void* dev[] = {ctx->d_Wr, ctx->d_br, ctx->d_Wp, ctx->d_bp, ctx->d_w, ctx->d_theta, ctx->d_cache, ctx->d_slot_ready, ctx->d_zp,
-                 ctx->d_qp, ctx->d_zr, ctx->d_demand, ctx->d_pi, ctx->d_ncand, ctx->d_stats, ctx->d_counters, ctx->d_tickets, ctx->d_spec, ctx->d_pair_tok,
-                 ctx->d_pair_gate, ctx->d_grp, ctx->d_tc_sync, ctx->d_plan_masks, ctx->d_xb, ctx->d_act, ctx->d_cand,
+                 ctx->d_qp, ctx->d_zr, ctx->d_demand, ctx->d_pi, ctx->d_ncand, ctx->d_stats, ctx->d_counters, ctx->d_tickets, ctx->d_spec,
+                 ctx->d_tc_sync, ctx->d_sgate, ctx->d_xb, ctx->d_act, ctx->d_cand,
                  ctx->d_idx, ctx->d_exec_idx, ctx->d_alpha, ctx->d_exec_gate, ctx->d_cand_ncand, ctx->d_attn, ctx->d_attn_sink,
                  ctx->d_h_stage, ctx->d_hp_stage, ctx->d_y_stage};
   for (void* p : dev)

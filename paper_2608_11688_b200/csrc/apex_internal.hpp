@@ -3,6 +3,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdint>
 #include <string>
 #include <vector>
@@ -114,13 +115,6 @@ struct FfnParams {
   const uint8_t* shared_w;  // or null
   const float* shared_gate; // [d] gate vector of the shared expert, or null: weight 1
   const uint32_t* slot_ready;  // [C]
-  // batched plan (B > 1), context-owned
-  int32_t* pair_tok;        // [B*k + B] token of each (expert, token) pair, sorted by expert; the shared expert's pairs last
-  float* pair_gate;         // [B*k + B]
-  int32_t* grp;             // [4 + 3*(N+1)]: routed groups, all groups, 0, 0, then (expert, pair offset, tokens) per group
-  unsigned* tc_sync;        // [kTcSyncWords] zeroed by the plan
-  unsigned long long* plan_masks;  // [2] union of the routed sets, of the execution sets
-  __nv_bfloat16* xb;        // [B][d] h' in bf16
   uint32_t* mbox_rec;       // mapped host: two 16-byte records {mask lo, mask hi, sequence number, 0}: routed set, execution set (B > 1: their unions)
   volatile uint32_t* mbox_status;
   uint32_t seq_value;
@@ -145,22 +139,42 @@ struct FfnParams {
 
 constexpr int kMaxDevices = 64;  // per-device launch attributes are remembered for this many devices
 
+// Kernels of one step run side by side (programmatic dependent launch), but an SM changes the split between L1 and shared
+// memory only when it is idle: a kernel that needs little of it, left to its own preference, may have to wait for the end
+// of the kernel it was to run beside.  So the small kernels ask for the split that the large ones need.
+template <auto* kernel>
+inline void prefer_max_shared() {
+  static std::atomic<bool> done[kMaxDevices];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices || done[dev].load(std::memory_order_relaxed)) return;
+  cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  done[dev].store(true, std::memory_order_relaxed);
+}
+
 // Batched tensor-core path (kernels_ffn_tc.cu): B > 1
-// Words of the synchronisation block, zeroed by the plan kernel of every step
+// Words of the synchronisation block: zero between launches (the last CTA of one clears them)
 constexpr int kTcTicket = 0;                 // units handed out
 constexpr int kTcAbort = 1;                  // somebody gave up
-constexpr int kTcDone = 2;                   // [N + 1] gate/up units counted in, per group
+constexpr int kTcExits = 2;                  // CTAs that have finished
+constexpr int kTcRows = 3;                   // tokens whose row of X is there and whose row of y is zero
+constexpr int kTcDone = 4;                   // [N + 1] gate/up units counted in, per group
 constexpr int kTcSyncWords = kTcDone + APEX_MAX_EXPERTS + 1;
 struct TcShifts { uint32_t up2, up4, up6, up8, up12; };  // powers of two (see the code converters)
+// Units of a group, per kind of expert (0 routed, 1 shared): gate/up row blocks, K tiles of the down projection, tiles per
+// down unit, units along K and 2^32 / that (0 for one)
+struct TcGeometry { int blocks1, tiles, chunk, kch; uint32_t kch_inv; };
 struct TcParams {
   FfnParams f;
   unsigned* sync;                        // [kTcSyncWords]
-  const unsigned long long* plan_masks;  // union of the routed sets, of the execution sets
+  __nv_bfloat16* xb;                     // [B][d] h' in bf16
+  float* sgate;                          // [B] weight of the shared expert per token (gated variant)
   __nv_bfloat16* act;                    // the intermediate, two planes [2][act_rows][act_stride]: bf16(a) and bf16(a - bf16(a))
   size_t act_plane;                      // elements per plane
   int act_rows, act_stride;
   int layer_slot0;                       // index of this layer's slot 0 in the all-layers weight tensor map
   int nmax1, nmax2;                      // tokens per unit of the gate/up and of the down projection (set by the launcher)
+  int shift1, shift2;                    // a group of n tokens has (n + 2^shift - 1) >> shift parts
+  TcGeometry geo[2];
   int nstage, nraw, stage_bytes;         // ring depths and stage size
   TcShifts shifts;
 };
@@ -241,7 +255,6 @@ struct AttnParams {
 cudaError_t launch_router(const RouterParams& p, cudaStream_t s);
 cudaError_t launch_select(const SelectParams& p, cudaStream_t s);
 cudaError_t launch_attention(const AttnParams& p, int n_sm, cudaStream_t s);
-cudaError_t launch_ffn_plan(const FfnParams& p, int n_sm, cudaStream_t s);
 cudaError_t launch_ffn(const FfnParams& p, int n_ctas, cudaStream_t s);  // n_ctas: grid size, at most ffn_grid_ctas(SM count)
 int ffn_grid_ctas(int n_sm);  // CTAs of one streaming-kernel launch (each adds one to the zero counter)
 cudaError_t launch_ffn_tc(const TcParams& p, const TcMaps& m, int n_sm, cudaStream_t s);
@@ -282,10 +295,8 @@ struct apex_ctx {
   apex::DevStats* d_stats = nullptr;                        // [L]
   unsigned long long* d_counters = nullptr;                 // [2]: -, zero
   // batched path (max_batch > 1)
-  int32_t *d_pair_tok = nullptr, *d_grp = nullptr;
-  float* d_pair_gate = nullptr;
   unsigned* d_tc_sync = nullptr;
-  unsigned long long* d_plan_masks = nullptr;
+  float* d_sgate = nullptr;
   __nv_bfloat16 *d_xb = nullptr, *d_act = nullptr;
   int act_stride = 0, act_rows = 0;
   size_t act_plane = 0;

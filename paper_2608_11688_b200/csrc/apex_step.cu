@@ -403,13 +403,13 @@ cudaError_t launch_stream(apex_ctx* ctx, FfnParams p, cudaStream_t cs) {
 }
 
 
-// B > 1: plan kernel, then the tensor-core grouped GEMM.
+// B > 1: the tensor-core grouped GEMM.
 int launch_batched(apex_ctx* ctx, int layer, const FfnParams& p, cudaStream_t cs) {
-  CU_TRY(ctx, launch_ffn_plan(p, ctx->n_sm, cs));
   TcParams t{};
   t.f = p;
   t.sync = ctx->d_tc_sync;
-  t.plan_masks = ctx->d_plan_masks;
+  t.xb = ctx->d_xb;
+  t.sgate = ctx->d_sgate;
   t.act = ctx->d_act;
   t.act_rows = ctx->act_rows;
   t.act_stride = ctx->act_stride;
@@ -421,7 +421,7 @@ int launch_batched(apex_ctx* ctx, int layer, const FfnParams& p, cudaStream_t cs
   ctx->last_ffn_y_hi = (uintptr_t)p.y + (size_t)p.B * p.d * sizeof(float);
   ctx->last_pred_layer = -1;
   ctx->last_stream = cs;
-  ctx->launches += 2;
+  ++ctx->launches;
   return APEX_OK;
 }
 
@@ -449,12 +449,6 @@ int ffn_launch(apex_ctx* ctx, int layer, int mode, const float* hpost_dev, int B
   p.shared_w = ctx->shared_dev[layer];
   p.shared_gate = ctx->shared_gate_on[layer] ? ctx->shared_gate_dev[layer] : nullptr;
   p.slot_ready = ctx->d_slot_ready + (size_t)layer * C;
-  p.pair_tok = ctx->d_pair_tok;
-  p.pair_gate = ctx->d_pair_gate;
-  p.grp = ctx->d_grp;
-  p.tc_sync = ctx->d_tc_sync;
-  p.plan_masks = ctx->d_plan_masks;
-  p.xb = ctx->d_xb;
   p.mbox_rec = const_cast<uint32_t*>(mbox_exec_rec(ctx, layer));
   p.mbox_status = &mhdr(ctx)->status;
   p.seq_value = ++ctx->exec_seq[layer];

@@ -15,7 +15,8 @@
 //   down       D [256 cols of d x 2n] = downT[K x 256]^T . [a_hi ; a_lo]^T  (downT is MN-major, two M = 128 halves; both
 //              y[token][col] += D[:, j] + D[:, n + j]      fp32 atomics       planes in one MMA: N = 2n)
 //
-// ONE persistent kernel runs both: the units of both projections form one list, gate/up first, and the CTAs take
+// Every CTA first derives the step's plan (execution sets, tokens per expert, pair list) from the gate's outputs.
+// ONE persistent kernel runs both projections: the units of both projections form one list, gate/up first, and the CTAs take
 // tickets.  A down unit needs its group's intermediate, so its activations are loaded once the group's gate/up units have
 // been counted in (its weights, which wait for nothing, are already on their way); the tickets are handed out in list
 // order, so whatever a unit waits for is already running somewhere and no co-residency is assumed.  As two kernels the
@@ -47,6 +48,7 @@
 
 #include "apex_internal.hpp"
 #include "ptx.cuh"
+#include "token_plan.cuh"
 
 namespace apex {
 
@@ -102,7 +104,7 @@ __device__ __forceinline__ void tma_gather4(void* dst, const CUtensorMap* map, i
 // multiply-adds, which run beside it (by kernel parameters: multiplications by constants the compiler knows would be
 // turned back into shifts): two masks per pair of codes instead of five integer operations.  A pair is made of
 // the codes that lie 16 bits apart in their word, so the values come out in the order 0 2 1 3 (e4m3: within four) and
-// 0 4 1 5 2 6 3 7 (e2m1: within eight): the activations a gate/up tile meets are stored in that order (by the plan kernel), and for a
+// 0 4 1 5 2 6 3 7 (e2m1: within eight): the activations a gate/up tile meets are stored in that order, and for a
 // down tile, whose codes run along the output columns, the epilogue undoes it.
 __host__ __device__ constexpr int tc_column_of(int qf, int j) {  // value at position j
   return qf == 2 ? (j & ~7) | ((j & 1) << 2) | ((j >> 1) & 3) : qf == 1 ? (j & ~3) | ((j & 1) << 1) | ((j >> 1) & 1) : j;
@@ -239,6 +241,9 @@ __device__ unsigned long long g_tc_tl[148][64][8];
 
 // One unit of work: the (part of a) group, the M block and the K-tile range of one of the projections (phase 1: gate/up,
 // 2: down; 0: the list is at its end).
+struct GroupDesc {
+  int expert, pair_off, n_tok;
+};
 struct UnitDesc {
   int phase, group, expert, pair_off, n_tok, blk, kt_begin, kt_end;
 };
@@ -287,8 +292,13 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
   __shared__ UnitDesc s_unit[kUnitRing];
   __shared__ uint32_t tmem_base_s;
   __shared__ int s_abort;
-  __shared__ int s_u1[APEX_MAX_EXPERTS + 2], s_u2[APEX_MAX_EXPERTS + 2];  // first unit of each group, in list order, per projection
-  __shared__ int32_t s_grp[4 + 3 * (APEX_MAX_EXPERTS + 1)];
+  __shared__ int s_u[2][APEX_MAX_EXPERTS + 1], s_units[2];  // per projection: units before each group's in list order; all units
+  __shared__ GroupDesc s_grp[APEX_MAX_EXPERTS + 1];         // executed experts, then the shared one
+  constexpr int kTokWords = APEX_MAX_BATCH / 32;
+  __shared__ unsigned s_mask[APEX_MAX_EXPERTS][kTokWords];  // tokens of each expert
+  __shared__ short s_off[APEX_MAX_EXPERTS][kTokWords];
+  __shared__ float s_inv[APEX_MAX_BATCH];                // what its gates are divided by
+  __shared__ unsigned long long s_union[2];              // of the routed sets, of the execution sets
   __shared__ uint8_t s_tok[APEX_MAX_BATCH * (APEX_MAX_TOPK + 1)];  // token of each pair
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -296,6 +306,7 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
 
   if (tid == 0) {
     s_abort = 0;
+    s_union[0] = s_union[1] = 0ull;
     for (int s = 0; s < kMaxStages; ++s) {
       mbar_init(&full[s], QF ? 1 + kCvThreads / 32 : 2);  // the activations' bytes, and the weights' (bytes, or the converter warps)
       mbar_init(&empty[s], 1);
@@ -344,55 +355,12 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     ready_mask = ((unsigned long long)__ballot_sync(0xffffffffu, r1) << 32) | __ballot_sync(0xffffffffu, r0);
     asm volatile("fence.proxy.async;" ::: "memory");  // the tensor-map loads below read what the flags cover
   }
+  tc_fence_before();
+  __syncthreads();  // barriers initialised, TMEM allocated
+  tc_fence_after();
   // everything above (barriers, TMEM, tensor-map prefetch, flags) is independent of the preceding kernel
   pdl_wait();
   pdl_launch_dependents();
-
-  // the group table and the pairs' tokens go to shared memory once: a global load per unit (1 to 2 us while the GPU
-  // streams) would sit on every role's path
-  for (int i = tid; i < 4 + 3 * (N + 1); i += (int)blockDim.x) s_grp[i] = p.f.grp[i];
-  for (int i = tid; i < p.f.B * (p.f.k + 1); i += (int)blockDim.x) s_tok[i] = (uint8_t)p.f.pair_tok[i];  // (past the last pair: unused)
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = tmem_base_s;
-  const int n_g = s_grp[1];
-  // Unit list: both projections take the groups from the end of the table -- the shared expert (the widest token tiles,
-  // the longest epilogues) first, so that its epilogues overlap later units.  A group of n tokens is cut into
-  // ceil(n / nmax) parts; parts fastest, so the CTAs that share a weight block run at the same time and the second
-  // reader hits L2.  The K of a down unit is cut into equal chunks of at most kDownTiles tiles (partial sums meet in y).
-  auto k_tiles = [&](int expert) { return ((expert >= N ? I_s : I) + kKTile - 1) / kKTile; };
-  auto down_chunk = [&](int tiles) {  // K tiles per down unit; whole raw tiles
-    const int n = (tiles + (QF ? kDownTilesQ : kDownTiles) - 1) / (QF ? kDownTilesQ : kDownTiles);
-    return ((tiles + n - 1) / n + SUB - 1) / SUB * SUB;
-  };
-  if (warp == 0) {  // two prefix sums over up to 65 groups: lanes own groups 2 lane, 2 lane + 1 (and lane 0 group 64)
-    auto units = [&](int o, int phase) -> int {
-      if (o >= n_g) return 0;
-      const int g = n_g - 1 - o, e = s_grp[4 + 3 * g], n = s_grp[6 + 3 * g];
-      if (phase == 1) return ((e >= N ? I_s : I) + 127) / 128 * ((n + p.nmax1 - 1) / p.nmax1);
-      const int t = k_tiles(e), c = down_chunk(t);
-      return d / 256 * ((t + c - 1) / c) * ((n + p.nmax2 - 1) / p.nmax2);
-    };
-    for (int phase = 1; phase <= 2; ++phase) {
-      int* su = phase == 1 ? s_u1 : s_u2;
-      const int a = units(2 * lane, phase), b = units(2 * lane + 1, phase);
-      int v = a + b;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int w = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += w;
-      }
-      su[2 * lane] = v - a - b;
-      su[2 * lane + 1] = v - b;
-      if (lane == 31) {
-        su[64] = v;
-        su[65] = v + units(64, phase);
-      }
-    }
-  }
-  __syncthreads();
-  const int n1 = s_u1[APEX_MAX_EXPERTS + 1], n2 = s_u2[APEX_MAX_EXPERTS + 1];
 
   bool ok = true;
   auto give_up = [&]() {  // a wait ran out: tell the CTA, the other CTAs and the host
@@ -400,6 +368,227 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     atomicExch(p.sync + kTcAbort, 1u);
     *p.f.mbox_status = 1u;
     if (p.f.stats) atomicAdd(&p.f.stats->timeouts, 1ull);
+  };
+  // ---- The step's plan, by every CTA for itself: all of them need it, and as a kernel of its own (one cluster, then the
+  // boundary) it was 4 to 16 us before the first weight was asked for.  The weight warp meanwhile takes the first
+  // tickets: a token each, whose h' it rounds to bf16 for the gathers and whose row of y it zeroes.
+  const int B = p.f.B, k = p.f.k;
+  int ticket = 0;
+  auto unit_list_barrier = [&]() { asm volatile("bar.sync 4, %0;" ::"r"((int)blockDim.x) : "memory"); };
+  if (warp == kWWarp) {
+    ticket = lane == 0 ? (int)atomicAdd(p.sync + kTcTicket, 1u) : 0;
+    for (;;) {
+      const int t = __shfl_sync(0xffffffffu, ticket, 0);
+      if (t >= B) break;
+      if (lane == 0) ticket = (int)atomicAdd(p.sync + kTcTicket, 1u);
+      const float4* h4 = reinterpret_cast<const float4*>(p.f.hpost + (size_t)t * d);
+      float4* y4 = reinterpret_cast<float4*>(p.f.y + (size_t)t * d);
+      uint4* x4 = reinterpret_cast<uint4*>(p.xb + (size_t)t * d);
+      auto pack = [](float a, float b) {
+        const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+        return *reinterpret_cast<const uint32_t*>(&v);
+      };
+#pragma unroll 4
+      for (int i = lane; i < d / 8; i += 32) {
+        const float4 a = __ldg(h4 + 2 * i), b = __ldg(h4 + 2 * i + 1);
+        // in the order in which the converters leave the weights
+        x4[i] = QF == 2   ? make_uint4(pack(a.x, b.x), pack(a.y, b.y), pack(a.z, b.z), pack(a.w, b.w))
+                : QF == 1 ? make_uint4(pack(a.x, a.z), pack(a.y, a.w), pack(b.x, b.z), pack(b.y, b.w))
+                          : make_uint4(pack(a.x, a.y), pack(a.z, a.w), pack(b.x, b.y), pack(b.z, b.w));
+        if (!p.f.accumulate) y4[2 * i] = y4[2 * i + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+      if (p.f.run_shared && p.f.shared_gate) {
+        const float sg = shared_gate_weight(p.f.shared_gate, p.f.hpost + (size_t)t * d, d, lane);
+        if (lane == 0) p.sgate[t] = sg;
+      }
+      __syncwarp();
+      if (lane == 0) asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p.sync + kTcRows), "r"(1u) : "memory");
+    }
+    unit_list_barrier();
+  } else {
+    const int pt = tid - 32, pn = (int)blockDim.x - 32, pwarp = warp - 1, pwarps = pn / 32;
+    auto plan_barrier = [&]() { asm volatile("bar.sync 3, %0;" ::"r"(pn) : "memory"); };  // everybody but the weight warp
+    // a thread per token: K_r, the execution set (S6), the sum of its gates
+    unsigned long long kr_all = 0ull, ex_all = 0ull;
+    for (int w = pwarp; w * 32 < B; w += pwarps) {
+      const int t = w * 32 + lane;
+      const bool on = t < B;
+      int id[APEX_MAX_TOPK];
+      float al[APEX_MAX_TOPK];
+#pragma unroll
+      for (int j = 0; j < APEX_MAX_TOPK; ++j) id[j] = on && j < k ? __ldg(p.f.idx + (size_t)t * k + j) : -1;
+#pragma unroll
+      for (int j = 0; j < APEX_MAX_TOPK; ++j) al[j] = id[j] >= 0 ? __ldg(p.f.alpha + (size_t)t * N + id[j]) : 0.f;
+      unsigned long long kr = 0ull;
+      float den = 0.f;  // sum of the executed experts' weights
+#pragma unroll
+      for (int j = 0; j < APEX_MAX_TOPK; ++j) {
+        if (id[j] >= 0) kr |= 1ull << id[j];
+        den += al[j];
+      }
+      unsigned long long ex = kr;
+      const unsigned long long resident = p.f.snap.resident_mask;
+      if (on && p.f.mode == APEX_MODE_STALL_FREE && (kr & ~resident)) {
+        // Algorithm 1: the |M| best remaining resident experts by router weight, i.e. by (logit descending, index ascending)
+        ex = kr & resident;
+        unsigned long long cand = resident & ~kr;
+        const float* z = p.f.z_r + (size_t)t * N;
+        for (int miss = __popcll(kr & ~resident); miss > 0 && cand; --miss) {
+          int best = -1;
+          float zb = 0.f;
+          for (unsigned long long rest = cand; rest; rest &= rest - 1) {
+            const int e = __ffsll((long long)rest) - 1;
+            const float ze = __ldg(z + e);
+            if (best < 0 || ze > zb) {
+              best = e;
+              zb = ze;
+            }
+          }
+          ex |= 1ull << best;
+          cand &= ~(1ull << best);
+        }
+        den = 0.f;
+        for (unsigned long long rest = ex; rest; rest &= rest - 1) den += __ldg(p.f.alpha + (size_t)t * N + __ffsll((long long)rest) - 1);
+      }
+      if (!p.f.norm_topk) den = 1.f;
+      if (on) s_inv[t] = den;
+      kr_all |= kr;
+      ex_all |= ex;
+      // the transpose: lane e (and e + 32) keeps the tokens of its two experts as a 32-bit word
+      const unsigned long long rx = on ? ex & p.f.run_mask : 0ull;
+      unsigned m0 = 0u, m1 = 0u;
+#pragma unroll
+      for (int e = 0; e < 32; ++e) {
+        const unsigned a = __ballot_sync(0xffffffffu, (rx >> e) & 1), b = __ballot_sync(0xffffffffu, (rx >> (e + 32)) & 1);
+        if (lane == e) {
+          m0 = a;
+          m1 = b;
+        }
+      }
+      s_mask[lane][w] = m0;
+      s_mask[lane + 32][w] = m1;
+      if (on && blockIdx.x == 0 && p.f.post_exec) {
+        int pos = 0;
+        for (unsigned long long rest = ex; rest; rest &= rest - 1, ++pos) {
+          const int e = __ffsll((long long)rest) - 1;
+          if (p.f.exec_idx) p.f.exec_idx[(size_t)t * k + pos] = e;
+          if (p.f.exec_gate) p.f.exec_gate[(size_t)t * k + pos] = __ldg(p.f.alpha + (size_t)t * N + e) / den;
+        }
+        if (p.f.stats) {
+          const int subst = __popcll(ex & ~kr), hits = __popcll(kr & resident);
+          if (subst) atomicAdd(&p.f.stats->substitutions, (unsigned long long)subst);
+          if (hits) atomicAdd(&p.f.stats->hits_R, (unsigned long long)hits);
+        }
+      }
+    }
+    if (blockIdx.x == 0 && p.f.post_exec) {
+      atomicOr(&s_union[0], kr_all);
+      atomicOr(&s_union[1], ex_all);
+    }
+    plan_barrier();
+    if (tid == 32 && blockIdx.x == 0 && p.f.post_exec) {
+      // the unions for the host: one 16-byte store each, with the sequence number
+      const unsigned long long kr = s_union[0], ex = s_union[1];
+      asm volatile("st.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p.f.mbox_rec), "r"((uint32_t)kr), "r"((uint32_t)(kr >> 32)), "r"(p.f.seq_value), "r"(0u) : "memory");
+      asm volatile("st.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p.f.mbox_rec + 4), "r"((uint32_t)ex), "r"((uint32_t)(ex >> 32)), "r"(p.f.seq_value), "r"(0u) : "memory");
+    }
+    if (pwarp == 0) {
+      // exclusive prefix over the experts (lane owns experts lane and lane + 32), then the groups
+      int c0 = 0, c1 = 0, units_after[2][2], units_all[2];
+      for (int w = 0; w * 32 < B; ++w) {
+        c0 += __popc(s_mask[lane][w]);
+        c1 += __popc(s_mask[lane + 32][w]);
+      }
+      int i0 = c0, i1 = c1;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u0 = __shfl_up_sync(0xffffffffu, i0, o), u1 = __shfl_up_sync(0xffffffffu, i1, o);
+        if (lane >= o) {
+          i0 += u0;
+          i1 += u1;
+        }
+      }
+      const int tot0 = __shfl_sync(0xffffffffu, i0, 31), all = tot0 + __shfl_sync(0xffffffffu, i1, 31);
+      const int off0 = i0 - c0, off1 = tot0 + i1 - c1;
+      for (int w = 0, a = off0, b = off1; w * 32 < B; ++w) {  // first pair of each expert and 32 tokens
+        s_off[lane][w] = (short)a;
+        s_off[lane + 32][w] = (short)b;
+        a += __popc(s_mask[lane][w]);
+        b += __popc(s_mask[lane + 32][w]);
+      }
+      // Unit list: both projections take the groups from the end of the table -- the shared expert (the widest token tiles,
+      // the longest epilogues) first, so that its epilogues overlap later units.  A group of n tokens is cut into parts;
+      // parts fastest, so the CTAs that share a weight block run at the same time and the second reader hits L2.  The K of
+      // a down unit is cut into equal chunks of at most kDownTiles tiles (partial sums meet in y).  s_u[q][g]: the units of
+      // the groups after g; the units of group g end at s_u[q][g - 1].
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int per = q == 0 ? p.geo[0].blocks1 : (d >> 8) * p.geo[0].kch, round = (1 << (q == 0 ? p.shift1 : p.shift2)) - 1;
+        const int sh = q == 0 ? p.shift1 : p.shift2;
+        const int a = per * ((c0 + round) >> sh), b = per * ((c1 + round) >> sh);
+        int va = a, vb = b;  // suffix sums over the experts
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int u0 = __shfl_down_sync(0xffffffffu, va, o), u1 = __shfl_down_sync(0xffffffffu, vb, o);
+          if (lane + o < 32) {
+            va += u0;
+            vb += u1;
+          }
+        }
+        const int tb = __shfl_sync(0xffffffffu, vb, 0);
+        const int sh_units = p.f.run_shared ? (q == 0 ? p.geo[1].blocks1 : (d >> 8) * p.geo[1].kch) * ((B + round) >> sh) : 0;
+        units_after[q][0] = sh_units + tb + va - a;
+        units_after[q][1] = sh_units + vb - b;
+        units_all[q] = sh_units + tb + __shfl_sync(0xffffffffu, va, 0);
+      }
+      const unsigned g0m = __ballot_sync(0xffffffffu, c0 > 0), g1m = __ballot_sync(0xffffffffu, c1 > 0);
+      const int n_routed = __popc(g0m) + __popc(g1m);
+      auto put = [&](int g, int expert, int off, int n, int u1, int u2) {
+        s_grp[g] = GroupDesc{expert, off, n};
+        s_u[0][g] = u1;
+        s_u[1][g] = u2;
+      };
+      if (c0 > 0) put(__popc(g0m & ((1u << lane) - 1u)), lane, off0, c0, units_after[0][0], units_after[1][0]);
+      if (c1 > 0) put(__popc(g0m) + __popc(g1m & ((1u << lane) - 1u)), lane + 32, off1, c1, units_after[0][1], units_after[1][1]);
+      if (lane == 0) {
+        if (p.f.run_shared) put(n_routed, N, all, B, 0, 0);
+        s_units[0] = units_all[0];
+        s_units[1] = units_all[1];
+      }
+    }
+    unit_list_barrier();  // the ticket taker may go on
+    // the pair list, sorted by (expert, token)
+    for (int e = pt >> 3; e < N; e += pn >> 3) {
+      const int w = pt & 7;
+      if (w * 32 >= B) continue;
+      int o = s_off[e][w];
+      for (unsigned m = s_mask[e][w]; m; m &= m - 1) s_tok[o++] = (uint8_t)(w * 32 + __ffs((int)m) - 1);
+    }
+    if (p.f.run_shared && pt < 32) {
+      int at = 0;  // the shared expert's pairs follow all others
+      for (int w = 0; w * 32 < B; ++w) at += __popc(s_mask[lane][w]) + __popc(s_mask[lane + 32][w]);
+      at = (int)__reduce_add_sync(0xffffffffu, (unsigned)at);
+      for (int t = lane; t < B; t += 32) s_tok[at + t] = (uint8_t)t;
+    }
+    plan_barrier();
+  }
+  const uint32_t tmem_base = tmem_base_s;
+  const int n1 = s_units[0], n2 = s_units[1];
+
+  // a count that other CTAs raise (one thread; bounded)
+  auto wait_count = [&](const unsigned* ctr, unsigned want) -> bool {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
+    if (v >= want) return true;
+    const unsigned long long t0 = globaltimer_ns();
+    for (uint32_t n_poll = 1; v < want; ++n_poll) {
+      if ((n_poll & 31u) == 0u && (*(volatile int*)&s_abort || *(volatile unsigned*)(p.sync + kTcAbort) ||
+                                   (long long)(globaltimer_ns() - t0) > p.f.wait_limit_ns))
+        return false;
+      __nanosleep(40);
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
+    }
+    return true;
   };
   // the descriptor of this role's n-th unit; phase 0 at the end of the list and after an abort
   auto next_unit = [&](uint32_t n) -> UnitDesc {
@@ -420,33 +609,34 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     // The next ticket is taken a ring's depth before the end of a unit: the answer is there when the unit's last load has
     // been issued (taken only then, it left the ring empty for 1.5 us per unit), and no unit waits long for its CTA.
     const int ahead = (QF ? NR : NS) * SUB;
-    int ticket = lane == 0 ? (int)atomicAdd(p.sync + kTcTicket, 1u) : 0;
+    // (lane 0 holds one from the rows above)
     for (uint32_t n = 0; ok; ++n) {
-      const int t = __shfl_sync(0xffffffffu, ticket, 0);
+      const int t = __shfl_sync(0xffffffffu, ticket, 0) - B;
       bool taken = false;
       UnitDesc ud = {};
       if (t < n1 + n2) {
         const bool down = t >= n1;
         const int u = down ? t - n1 : t;
-        const int* su = down ? s_u2 : s_u1;
-        // order index of the group: the number of groups that end at or before u
-        const int o = __popc(__ballot_sync(0xffffffffu, su[lane + 1] <= u)) + __popc(__ballot_sync(0xffffffffu, su[lane + 33] <= u)) +
-                      (su[65] <= u ? 1 : 0);
-        const int g = n_g - 1 - o, nt = s_grp[6 + 3 * g], nmax = down ? p.nmax2 : p.nmax1;
-        const int parts = (nt + nmax - 1) / nmax;
-        int local = u - su[o];
-        const int part = local % parts;
-        local /= parts;
+        const int* su = s_u[down ? 1 : 0];
+        // the group: the first one (in table order) whose units begin at or before u.  Entries fall along the table
+        const unsigned m0 = __ballot_sync(0xffffffffu, su[lane] <= u), m1 = __ballot_sync(0xffffffffu, su[lane + 32] <= u);
+        const int g = m0 ? __ffs((int)m0) - 1 : m1 ? 31 + __ffs((int)m1) : 64;
+        const GroupDesc gr = s_grp[g];
+        const int sh = down ? p.shift2 : p.shift1, nmax = down ? p.nmax2 : p.nmax1;
+        const int parts = (gr.n_tok + (1 << sh) - 1) >> sh;  // (at most four)
+        const uint32_t parts_inv = parts == 2 ? 0x80000000u : parts == 3 ? 0x55555556u : 0x40000000u;
+        const int rest = u - su[g];
+        const int local = parts == 1 ? rest : (int)__umulhi((uint32_t)rest, parts_inv), part = rest - local * parts;
+        const TcGeometry& geo = p.geo[gr.expert >= N ? 1 : 0];
         ud.phase = down ? 2 : 1;
         ud.group = g;
-        ud.expert = s_grp[4 + 3 * g];
-        ud.pair_off = s_grp[5 + 3 * g] + part * nmax;
-        ud.n_tok = nt - part * nmax < nmax ? nt - part * nmax : nmax;
+        ud.expert = gr.expert;
+        ud.pair_off = gr.pair_off + part * nmax;
+        ud.n_tok = min(gr.n_tok - part * nmax, nmax);
         if (down) {
-          const int tiles = k_tiles(ud.expert), c = down_chunk(tiles), kch = (tiles + c - 1) / c;
-          ud.blk = local / kch;
-          ud.kt_begin = local % kch * c;
-          ud.kt_end = ud.kt_begin + c < tiles ? ud.kt_begin + c : tiles;
+          ud.blk = geo.kch == 1 ? local : (int)__umulhi((uint32_t)local, geo.kch_inv);
+          ud.kt_begin = (local - ud.blk * geo.kch) * geo.chunk;
+          ud.kt_end = min(ud.kt_begin + geo.chunk, geo.tiles);
         } else {
           ud.blk = local;
           ud.kt_end = d / kKTile;
@@ -544,25 +734,12 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
       if (ud.phase == 1) {  // lane j: rows 4 j .. 4 j + 3 (past the last token: any row, the result is not used)
 #pragma unroll
         for (int i = 0; i < 4; ++i) tok[i] = s_tok[ud.pair_off + min(4 * lane + i, ud.n_tok - 1)];
-      } else {
-        // the group's intermediate must be complete: every gate/up unit of the group has been counted in
+      }
+      // what is loaded must be complete: the rows of X (once), or every gate/up unit of the group
+      if (ud.phase == 2 || n == 0) {
         if (lane == 0) {
-          const unsigned want = (unsigned)(((ud.expert >= N ? I_s : I) + 127) / 128 * ((s_grp[6 + 3 * ud.group] + p.nmax1 - 1) / p.nmax1));
-          const unsigned* done = p.sync + kTcDone + ud.group;
-          unsigned v;
-          asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(done) : "memory");
-          if (v < want) {
-            const unsigned long long t0 = globaltimer_ns();
-            for (uint32_t n_poll = 1; v < want; ++n_poll) {
-              if ((n_poll & 31u) == 0u && (*(volatile int*)&s_abort || *(volatile unsigned*)(p.sync + kTcAbort) ||
-                                           (long long)(globaltimer_ns() - t0) > p.f.wait_limit_ns)) {
-                ok = false;
-                break;
-              }
-              __nanosleep(40);
-              asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(done) : "memory");
-            }
-          }
+          const unsigned want = ud.phase == 1 ? (unsigned)B : (unsigned)(p.geo[ud.expert >= N ? 1 : 0].blocks1 * ((s_grp[ud.group].n_tok + (1 << p.shift1) - 1) >> p.shift1));
+          if (!wait_count(p.sync + (ud.phase == 1 ? kTcRows : kTcDone + ud.group), want)) ok = false;
           asm volatile("fence.proxy.async;" ::: "memory");  // the bulk loads below read what other CTAs' threads have stored
         }
         ok = __all_sync(0xffffffffu, ok);
@@ -749,23 +926,31 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     if (!ok && lane == 0) atomicExch(&s_abort, 1);
   } else {
     // ================= epilogue: warp w owns TMEM lanes 32*(w%4) .. +31
-    if (warp == kEpiWarp0 && blockIdx.x == 0 && lane == 0 && p.f.post_exec) {
-      // the unions of the routed and of the execution sets for the host: one 16-byte store each, with the sequence number
-      const unsigned long long kr = p.plan_masks[0], ex = p.plan_masks[1];
-      asm volatile("st.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p.f.mbox_rec), "r"((uint32_t)kr), "r"((uint32_t)(kr >> 32)), "r"(p.f.seq_value), "r"(0u) : "memory");
-      asm volatile("st.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p.f.mbox_rec + 4), "r"((uint32_t)ex), "r"((uint32_t)(ex >> 32)), "r"(p.f.seq_value), "r"(0u) : "memory");
-    }
     const int quad = warp & 3;
     const int row = quad * 32 + lane;  // row of the 128-row tile
     AccBuffers acc;
+    bool rows_seen = false;  // every row of y has been zeroed (and the shared expert's gates are there)
     for (uint32_t n = 0;; ++n) {
       const UnitDesc ud = next_unit(n);
       if (ud.phase == 0) break;
+      if (!rows_seen) {
+        if (!__shfl_sync(0xffffffffu, lane == 0 ? (wait_count(p.sync + kTcRows, (unsigned)B) ? 1 : 0) : 0, 0)) {
+          if (lane == 0) give_up();
+          break;
+        }
+        rows_seen = true;
+      }
       const bool shared = ud.expert >= N;
       const bool wide = unit_is_wide<QF>(ud);
       const uint32_t b0 = wide ? 0u : acc.next, b1 = wide ? 1u : acc.next;
       // the pairs' weights, sixteen at a time, asked for before the wait and then one batch ahead
-      auto load_gates = [&](int c0) { return ud.phase == 1 && c0 + (lane & 15) < ud.n_tok ? __ldg(p.f.pair_gate + ud.pair_off + c0 + (lane & 15)) : 0.f; };
+      auto load_gates = [&](int c0) {
+        const int c = c0 + (lane & 15);
+        if (ud.phase != 1 || c >= ud.n_tok) return 0.f;
+        const int t = s_tok[ud.pair_off + c];
+        if (shared) return p.f.shared_gate ? __ldcg(p.sgate + t) : 1.f;
+        return __ldg(p.f.alpha + (size_t)t * N + ud.expert) / s_inv[t];
+      };
       float gates_next = load_gates(0);
       bool landed = true;
       for (uint32_t b = b0; b <= b1; ++b) landed = landed && mbar_wait(&tmem_full[b], acc.uses[b]++ & 1, &s_abort, p.f.wait_limit_ns);
@@ -848,6 +1033,13 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     while (globaltimer_ns() - t0 < 1000000ull) __nanosleep(1000);
     __syncthreads();
   }
+  if (tid == 0) {  // the last CTA leaves the counters zero for the next launch (which waits for this one)
+    __threadfence();
+    if (atomicAdd(p.sync + kTcExits, 1u) == gridDim.x - 1) {
+      for (int i = 0; i < kTcSyncWords; ++i) p.sync[i] = 0u;
+      __threadfence();
+    }
+  }
   if (warp == kMmaWarp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
   SPAN_END(8);
 }
@@ -912,7 +1104,7 @@ bool tc_make_store_maps(int fmt, void* weights, void* scales, const void* base, 
 }
 
 namespace {
-constexpr int kTcSmemBudget = 216 * 1024;  // rings of a CTA, 1 KB of alignment included
+constexpr int kTcSmemBudget = 215 * 1024;  // rings of a CTA, 1 KB of alignment included
 
 template <int QF>
 cudaError_t launch_tc(const TcParams& p, const TcMaps& m, cudaLaunchConfig_t& cfg) {
@@ -944,6 +1136,19 @@ cudaError_t launch_ffn_tc(const TcParams& p_in, const TcMaps& m, int n_sm, cudaS
   const int b16 = (p.f.B + 15) & ~15;
   p.nmax1 = b16 < 128 ? b16 : 128;
   p.nmax2 = b16 < 64 ? b16 : 64;
+  p.shift1 = p.f.B <= p.nmax1 ? 20 : 7;  // (more tokens than a unit takes: the unit takes 128 or 64)
+  p.shift2 = p.f.B <= p.nmax2 ? 20 : 6;
+  for (int q = 0; q < 2; ++q) {
+    TcGeometry& g = p.geo[q];
+    const int rows = q ? p.f.I_shared : p.f.I, most = qf ? kDownTilesQ : kDownTiles, sub = tc_sub(qf);
+    g.blocks1 = (rows + 127) / 128;
+    g.tiles = (rows + kKTile - 1) / kKTile;
+    if (!g.tiles) continue;
+    const int n = (g.tiles + most - 1) / most;
+    g.chunk = ((g.tiles + n - 1) / n + sub - 1) / sub * sub;  // whole raw tiles
+    g.kch = (g.tiles + g.chunk - 1) / g.chunk;
+    g.kch_inv = g.kch > 1 ? (uint32_t)((0x100000000ull + g.kch - 1) / g.kch) : 0u;
+  }
   const int b_bytes = p.nmax1 * 128 > 2 * p.nmax2 * 128 ? p.nmax1 * 128 : 2 * p.nmax2 * 128;
   p.stage_bytes = kABytes + ((b_bytes + 1023) & ~1023);
   const int budget = kTcSmemBudget - 1024;

@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(256) router_kernel(const RouterParams p) {
 }
 
 // The same for a batch (B > 1): a cluster takes TT tokens, its CTA r the experts r * wpc .. r * wpc + wpc - 1 (wpc <= 8).
-// Rows of W and of x come into shared memory by bulk copies in chunks of kChunk columns, two buffers (the W rows are
+// Rows of W and of x come into shared memory by bulk copies in chunks of 512 or 1024 columns, two buffers (the W rows are
 // parameters and are asked for before the dependency wait).  A warp takes a tile of tokens x experts with its lanes along
 // the columns: per (token, expert) every lane runs the multiply-add chain of router_kernel and the lanes are added by the
 // same xor tree -- halving the set of values a lane keeps at every level, which pairs the same partial sums -- so the
@@ -113,7 +113,9 @@ __global__ void __launch_bounds__(256) router_kernel(const RouterParams p) {
 //
 // Bound by latency: two rounds of loads, 16 multiply-adds per lane, token and expert at d = 2048, one cluster barrier, a
 // serial epilogue.  As one token per pass over register-held rows it took 29 us at B = 256, N = 60, d = 2048.
-constexpr int kChunk = 1024;
+// columns per chunk: with 512 two of the largest CTAs share an SM (a GPU holds 15 clusters of eight CTAs, one to an SM, and
+// 16 are needed at B = 256: the last one ran behind the others)
+__host__ __device__ constexpr int router_chunk(int tt) { return tt >= 16 ? 512 : 1024; }
 constexpr int kRouterWarps = 8;
 
 __host__ __device__ constexpr int router_tile_tok(int tt) { return tt < 4 ? tt : 4; }
@@ -125,32 +127,33 @@ __global__ void __launch_bounds__(kRouterWarps * 32, 2) router_batched_kernel(co
   cg::cluster_group cluster = cg::this_cluster();
   const unsigned crank = cluster.block_rank(), csize = cluster.num_blocks();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int CH = router_chunk(TT);
   constexpr int NT = router_tile_tok(TT), NX = router_tile_exp(TT);
   __shared__ float zs[TT][APEX_MAX_EXPERTS];   // tokens finished here (at most all of them)
   __shared__ float qs[kRouterWarps][APEX_MAX_EXPERTS];
   __shared__ int pis[kRouterWarps][APEX_MAX_EXPERTS];
   __shared__ int posp[kRouterWarps][APEX_MAX_EXPERTS];
   __shared__ uint64_t s_bar[2];
-  extern __shared__ __align__(128) float tiles[];  // [2][TT + 8][kChunk]: x rows, W rows
+  extern __shared__ __align__(128) float tiles[];  // [2][TT + 8][CH]: x rows, W rows
   const int b0 = blockIdx.y * TT, nt = min(TT, p.B - b0);
   const int e0 = (int)crank * p.warps_per_cta, ne = max(0, min(p.warps_per_cta, p.N - e0));
-  const int n_chunks = (p.d + kChunk - 1) / kChunk;
+  const int n_chunks = (p.d + CH - 1) / CH;
   if (threadIdx.x == 0) {
     mbar_init(&s_bar[0], 2);
     mbar_init(&s_bar[1], 2);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  auto chunk_bytes = [&](int c) { return (uint32_t)(min(kChunk, p.d - c * kChunk) * 4); };
+  auto chunk_bytes = [&](int c) { return (uint32_t)(min(CH, p.d - c * CH) * 4); };
   auto load_w = [&](int c) {  // warp 0
     if (lane == 0) mbar_expect_tx(&s_bar[c & 1], ne * chunk_bytes(c));
     __syncwarp();
-    if (lane < ne) bulk_g2s(tiles + ((c & 1) * (TT + 8) + TT + lane) * kChunk, p.W + (size_t)(e0 + lane) * p.d + c * kChunk, chunk_bytes(c), &s_bar[c & 1]);
+    if (lane < ne) bulk_g2s(tiles + ((c & 1) * (TT + 8) + TT + lane) * CH, p.W + (size_t)(e0 + lane) * p.d + c * CH, chunk_bytes(c), &s_bar[c & 1]);
   };
   auto load_x = [&](int c) {
     if (lane == 0) mbar_expect_tx(&s_bar[c & 1], nt * chunk_bytes(c));
     __syncwarp();
-    if (lane < nt) bulk_g2s(tiles + ((c & 1) * (TT + 8) + lane) * kChunk, p.x + (size_t)(b0 + lane) * p.d + c * kChunk, chunk_bytes(c), &s_bar[c & 1]);
+    if (lane < nt) bulk_g2s(tiles + ((c & 1) * (TT + 8) + lane) * CH, p.x + (size_t)(b0 + lane) * p.d + c * CH, chunk_bytes(c), &s_bar[c & 1]);
   };
   if (warp == 0)
     for (int c = 0; c < 2 && c < n_chunks; ++c) load_w(c);
@@ -174,16 +177,16 @@ __global__ void __launch_bounds__(kRouterWarps * 32, 2) router_batched_kernel(co
   for (int c = 0; c < n_chunks; ++c) {
     mbar_wait(&s_bar[c & 1], (c >> 1) & 1, nullptr, 2000000000ll);
     if (active) {
-      const int nv = min(kChunk, p.d - c * kChunk) >> 2;
-      const float4* xt = reinterpret_cast<const float4*>(tiles + ((c & 1) * (TT + 8) + t0) * kChunk) + lane;
-      const float4* wt = reinterpret_cast<const float4*>(tiles + ((c & 1) * (TT + 8) + TT + x0) * kChunk) + lane;
+      const int nv = min(CH, p.d - c * CH) >> 2;
+      const float4* xt = reinterpret_cast<const float4*>(tiles + ((c & 1) * (TT + 8) + t0) * CH) + lane;
+      const float4* wt = reinterpret_cast<const float4*>(tiles + ((c & 1) * (TT + 8) + TT + x0) * CH) + lane;
       auto step = [&](int i) {
         float4 xv[NT];
 #pragma unroll
-        for (int t = 0; t < NT; ++t) xv[t] = xt[t * (kChunk / 4) + i];
+        for (int t = 0; t < NT; ++t) xv[t] = xt[t * (CH / 4) + i];
 #pragma unroll
         for (int x = 0; x < NX; ++x) {
-          const float4 wv = wt[x * (kChunk / 4) + i];
+          const float4 wv = wt[x * (CH / 4) + i];
 #pragma unroll
           for (int t = 0; t < NT; ++t) {
             float a = acc[x * NT + t];
@@ -257,7 +260,7 @@ __global__ void __launch_bounds__(kRouterWarps * 32, 2) router_batched_kernel(co
 
 template <int TT>
 cudaError_t launch_router_batched(const RouterParams& p, cudaLaunchConfig_t& cfg, int csize) {
-  constexpr int smem = 2 * (TT + 8) * kChunk * (int)sizeof(float);
+  constexpr int smem = 2 * (TT + 8) * router_chunk(TT) * (int)sizeof(float);
   static bool configured[kMaxDevices];
   static std::mutex setup_mutex;  // contexts of several host threads (and the context-free gate) share this set-up
   int dev = 0;
@@ -271,6 +274,7 @@ cudaError_t launch_router_batched(const RouterParams& p, cudaLaunchConfig_t& cfg
       configured[dev] = true;
     }
   }
+  prefer_max_shared<router_batched_kernel<TT>>();
   cfg.gridDim = dim3(csize, (p.B + TT - 1) / TT, 1);
   cfg.dynamicSmemBytes = smem;
   return cudaLaunchKernelEx(&cfg, router_batched_kernel<TT>, p);
@@ -296,10 +300,13 @@ cudaError_t launch_router(const RouterParams& p, cudaStream_t s) {
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  if (p.B == 1) return cudaLaunchKernelEx(&cfg, router_kernel, q);
-  // Tokens per cluster: as few as let all clusters run at once on 148 SMs (18 clusters of eight CTAs), since a cluster's
-  // time grows with its tokens; at most 16
-  const int clusters = 144 / csize;
+  if (p.B == 1) {
+    prefer_max_shared<router_kernel>();
+    return cudaLaunchKernelEx(&cfg, router_kernel, q);
+  }
+  // Tokens per cluster: as few as let all clusters run at once (15 of eight CTAs), since a cluster's time grows with its
+  // tokens; at most 16
+  const int clusters = 120 / csize;
   if (p.B <= clusters) return launch_router_batched<1>(q, cfg, csize);
   if (p.B <= 2 * clusters) return launch_router_batched<2>(q, cfg, csize);
   if (p.B <= 4 * clusters) return launch_router_batched<4>(q, cfg, csize);
@@ -335,6 +342,7 @@ __global__ void __launch_bounds__(128) select_kernel(const SelectParams p) {
 }
 
 cudaError_t launch_select(const SelectParams& p, cudaStream_t s) {
+  prefer_max_shared<select_kernel>();
   const int wpb = 4;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((p.B + wpb - 1) / wpb, 1, 1);
@@ -380,6 +388,7 @@ __global__ void __launch_bounds__(512) attention_standin_kernel(const AttnParams
 }
 
 cudaError_t launch_attention(const AttnParams& p, int n_sm, cudaStream_t s) {
+  prefer_max_shared<attention_standin_kernel>();
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(n_sm * 2, 1, 1);
   cfg.blockDim = dim3(512, 1, 1);

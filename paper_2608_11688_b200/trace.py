@@ -25,10 +25,7 @@ KERNEL_NAMES = {
     3: "attention stand-in",
     4: "gate",
     5: "expert FFN, streaming",
-    6: "FFN plan (B > 1)",
-    7: "gather (B > 1)",
-    8: "gate/up GEMM (B > 1)",
-    9: "down GEMM (B > 1)",
+    8: "expert FFN, grouped GEMM (B > 1)",
     10: "persistent token kernel (all layers, B = 1)",
 }
 LOG_RECORDS = 4096
