@@ -1,5 +1,8 @@
 """ctypes binding of libapex.so: the same names as the C entry points, argument marshalling only.
 
+The calls of the decode step go through a small extension module (``_pycall``, csrc/pycall.c) that marshals in C; the
+others through ctypes.
+
 Device buffers are torch CUDA tensors (``data_ptr()``), streams are ``torch.cuda.Stream`` objects
 (or None for the current stream).  There is no CPU fallback: loading fails loudly when the
 library has not been built.
@@ -7,13 +10,18 @@ library has not been built.
 from __future__ import annotations
 
 import ctypes as C
+import importlib.machinery
+import importlib.util
 import os
+import sys
+import threading
 from typing import Optional
 
 import numpy as np
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libapex.so")
+PYCALL_PATH = os.path.join(_HERE, "_pycall.so")
 
 APEX_OK, APEX_EINVAL, APEX_ENOMEM, APEX_ECUDA, APEX_ETIMEOUT, APEX_ESTATE, APEX_ENOTIMPL = 0, -1, -2, -3, -4, -5, -6
 MODE_EXACT, MODE_STALL_FREE = 0, 1
@@ -92,7 +100,38 @@ SIGNATURES = {
     "apex_slots_set": (_I, [_P, _P, _P, C.c_int64]),
 }
 
+# the calls of the decode step: signature in the notation of csrc/pycall.c
+FAST = {
+    "apex_predict": "iipis", "apex_select_candidates": "iiifpps", "apex_prefetch": "iiii", "apex_attention_standin": "iis",
+    "apex_route_topk": "iipipps", "apex_moe_ffn": "iiipippps", "apex_moe_ffn_begin": "iiipippps", "apex_moe_ffn_end": "ii",
+    "apex_decode_token": "ippifips", "apex_decode_token_host": "ippifips", "apex_route_topk_static": "pppiiiippsii",
+}
 _lib = None
+_fast = {}       # name -> callable
+_pycall = None
+
+
+def _setup_pycall(with_stream=False):
+    """Hands the extension module torch's types and getters (what there is of them yet: torch may be imported later)."""
+    torch = sys.modules.get("torch")
+    tensor = getattr(torch, "Tensor", None)
+    c = getattr(torch, "_C", None) if with_stream else None
+    raw, dev = getattr(c, "_cuda_getCurrentRawStream", None), getattr(c, "_cuda_getDevice", None)
+    if raw is None or dev is None:
+        raw = dev = None
+    _pycall.setup(_ptr, _stream, tensor, raw, dev)
+
+
+def _load_pycall(lib):
+    global _pycall
+    if not os.path.exists(PYCALL_PATH):
+        raise RuntimeError(f"{PYCALL_PATH} not found: build it with `python -m paper_2608_11688_b200.build`")
+    loader = importlib.machinery.ExtensionFileLoader("_pycall", PYCALL_PATH)
+    _pycall = importlib.util.module_from_spec(importlib.util.spec_from_loader("_pycall", loader))
+    loader.exec_module(_pycall)
+    _setup_pycall()
+    for name, sig in FAST.items():
+        _fast[name] = _pycall.make(C.cast(getattr(lib, name), C.c_void_p).value, sig)
 
 
 def load_library(path: str = LIB_PATH) -> C.CDLL:
@@ -108,6 +147,7 @@ def load_library(path: str = LIB_PATH) -> C.CDLL:
         fn = getattr(lib, name)
         fn.restype = res
         fn.argtypes = args
+    _load_pycall(lib)
     _lib = lib
     return lib
 
@@ -132,7 +172,9 @@ def _ptr(t) -> Optional[int]:
 def _stream(s) -> Optional[int]:
     if s is None:
         import torch
-        return torch.cuda.current_stream().cuda_stream
+        stream = torch.cuda.current_stream().cuda_stream
+        _setup_pycall(with_stream=True)   # CUDA is initialised from here on
+        return stream
     if isinstance(s, int):
         return s
     return s.cuda_stream
@@ -152,6 +194,7 @@ class Apex:
         if rc != APEX_OK:
             raise ApexError(rc, self.lib.apex_last_error(None).decode() or "apex_create failed")
         self.h = h
+        self._h = h.value
         self._keep = []   # borrowed buffers that must outlive the context
 
     # -- plumbing
@@ -163,7 +206,7 @@ class Apex:
     def destroy(self):
         if getattr(self, "h", None):
             self.lib.apex_destroy(self.h)
-            self.h = None
+            self.h, self._h = None, 0
             self._keep = []
 
     def __del__(self):
@@ -208,26 +251,35 @@ class Apex:
 
     # -- the layer-step
     def predict(self, layer, h_dev, B, stream=None):
-        self._chk(self.lib.apex_predict(self.h, layer, _ptr(h_dev), B, _stream(stream)))
+        rc = _fast["apex_predict"](self._h, layer, h_dev, B, stream)
+        if rc:
+            self._chk(rc)
 
     def select_candidates(self, layer, B, tau, cand_dev, ncand_dev, stream=None):
-        self._chk(self.lib.apex_select_candidates(self.h, layer, B, float(tau), _ptr(cand_dev), _ptr(ncand_dev),
-                                                  _stream(stream)))
+        rc = _fast["apex_select_candidates"](self._h, layer, B, tau, cand_dev, ncand_dev, stream)
+        if rc:
+            self._chk(rc)
 
     def prefetch(self, layer, B, copy_stream=None):
-        self._chk(self.lib.apex_prefetch(self.h, layer, B, None if copy_stream is None else _stream(copy_stream)))
+        rc = _fast["apex_prefetch"](self._h, layer, B, 0 if copy_stream is None else _stream(copy_stream))
+        if rc:
+            self._chk(rc)
 
     def attention_standin(self, layer, stream=None):
-        self._chk(self.lib.apex_attention_standin(self.h, layer, _stream(stream)))
+        rc = _fast["apex_attention_standin"](self._h, layer, stream)
+        if rc:
+            self._chk(rc)
 
     def route_topk(self, layer, hpost_dev, B, idx_dev, alpha_dev, stream=None):
-        self._chk(self.lib.apex_route_topk(self.h, layer, _ptr(hpost_dev), B, _ptr(idx_dev), _ptr(alpha_dev),
-                                           _stream(stream)))
+        rc = _fast["apex_route_topk"](self._h, layer, hpost_dev, B, idx_dev, alpha_dev, stream)
+        if rc:
+            self._chk(rc)
 
     def moe_ffn(self, layer, mode, hpost_dev, B, y_dev, exec_idx_dev=None, exec_gate_dev=None, stream=None):
         m = MODES[mode] if isinstance(mode, str) else mode
-        self._chk(self.lib.apex_moe_ffn(self.h, layer, m, _ptr(hpost_dev), B, _ptr(y_dev), _ptr(exec_idx_dev),
-                                        _ptr(exec_gate_dev), _stream(stream)))
+        rc = _fast["apex_moe_ffn"](self._h, layer, m, hpost_dev, B, y_dev, exec_idx_dev, exec_gate_dev, stream)
+        if rc:
+            self._chk(rc)
 
     def moe_ffn_begin_raw(self, layer, mode_int, hpost_ptr, B, y_ptr, stream_int):
         """apex_moe_ffn_begin with raw addresses (no per-call marshalling): for tight timing loops."""
@@ -237,21 +289,26 @@ class Apex:
 
     def moe_ffn_begin(self, layer, mode, hpost_dev, B, y_dev, exec_idx_dev=None, exec_gate_dev=None, stream=None):
         m = MODES[mode] if isinstance(mode, str) else mode
-        self._chk(self.lib.apex_moe_ffn_begin(self.h, layer, m, _ptr(hpost_dev), B, _ptr(y_dev), _ptr(exec_idx_dev),
-                                              _ptr(exec_gate_dev), _stream(stream)))
+        rc = _fast["apex_moe_ffn_begin"](self._h, layer, m, hpost_dev, B, y_dev, exec_idx_dev, exec_gate_dev, stream)
+        if rc:
+            self._chk(rc)
 
     def moe_ffn_end(self, layer):
-        self._chk(self.lib.apex_moe_ffn_end(self.h, layer))
+        rc = _fast["apex_moe_ffn_end"](self._h, layer)
+        if rc:
+            self._chk(rc)
 
     def decode_token(self, h_dev, hpost_dev, B, tau, mode, y_dev, stream=None):
         m = MODES[mode] if isinstance(mode, str) else mode
-        self._chk(self.lib.apex_decode_token(self.h, _ptr(h_dev), _ptr(hpost_dev), B, float(tau), m, _ptr(y_dev),
-                                             _stream(stream)))
+        rc = _fast["apex_decode_token"](self._h, h_dev, hpost_dev, B, tau, m, y_dev, stream)
+        if rc:
+            self._chk(rc)
 
     def decode_token_host(self, h_host, hpost_host, B, tau, mode, y_host, stream=None):
         m = MODES[mode] if isinstance(mode, str) else mode
-        self._chk(self.lib.apex_decode_token_host(self.h, _ptr(h_host), _ptr(hpost_host), B, float(tau), m,
-                                                  _ptr(y_host), _stream(stream)))
+        rc = _fast["apex_decode_token_host"](self._h, h_host, hpost_host, B, tau, m, y_host, stream)
+        if rc:
+            self._chk(rc)
 
     # -- observation
     def get_stats(self, layer=-1):
@@ -300,14 +357,24 @@ def route_topk_static(W_r_dev, b_r_dev, hpost_dev, k, idx_dev, alpha_dev, stream
     """apex_route_topk_static: the gate without a context and without any allocation.  W_r_dev [N][d],
     b_r_dev [N] or None, hpost_dev [B][d] are CUDA tensors; idx_dev [B][k] int32 and alpha_dev [B][N]
     fp32 receive the result.  Raises ApexError with the library's message on failure."""
-    lib = load_library()
+    load_library()
     N, d = W_r_dev.shape
-    B = hpost_dev.shape[0]
-    err = C.create_string_buffer(256)
-    rc = lib.apex_route_topk_static(_ptr(W_r_dev), _ptr(b_r_dev), _ptr(hpost_dev), N, d, k, B, _ptr(idx_dev),
-                                    _ptr(alpha_dev), _stream(stream), err, len(err))
-    if rc != APEX_OK:
-        raise ApexError(rc, err.value.decode())
+    err = _err_buffer()
+    rc = _fast["apex_route_topk_static"](W_r_dev, b_r_dev, hpost_dev, N, d, k, hpost_dev.shape[0], idx_dev, alpha_dev, stream, err[1], 256)
+    if rc:
+        raise ApexError(rc, err[0].value.decode())
+
+
+_tls = threading.local()
+
+
+def _err_buffer():
+    """(ctypes buffer of 256 bytes, its address), one per thread."""
+    err = getattr(_tls, "err", None)
+    if err is None:
+        buf = C.create_string_buffer(256)
+        err = _tls.err = (buf, C.addressof(buf))
+    return err
 
 
 def fit_cdf(X_dev, dstar_dev, k, iters=600, lr=0.05, stream=None):

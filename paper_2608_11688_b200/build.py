@@ -4,10 +4,12 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libapex.so")
+PYCALL = os.path.join(HERE, "_pycall.so")            # argument marshalling of the Python binding (csrc/pycall.c)
 TRACE_LIB = os.path.join(HERE, "libapex_trace.so")   # the same sources with the kernels' time stamps compiled in (trace.py)
 SOURCES = ["apex_ctx.cu", "apex_step.cu", "apex_observe.cu", "apex_decode.cu", "kernels_decode.cu", "kernels_router.cu", "kernels_ffn.cu", "kernels_ffn_tc.cu", "apex_noalloc.cu", "fit_cdf.cu", "distill.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -25,12 +27,27 @@ def _stale(lib: str = LIB) -> bool:
     if not os.path.exists(lib):
         return True
     t = os.path.getmtime(lib)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(HERE, "..", "include", "apex.h")]
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cu", ".cuh", ".hpp"))] + [os.path.join(HERE, "..", "include", "apex.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def build_pycall(force: bool = False) -> str:
+    """The binding's extension module (C, CPython API)."""
+    src = os.path.join(CSRC, "pycall.c")
+    if not force and os.path.exists(PYCALL) and os.path.getmtime(src) <= os.path.getmtime(PYCALL):
+        return PYCALL
+    cmd = [os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I" + sysconfig.get_paths()["include"], src, "-o", PYCALL]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        sys.stderr.write(r.stdout + r.stderr)
+        raise RuntimeError("the compiler failed on pycall.c")
+    return PYCALL
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compiles every .cu of the package for sm_100a and links libapex.so.  Returns its path."""
+    """Compiles every .cu of the package for sm_100a and links libapex.so (and builds the binding's extension module).
+    Returns its path."""
+    build_pycall(force)
     if not force and not _stale():
         return LIB
     flags = [f for f in NVCC_FLAGS if not f.startswith("--use_fast_math")]

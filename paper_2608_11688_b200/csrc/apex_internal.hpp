@@ -97,6 +97,8 @@ struct RouterParams {
   const int32_t* pi_pred;     // [B][N] ranking of the prefetch router for this step, or null
   const int32_t* ncand_pred;  // [B]
   DevStats* stats;
+  uint32_t* mbox_rec;  // mapped host, B == 1: {routed set lo, hi, sequence number, 0} in one 16-byte store, or null
+  uint32_t seq_value;
   int C;
   int fuse_select;   // 1: the leader warp also runs the budget selection (sel) for its token
   SelectParams sel;
@@ -353,6 +355,7 @@ struct apex_ctx {
   struct StepState {
     int B = 0;
     bool predicted = false, selected = false, prefetched = false, routed = false;
+    uint32_t route_seq = 0;                // sequence number of the gate's record of K_r (B == 1)
     cudaStream_t route_stream = nullptr;   // stream of this step's gate kernel
     const int32_t* idx_dev = nullptr;
     const float* alpha_dev = nullptr;

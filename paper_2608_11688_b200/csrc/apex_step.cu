@@ -355,6 +355,10 @@ int apex_route_topk(apex_ctx* ctx, int layer, const float* hpost_dev, int B, int
   p.pi_pred = st.selected ? ctx->d_pi : nullptr;
   p.ncand_pred = st.selected ? ctx->d_ncand : nullptr;
   p.stats = ctx->d_stats + layer;
+  if (B == 1) {  // K_r goes to the host from here: the expert FFN's host half finds it when it is called
+    p.mbox_rec = const_cast<uint32_t*>(mbox_exec_rec(ctx, layer));
+    p.seq_value = st.route_seq = ++ctx->exec_seq[layer];
+  }
   CU_TRY(ctx, launch_router(p, (cudaStream_t)stream));
   ctx->last_was_ffn = false;
   ctx->last_pred_layer = -1;
@@ -498,10 +502,12 @@ int ffn_finalize(apex_ctx* ctx, int layer) {
   cudaStream_t cs = st.pend_stream;
   auto& tab = ctx->tables[layer];
   const FfnParams& p = ctx->ffn_params[layer];
-  // the FFN posts the routed and the execution set of the layer-step as masks (B > 1: the unions over the tokens), each
-  // with its sequence number in one 16-byte record
+  // The routed and the execution set of the layer-step arrive as masks, each with its sequence number in one 16-byte
+  // record.  One token: the gate posts the routed set (exact mode needs no more), the FFN the execution set; a batch: the
+  // FFN posts both, the unions over the tokens.
   volatile uint32_t* rec = mbox_exec_rec(ctx, layer);
-  if (!host_wait_seq(ctx, rec + 2, ctx->exec_seq[layer]) || !host_wait_seq(ctx, rec + 6, ctx->exec_seq[layer]))
+  if (!host_wait_seq(ctx, rec + 2, B == 1 ? st.route_seq : ctx->exec_seq[layer]) ||
+      (st.pend_mode != APEX_MODE_EXACT && !host_wait_seq(ctx, rec + 6, ctx->exec_seq[layer])))
     return fail(ctx, APEX_ETIMEOUT, "apex_moe_ffn: K_r did not arrive");
   const uint64_t need = ((uint64_t)rec[1] << 32) | rec[0], ex_mask = ((uint64_t)rec[5] << 32) | rec[4];
   if (st.pend_mode == APEX_MODE_EXACT) {

@@ -358,9 +358,9 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
   };
 
   auto post_plan = [&]() {
-    // The routed and the execution set go to the caller's buffers and, as masks, to the host mailbox: each in ONE
-    // aligned 16-byte store that carries its own sequence number, so no system-scope fence (a round trip over the
-    // host link) sits in this warp's way -- it has rows to stream like every other warp.
+    // The execution set goes to the caller's buffers and, as a mask, to the host mailbox: in ONE aligned 16-byte store that
+    // carries its own sequence number, so no system-scope fence (a round trip over the host link) sits in this warp's
+    // way -- it has rows to stream like every other warp.  (The host has the routed set from the gate kernel.)
     store_token_plan(tp1, lane, k, p.exec_idx, p.exec_gate, nullptr);
     if (lane == 0) {
       if (p.stats) {
@@ -368,19 +368,12 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
         if (ns) atomicAdd(&p.stats->substitutions, (unsigned long long)ns);
         atomicAdd(&p.stats->hits_R, (unsigned long long)__popcll(tp1.kr_mask & p.snap.resident_mask));
       }
-      asm volatile("st.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p.mbox_rec), "r"((uint32_t)tp1.kr_mask),
-                   "r"((uint32_t)(tp1.kr_mask >> 32)), "r"(p.seq_value), "r"(0u)
-                   : "memory");
       asm volatile("st.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p.mbox_rec + 4), "r"((uint32_t)tp1.exec_mask),
                    "r"((uint32_t)(tp1.exec_mask >> 32)), "r"(p.seq_value), "r"(0u)
                    : "memory");
     }
   };
   const bool poster = cta == 0 && warp == 0 && p.post_exec;
-  // If an expert of this launch still has to be fetched, the host cannot start before it has seen
-  // K_r: post first.  Otherwise post while the first rows are in flight.
-  const bool will_wait_for_host = p.demand_in_kernel && (run & ~p.snap.resident_mask) != 0ull;
-  if (poster && will_wait_for_host) post_plan();
   // ---- row supply of this warp (state lives in lane 0; the other lanes learn the outcome by shuffle)
   int next_static = 0;                 // static rows of this warp already started
   int dyn_cur = 0, dyn_end = 0;  // rows of the current ticket
@@ -433,7 +426,7 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
   __syncwarp();
   int tail = first_fill;  // rows of this warp whose copy has been started (uniform across the warp)
   next_static = first_fill;
-  if (poster && !will_wait_for_host) post_plan();
+  if (poster) post_plan();
   // a warp with fewer static rows than stages tops up from the dynamic part
   while (tail < NSW) {
     int more = 0;

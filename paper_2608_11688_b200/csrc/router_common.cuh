@@ -203,6 +203,11 @@ __device__ __forceinline__ void router_epilogue(const RouterParams& p, const Epi
     RTL(5);
     return;
   }
+  if (p.mbox_rec) {  // the host waits for the routed set: first of all
+    const unsigned lo = __ballot_sync(0xffffffffu, e0 < N && r0 < k), hi = __ballot_sync(0xffffffffu, e1 < N && r1 < k);
+    if (lane == 0)
+      asm volatile("st.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p.mbox_rec), "r"(lo), "r"(hi), "r"(p.seq_value), "r"(0u) : "memory");
+  }
   outputs();
   if (!p.topk_out || !p.stats) return;
 

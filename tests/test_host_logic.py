@@ -148,3 +148,34 @@ def test_slot_planner_set_rejects_inconsistent_tables(lib):
     assert s.set([1, -1, 0, -1], [3, 4], 7) == 0
     es, st, clk = s.get()
     assert list(es) == [1, -1, 0, -1] and list(st) == [3, 4] and clk == 7
+
+
+@pytest.mark.parametrize("sig,args,want", [
+    ("i", (-3,), [-3]), ("iip", (1, 2, None), [1, 2, 0]), ("ifip", (7, 0.5, 9, "array"), [7, 9, "array", 0.5]),
+    ("iiiiiiiiipsi", (1, 2, 3, 4, 5, 6, 7, 8, 2**31 - 1, "tensor", 77, 5), [1, 2, 3, 4, 5, 6, 7, 8, 2**31 - 1, "tensor", 77, 5])])
+def test_pycall_marshals_every_argument(sig, args, want):
+    """The extension module behind the decode calls: integers, None, buffers, streams and fp32 values in registers and on
+    the stack arrive as the C function expects them; wrong counts and types raise."""
+    import ctypes as C
+    import torch
+    from paper_2608_11688_b200 import binding, build
+    build.build_pycall()
+    binding.load_library()
+    bufs = {"array": np.zeros(4, np.float32), "tensor": torch.zeros(4)}
+    seen = []
+    types = [C.c_float if c == "f" else C.c_int if c == "i" else C.c_uint64 for c in sig]
+
+    @C.CFUNCTYPE(C.c_int, *types)
+    def entry(*a):
+        seen.extend([v for v, c in zip(a, sig) if c != "f"] + [v for v, c in zip(a, sig) if c == "f"])
+        return -5
+
+    f = binding._pycall.make(C.cast(entry, C.c_void_p).value, sig)
+    assert f(*[bufs.get(a, a) if isinstance(a, str) else a for a in args]) == -5
+    assert seen == [binding._ptr(bufs[w]) if isinstance(w, str) else w for w in want]
+    with pytest.raises(TypeError):
+        f(*args, 0)
+    with pytest.raises(TypeError):
+        f(*[object()] * len(sig))
+    with pytest.raises(AssertionError):
+        binding._pycall.make(C.cast(entry, C.c_void_p).value, "p")(torch.zeros(4, 4).t())
