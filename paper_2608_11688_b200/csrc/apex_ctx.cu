@@ -140,7 +140,6 @@ int apex_create(const apex_config* cfg, apex_ctx** out) {
   ctx->attn_layers = L < 8 ? L : 8;
   CR(dev_alloc(&ctx->d_attn, ctx->attn_bytes * ctx->attn_layers));
   CR(cudaMemset(ctx->d_attn, 0, ctx->attn_bytes * ctx->attn_layers));
-  CR(dev_alloc(&ctx->d_attn_sink, 4));
 
   // mapped mailbox
   MailboxLayout& ml = ctx->ml;
@@ -210,7 +209,7 @@ int apex_destroy(apex_ctx* ctx) {
   void* dev[] = {ctx->d_Wr, ctx->d_br, ctx->d_Wp, ctx->d_bp, ctx->d_w, ctx->d_theta, ctx->d_cache, ctx->d_slot_ready, ctx->d_zp,
                  ctx->d_qp, ctx->d_zr, ctx->d_demand, ctx->d_pi, ctx->d_ncand, ctx->d_stats, ctx->d_counters, ctx->d_tickets, ctx->d_spec,
                  ctx->d_tc_sync, ctx->d_sgate, ctx->d_xb, ctx->d_act, ctx->d_cand,
-                 ctx->d_idx, ctx->d_exec_idx, ctx->d_alpha, ctx->d_exec_gate, ctx->d_cand_ncand, ctx->d_attn, ctx->d_attn_sink,
+                 ctx->d_idx, ctx->d_exec_idx, ctx->d_alpha, ctx->d_exec_gate, ctx->d_cand_ncand, ctx->d_attn,
                  ctx->d_h_stage, ctx->d_hp_stage, ctx->d_y_stage};
   for (void* p : dev)
     if (p) cudaFree(p);

@@ -100,6 +100,7 @@ struct RouterParams {
   uint32_t* mbox_rec;  // mapped host, B == 1: {routed set lo, hi, sequence number, 0} in one 16-byte store, or null
   uint32_t seq_value;
   int C;
+  int wait_last;      // 1: x does not come from the preceding kernel (the attention stand-in): wait for it before exiting only
   int fuse_select;   // 1: the leader warp also runs the budget selection (sel) for its token
   SelectParams sel;
 };
@@ -247,10 +248,10 @@ struct DecodeParams {
 };
 
 struct AttnParams {
-  const uint4* buf;
-  size_t n_vec;  // 16-byte vectors
-  float* sink;
+  const uint8_t* buf;
+  size_t bytes;         // a multiple of 16
   int wait_first;       // 1: wait for the preceding kernel before streaming; 0: stream beside it, wait before exiting
+  unsigned* status;     // mapped: 1 when a wait ran out
 };
 
 // launchers (kernels_*.cu).  Each returns the cudaError_t of the launch.
@@ -306,7 +307,6 @@ struct apex_ctx {
   std::vector<apex::TcMaps> tc_shared_maps;  // per layer: ws / ssc filled
   uint8_t* d_attn = nullptr;
   size_t attn_bytes = 0, attn_layers = 1;
-  float* d_attn_sink = nullptr;
   // scratch for apex_decode_token
   int32_t *d_cand = nullptr, *d_cand_ncand = nullptr, *d_exec_idx = nullptr;
   float* d_exec_gate = nullptr;

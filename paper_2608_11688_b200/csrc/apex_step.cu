@@ -174,12 +174,13 @@ int fill_select(apex_ctx* ctx, int layer, int B, float tau, int32_t* cand_dev, i
 // S1-S3 in one launch (used by apex_decode_token): the leader warp of the prefetch-router kernel
 // goes on with the budget selection of its token.
 int predict_select_fused(apex_ctx* ctx, int layer, const float* h_dev, int B, float tau, int32_t* cand_dev,
-                         int32_t* ncand_dev, cudaStream_t cs) {
+                         int32_t* ncand_dev, bool beside_standin, cudaStream_t cs) {
   RouterParams p;
   int r = begin_predict(ctx, layer, h_dev, B, &p);
   if (r != APEX_OK) return r;
   if ((r = fill_select(ctx, layer, B, tau, cand_dev, ncand_dev, &p.sel)) != APEX_OK) return r;
   p.fuse_select = 1;
+  p.wait_last = beside_standin ? 1 : 0;
   CU_TRY(ctx, launch_router(p, cs));
   ctx->last_was_ffn = false;
   ctx->last_pred_layer = layer;
@@ -313,9 +314,9 @@ int apex_attention_standin(apex_ctx* ctx, int layer, void* stream) {
   CHECK_CTX(ctx);
   CHECK_LAYER(ctx, layer);
   AttnParams p{};
-  p.buf = reinterpret_cast<const uint4*>(ctx->d_attn + (size_t)(layer % ctx->attn_layers) * ctx->attn_bytes);
-  p.n_vec = ctx->attn_bytes / 16;
-  p.sink = ctx->d_attn_sink;
+  p.buf = ctx->d_attn + (size_t)(layer % ctx->attn_layers) * ctx->attn_bytes;
+  p.bytes = ctx->attn_bytes;
+  p.status = const_cast<unsigned*>(&mhdr(ctx)->status);
   // The attention block of a layer reads the layer's input, not the prefetch router's output: when the kernel
   // just before it on this stream is this layer-step's prefetch stage, the two may run side by side (Sec. IV-A:
   // prediction and prefetch are hidden under attention).  Anything else in front of it is waited for first.
@@ -648,10 +649,15 @@ int apex_decode_token(apex_ctx* ctx, const float* h_dev, const float* hpost_dev,
     int32_t* idx = ctx->d_idx + (size_t)l * MB * k;
     float* alpha = ctx->d_alpha + (size_t)l * MB * N;
     const bool prefetching = !(tau < 0.f);  // tau < 0: the conventional scheme, expert loading on the critical path
-    if (prefetching &&
-        (r = predict_select_fused(ctx, l, h_dev + l * step, B, tau, ctx->d_cand, ctx->d_cand_ncand, (cudaStream_t)stream)) != APEX_OK)
+    // A batch: the stand-in goes first and waits for the previous layer (its window opens when that layer's output exists);
+    // the prefetch stage is launched when every CTA of it has passed that wait and runs beside it.  The other way round
+    // the stand-in started 3 to 6 us later, a launch behind the router.  (One token: its candidate record is waited for
+    // by the host, so its router, which is small, goes first.)
+    const bool standin_first = standin && B > 1;
+    if (standin_first && (r = apex_attention_standin(ctx, l, stream)) != APEX_OK) return r;
+    if (prefetching && (r = predict_select_fused(ctx, l, h_dev + l * step, B, tau, ctx->d_cand, ctx->d_cand_ncand, standin_first, (cudaStream_t)stream)) != APEX_OK)
       return r;
-    if (standin && (r = apex_attention_standin(ctx, l, stream)) != APEX_OK) return r;
+    if (standin && !standin_first && (r = apex_attention_standin(ctx, l, stream)) != APEX_OK) return r;
     if ((r = apex_route_topk(ctx, l, hpost_dev + l * step, B, idx, alpha, stream)) != APEX_OK) return r;
     if (l > 0 && (r = ffn_finalize(ctx, l - 1)) != APEX_OK) return r;
     if (prefetching && (r = apex_prefetch(ctx, l, B, nullptr)) != APEX_OK) return r;

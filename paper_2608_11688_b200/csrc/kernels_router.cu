@@ -63,8 +63,8 @@ __global__ void __launch_bounds__(256) router_kernel(const RouterParams p) {
   EpilogueVals ev;
   if (p.fuse_select && crank == 0 && warp == 0) ev.sel = load_select_vals(p.sel, lane);
   RTL(0);
-  pdl_wait();               // everything queued before this kernel is complete: x may be read
-  pdl_launch_dependents();  // the next kernel may begin its own prologue
+  if (!p.wait_last) pdl_wait();  // everything queued before this kernel is complete: x may be read
+  pdl_launch_dependents();       // the next kernel may begin its own prologue
   RTL(1);
   if (crank == 0 && warp == 0) load_prediction(p, b, lane, &ev);
 
@@ -97,10 +97,14 @@ __global__ void __launch_bounds__(256) router_kernel(const RouterParams p) {
   RTL(2);
   cluster.sync();
   RTL(3);
-  if (crank != 0 || warp != 0) return;
+  if (crank != 0 || warp != 0) {
+    if (p.wait_last) pdl_wait();
+    return;
+  }
 
   // ---- leader warp
   router_epilogue(p, ev, b, lane, zs, qs, pis, posp);
+  if (p.wait_last) pdl_wait();
   SPAN_END((p.fuse_select || !p.topk_out || !p.stats) ? 1 : 4);
 }
 
@@ -161,7 +165,7 @@ __global__ void __launch_bounds__(kRouterWarps * 32, 2) router_batched_kernel(co
   EpilogueVals ev;
   if (p.fuse_select && te < nt) ev.sel = load_select_vals(p.sel, lane);
   RTL(0);
-  pdl_wait();
+  if (!p.wait_last) pdl_wait();
   pdl_launch_dependents();
   RTL(1);
   if (te < nt) load_prediction(p, b0 + te, lane, &ev);
@@ -254,6 +258,7 @@ __global__ void __launch_bounds__(kRouterWarps * 32, 2) router_batched_kernel(co
     load_prediction(p, b0 + t, lane, &ev);
     router_epilogue(p, ev, b0 + t, lane, zs[t / csize], qs[warp], pis[warp], posp[warp]);
   }
+  if (p.wait_last) pdl_wait();
   RTL(6);
   SPAN_END((p.fuse_select || !p.topk_out || !p.stats) ? 1 : 4);
 }
@@ -356,31 +361,36 @@ cudaError_t launch_select(const SelectParams& p, cudaStream_t s) {
   return cudaLaunchKernelEx(&cfg, select_kernel, p);
 }
 
-// Streams attn_bytes once (the weight and KV bytes an attention block of this shape reads).  The
-// xor of everything read is stored only if it equals one fixed pattern, which keeps the loads live.
-__global__ void __launch_bounds__(512) attention_standin_kernel(const AttnParams p) {
+// Streams the bytes of an attention block once, through shared memory by bulk copies: four threads keep a 16 KB copy
+// each in flight (64 KB per SM, 9.5 MB on the GPU against the 8 MB that latency times bandwidth asks for).  Few
+// registers and 64 KB, so a router's CTAs fit beside it; as 512-thread CTAs with loads in registers it took 12 to 17 us for the
+// 42 MB of d = 2048, and no router fitted beside two of them.
+constexpr int kAttnChunk = 16 * 1024, kAttnWarps = 4;
+
+__global__ void __launch_bounds__(kAttnWarps * 32) attention_standin_kernel(const AttnParams p) {
   SPAN_BEGIN();
+  extern __shared__ __align__(128) uint8_t attn_smem[];
+  __shared__ uint64_t s_bar[kAttnWarps];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (lane == 0) {
+    mbar_init(&s_bar[warp], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
   if (p.wait_first) pdl_wait();
   pdl_launch_dependents();
-  const size_t stride = (size_t)gridDim.x * blockDim.x;
-  uint4 a = make_uint4(0, 0, 0, 0);
-  auto take = [&](const uint4& v) {
-    a.x ^= v.x;
-    a.y ^= v.y;
-    a.z ^= v.z;
-    a.w ^= v.w;
-  };
-  // eight loads of a thread in flight: with one, 2.4 MB under way on the whole GPU were 14 us for the 42 MB of d = 2048
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  for (; i + 7 * stride < p.n_vec; i += 8 * stride) {
-    uint4 v[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = __ldcs(p.buf + i + u * stride);
-#pragma unroll
-    for (int u = 0; u < 8; ++u) take(v[u]);
+  if (lane == 0) {
+    uint32_t parity = 0;
+    const size_t stride = (size_t)gridDim.x * kAttnWarps * kAttnChunk;
+    for (size_t off = ((size_t)warp * gridDim.x + blockIdx.x) * kAttnChunk; off < p.bytes; off += stride, parity ^= 1u) {
+      const uint32_t n = p.bytes - off < (size_t)kAttnChunk ? (uint32_t)(p.bytes - off) : (uint32_t)kAttnChunk;
+      mbar_expect_tx(&s_bar[warp], n);
+      bulk_g2s(attn_smem + warp * kAttnChunk, p.buf + off, n, &s_bar[warp]);
+      if (!mbar_wait(&s_bar[warp], parity, nullptr, 2000000000ll)) {  // (bounded like every wait; a copy of this GPU's own memory)
+        *(volatile unsigned*)p.status = 1u;
+        break;
+      }
+    }
   }
-  for (; i < p.n_vec; i += stride) take(__ldcs(p.buf + i));
-  if (a.x == 0x12345678u && a.y == 0x9abcdef0u && a.z == 0x0fedcba9u && a.w == 0x87654321u) p.sink[0] = 1.f;
   // Streamed beside the preceding kernel: wait for it now, so that whoever waits for this kernel has, as
   // always, everything before it on the stream complete.
   if (!p.wait_first) pdl_wait();
@@ -388,10 +398,21 @@ __global__ void __launch_bounds__(512) attention_standin_kernel(const AttnParams
 }
 
 cudaError_t launch_attention(const AttnParams& p, int n_sm, cudaStream_t s) {
+  static std::atomic<bool> configured[kMaxDevices];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  if (!configured[dev].load(std::memory_order_acquire)) {
+    if ((e = cudaFuncSetAttribute(attention_standin_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttnWarps * kAttnChunk)) != cudaSuccess) return e;
+    configured[dev].store(true, std::memory_order_release);
+  }
   prefer_max_shared<attention_standin_kernel>();
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(n_sm * 2, 1, 1);
-  cfg.blockDim = dim3(512, 1, 1);
+  const size_t chunks = (p.bytes + kAttnChunk - 1) / kAttnChunk;
+  cfg.gridDim = dim3((unsigned)(chunks < (size_t)n_sm ? chunks : (size_t)n_sm), 1, 1);
+  cfg.blockDim = dim3(kAttnWarps * 32, 1, 1);
+  cfg.dynamicSmemBytes = kAttnWarps * kAttnChunk;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
