@@ -209,7 +209,8 @@ struct DecodeMbox {
 struct DecodeParams {
   const float* h;       // [L][d] pre-attention states
   const float* hpost;   // [L][d] post-attention states
-  float* y;             // [L][d], zero at launch
+  float* y;             // [L][d]
+  int zero_y;           // 1: the kernel zeroes y (before the stand-in is counted in; without one the host does it)
   const float *W_p, *b_p, *W_r, *b_r;  // [L][N][d], [L][N] (zeros where a layer has no bias)
   const float *w, *theta;               // [L][N], [L][N-k+1]
   const uint8_t* cache;                 // [L][C][slot_stride]
@@ -388,7 +389,7 @@ struct apex_ctx {
   std::vector<uint8_t> dec_opt_host, dec_opt_last;  // expectation per layer: now / as uploaded
   apex::SlotSnapshot* dec_tab_stage = nullptr;  // pinned [2][L]: staging of the table upload
   std::vector<apex::SlotSnapshot> dec_tab_last;  // what the device holds
-  bool dec_tab_valid = false;
+  std::vector<uint64_t> dec_tab_version;         // table versions dec_tab_last was taken from (0: never)
   int dec_stage_sel = 0;
   apex::DecodeHostSnap* dec_snap = nullptr;   // mapped [L]
   apex::DecodeHostSnap* d_dec_snap = nullptr; // device [L]

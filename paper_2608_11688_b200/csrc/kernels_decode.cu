@@ -171,6 +171,12 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_token_kernel(const Deco
     mbar_init(&s_rbar, kDecWarps);
   }
   if (tid < APEX_MAX_EXPERTS / 4) s_rank[tid] = 0u;
+  if (p.zero_y) {
+    // y of all layers, a slice per CTA.  Nobody adds to it before the first layer's cluster barrier, which follows the count
+    // of the stand-in by every CTA, and a CTA counts itself in behind the barrier below.
+    float4* y4 = reinterpret_cast<float4*>(p.y);
+    for (int i = cta * (int)blockDim.x + tid; i < L * (d / 4); i += G * (int)blockDim.x) y4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
   if (tid < NS) mbar_init(&s_full[tid], 1);
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   __syncthreads();

@@ -37,12 +37,16 @@ class SlotTable {
     return m;
   }
 
+  // Changes whenever an expert enters or leaves the table.
+  uint64_t version() const { return version_; }
+
   void begin_step() {
     ++clock_;
     if (!reuse_) clear();
   }
 
   void clear() {
+    ++version_;
     std::fill(slot_expert_.begin(), slot_expert_.end(), -1);
     std::fill(expert_slot_.begin(), expert_slot_.end(), -1);
     std::fill(slot_stamp_.begin(), slot_stamp_.end(), (int64_t)-1);
@@ -57,6 +61,7 @@ class SlotTable {
   void drop(int e) {
     if (e < 0 || e >= N_ || expert_slot_[e] < 0) return;
     const int s = expert_slot_[e];
+    ++version_;
     expert_slot_[e] = -1;
     slot_expert_[s] = -1;
     slot_stamp_[s] = -1;
@@ -141,6 +146,7 @@ class SlotTable {
         se[s] = e;
       }
     }
+    ++version_;
     slot_expert_ = se;
     expert_slot_.assign(expert_slot, expert_slot + N_);
     slot_stamp_.assign(slot_stamp, slot_stamp + C_);
@@ -169,6 +175,7 @@ class SlotTable {
     }
     if (best < 0) return false;
     if (slot_expert_[best] >= 0) expert_slot_[slot_expert_[best]] = -1;
+    ++version_;
     slot_expert_[best] = e;
     expert_slot_[e] = best;
     slot_stamp_[best] = clock_;
@@ -181,6 +188,7 @@ class SlotTable {
   std::vector<int32_t> slot_expert_, expert_slot_;
   std::vector<int64_t> slot_stamp_;
   int64_t clock_ = 0;
+  uint64_t version_ = 1;
 };
 
 }  // namespace apex
