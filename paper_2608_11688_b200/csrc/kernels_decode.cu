@@ -101,6 +101,9 @@ __device__ __forceinline__ void st_async_remote(void* local_dst, uint64_t* local
 __device__ __forceinline__ void red_release_gpu_u64(unsigned long long* p, unsigned long long v) {
   asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
+__device__ __forceinline__ void red_relaxed_gpu_u64(unsigned long long* p, unsigned long long v) {
+  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
 __device__ __forceinline__ uint32_t ld_acquire_gpu_u32(const uint32_t* p) {
   uint32_t v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -129,6 +132,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_token_kernel(const Deco
   __shared__ uint64_t s_full[kDecMaxStages];
   __shared__ uint64_t s_xbar[2];   // logits of the prefetch router / of the gate have arrived from the whole cluster
   __shared__ uint64_t s_pbar;      // warp 0 has derived the candidate set of this layer
+  __shared__ uint64_t s_cbar[2];   // the CTA's polling warp has seen: the previous layer's y complete / the stand-in complete
   __shared__ uint64_t s_rbar;      // every warp has added its share of the gate's rank counts
   __shared__ unsigned s_rank[APEX_MAX_EXPERTS / 4];  // rank of each expert's gate logit, four 8-bit counts to a word (zero between layers)
   __shared__ float s_zp[APEX_MAX_EXPERTS], s_zr[APEX_MAX_EXPERTS];
@@ -168,6 +172,8 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_token_kernel(const Deco
     mbar_init(&s_xbar[0], 1);
     mbar_init(&s_xbar[1], 1);
     mbar_init(&s_pbar, 1);
+    mbar_init(&s_cbar[0], 1);
+    mbar_init(&s_cbar[1], 1);
     mbar_init(&s_rbar, kDecWarps);
   }
   if (tid < APEX_MAX_EXPERTS / 4) s_rank[tid] = 0u;
@@ -260,13 +266,14 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_token_kernel(const Deco
       }
     }
   };
-  // bounded wait for a device-wide counter (one lane calls it).  Hundreds of warps wait for the same word while the
-  // CTAs are still adding to it: poll gently.
+  // Bounded wait for a device-wide counter (one lane calls it).  One warp of a CTA polls and lets the others know through
+  // shared memory: with every warp polling (960 of them, on the words the CTAs are still adding to) a count was seen 0.5 us later.
+  const bool poller = warp == kDecWarps - 1;
   auto wait_counter = [&](const unsigned long long* ctr, unsigned long long target) -> bool {
     if (ld_acquire_gpu_u64(ctr) >= target) return true;
     const unsigned long long t0 = globaltimer_ns();
     for (uint32_t it = 1;; ++it) {
-      __nanosleep(40);
+      __nanosleep(20);
       if (ld_acquire_gpu_u64(ctr) >= target) return true;
       if ((it & 15u) == 0u) {
         if (stop_requested()) return false;
@@ -482,20 +489,36 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_token_kernel(const Deco
       DTL(3);
       if (lane == 0 && p.run_attn) {
         const unsigned old = atomicAdd(&s_attn_done, 1u);
-        if ((old + 1u) % kDecWarps == 0u) red_release_gpu_u64(bar_attn, 1ull);
+        // (nothing but the zeroes of y, before the first layer, is published by this count: the others need no fence, 0.5 us)
+        if ((old + 1u) % kDecWarps == 0u) {
+          if (l == 0) red_release_gpu_u64(bar_attn, 1ull);
+          else red_relaxed_gpu_u64(bar_attn, 1ull);
+        }
       }
     };
     // The stand-in is this layer's attention block: its window opens when the previous layer's y is complete.  (With
     // standin_ahead the chunks were requested earlier, while the previous layer was still finishing: the window then
     // overlaps that layer's tail -- including any wait for its experts -- which is not what Eq. (12) describes.)
-    if ((J > 0 || has_wp) && running && bar_prev_ffn) {
+    // (polling warp: wait for a counter, then release the CTA's barrier `b`; other warps: wait for that)
+    auto wait_counted = [&](int b, const unsigned long long* ctr, const unsigned long long* ctr2, uint32_t parity) -> bool {
       bool go = true;
-      if (lane == 0) go = wait_counter(bar_prev_ffn, p.bar_target);
-      go = __shfl_sync(0xffffffffu, go ? 1 : 0, 0) != 0;
+      if (poller) {
+        if (lane == 0) {
+          go = wait_counter(ctr, p.bar_target) && (!ctr2 || wait_counter(ctr2, p.bar_target));
+          if (go) mbar_arrive(&s_cbar[b]);
+        }
+        go = __shfl_sync(0xffffffffu, go ? 1 : 0, 0) != 0;
+      } else {
+        go = __all_sync(0xffffffffu, wait_bar(&s_cbar[b], parity));
+      }
       if (!go) {
         if (lane == 0 && !stop_requested()) gave_up();
         ok = false;
       }
+      return go;
+    };
+    if ((J > 0 || has_wp || poller) && running && bar_prev_ffn) {
+      wait_counted(0, bar_prev_ffn, nullptr, (uint32_t)((l - 1) & 1));
       DTL(15);
     }
     if (ok && running) start_seg1(l, NSW);  // this layer's chunks: on their way while the prefetch logit is computed
@@ -528,22 +551,17 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_token_kernel(const Deco
     }
     // exact gate: this warp's logit, once the whole stand-in has been streamed (a real attention block would only then
     // have produced h') and the previous layer's y is complete
-    if (has_wr && ok && !cta_stopped()) {
+    if ((has_wr || (poller && (int)crank * kDecWarps < N)) && ok && !cta_stopped()) {
       // (a wide gate row comes into registers only now, from L2: its latency passes while the counters are waited for,
       // and the registers were free for the stand-in's segment and are free again for the expert rows)
-      if (WR_LATE && p.run_attn) load_row(Wr_row, wr_row);  // (without a window to wait for, the row is read with x)
+      if (WR_LATE && p.run_attn && has_wr) load_row(Wr_row, wr_row);  // (without a window to wait for, the row is read with x)
+      // (without a stand-in: the previous layer's counter, which nobody may have waited for yet)
       bool go = true;
-      if (lane == 0) {
-        if (p.run_attn) go = wait_counter(bar_attn, p.bar_target);
-        if (go && bar_prev_ffn) go = wait_counter(bar_prev_ffn, p.bar_target);
-      }
-      go = __shfl_sync(0xffffffffu, go ? 1 : 0, 0) != 0;
-      if (!go) {
-        if (lane == 0 && !stop_requested()) gave_up();
-        ok = false;
-      } else {
+      if (p.run_attn) go = wait_counted(1, bar_attn, bar_prev_ffn, lpar);
+      else if (bar_prev_ffn && !(J > 0 || has_wp || poller)) go = wait_counted(0, bar_prev_ffn, nullptr, (uint32_t)((l - 1) & 1));
+      if (go) {
         DTL(14);
-        row_logit(Wr_row, wr_row, !WR_LATE || p.run_attn != 0, hpl, bias_r, s_zr, &s_xbar[1], 0, kDecCluster);
+        if (has_wr) row_logit(Wr_row, wr_row, !WR_LATE || p.run_attn != 0, hpl, bias_r, s_zr, &s_xbar[1], 0, kDecCluster);
         DTL(4);
       }
     }
