@@ -176,14 +176,16 @@ struct TcParams {
   int act_rows, act_stride;
   int layer_slot0;                       // index of this layer's slot 0 in the all-layers weight tensor map
   int nmax1, nmax2;                      // tokens per unit of the gate/up and of the down projection (set by the launcher)
+  int rows1;                             // rows of I per gate/up unit: 128 or 32 (set by the launcher)
   int shift1, shift2;                    // a group of n tokens has (n + 2^shift - 1) >> shift parts
   TcGeometry geo[2];
   int nstage, nraw, stage_bytes;         // ring depths and stage size
   TcShifts shifts;
 };
 struct TcMaps {          // opaque 128-byte CUtensorMap objects
-  alignas(64) unsigned char w[128], ws[128];    // weights of the slots / of the layer's shared expert
-  alignas(64) unsigned char sc[128], ssc[128];  // quantised stores: the same bytes in 16-byte boxes, for the e2m1 block scales
+  // weights of the slots / of the layer's shared expert: boxes of the largest height and of 32 rows
+  alignas(64) unsigned char w[2][128], ws[2][128];
+  alignas(64) unsigned char sc[2][128], ssc[2][128];  // quantised stores: the same bytes in 16-byte boxes, for the e2m1 block scales
   alignas(64) unsigned char x[128], xc[128], act[128];
 };
 
@@ -263,7 +265,7 @@ cudaError_t launch_ffn(const FfnParams& p, int n_ctas, cudaStream_t s);  // n_ct
 int ffn_grid_ctas(int n_sm);  // CTAs of one streaming-kernel launch (each adds one to the zero counter)
 cudaError_t launch_ffn_tc(const TcParams& p, const TcMaps& m, int n_sm, cudaStream_t s);
 bool tc_make_activation_maps(TcMaps* m, const void* xb, int d, int max_batch, const void* act, size_t act_rows, int act_stride);
-bool tc_make_store_maps(int fmt, void* weights, void* scales, const void* base, int d, int I, size_t n_slots, size_t slot_bytes);  // one store, in storage format fmt
+bool tc_make_store_maps(int fmt, unsigned char (*weights)[128], unsigned char (*scales)[128], const void* base, int d, int I, size_t n_slots, size_t slot_bytes);  // one store, in storage format fmt
 bool ffn_shape_supported(int d);
 bool ffn_quantised_shape_supported(int d);   // widths the e4m3 / e2m1 kernels were built for
 size_t ffn_row_bytes(int fmt, int d);        // bytes of one intermediate index (three vectors and their scales)

@@ -61,6 +61,11 @@ constexpr int kEpiWarp0 = 3;   // four epilogue warps
 constexpr int kCvWarp0 = 7;    // sixteen converter warps (quantised stores only): four per scheduler hide the latency of shared memory and ALU
 constexpr int kCvThreads = 512;
 __host__ __device__ constexpr int tc_threads(int qf) { return kCvWarp0 * 32 + (qf ? kCvThreads : 0); }
+// Gate/up units of kRowsSmall rows: a stage takes tc_wide(QF) K tiles (8 KB of operand each), which on the quantised stores
+// is a whole raw tile.
+constexpr int kRowsSmall = 32;
+constexpr int kHandBytes = 2 * 16 * 32 * 4;  // their epilogue: up values handed from one warp to another, two batches of 16 columns
+__host__ __device__ constexpr int tc_wide(int qf) { return qf == 1 ? 2 : 4; }
 constexpr int kKTile = 64;           // K values per stage (128 bytes of bf16: one swizzle span)
 constexpr int kABytes = 2 * 128 * 128;  // the two weight tiles of a stage
 constexpr int kMaxStages = 8, kMaxRaw = 4;
@@ -239,6 +244,10 @@ __device__ unsigned long long g_tc_tl[148][64][8];
 #define TCTL(u, i) do { } while (0)
 #endif
 
+// weight maps, by projection (boxes differ in height) and store (slots, shared expert)
+struct TcWeightMaps {
+  CUtensorMap codes[2][2], scales[2][2];
+};
 // One unit of work: the (part of a) group, the M block and the K-tile range of one of the projections (phase 1: gate/up,
 // 2: down; 0: the list is at its end).
 struct GroupDesc {
@@ -272,19 +281,19 @@ __device__ __forceinline__ bool unit_is_wide(const UnitDesc& ud) { return QF != 
 
 }  // namespace
 
-// tm_w, tm_ws: weights of the slots / of the shared expert.  bf16: boxes of 64 columns x 64 rows; quantised: the raw row
-// bytes, boxes of 128 bytes x 128 rows.  tm_sc, tm_ssc: the same bytes in boxes of 16 bytes x 128 rows (e2m1 block scales).
+// tm_w: weights of the slots and of the shared expert.  bf16: boxes of 64 columns x 64 rows; quantised: the raw row
+// bytes, boxes of 128 bytes x 128 rows, and the same bytes in boxes of 16 bytes x 128 rows (e2m1 block scales); for gate/up
+// units of fewer rows, boxes of that many.
 // tm_x, tm_xc: h' in bf16, boxes of one row (gathered) and of kARowsPerLoad.  tm_act: the intermediate, plane a_lo below plane a_hi.
 template <int QF>
 __global__ void __launch_bounds__(tc_threads(QF), 1)
-ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_ws,
-              const __grid_constant__ CUtensorMap tm_sc, const __grid_constant__ CUtensorMap tm_ssc,
-              const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_xc, const __grid_constant__ CUtensorMap tm_act, const TcParams p) {
+ffn_tc_kernel(const __grid_constant__ TcWeightMaps tm_w, const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_xc,
+              const __grid_constant__ CUtensorMap tm_act, const TcParams p) {
   SPAN_BEGIN();
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   constexpr int SUB = tc_sub(QF);
-  constexpr int RAW_BYTES = tc_raw_bytes(QF);
+  constexpr int RAW_BYTES = tc_raw_bytes(QF), WIDE = tc_wide(QF);
   const int STAGE_BYTES = p.stage_bytes, NS = p.nstage, NR = p.nraw;
   uint8_t* raw_ring = smem + (size_t)NS * STAGE_BYTES;
   __shared__ uint64_t full[kMaxStages], empty[kMaxStages], rawfull[kMaxRaw], rawempty[kMaxRaw], tmem_full[2], tmem_empty[2];
@@ -324,14 +333,14 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
       mbar_init(&unit_empty[u], 6 + (QF ? kCvThreads / 32 : 0));  // every warp that reads the descriptor
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_w) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_ws) : "memory");
+    for (int ph = 0; ph < 2; ++ph) {
+      for (int st = 0; st <= (p.f.run_shared ? 1 : 0); ++st) {
+        asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_w.codes[ph][st]) : "memory");
+        if (QF == 2) asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_w.scales[ph][st]) : "memory");
+      }
+    }
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_x) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_act) : "memory");
-    if (QF == 2) {
-      asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_sc) : "memory");
-      asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_ssc) : "memory");
-    }
   }
   if (warp == kMmaWarp) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(512) : "memory");
@@ -603,8 +612,8 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
   };
 
   if (warp == kWWarp) {
-    // ================= tickets and weight loads.  Each load of a stage is issued by a different lane (one thread
-    // sustains only about one bulk copy per 570 cycles).
+    // ================= tickets and weight loads.  One elected lane issues the loads of a stage, from warp-uniform registers: issued
+    // by lanes under a condition on the lane number the loop took 800 cycles per stage, the pace of a launch of few units.
     RingPos rp;  // over the stages (bf16) or the raw tiles (quantised)
     // The next ticket is taken a ring's depth before the end of a unit: the answer is there when the unit's last load has
     // been issued (taken only then, it left the ring empty for 1.5 us per unit), and no unit waits long for its CTA.
@@ -677,46 +686,55 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         if (!ok) break;
         slot += p.layer_slot0;  // the tensor map covers the slots of all layers
       }
-      const CUtensorMap* wmap = shared ? &tm_ws : &tm_w;
-      for (int kt = ud.kt_begin; kt < ud.kt_end; kt += SUB, rp.next(QF ? NR : NS)) {
-        uint64_t* bar;
-        uint8_t* dst;
-        if (QF == 0) {
-          if (lane == 0 && !mbar_wait(&empty[rp.s], rp.parity ^ 1, &s_abort, p.f.wait_limit_ns)) ok = false;
-          bar = &full[rp.s];
-          dst = smem + rp.s * STAGE_BYTES;
-        } else {
-          if (lane == 0 && !mbar_wait(&rawempty[rp.s], rp.parity ^ 1, &s_abort, p.f.wait_limit_ns)) ok = false;
-          bar = &rawfull[rp.s];
-          dst = raw_ring + rp.s * RAW_BYTES;
-        }
-        ok = __all_sync(0xffffffffu, ok);
+      // (shuffles: the compiler keeps what comes out of them in uniform registers)
+      const int phase = __shfl_sync(0xffffffffu, ud.phase, 0), blk = __shfl_sync(0xffffffffu, ud.blk, 0), usl = __shfl_sync(0xffffffffu, slot, 0);
+      const int kt_begin = __shfl_sync(0xffffffffu, ud.kt_begin, 0), kt_end = __shfl_sync(0xffffffffu, ud.kt_end, 0);
+      const int store = __shfl_sync(0xffffffffu, shared ? 1 : 0, 0);
+      const CUtensorMap* wmap = &tm_w.codes[phase - 1][store];
+      const CUtensorMap* smap = &tm_w.scales[phase - 1][store];
+      const int rows1 = p.rows1;
+      const bool small = phase == 1 && rows1 == kRowsSmall;
+      const uint32_t tile_bytes = QF == 0 ? kABytes : small ? RAW_BYTES / 128 * kRowsSmall : RAW_BYTES;
+      const int step = QF == 0 && small ? WIDE : SUB;
+      for (int kt = kt_begin; kt < kt_end; kt += step, rp.next(QF ? NR : NS)) {
+        uint64_t* bar = QF ? &rawfull[rp.s] : &full[rp.s];
+        uint8_t* dst = QF ? raw_ring + rp.s * RAW_BYTES : smem + rp.s * STAGE_BYTES;
+        ok = __all_sync(0xffffffffu, mbar_wait(QF ? &rawempty[rp.s] : &empty[rp.s], rp.parity ^ 1, &s_abort, p.f.wait_limit_ns));
         if (!ok) break;
-        if (!taken && kt + ahead >= ud.kt_end) {
+        if (!taken && kt + ahead >= kt_end) {
           taken = true;
           if (lane == 0) ticket = (int)atomicAdd(p.sync + kTcTicket, 1u);
         }
-        if (lane == 0) mbar_expect_tx(bar, QF ? RAW_BYTES : kABytes);
-        __syncwarp();
-        if (QF == 0) {
-          if (lane < 4) {
-            if (ud.phase == 1) tma_load_4d(dst + lane * 8192, wmap, kt * kKTile, lane >> 1, ud.blk * 128 + (lane & 1) * 64, slot, bar);  // gate | up, two row halves each
-            else tma_load_4d(dst + lane * 8192, wmap, ud.blk * 256 + lane * 64, 2, kt * kKTile, slot, bar);                               // downT, 64 columns each
-          }
-        } else if (QF == 1) {  // row: gate | up | downT codes (d bytes each), then the scales
-          if (lane < 2) {
-            if (ud.phase == 1) tma_load_3d(dst + lane * 16384, wmap, lane * d + kt * kKTile, ud.blk * 128, slot, bar);
-            else tma_load_3d(dst + lane * 16384, wmap, 2 * d + ud.blk * 256 + lane * 128, kt * kKTile, slot, bar);
-          }
-        } else {  // row: gate | up | downT codes (d/2 bytes each), then their scale bytes (d/32 each)
-          const CUtensorMap* smap = shared ? &tm_ssc : &tm_sc;
-          if (lane < 2) {
-            if (ud.phase == 1) tma_load_3d(dst + lane * 16384, wmap, lane * (d / 2) + kt * (kKTile / 2), ud.blk * 128, slot, bar);
-            else tma_load_3d(dst + lane * 16384, wmap, d + ud.blk * 128, kt * kKTile + lane * 128, slot, bar);
-          } else if (lane < 4) {
-            const int h = lane - 2;
-            if (ud.phase == 1) tma_load_3d(dst + 32768 + h * 2048, smap, 3 * (d / 2) + h * (d / 32) + ((kt * 2) & ~15), ud.blk * 128, slot, bar);
-            else tma_load_3d(dst + 32768 + h * 2048, smap, 3 * (d / 2) + 2 * (d / 32) + ((ud.blk * 8) & ~15), kt * kKTile + h * 128, slot, bar);
+        if (elect_one()) {
+          mbar_expect_tx(bar, tile_bytes);
+          if (QF == 0) {
+            if (phase == 2) {
+#pragma unroll
+              for (int i = 0; i < 4; ++i) tma_load_4d(dst + i * 8192, wmap, blk * 256 + i * 64, 2, kt * kKTile, usl, bar);  // downT, 64 columns each
+            } else if (!small) {
+#pragma unroll
+              for (int i = 0; i < 4; ++i) tma_load_4d(dst + i * 8192, wmap, kt * kKTile, i >> 1, blk * 128 + (i & 1) * 64, usl, bar);  // gate | up, two row halves each
+            } else {
+#pragma unroll
+              for (int i = 0; i < 2 * WIDE; ++i) tma_load_4d(dst + i * (kRowsSmall * 128), wmap, (kt + (i >> 1)) * kKTile, i & 1, blk * kRowsSmall, usl, bar);  // per K tile: gate, up
+            }
+          } else if (QF == 1) {  // row: gate | up | downT codes (d bytes each), then the scales
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              if (phase == 1) tma_load_3d(dst + i * 16384, wmap, i * d + kt * kKTile, blk * rows1, usl, bar);
+              else tma_load_3d(dst + i * 16384, wmap, 2 * d + blk * 256 + i * 128, kt * kKTile, usl, bar);
+            }
+          } else {  // row: gate | up | downT codes (d/2 bytes each), then their scale bytes (d/32 each)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              if (phase == 1) {
+                tma_load_3d(dst + i * 16384, wmap, i * (d / 2) + kt * (kKTile / 2), blk * rows1, usl, bar);
+                tma_load_3d(dst + 32768 + i * 2048, smap, 3 * (d / 2) + i * (d / 32) + ((kt * 2) & ~15), blk * rows1, usl, bar);
+              } else {
+                tma_load_3d(dst + i * 16384, wmap, d + blk * 128, kt * kKTile + i * 128, usl, bar);
+                tma_load_3d(dst + 32768 + i * 2048, smap, 3 * (d / 2) + 2 * (d / 32) + ((blk * 8) & ~15), kt * kKTile + i * 128, usl, bar);
+              }
+            }
           }
         }
         __syncwarp();
@@ -730,10 +748,15 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
       const UnitDesc ud = next_unit(n);
       if (ud.phase == 0) break;
       const int n_pad = (ud.n_tok + 15) & ~15;
+      const bool gather = ud.phase == 1 && ud.expert < N;
+      const int n_loads = gather ? (ud.n_tok + 3) / 4 : n_pad / kARowsPerLoad;
+      // load number and K tile of the stage this lane issues, where it takes a lane each
+      const bool small = ud.phase == 1 && p.rows1 == kRowsSmall;
+      const int li = small ? lane % n_loads : lane, kj = small ? lane / n_loads : 0;
       int tok[4] = {0, 0, 0, 0};
-      if (ud.phase == 1) {  // lane j: rows 4 j .. 4 j + 3 (past the last token: any row, the result is not used)
+      if (ud.phase == 1) {  // load j: rows 4 j .. 4 j + 3 (past the last token: any row, the result is not used)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) tok[i] = s_tok[ud.pair_off + min(4 * lane + i, ud.n_tok - 1)];
+        for (int i = 0; i < 4; ++i) tok[i] = s_tok[ud.pair_off + min(4 * li + i, ud.n_tok - 1)];
       }
       // what is loaded must be complete: the rows of X (once), or every gate/up unit of the group
       if (ud.phase == 2 || n == 0) {
@@ -746,25 +769,56 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         if (!ok) break;
       }
       // The shared expert runs all tokens in order: plain boxes (32 gathers per stage were its pace, 1.3 us at 128 tokens)
-      const bool gather = ud.phase == 1 && ud.expert < N;
-      const int n_loads = gather ? (ud.n_tok + 3) / 4 : n_pad / kARowsPerLoad;
-      const uint32_t bytes = gather ? n_loads * 512u : (uint32_t)(ud.phase * n_pad * 128);
-      for (int kt = ud.kt_begin; kt < ud.kt_end; ++kt, rp.next(NS)) {
+      const int tiles = __shfl_sync(0xffffffffu, small ? WIDE : 1, 0);   // K tiles of a stage
+      const uint32_t bytes = (uint32_t)tiles * (gather ? n_loads * 512u : (uint32_t)(ud.phase * n_pad * 128));
+      const int phase = __shfl_sync(0xffffffffu, ud.phase, 0), loads = __shfl_sync(0xffffffffu, n_loads, 0), pads = __shfl_sync(0xffffffffu, n_pad, 0);
+      const int kt_begin = __shfl_sync(0xffffffffu, ud.kt_begin, 0), kt_end = __shfl_sync(0xffffffffu, ud.kt_end, 0);
+      const int row0 = __shfl_sync(0xffffffffu, phase == 2 ? ud.pair_off : tok[0], 0);  // (the shared expert's tokens follow one another)
+      const bool few = loads <= 2;  // one elected lane issues them; otherwise a lane each
+      int t0[4], t1[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        t0[i] = __shfl_sync(0xffffffffu, tok[i], 0);
+        t1[i] = __shfl_sync(0xffffffffu, tok[i], 1);
+      }
+      for (int kt = kt_begin; kt < kt_end; kt += tiles, rp.next(NS)) {
         const uint32_t s = rp.s;
-        if (lane == 0 && !mbar_wait(&empty[s], rp.parity ^ 1, &s_abort, p.f.wait_limit_ns)) ok = false;
-        ok = __all_sync(0xffffffffu, ok);
+        ok = __all_sync(0xffffffffu, mbar_wait(&empty[s], rp.parity ^ 1, &s_abort, p.f.wait_limit_ns));
         if (!ok) break;
-        if (lane == 0) mbar_expect_tx(&full[s], bytes);
-        __syncwarp();
         uint8_t* dst = smem + s * STAGE_BYTES + kABytes;
-        if (ud.phase == 1 && !gather) {
-          if (lane < n_loads)
-            tma_load_2d(dst + lane * kARowsPerLoad * 128, &tm_xc, kt * kKTile, s_tok[ud.pair_off] + lane * kARowsPerLoad, &full[s]);
-        } else if (ud.phase == 1) {
-          if (lane < n_loads) tma_gather4(dst + lane * 512, &tm_x, kt * kKTile, tok[0], tok[1], tok[2], tok[3], &full[s]);
-        } else if (lane < 2 * n_loads) {  // (at most 64 tokens: 4 boxes per plane)
-          const int pl = lane >= n_loads ? 1 : 0, r = lane - pl * n_loads;
-          tma_load_2d(dst + (pl * n_pad + r * kARowsPerLoad) * 128, &tm_act, kt * kKTile, pl * p.act_rows + ud.pair_off + r * kARowsPerLoad, &full[s]);
+        if (few) {
+          if (elect_one()) {
+            mbar_expect_tx(&full[s], bytes);
+            if (phase == 2) {
+              tma_load_2d(dst, &tm_act, kt * kKTile, row0, &full[s]);
+              tma_load_2d(dst + pads * 128, &tm_act, kt * kKTile, p.act_rows + row0, &full[s]);
+              if (loads == 2) {
+                tma_load_2d(dst + kARowsPerLoad * 128, &tm_act, kt * kKTile, row0 + kARowsPerLoad, &full[s]);
+                tma_load_2d(dst + (pads + kARowsPerLoad) * 128, &tm_act, kt * kKTile, p.act_rows + row0 + kARowsPerLoad, &full[s]);
+              }
+            } else if (gather) {
+              for (int j = 0; j < tiles; ++j) {
+                tma_gather4(dst + j * pads * 128, &tm_x, (kt + j) * kKTile, t0[0], t0[1], t0[2], t0[3], &full[s]);
+                if (loads == 2) tma_gather4(dst + j * pads * 128 + 512, &tm_x, (kt + j) * kKTile, t1[0], t1[1], t1[2], t1[3], &full[s]);
+              }
+            } else {
+              for (int j = 0; j < tiles; ++j) {
+                tma_load_2d(dst + j * pads * 128, &tm_xc, (kt + j) * kKTile, row0, &full[s]);
+                if (loads == 2) tma_load_2d(dst + (j * pads + kARowsPerLoad) * 128, &tm_xc, (kt + j) * kKTile, row0 + kARowsPerLoad, &full[s]);
+              }
+            }
+          }
+        } else {
+          if (lane == 0) mbar_expect_tx(&full[s], bytes);
+          __syncwarp();
+          if (phase == 1 && !gather) {
+            if (lane < tiles * loads) tma_load_2d(dst + (kj * pads + li * kARowsPerLoad) * 128, &tm_xc, (kt + kj) * kKTile, row0 + li * kARowsPerLoad, &full[s]);
+          } else if (phase == 1) {
+            if (lane < tiles * loads) tma_gather4(dst + kj * pads * 128 + li * 512, &tm_x, (kt + kj) * kKTile, tok[0], tok[1], tok[2], tok[3], &full[s]);
+          } else if (lane < 2 * loads) {  // (at most 64 tokens: 4 boxes per plane)
+            const int pl = lane >= loads ? 1 : 0, r = lane - pl * loads;
+            tma_load_2d(dst + (pl * pads + r * kARowsPerLoad) * 128, &tm_act, kt * kKTile, pl * p.act_rows + row0 + r * kARowsPerLoad, &full[s]);
+          }
         }
         __syncwarp();
       }
@@ -799,7 +853,9 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
       const uint32_t idesc = umma_idesc(128, down ? 2 * n_pad : n_pad, down ? 1 : 0);
       const uint64_t desc_a = down ? desc_a2 : desc_a1;
       const uint64_t a_step = down ? 128 : 2;   // per 16 K values: 16 rows of 128 bytes (MN-major) | 32 bytes of a row
-      for (int kt = kt_begin; kt < kt_end; ++kt, rp.next(NS)) {
+      const bool small = !down && p.rows1 == kRowsSmall;
+      const int tiles = small ? WIDE : 1;
+      for (int kt = kt_begin; kt < kt_end; kt += tiles, rp.next(NS)) {
         const uint32_t s = rp.s;
         ok = __all_sync(0xffffffffu, mbar_wait(&full[s], rp.parity, &s_abort, p.f.wait_limit_ns));
         if (!ok) break;
@@ -810,7 +866,19 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         const uint64_t soff = (uint64_t)(s * (uint32_t)STAGE_BYTES >> 4);
         const uint64_t da = desc_a + soff, db = desc_b + soff;
         if (elect_one()) {
-          if (QF != 0 && !down) {
+          if (small) {
+            // Gate and up rows in one MMA (TMEM lanes 0 .. 31 and 32 .. 63); M = 128 all the same: the rows past the 64 are
+            // whatever lies behind them (inside the stage: 8 KB of activations at least), and nobody reads theirs of the result.
+#pragma unroll
+            for (int j = 0; j < WIDE; ++j) {
+              const uint64_t daj = da + (uint64_t)(j * (2 * kRowsSmall * 128 / 16)), dbj = db + (uint64_t)(j * n_pad * (128 / 16));
+#pragma unroll
+              for (int ks = 0; ks < kKTile / 16; ++ks) {
+                const uint32_t a = (kt > kt_begin || j > 0 || ks > 0) ? 1u : 0u;
+                umma(tacc, daj + (uint64_t)(ks * 2), dbj + (uint64_t)(ks * 2), idesc, a);
+              }
+            }
+          } else if (QF != 0 && !down) {
             const uint32_t ta = tbase + kTmemA + s * 64u;  // gate, then up: 32 columns each
 #pragma unroll
             for (int ks = 0; ks < kKTile / 16; ++ks) {
@@ -827,7 +895,7 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
             }
           }
           umma_commit(&empty[s]);  // the stage is free once these MMAs have read it
-          if (kt + 1 == kt_end) {
+          if (kt + tiles >= kt_end) {
             umma_commit(&tmem_full[b0]);
             if (wide) umma_commit(&tmem_full[1]);
           }
@@ -849,6 +917,51 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     for (uint32_t n = 0; ok; ++n) {
       const UnitDesc ud = next_unit(n);
       if (ud.phase == 0) break;
+      if (ud.phase == 1 && p.rows1 == kRowsSmall) {
+        // 32 rows of gate and up: all of the raw tile into one stage's shared memory (K-major, a K tile's gate rows, then
+        // its up rows).  Through TMEM, whose lanes are rows, the four warps of one scheduler would do all of it.
+        for (int kt = ud.kt_begin; kt < ud.kt_end; kt += SUB, rr.next(NR)) {
+          const uint32_t r = rr.s;
+          ok = __all_sync(0xffffffffu, mbar_wait(&rawfull[r], rr.parity, &s_abort, p.f.wait_limit_ns));
+          if (!ok) break;
+          const uint8_t* raw = raw_ring + r * RAW_BYTES;
+          const uint32_t s = rp.s;
+          ok = __all_sync(0xffffffffu, mbar_wait(&empty[s], rp.parity ^ 1, &s_abort, p.f.wait_limit_ns));
+          if (!ok) break;
+          tc_fence_after();
+          const int cw = ct >> 5, t = cw & 1, x = lane & 7;
+          const uint8_t* src = raw + t * 16384 + lane * 128;
+          uint8_t* dst = smem + s * STAGE_BYTES + t * (kRowsSmall * 128) + lane * 128;
+          if (QF == 1) {  // warp: gate | up, 16-value quarter, K tile
+            const int q = (cw >> 1) & 3, j = cw >> 3;
+            const uint4 v = *reinterpret_cast<const uint4*>(src + (((4 * j + q) ^ x) << 4));
+            uint4 o0, o1;
+            e4m3x4_to_bf16(p.shifts, v.x, o0.x, o0.y);
+            e4m3x4_to_bf16(p.shifts, v.y, o0.z, o0.w);
+            e4m3x4_to_bf16(p.shifts, v.z, o1.x, o1.y);
+            e4m3x4_to_bf16(p.shifts, v.w, o1.z, o1.w);
+            dst += j * (2 * kRowsSmall * 128);
+            *reinterpret_cast<uint4*>(dst + (((2 * q) ^ x) << 4)) = o0;
+            *reinterpret_cast<uint4*>(dst + (((2 * q + 1) ^ x) << 4)) = o1;
+          } else {  // warp: gate | up, 32-value half (one scale block), K tile
+            const int h = (cw >> 1) & 1, j = cw >> 2;
+            const uint4 v = *reinterpret_cast<const uint4*>(src + (((2 * j + h) ^ x) << 4));
+            uint4 o[4];
+            e2m1x32_to_bf16(p.shifts, v, raw[32768 + t * 2048 + lane * 16 + ((kt * 2) & 15) + 2 * j + h], o);
+            dst += j * (2 * kRowsSmall * 128);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) *reinterpret_cast<uint4*>(dst + (((4 * h + i) ^ x) << 4)) = o[i];
+          }
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) {
+            mbar_arrive(&full[s]);
+            mbar_arrive(&rawempty[r]);
+          }
+          rp.next(NS);
+        }
+        continue;
+      }
       for (int kt = ud.kt_begin; kt < ud.kt_end && ok; kt += SUB, rr.next(NR)) {
         const uint32_t r = rr.s;
         ok = __all_sync(0xffffffffu, mbar_wait(&rawfull[r], rr.parity, &s_abort, p.f.wait_limit_ns));
@@ -929,6 +1042,9 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     const int quad = warp & 3;
     const int row = quad * 32 + lane;  // row of the 128-row tile
     AccBuffers acc;
+    // (behind the rings)
+    float* s_up = reinterpret_cast<float*>(raw_ring + (size_t)NR * RAW_BYTES);
+    uint32_t handed = 0;     // batches of accumulator columns passed between the two warps
     bool rows_seen = false;  // every row of y has been zeroed (and the shared expert's gates are there)
     for (uint32_t n = 0;; ++n) {
       const UnitDesc ud = next_unit(n);
@@ -965,8 +1081,8 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
       if (warp == kEpiWarp0 && lane == 0) TCTL(n, 3);
       const uint32_t tacc = tmem_base + b0 * tc_acc_cols(QF) + ((uint32_t)(quad * 32) << 16);
       if (ud.phase == 1) {
-        const int i = ud.blk * 128 + row;
-        const bool row_ok = i < (shared ? I_s : I);
+        const int i = ud.blk * p.rows1 + row;
+        const bool row_ok = row < p.rows1 && i < (shared ? I_s : I);
         float sg = 1.f, su = 1.f, sd = 1.f;
         if (QF == 1 && row_ok) {  // the row's three fp32 scales follow its 3 d code bytes
           const uint8_t* wb = shared ? p.f.shared_w : p.f.cache + (size_t)p.f.snap.expert_slot[ud.expert] * p.f.slot_stride;
@@ -975,10 +1091,19 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
           su = __ldg(sc + 1);
           sd = __ldg(sc + 2);
         }
-        for (int c0 = 0; c0 < ud.n_tok; c0 += 16) {
+        const bool small = p.rows1 == kRowsSmall;
+        // (32 rows: the up half of the accumulator is the second warp's; it passes its values on, two batches in turn)
+        for (int c0 = 0; c0 < ud.n_tok && !(small && quad > 0); c0 += 16) {
           uint32_t a[16], b2[16];
           tmem_ld16(tacc + (uint32_t)c0, a);
-          tmem_ld16(tacc + second + (uint32_t)c0, b2);
+          if (small) {
+            const float* up = s_up + (handed++ & 1u) * 512 + lane;
+            asm volatile("bar.sync 2, 64;" ::: "memory");
+#pragma unroll
+            for (int j = 0; j < 16; ++j) b2[j] = __float_as_uint(up[j * 32]);
+          } else {
+            tmem_ld16(tacc + second + (uint32_t)c0, b2);
+          }
           const float gates = gates_next;
           gates_next = load_gates(c0 + 16);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
@@ -998,6 +1123,17 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
                 dst[(size_t)j * p.act_stride + p.act_plane] = __float2bfloat16(v[j] - __bfloat162float(hi));
               }
             }
+          }
+        }
+        if (small && quad == 1) {
+          for (int c0 = 0; c0 < ud.n_tok; c0 += 16) {
+            uint32_t u[16];
+            tmem_ld16(tacc + (uint32_t)c0, u);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            float* up = s_up + (handed++ & 1u) * 512 + lane;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) up[j * 32] = __uint_as_float(u[j]);
+            asm volatile("bar.sync 2, 64;" ::: "memory");
           }
         }
         release();
@@ -1088,19 +1224,27 @@ bool tc_make_activation_maps(TcMaps* m, const void* xb, int d, int max_batch, co
 
 // The weight maps of one store (the slots of all layers, or one shared expert): n_slots consecutive slots of I rows.  Rows
 // past I (the last tile of an I that is not a multiple of the tile) read as zero.
-bool tc_make_store_maps(int fmt, void* weights, void* scales, const void* base, int d, int I, size_t n_slots, size_t slot_bytes) {
+bool tc_make_store_maps(int fmt, unsigned char (*weights)[128], unsigned char (*scales)[128], const void* base, int d, int I, size_t n_slots, size_t slot_bytes) {
+  const cuuint32_t rows[2] = {fmt == 0 ? 64u : 128u, (cuuint32_t)kRowsSmall};
   if (fmt == 0) {  // [I][3][d] bf16
     const cuuint64_t dims[4] = {(cuuint64_t)d, 3, (cuuint64_t)I, (cuuint64_t)n_slots};
     const cuuint64_t strides[3] = {(cuuint64_t)d * 2, (cuuint64_t)d * 6, (cuuint64_t)slot_bytes};
-    const cuuint32_t box[4] = {64, 1, 64, 1};
-    return encode(weights, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
+    for (int i = 0; i < 2; ++i) {
+      const cuuint32_t box[4] = {64, 1, rows[i], 1};
+      if (!encode(weights[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B)) return false;
+    }
+    return true;
   }
   const size_t rb = ffn_row_bytes(fmt, d);  // raw bytes [I][row bytes]
   const cuuint64_t dims[3] = {(cuuint64_t)rb, (cuuint64_t)I, (cuuint64_t)n_slots};
   const cuuint64_t strides[2] = {(cuuint64_t)rb, (cuuint64_t)slot_bytes};
-  const cuuint32_t box[3] = {128, 128, 1}, sbox[3] = {16, 128, 1};
-  return encode(weights, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B) &&
-         encode(scales, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, base, dims, strides, sbox, CU_TENSOR_MAP_SWIZZLE_NONE);
+  for (int i = 0; i < 2; ++i) {
+    const cuuint32_t box[3] = {128, rows[i], 1}, sbox[3] = {16, rows[i], 1};
+    if (!encode(weights[i], CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !encode(scales[i], CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, base, dims, strides, sbox, CU_TENSOR_MAP_SWIZZLE_NONE))
+      return false;
+  }
+  return true;
 }
 
 namespace {
@@ -1116,13 +1260,18 @@ cudaError_t launch_tc(const TcParams& p, const TcMaps& m, cudaLaunchConfig_t& cf
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < kMaxDevices) configured[dev] = true;
   }
-  const CUtensorMap* w = reinterpret_cast<const CUtensorMap*>(m.w);
-  const CUtensorMap* ws = reinterpret_cast<const CUtensorMap*>(p.f.shared_w ? m.ws : m.w);
-  // the 16-byte-box maps are used for the e2m1 store only; bf16 passes the weight maps again
-  const CUtensorMap* sc = QF ? reinterpret_cast<const CUtensorMap*>(m.sc) : w;
-  const CUtensorMap* ssc = QF ? reinterpret_cast<const CUtensorMap*>(p.f.shared_w ? m.ssc : m.sc) : w;
+  TcWeightMaps w;
+  const int v1 = p.rows1 == kRowsSmall ? 1 : 0;
+  for (int ph = 0; ph < 2; ++ph) {
+    const int v = ph ? 0 : v1;
+    memcpy(&w.codes[ph][0], m.w[v], 128);
+    memcpy(&w.codes[ph][1], p.f.shared_w ? m.ws[v] : m.w[v], 128);
+    // the 16-byte-box maps are used for the e2m1 store only; the others pass the weight maps again
+    memcpy(&w.scales[ph][0], QF == 2 ? m.sc[v] : m.w[v], 128);
+    memcpy(&w.scales[ph][1], QF == 2 ? (p.f.shared_w ? m.ssc[v] : m.sc[v]) : m.w[v], 128);
+  }
   cfg.blockDim = dim3(tc_threads(QF), 1, 1);
-  return cudaLaunchKernelEx(&cfg, ffn_tc_kernel<QF>, *w, *ws, *sc, *ssc, *reinterpret_cast<const CUtensorMap*>(m.x), *reinterpret_cast<const CUtensorMap*>(m.xc),
+  return cudaLaunchKernelEx(&cfg, ffn_tc_kernel<QF>, w, *reinterpret_cast<const CUtensorMap*>(m.x), *reinterpret_cast<const CUtensorMap*>(m.xc),
                             *reinterpret_cast<const CUtensorMap*>(m.act), p);
 }
 }  // namespace
@@ -1138,10 +1287,20 @@ cudaError_t launch_ffn_tc(const TcParams& p_in, const TcMaps& m, int n_sm, cudaS
   p.nmax2 = b16 < 64 ? b16 : 64;
   p.shift1 = p.f.B <= p.nmax1 ? 20 : 7;  // (more tokens than a unit takes: the unit takes 128 or 64)
   p.shift2 = p.f.B <= p.nmax2 ? 20 : 6;
+  // Rows of I per gate/up unit: 32 where that still gives every CTA at most one unit, were all experts executed that B tokens
+  // can ask for.  A unit is a chain over all of d, so with fewer units than CTAs the launch takes as long as one unit does,
+  // and what a stage costs is the loops of its roles, 800 cycles whatever it holds: at d = 4096, I = 256 a step of
+  // two tokens was 79 us per layer (bf16) and 99 (e2m1) with 128 rows and one K tile per stage, 65 and 77 so.  With
+  // more units than CTAs 128 rows read the activations a quarter as often.  (More than 128 rows of X in a stage of several
+  // K tiles would leave no room for a ring.)
+  const int experts = p.f.N < p.f.B * p.f.k ? p.f.N : p.f.B * p.f.k;
+  const int small_units = experts * ((p.f.I + kRowsSmall - 1) / kRowsSmall) + (p.f.run_shared ? (p.f.I_shared + kRowsSmall - 1) / kRowsSmall : 0);
+  const bool small = small_units <= n_sm && p.nmax1 * tc_wide(qf) <= 128;
+  p.rows1 = small ? kRowsSmall : 128;
   for (int q = 0; q < 2; ++q) {
     TcGeometry& g = p.geo[q];
     const int rows = q ? p.f.I_shared : p.f.I, most = qf ? kDownTilesQ : kDownTiles, sub = tc_sub(qf);
-    g.blocks1 = (rows + 127) / 128;
+    g.blocks1 = (rows + p.rows1 - 1) / p.rows1;
     g.tiles = (rows + kKTile - 1) / kKTile;
     if (!g.tiles) continue;
     const int n = (g.tiles + most - 1) / most;
@@ -1149,9 +1308,11 @@ cudaError_t launch_ffn_tc(const TcParams& p_in, const TcMaps& m, int n_sm, cudaS
     g.kch = (g.tiles + g.chunk - 1) / g.chunk;
     g.kch_inv = g.kch > 1 ? (uint32_t)((0x100000000ull + g.kch - 1) / g.kch) : 0u;
   }
-  const int b_bytes = p.nmax1 * 128 > 2 * p.nmax2 * 128 ? p.nmax1 * 128 : 2 * p.nmax2 * 128;
+  const int b1 = p.nmax1 * (small ? tc_wide(qf) : 1);
+  const int b_bytes = b1 * 128 > 2 * p.nmax2 * 128 ? b1 * 128 : 2 * p.nmax2 * 128;
   p.stage_bytes = kABytes + ((b_bytes + 1023) & ~1023);
-  const int budget = kTcSmemBudget - 1024;
+  const int behind = small ? kHandBytes : 0;
+  const int budget = kTcSmemBudget - 1024 - behind;
   if (qf == 0) {
     p.nraw = 0;
     p.nstage = budget / p.stage_bytes < kMaxStages ? budget / p.stage_bytes : kMaxStages;
@@ -1170,7 +1331,7 @@ cudaError_t launch_ffn_tc(const TcParams& p_in, const TcMaps& m, int n_sm, cudaS
   cfg.gridDim = dim3(n_sm, 1, 1);
   // Each CTA allocates all 512 TMEM columns, so two CTAs must never share an SM (the second would sit in
   // tcgen05.alloc until the first has finished): the rings take more than half an SM's shared memory in any case.
-  cfg.dynamicSmemBytes = (size_t)p.nstage * p.stage_bytes + (size_t)p.nraw * tc_raw_bytes(qf) + 1024;
+  cfg.dynamicSmemBytes = (size_t)p.nstage * p.stage_bytes + (size_t)p.nraw * tc_raw_bytes(qf) + 1024 + behind;
   return qf == 1 ? launch_tc<1>(p, m, cfg) : qf == 2 ? launch_tc<2>(p, m, cfg) : launch_tc<0>(p, m, cfg);
 }
 

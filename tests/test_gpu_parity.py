@@ -240,10 +240,12 @@ def test_fp8_store_of_subnormal_codes(B):
 
 
 @pytest.mark.parametrize("fmt", ["bf16", "fp8", "fp4"])
-@pytest.mark.parametrize("N,k,I,I_shared,B", [(4, 2, 72, 200, 2), (5, 2, 200, 0, 31), (3, 1, 130, 72, 130), (2, 2, 1100, 64, 256)])
+@pytest.mark.parametrize("N,k,I,I_shared,B", [(4, 2, 72, 200, 2), (5, 2, 200, 0, 31), (3, 1, 130, 72, 130), (2, 2, 1100, 64, 256),
+                                                  (6, 2, 700, 90, 40), (16, 3, 648, 200, 24)])
 def test_grouped_gemm_tile_edges(fmt, N, k, I, I_shared, B):
-    """Intermediate sizes off the 64- and 128-row tiles (the rest reads as zero), one and several chunks of K in the down
-    projection, and groups of 2 to 256 tokens: one part or several, and on the quantised stores both accumulator layouts."""
+    """Intermediate sizes off the 64- and 128-row tiles (the rest reads as zero), gate/up units of 32 rows (the first two, and
+    on the e4m3 store the fifth) and of 128, one and several chunks of K in the down projection, and groups of 2 to 256
+    tokens: one part or several, and on the quantised stores both accumulator layouts."""
     cfg = synth.tiny_config(d=512, N=N, k=k, I=I, C=N, T=2, I_shared=I_shared, sigma_p=1.0, cfg_id=279)
     run = {"bf16": _run, "fp8": _run_fp8, "fp4": _run_fp4}[fmt]
     rep, stats = run(cfg, mode="exact", tau=0.8, T=2, B=B, ffn_token_stride=max(1, B // 16))
