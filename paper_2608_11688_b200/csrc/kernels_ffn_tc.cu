@@ -1108,19 +1108,24 @@ ffn_tc_kernel(const __grid_constant__ TcWeightMaps tm_w, const __grid_constant__
           gates_next = load_gates(c0 + 16);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
           __nv_bfloat16* dst = p.act + (size_t)(ud.pair_off + c0) * p.act_stride + i;
-          float v[16];
+          // (eight independent chains at a time; columns past the last token are not stored)
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {  // (no branches: sixteen independent chains; columns past the last token are not stored)
-            const float gq = sg * __uint_as_float(a[j]), uq = su * __uint_as_float(b2[j]);
-            v[j] = __shfl_sync(0xffffffffu, gates, j) * (gq / (1.f + expf(-gq))) * uq * sd;
-          }
-          if (row_ok) {
+          for (int j0 = 0; j0 < 16; j0 += 8) {
+            if (c0 + j0 >= ud.n_tok) break;
+            float v[8];
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              if (c0 + j < ud.n_tok) {
-                const __nv_bfloat16 hi = __float2bfloat16(v[j]);
-                dst[(size_t)j * p.act_stride] = hi;
-                dst[(size_t)j * p.act_stride + p.act_plane] = __float2bfloat16(v[j] - __bfloat162float(hi));
+            for (int j = 0; j < 8; ++j) {
+              const float gq = sg * __uint_as_float(a[j0 + j]), uq = su * __uint_as_float(b2[j0 + j]);
+              v[j] = __shfl_sync(0xffffffffu, gates, j0 + j) * (gq / (1.f + expf(-gq))) * uq * sd;
+            }
+            if (row_ok) {
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                if (c0 + j0 + j < ud.n_tok) {
+                  const __nv_bfloat16 hi = __float2bfloat16(v[j]);
+                  dst[(size_t)(j0 + j) * p.act_stride] = hi;
+                  dst[(size_t)(j0 + j) * p.act_stride + p.act_plane] = __float2bfloat16(v[j] - __bfloat162float(hi));
+                }
               }
             }
           }
