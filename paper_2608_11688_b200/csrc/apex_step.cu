@@ -660,10 +660,15 @@ int apex_decode_token(apex_ctx* ctx, const float* h_dev, const float* hpost_dev,
     if (standin && !standin_first && (r = apex_attention_standin(ctx, l, stream)) != APEX_OK) return r;
     if ((r = apex_route_topk(ctx, l, hpost_dev + l * step, B, idx, alpha, stream)) != APEX_OK) return r;
     if (l > 0 && (r = ffn_finalize(ctx, l - 1)) != APEX_OK) return r;
-    if (prefetching && (r = apex_prefetch(ctx, l, B, nullptr)) != APEX_OK) return r;
+    // With every expert of the layer in a slot no candidate set changes the table (only its LRU stamps): the expert FFN of a
+    // batch is launched without waiting for the candidate records, a host round trip of 5 to 10 us that short layers
+    // (small d, short context) do not hide.
+    const bool settled = B > 1 && ctx->tables[l].all_resident();
+    if (prefetching && !settled && (r = apex_prefetch(ctx, l, B, nullptr)) != APEX_OK) return r;
     if ((r = ffn_launch(ctx, l, mode, hpost_dev + l * step, B, y_dev + l * step, ctx->d_exec_idx, ctx->d_exec_gate,
                         (cudaStream_t)stream)) != APEX_OK)
       return r;
+    if (prefetching && settled && (r = apex_prefetch(ctx, l, B, nullptr)) != APEX_OK) return r;
   }
   return ffn_finalize(ctx, ctx->cfg.L - 1);
 }

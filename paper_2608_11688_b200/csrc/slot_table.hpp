@@ -80,6 +80,11 @@ class SlotTable {
       }
     return plan_prefetch(count, copies, U_mask_out);
   }
+  bool all_resident() const {
+    for (int e = 0; e < N_; ++e)
+      if (expert_slot_[e] < 0) return false;
+    return true;
+  }
   // The same from the number of tokens that want each expert.
   bool plan_prefetch(const int* count, std::vector<SlotCopy>* copies, uint64_t* U_mask_out = nullptr) {
     std::vector<int> wanted;
