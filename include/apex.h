@@ -38,8 +38,8 @@
  * to a multiple of 16 bytes,
  *   [I][ gate_i (d/2 bytes) | up_i (d/2) | downT_i (d/2) | gate scales (d/32) | up scales | downT scales | pad ],
  * weight = scale of its block * code.
- * Both need d in {512, 1024, 1536, 2048, 4096} and exclude each other; batched steps then run the
- * streaming kernel per (token, expert) pair (no tensor-core path for these formats yet).
+ * Both need d in {512, 1024, 1536, 2048, 4096} and exclude each other; batched steps run on the tensor
+ * cores in every format (codes are expanded to bf16 on chip, which is exact).
  */
 #ifndef APEX_H
 #define APEX_H
