@@ -1082,7 +1082,10 @@ ffn_tc_kernel(const __grid_constant__ TcWeightMaps tm_w, const __grid_constant__
       const uint32_t tacc = tmem_base + b0 * tc_acc_cols(QF) + ((uint32_t)(quad * 32) << 16);
       if (ud.phase == 1) {
         const int i = ud.blk * p.rows1 + row;
+        // Rows between I and the end of its last K tile are stored as zeroes: the down projection reads them, and what a wider
+        // group of an earlier step left there may be an Inf or NaN, which zero weights do not cancel.
         const bool row_ok = row < p.rows1 && i < (shared ? I_s : I);
+        const bool row_read = row < p.rows1 && i < p.geo[shared ? 1 : 0].tiles * kKTile;
         float sg = 1.f, su = 1.f, sd = 1.f;
         if (QF == 1 && row_ok) {  // the row's three fp32 scales follow its 3 d code bytes
           const uint8_t* wb = shared ? p.f.shared_w : p.f.cache + (size_t)p.f.snap.expert_slot[ud.expert] * p.f.slot_stride;
@@ -1117,8 +1120,9 @@ ffn_tc_kernel(const __grid_constant__ TcWeightMaps tm_w, const __grid_constant__
             for (int j = 0; j < 8; ++j) {
               const float gq = sg * __uint_as_float(a[j0 + j]), uq = su * __uint_as_float(b2[j0 + j]);
               v[j] = __shfl_sync(0xffffffffu, gates, j0 + j) * (gq / (1.f + expf(-gq))) * uq * sd;
+              if (!row_ok) v[j] = 0.f;
             }
-            if (row_ok) {
+            if (row_read) {
 #pragma unroll
               for (int j = 0; j < 8; ++j) {
                 if (c0 + j0 + j < ud.n_tok) {
@@ -1305,8 +1309,8 @@ cudaError_t launch_ffn_tc(const TcParams& p_in, const TcMaps& m, int n_sm, cudaS
   for (int q = 0; q < 2; ++q) {
     TcGeometry& g = p.geo[q];
     const int rows = q ? p.f.I_shared : p.f.I, most = qf ? kDownTilesQ : kDownTiles, sub = tc_sub(qf);
-    g.blocks1 = (rows + p.rows1 - 1) / p.rows1;
     g.tiles = (rows + kKTile - 1) / kKTile;
+    g.blocks1 = (g.tiles * kKTile + p.rows1 - 1) / p.rows1;  // whole K tiles of the down projection (zeroes past I)
     if (!g.tiles) continue;
     const int n = (g.tiles + most - 1) / most;
     g.chunk = ((g.tiles + n - 1) / n + sub - 1) / sub * sub;  // whole raw tiles
