@@ -38,8 +38,12 @@
  * to a multiple of 16 bytes,
  *   [I][ gate_i (d/2 bytes) | up_i (d/2) | downT_i (d/2) | gate scales (d/32) | up scales | downT scales | pad ],
  * weight = scale of its block * code.
- * Both need d in {512, 1024, 1536, 2048, 4096} and exclude each other; batched steps run on the tensor
- * cores in every format (codes are expanded to bf16 on chip, which is exact).
+ * Both need d in {512, 1024, 1536, 2048, 4096} and exclude each other.
+ *
+ * Batched expert FFN (B > 1, every format): where I and I_shared are multiples of 128 it runs on the tensor cores (codes
+ * are expanded to bf16 on chip, which is exact); h' is then rounded to bf16 and the gated intermediate carried as two bf16
+ * values (2^-17).  Other sizes stream the rows of each (expert, token) pair, with h' and the intermediate in fp32, as a
+ * single token does.
  */
 #ifndef APEX_H
 #define APEX_H

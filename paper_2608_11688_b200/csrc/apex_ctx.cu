@@ -117,11 +117,17 @@ int apex_create(const apex_config* cfg, apex_ctx** out) {
   CR(dev_alloc(&ctx->d_alpha, L * MB * N));
   CR(dev_alloc(&ctx->d_exec_gate, MB * k));
   CR(dev_alloc(&ctx->d_cand_ncand, MB));
-  // batched path (only for contexts that will see batches): scratch and tensor maps of the grouped GEMM
-  if (MB > 1) {
-    const size_t max_pairs = MB * (k + 1);
+  // batched path (only for contexts that will see batches): scratch and tensor maps of the grouped GEMM, or the pair list of
+  // the streaming kernel
+  const size_t max_pairs = MB * (k + 1);
+  if (MB > 1 && !tc_shape_supported(c.I, c.I_shared)) {
+    CR(dev_alloc(&ctx->d_pair_tok, max_pairs));
+    CR(dev_alloc(&ctx->d_pair_expert, max_pairs));
+    CR(dev_alloc(&ctx->d_pair_gate, max_pairs));
+    CR(dev_alloc(&ctx->d_n_pairs, 4));
+  } else if (MB > 1) {
     const size_t rows = max_pairs + 64;  // (boxes of the last group reach past its rows)
-    const size_t i_max = ((size_t)(c.I > c.I_shared ? c.I : c.I_shared) + 63) / 64 * 64;
+    const size_t i_max = (size_t)(c.I > c.I_shared ? c.I : c.I_shared);
     CR(dev_alloc(&ctx->d_tc_sync, (size_t)kTcSyncWords));
     CR(cudaMemset(ctx->d_tc_sync, 0, kTcSyncWords * sizeof(unsigned)));
     CR(dev_alloc(&ctx->d_sgate, MB));
@@ -135,6 +141,7 @@ int apex_create(const apex_config* cfg, apex_ctx** out) {
         !tc_make_activation_maps(&ctx->tc_maps, ctx->d_xb, c.d, (int)MB, ctx->d_act, rows, (int)i_max))
       return bail(APEX_ECUDA, "apex_create: a tensor map of the batched path could not be encoded", cudaSuccess);
     ctx->tc_shared_maps.assign(L, ctx->tc_maps);
+    ctx->tc_ok = true;
   }
   ctx->attn_bytes = (4 * d * d + 2 * (size_t)ctx->cfg.ctx_len * d) * 2;
   ctx->attn_layers = L < 8 ? L : 8;
@@ -208,7 +215,7 @@ int apex_destroy(apex_ctx* ctx) {
   cudaGetLastError();
   void* dev[] = {ctx->d_Wr, ctx->d_br, ctx->d_Wp, ctx->d_bp, ctx->d_w, ctx->d_theta, ctx->d_cache, ctx->d_slot_ready, ctx->d_zp,
                  ctx->d_qp, ctx->d_zr, ctx->d_demand, ctx->d_pi, ctx->d_ncand, ctx->d_stats, ctx->d_counters, ctx->d_tickets, ctx->d_spec,
-                 ctx->d_tc_sync, ctx->d_sgate, ctx->d_xb, ctx->d_act, ctx->d_cand,
+                 ctx->d_pair_tok, ctx->d_pair_expert, ctx->d_pair_gate, ctx->d_n_pairs, ctx->d_tc_sync, ctx->d_sgate, ctx->d_xb, ctx->d_act, ctx->d_cand,
                  ctx->d_idx, ctx->d_exec_idx, ctx->d_alpha, ctx->d_exec_gate, ctx->d_cand_ncand, ctx->d_attn,
                  ctx->d_h_stage, ctx->d_hp_stage, ctx->d_y_stage};
   for (void* p : dev)
@@ -291,7 +298,7 @@ int apex_set_shared_expert(apex_ctx* ctx, int layer, const void* dev_weights) {
   ctx->shared_dev[layer] = static_cast<const uint8_t*>(dev_weights);
   if (ctx->d_shared_ptrs)
     CU_TRY(ctx, cudaMemcpy(ctx->d_shared_ptrs + layer, &dev_weights, sizeof(void*), cudaMemcpyHostToDevice));
-  if (!ctx->tc_shared_maps.empty()) {
+  if (ctx->tc_ok) {
     TcMaps& m = ctx->tc_shared_maps[layer];
     if (!tc_make_store_maps(ctx->fmt, m.ws, m.ssc, dev_weights, ctx->cfg.d, ctx->cfg.I_shared, 1, ctx->shared_bytes))
       return fail(ctx, APEX_ECUDA, "tensor map for the shared expert could not be encoded");

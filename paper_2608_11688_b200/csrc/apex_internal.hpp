@@ -133,6 +133,10 @@ struct FfnParams {
   int fmt;                      // storage format of the slots: 0 bf16, 1 e4m3 with per-row scales, 2 e2m1 with block scales
   int zero_early;               // 1: y may be zeroed before the dependency wait (the preceding kernel does not touch y)
   long long spec_delay_ns;      // the speculative first fill starts this long after the CTA does
+  // per-pair streaming of a batch: written by launch_ffn_plan
+  int32_t *pair_tok, *pair_expert;  // [B*k + B]; expert N = the shared one
+  float* pair_gate;                 // [B*k + B]
+  int32_t* n_pairs;                 // [1]
   const int32_t* spec;          // [k] predicted top-k of this layer-step (complete before the preceding kernel began), or null
   SlotSnapshot snap;
   size_t slot_stride;
@@ -154,7 +158,7 @@ inline void prefer_max_shared() {
   done[dev].store(true, std::memory_order_relaxed);
 }
 
-// Batched tensor-core path (kernels_ffn_tc.cu): B > 1
+// Batched tensor-core path (kernels_ffn_tc.cu): B > 1, I and I_shared multiples of 128
 // Words of the synchronisation block: zero between launches (the last CTA of one clears them)
 constexpr int kTcTicket = 0;                 // units handed out
 constexpr int kTcAbort = 1;                  // somebody gave up
@@ -261,9 +265,11 @@ struct AttnParams {
 cudaError_t launch_router(const RouterParams& p, cudaStream_t s);
 cudaError_t launch_select(const SelectParams& p, cudaStream_t s);
 cudaError_t launch_attention(const AttnParams& p, int n_sm, cudaStream_t s);
+cudaError_t launch_ffn_plan(const FfnParams& p, cudaStream_t s);  // B > 1, before launch_ffn
 cudaError_t launch_ffn(const FfnParams& p, int n_ctas, cudaStream_t s);  // n_ctas: grid size, at most ffn_grid_ctas(SM count)
 int ffn_grid_ctas(int n_sm);  // CTAs of one streaming-kernel launch (each adds one to the zero counter)
 cudaError_t launch_ffn_tc(const TcParams& p, const TcMaps& m, int n_sm, cudaStream_t s);
+bool tc_shape_supported(int I, int I_shared);  // does the grouped GEMM take these intermediate sizes
 bool tc_make_activation_maps(TcMaps* m, const void* xb, int d, int max_batch, const void* act, size_t act_rows, int act_stride);
 bool tc_make_store_maps(int fmt, unsigned char (*weights)[128], unsigned char (*scales)[128], const void* base, int d, int I, size_t n_slots, size_t slot_bytes);  // one store, in storage format fmt
 bool ffn_shape_supported(int d);
@@ -300,12 +306,14 @@ struct apex_ctx {
   int32_t *d_pi = nullptr, *d_ncand = nullptr;              // [maxB][N], [maxB]
   apex::DevStats* d_stats = nullptr;                        // [L]
   unsigned long long* d_counters = nullptr;                 // [2]: -, zero
-  // batched path (max_batch > 1)
+  // batched path (max_batch > 1): the grouped GEMM's scratch, or the pair list of the streaming kernel
+  bool tc_ok = false;
+  int32_t *d_pair_tok = nullptr, *d_pair_expert = nullptr, *d_n_pairs = nullptr;
+  float* d_pair_gate = nullptr;
   unsigned* d_tc_sync = nullptr;
   float* d_sgate = nullptr;
   __nv_bfloat16 *d_xb = nullptr, *d_act = nullptr;
   int act_stride = 0, act_rows = 0;
-  size_t act_plane = 0;
   apex::TcMaps tc_maps{};
   std::vector<apex::TcMaps> tc_shared_maps;  // per layer: ws / ssc filled
   uint8_t* d_attn = nullptr;

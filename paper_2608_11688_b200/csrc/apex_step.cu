@@ -408,8 +408,18 @@ cudaError_t launch_stream(apex_ctx* ctx, FfnParams p, cudaStream_t cs) {
 }
 
 
-// B > 1: the tensor-core grouped GEMM.
+// B > 1: the tensor-core grouped GEMM, or a plan and the streaming kernel over the (expert, token) pairs.
 int launch_batched(apex_ctx* ctx, int layer, const FfnParams& p, cudaStream_t cs) {
+  if (!ctx->tc_ok) {
+    CU_TRY(ctx, launch_ffn_plan(p, cs));
+    ctx->last_was_ffn = false;
+    ctx->last_pred_layer = -1;
+    ctx->last_stream = cs;
+    ++ctx->launches;
+    CU_TRY(ctx, launch_stream(ctx, p, cs));
+    ++ctx->launches;
+    return APEX_OK;
+  }
   TcParams t{};
   t.f = p;
   t.sync = ctx->d_tc_sync;
@@ -458,6 +468,10 @@ int ffn_launch(apex_ctx* ctx, int layer, int mode, const float* hpost_dev, int B
   p.mbox_status = &mhdr(ctx)->status;
   p.seq_value = ++ctx->exec_seq[layer];
   p.stats = ctx->d_stats + layer;
+  p.pair_tok = ctx->d_pair_tok;
+  p.pair_expert = ctx->d_pair_expert;
+  p.pair_gate = ctx->d_pair_gate;
+  p.n_pairs = ctx->d_n_pairs;
   p.zero_counter = ctx->d_counters + 1;
   p.snap = make_snapshot(ctx, layer);
   p.slot_stride = ctx->expert_bytes;

@@ -6,8 +6,10 @@
 // downT_i are contiguous (downT is W_down transposed) -- so one pass suffices and every CTA reads one
 // contiguous byte range:  a_i = g_e * silu(gate_i . h') * (up_i . h'),  y += a_i * downT_i.
 //
-// Kernel (one token; batches run kernels_ffn_tc.cu): persistent, one CTA per SM.  The (expert, i) row space is
-// cut into equal contiguous ranges, one per CTA.  Each of the eight warps streams its own rows
+// Kernel: persistent, one CTA per SM.  The (pair, i) row space -- a pair is (expert, token) -- is
+// cut into equal contiguous ranges, one per CTA.  One token plans its pairs itself (PAIRS false); a batch gets them from
+// kernels_plan.cu, sorted by expert (PAIRS true: batches whose intermediate sizes the grouped GEMM does not take, see
+// tc_shape_supported; h' and the intermediate are fp32 here).  Each of the eight warps streams its own rows
 // (row q of the CTA belongs to warp q mod 8) into its stages of a shared-memory ring with one bulk
 // asynchronous copy per row (TMA, mbarrier completion; issuing from eight threads instead of one
 // matters: one thread sustains only about one bulk copy per 570 cycles), does the two dot products
@@ -59,21 +61,23 @@ __host__ __device__ constexpr int ring_stages(uint32_t entry_bytes) {
 }
 
 // ---------------------------------------------------------------- the streaming FFN kernel
-// Row space of the step's one token: each executed routed expert owns I consecutive rows, then the shared expert its
-// I_shared; row r of an expert is intermediate index i = r - its first row.
+// Row space: pair p (a (token, expert) pair; routed pairs first, then the shared-expert pairs) owns
+// I (or I_shared) consecutive rows; row r of pair p is intermediate index i = r - its first row.
 struct RowMap {
-  int n_routed;          // executed routed experts
+  int n_routed;          // routed pairs
   int routed_rows;       // n_routed * I (the host refuses shapes whose row count does not fit 31 bits)
   int total_rows;
 };
 
 
-template <int NCH, bool H_REGS, int FMT>
+template <int NCH, bool H_REGS, int FMT, bool PAIRS>
 __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel(const FfnParams p) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ uint64_t s_full[kMaxStages];
   __shared__ int s_exp[kMaxStages];
-  __shared__ int s_pos[kConsumerWarps][APEX_MAX_TOPK];  // expert at each position of the row space (a copy per warp)
+  __shared__ float s_gate[PAIRS ? kMaxStages : 1];
+  __shared__ int s_tok[PAIRS ? kMaxStages : 1];
+  __shared__ int s_pos[kConsumerWarps][APEX_MAX_TOPK];  // one token: expert at each position of the row space (a copy per warp)
   __shared__ int s_abort;
 
   constexpr int d = NCH * 256;
@@ -103,7 +107,8 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   __syncthreads();  // barriers initialised
   float hreg[H_REGS ? NCH * 8 : 1];
-  if (H_REGS) {  // h' is an input of the gate kernel as well: complete long before this kernel
+  const float* hrow = p.hpost;
+  if (H_REGS && !PAIRS) {  // h' is an input of the gate kernel as well: complete long before this kernel
 #pragma unroll
     for (int c = 0; c < NCH; ++c) {
       const float4 a = __ldg(reinterpret_cast<const float4*>(p.hpost) + (c * 32 + lane) * 2);
@@ -117,7 +122,7 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
   // usual case: the gate kernel), after it otherwise.
   auto zero_slice = [&]() {
     if (p.accumulate) return;
-    const size_t n4 = (size_t)d / 4;
+    const size_t n4 = (size_t)(PAIRS ? p.B : 1) * d / 4;
     const size_t per = (n4 + G - 1) / G;
     const size_t lo = per * cta, hi = lo + per < n4 ? lo + per : n4;
     float4* y4 = reinterpret_cast<float4*>(p.y);
@@ -153,10 +158,10 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
   bool dynamic = false;
   int S = 0, chunk = 1, n_static = 0;
   int static_base = 0, dyn_begin = 0, dyn_rows = 0;
-  auto set_geometry = [&](int n_routed) {
+  auto set_geometry = [&](int n_routed, int n_shared) {
     rm.n_routed = n_routed;
     rm.routed_rows = n_routed * I;
-    rm.total_rows = rm.routed_rows + (p.run_shared ? p.I_shared : 0);
+    rm.total_rows = rm.routed_rows + n_shared * p.I_shared;
     const int per_cta = rm.total_rows / G, extra = rm.total_rows - per_cta * G;  // the first `extra` CTAs take one row more
     dynamic = per_cta >= 2 * NS;
     const int range_lo = cta * per_cta + (cta < extra ? cta : extra), range_hi = range_lo + per_cta + (cta < extra ? 1 : 0);
@@ -174,8 +179,9 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
       *pidx = (int)(r / I);
       *i = r - *pidx * I;
     } else {
-      *pidx = rm.n_routed;
-      *i = r - rm.routed_rows;
+      const int more = PAIRS ? (r - rm.routed_rows) / p.I_shared : 0;
+      *pidx = rm.n_routed + more;
+      *i = r - rm.routed_rows - more * p.I_shared;
     }
   };
 
@@ -184,7 +190,7 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
   // kernel is still running; after the dependency wait each guess is either confirmed (the copy is
   // already in flight or has landed) or dropped and its stage refilled.  Positions of the row space
   // that hold a confirmed guess keep it, so confirmed rows stay with the CTA that requested them.
-  bool spec_on = p.spec != nullptr;
+  bool spec_on = !PAIRS && p.spec != nullptr;
   int spec_e = -1;
   bool spec_issued = false;  // this lane started a speculative copy into its stage (stage index = lane)
   if (spec_on) {
@@ -204,7 +210,7 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
       const unsigned long long t0 = globaltimer_ns();
       while ((long long)(globaltimer_ns() - t0) < p.spec_delay_ns) __nanosleep(200);
     }
-    set_geometry(k);
+    set_geometry(k, p.run_shared ? 1 : 0);
     const int fill = n_static < NSW ? n_static : NSW;
     if (lane < fill) {
       int pidx;
@@ -234,15 +240,22 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
   if (!p.zero_early) zero_slice();  // a preceding launch of this library may still be adding to the same y
 
   // ---- every global load of the prologue is issued before the first use, so the latencies overlap.
-  const TokenLoads tl1 = load_token(p.idx, p.z_r, p.alpha, N, k, p.mode, lane);
+  TokenLoads tl1;
+  if (!PAIRS) tl1 = load_token(p.idx, p.z_r, p.alpha, N, k, p.mode, lane);
   if (tid == 0) TL(10);
 
-  // ---- plan: every warp derives the execution set itself
-  const TokenPlan tp1 = plan_token(tl1, p.mode, p.norm_topk, p.snap.resident_mask, lane);
+  // ---- plan: one token: every warp derives the execution set itself; a batch: the plan kernel wrote it
+  TokenPlan tp1;
+  tp1.exec_mask = tp1.kr_mask = 0ull;
+  tp1.g0 = tp1.g1 = 0.f;
+  if (!PAIRS) tp1 = plan_token(tl1, p.mode, p.norm_topk, p.snap.resident_mask, lane);
   const float g0 = tp1.g0, g1 = tp1.g1;
   const unsigned long long run = tp1.exec_mask & p.run_mask;
   bool spec_geometry = false;  // the speculative row space is the final one
-  {
+  if (PAIRS) {
+    const int n_shared = p.run_shared ? p.B : 0;
+    set_geometry(p.n_pairs[0] - n_shared, n_shared);
+  } else {
     const int n_routed = __popcll(run);
     spec_geometry = spec_on && n_routed == k;
     int pos_e = -1;
@@ -257,7 +270,7 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
       if (lane < k) pos_e = keep ? spec_e : nth_set_bit64(rest, __popc(gaps & ((1u << lane) - 1u)));
     } else {
       if (lane < n_routed) pos_e = nth_set_bit64(run, lane);
-      set_geometry(n_routed);
+      set_geometry(n_routed, p.run_shared ? 1 : 0);
     }
     if (lane < APEX_MAX_TOPK) s_pos[warp][lane] = pos_e;
     __syncwarp();
@@ -294,7 +307,7 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
   auto issue = [&](int r, int n) {
     int pidx, i;
     locate(r, &pidx, &i);
-    const int e = pidx < rm.n_routed ? s_pos[warp][pidx] : N;
+    const int e = PAIRS ? p.pair_expert[pidx] : pidx < rm.n_routed ? s_pos[warp][pidx] : N;
     const uint8_t* base;
     if (e < N) {
       int slot = p.snap.expert_slot[e];
@@ -353,6 +366,10 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
     }
     const int s = warp + kConsumerWarps * (n % NSW);
     s_exp[s] = e;
+    if (PAIRS) {
+      s_gate[s] = p.pair_gate[pidx];
+      s_tok[s] = p.pair_tok[pidx];
+    }
     mbar_expect_tx(&s_full[s], entry_bytes);
     bulk_g2s(smem + (size_t)s * entry_bytes, base + (size_t)i * entry_bytes, entry_bytes, &s_full[s]);
   };
@@ -373,7 +390,7 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
                    : "memory");
     }
   };
-  const bool poster = cta == 0 && warp == 0 && p.post_exec;
+  const bool poster = !PAIRS && cta == 0 && warp == 0 && p.post_exec;
   // ---- row supply of this warp (state lives in lane 0; the other lanes learn the outcome by shuffle)
   int next_static = 0;                 // static rows of this warp already started
   int dyn_cur = 0, dyn_end = 0;  // rows of the current ticket
@@ -443,7 +460,19 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
     ++tail;
   }
   bool polled = false;
-  float sgate = -1.f;  // value of the shared expert's gate, once computed
+  float sgate = -1.f;  // one token: value of the shared expert's gate, once computed
+  int cur_tok = -1;    // a batch: token whose h' and partial sums this warp holds
+  auto flush_token = [&]() {
+    if (lane == 0) poll_zeroed(true);
+    __syncwarp();
+    float4* y4 = reinterpret_cast<float4*>(p.y + (size_t)cur_tok * d);
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) {
+      const int col4 = (c * 32 + lane) * 2;
+      atomicAdd(y4 + col4, make_float4(acc[c * 8 + 0], acc[c * 8 + 1], acc[c * 8 + 2], acc[c * 8 + 3]));
+      atomicAdd(y4 + col4 + 1, make_float4(acc[c * 8 + 4], acc[c * 8 + 5], acc[c * 8 + 6], acc[c * 8 + 7]));
+    }
+  };
   for (int head = 0; head < tail; ++head) {
     if (__any_sync(0xffffffffu, *(volatile int*)&s_abort != 0)) break;
     const int s = warp + kConsumerWarps * (head % NSW);
@@ -455,10 +484,32 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
     if (lane == 0 && warp == 0 && head == 0) TL(5);
     if (lane == 0 && warp == 0) TL(6);
     const int e = s_exp[s];
-    float gate = __shfl_sync(0xffffffffu, e < 32 ? g0 : g1, e & 31);
-    if (e >= N) {  // the shared expert: weight 1, or its gate's value (computed when the warp meets its first shared row)
-      if (p.shared_gate && sgate < 0.f) sgate = shared_gate_weight(p.shared_gate, p.hpost, d, lane);
-      gate = p.shared_gate ? sgate : 1.f;
+    float gate;
+    if (PAIRS) {
+      gate = s_gate[s];
+      const int tok = s_tok[s];
+      if (tok != cur_tok) {
+        if (cur_tok >= 0) flush_token();
+#pragma unroll
+        for (int m = 0; m < NCH * 8; ++m) acc[m] = 0.f;
+        cur_tok = tok;
+        hrow = p.hpost + (size_t)tok * d;
+        if (H_REGS) {
+#pragma unroll
+          for (int c = 0; c < NCH; ++c) {
+            const float4 a = __ldg(reinterpret_cast<const float4*>(hrow) + (c * 32 + lane) * 2);
+            const float4 b2 = __ldg(reinterpret_cast<const float4*>(hrow) + (c * 32 + lane) * 2 + 1);
+            hreg[c * 8 + 0] = a.x; hreg[c * 8 + 1] = a.y; hreg[c * 8 + 2] = a.z; hreg[c * 8 + 3] = a.w;
+            hreg[c * 8 + 4] = b2.x; hreg[c * 8 + 5] = b2.y; hreg[c * 8 + 6] = b2.z; hreg[c * 8 + 7] = b2.w;
+          }
+        }
+      }
+    } else {
+      gate = __shfl_sync(0xffffffffu, e < 32 ? g0 : g1, e & 31);
+      if (e >= N) {  // the shared expert: weight 1, or its gate's value (computed when the warp meets its first shared row)
+        if (p.shared_gate && sgate < 0.f) sgate = shared_gate_weight(p.shared_gate, p.hpost, d, lane);
+        gate = p.shared_gate ? sgate : 1.f;
+      }
     }
     const uint8_t* gs = smem + (size_t)s * entry_bytes;
     const uint8_t* us = gs + row_bytes;
@@ -473,8 +524,8 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
 #pragma unroll
         for (int m = 0; m < 8; ++m) hh[m] = hreg[c * 8 + m];
       } else {
-        const float4 a = __ldg(reinterpret_cast<const float4*>(p.hpost) + (c * 32 + lane) * 2);
-        const float4 b2 = __ldg(reinterpret_cast<const float4*>(p.hpost) + (c * 32 + lane) * 2 + 1);
+        const float4 a = __ldg(reinterpret_cast<const float4*>(hrow) + (c * 32 + lane) * 2);
+        const float4 b2 = __ldg(reinterpret_cast<const float4*>(hrow) + (c * 32 + lane) * 2 + 1);
         hh[0] = a.x; hh[1] = a.y; hh[2] = a.z; hh[3] = a.w; hh[4] = b2.x; hh[5] = b2.y; hh[6] = b2.z; hh[7] = b2.w;
       }
       if (FMT == kFmtMxfp4) {  // the lane's eight elements share one block scale
@@ -550,6 +601,11 @@ __global__ void __launch_bounds__(kFfnThreads, kCtasPerSm) moe_ffn_stream_kernel
     }
   }
 
+  if (PAIRS) {
+    if (cur_tok >= 0 && !aborted) flush_token();
+    return;
+  }
+
   // ---- reduce the eight partial vectors in shared memory, then one vector atomic per float4
   __syncthreads();  // every ring entry has been consumed; the ring is free
   if (tid == 0) TL(7);
@@ -602,8 +658,8 @@ extern "C" int apex_debug_reset_spans() {
 }
 #endif
 
-template <int NCH, int FMT>
-static cudaError_t launch_ffn_t(const FfnParams& p, int n_ctas, cudaStream_t s) {
+template <int NCH, int FMT, bool PAIRS>
+static cudaError_t launch_ffn_p(const FfnParams& p, int n_ctas, cudaStream_t s) {
   constexpr bool HR = NCH <= 8;
   constexpr uint32_t entry = fmt_entry_bytes(FMT, NCH * 256);
   constexpr int NS = ring_stages(entry);
@@ -612,7 +668,7 @@ static cudaError_t launch_ffn_t(const FfnParams& p, int n_ctas, cudaStream_t s) 
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= kMaxDevices || !configured[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(moe_ffn_stream_kernel<NCH, HR, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(moe_ffn_stream_kernel<NCH, HR, FMT, PAIRS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < kMaxDevices) configured[dev] = true;
   }
@@ -626,7 +682,12 @@ static cudaError_t launch_ffn_t(const FfnParams& p, int n_ctas, cudaStream_t s) 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, moe_ffn_stream_kernel<NCH, HR, FMT>, p);
+  return cudaLaunchKernelEx(&cfg, moe_ffn_stream_kernel<NCH, HR, FMT, PAIRS>, p);
+}
+
+template <int NCH, int FMT>
+static cudaError_t launch_ffn_t(const FfnParams& p, int n_ctas, cudaStream_t s) {
+  return p.B > 1 ? launch_ffn_p<NCH, FMT, true>(p, n_ctas, s) : launch_ffn_p<NCH, FMT, false>(p, n_ctas, s);
 }
 
 bool ffn_shape_supported(int d) {

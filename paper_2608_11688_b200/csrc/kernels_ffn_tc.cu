@@ -311,7 +311,7 @@ ffn_tc_kernel(const __grid_constant__ TcWeightMaps tm_w, const __grid_constant__
   __shared__ uint8_t s_tok[APEX_MAX_BATCH * (APEX_MAX_TOPK + 1)];  // token of each pair
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int N = p.f.N, d = p.f.d, I = p.f.I, I_s = p.f.I_shared;
+  const int N = p.f.N, d = p.f.d;
 
   if (tid == 0) {
     s_abort = 0;
@@ -1082,10 +1082,7 @@ ffn_tc_kernel(const __grid_constant__ TcWeightMaps tm_w, const __grid_constant__
       const uint32_t tacc = tmem_base + b0 * tc_acc_cols(QF) + ((uint32_t)(quad * 32) << 16);
       if (ud.phase == 1) {
         const int i = ud.blk * p.rows1 + row;
-        // Rows between I and the end of its last K tile are stored as zeroes: the down projection reads them, and what a wider
-        // group of an earlier step left there may be an Inf or NaN, which zero weights do not cancel.
-        const bool row_ok = row < p.rows1 && i < (shared ? I_s : I);
-        const bool row_read = row < p.rows1 && i < p.geo[shared ? 1 : 0].tiles * kKTile;
+        const bool row_ok = row < p.rows1;
         float sg = 1.f, su = 1.f, sd = 1.f;
         if (QF == 1 && row_ok) {  // the row's three fp32 scales follow its 3 d code bytes
           const uint8_t* wb = shared ? p.f.shared_w : p.f.cache + (size_t)p.f.snap.expert_slot[ud.expert] * p.f.slot_stride;
@@ -1120,9 +1117,8 @@ ffn_tc_kernel(const __grid_constant__ TcWeightMaps tm_w, const __grid_constant__
             for (int j = 0; j < 8; ++j) {
               const float gq = sg * __uint_as_float(a[j0 + j]), uq = su * __uint_as_float(b2[j0 + j]);
               v[j] = __shfl_sync(0xffffffffu, gates, j0 + j) * (gq / (1.f + expf(-gq))) * uq * sd;
-              if (!row_ok) v[j] = 0.f;
             }
-            if (row_read) {
+            if (row_ok) {
 #pragma unroll
               for (int j = 0; j < 8; ++j) {
                 if (c0 + j0 + j < ud.n_tok) {
@@ -1227,12 +1223,17 @@ static bool rows_map(void* out, const void* base, int cols, size_t rows, size_t 
   return encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
+// Batches run here where I and I_shared are multiples of the 128-row tile.  This path rounds h' to bf16 and carries the
+// intermediate to 2^-17; the streaming kernel, which takes all other sizes a (expert, token) pair at a time, keeps both in
+// fp32, and so do its batches: relative error of y at d = 512 2e-7 .. 3e-7 there against 2e-3 here for h' with 24 bits
+// (for bf16-representable h' 2e-6 to 3e-6 here).
+bool tc_shape_supported(int I, int I_shared) { return I % 128 == 0 && I_shared % 128 == 0; }
+
 bool tc_make_activation_maps(TcMaps* m, const void* xb, int d, int max_batch, const void* act, size_t act_rows, int act_stride) {
   return rows_map(m->x, xb, d, max_batch, d, 1) && rows_map(m->xc, xb, d, max_batch, d, kARowsPerLoad) && rows_map(m->act, act, act_stride, 2 * act_rows, act_stride, kARowsPerLoad);
 }
 
-// The weight maps of one store (the slots of all layers, or one shared expert): n_slots consecutive slots of I rows.  Rows
-// past I (the last tile of an I that is not a multiple of the tile) read as zero.
+// The weight maps of one store (the slots of all layers, or one shared expert): n_slots consecutive slots of I rows.
 bool tc_make_store_maps(int fmt, unsigned char (*weights)[128], unsigned char (*scales)[128], const void* base, int d, int I, size_t n_slots, size_t slot_bytes) {
   const cuuint32_t rows[2] = {fmt == 0 ? 64u : 128u, (cuuint32_t)kRowsSmall};
   if (fmt == 0) {  // [I][3][d] bf16
@@ -1303,14 +1304,14 @@ cudaError_t launch_ffn_tc(const TcParams& p_in, const TcMaps& m, int n_sm, cudaS
   // more units than CTAs 128 rows read the activations a quarter as often.  (More than 128 rows of X in a stage of several
   // K tiles would leave no room for a ring.)
   const int experts = p.f.N < p.f.B * p.f.k ? p.f.N : p.f.B * p.f.k;
-  const int small_units = experts * ((p.f.I + kRowsSmall - 1) / kRowsSmall) + (p.f.run_shared ? (p.f.I_shared + kRowsSmall - 1) / kRowsSmall : 0);
+  const int small_units = experts * (p.f.I / kRowsSmall) + (p.f.run_shared ? p.f.I_shared / kRowsSmall : 0);
   const bool small = small_units <= n_sm && p.nmax1 * tc_wide(qf) <= 128;
   p.rows1 = small ? kRowsSmall : 128;
   for (int q = 0; q < 2; ++q) {
     TcGeometry& g = p.geo[q];
     const int rows = q ? p.f.I_shared : p.f.I, most = qf ? kDownTilesQ : kDownTiles, sub = tc_sub(qf);
-    g.tiles = (rows + kKTile - 1) / kKTile;
-    g.blocks1 = (g.tiles * kKTile + p.rows1 - 1) / p.rows1;  // whole K tiles of the down projection (zeroes past I)
+    g.blocks1 = rows / p.rows1;
+    g.tiles = rows / kKTile;
     if (!g.tiles) continue;
     const int n = (g.tiles + most - 1) / most;
     g.chunk = ((g.tiles + n - 1) / n + sub - 1) / sub * sub;  // whole raw tiles

@@ -25,6 +25,7 @@ KERNEL_NAMES = {
     3: "attention stand-in",
     4: "gate",
     5: "expert FFN, streaming",
+    6: "FFN plan (B > 1, per-pair streaming)",
     8: "expert FFN, grouped GEMM (B > 1)",
     10: "persistent token kernel (all layers, B = 1)",
 }

@@ -50,3 +50,41 @@ def test_an_overflowing_step_leaves_nothing_for_the_next():
         assert np.isfinite(y).all() and _rel(y, ref) <= 3e-5
     finally:
         ctx.destroy()
+
+
+@pytest.mark.parametrize("fmt", ["bf16", "fp8", "fp4"])
+@pytest.mark.parametrize("I,I_shared,B", [(72, 0, 2), (192, 128, 5), (128, 200, 7), (320, 0, 40), (130, 72, 256)])
+def test_batches_off_the_128_row_tiles_keep_fp32_hidden_states(fmt, I, I_shared, B):
+    # h' with all 24 bits: rounding it to bf16 would show as about 2^-9.  The sums: a lane's chains of 16 products and 5 levels
+    # of a tree per dot product, then at most I + I_shared fp32 additions into y, every one to half an ulp (2^-24) in
+    # either direction; 2^-24 (16 + 5 + sqrt(I + I_shared)) of the terms' size is below 3e-6 for these shapes
+    prob = _problem(fmt, d=512, N=8, k=2, I=I, I_shared=I_shared, cfg_id=321)
+    ctx = prob.make_ctx(max_batch=B)
+    try:
+        ctx.warm_all()
+        y, ref = _step(prob, ctx, np.random.default_rng(321 + B).standard_normal((B, 512)).astype(np.float32))
+        rel = _rel(y, ref)
+        print("fp32 h'", fmt, I, I_shared, B, rel)
+        assert rel <= 3e-6
+    finally:
+        ctx.destroy()
+
+
+@pytest.mark.parametrize("fmt", ["bf16", "fp8", "fp4"])
+@pytest.mark.parametrize("N,k,I,I_shared,B", [(4, 2, 128, 256, 2), (5, 2, 256, 0, 31), (3, 1, 128, 384, 130), (2, 2, 1152, 128, 256),
+                                              (6, 2, 768, 128, 40), (16, 3, 640, 256, 24)])
+def test_grouped_gemm_tiles(fmt, N, k, I, I_shared, B):
+    # the sizes the grouped GEMM takes: gate/up units of 32 rows (the first two, and on the e4m3 store the fifth) and of 128,
+    # one and several chunks of K in the down projection, groups of 2 to 256 tokens: one part or several, and on the
+    # quantised stores both accumulator layouts.  h' is bf16-representable; the intermediate is carried to 2^-17 (7.6e-6)
+    prob = _problem(fmt, d=512, N=N, k=k, I=I, I_shared=I_shared, cfg_id=322)
+    ctx = prob.make_ctx(max_batch=B)
+    try:
+        ctx.warm_all()
+        hp = torch.from_numpy(np.random.default_rng(322 + B).standard_normal((B, 512)).astype(np.float32)).bfloat16().float().numpy()
+        y, ref = _step(prob, ctx, hp)
+        rel = _rel(y, ref)
+        print("bf16 h'", fmt, I, I_shared, B, rel)
+        assert rel <= 7.6e-6
+    finally:
+        ctx.destroy()
