@@ -268,7 +268,8 @@ int apex_set_slot_table(apex_ctx* ctx, int layer, const int32_t* expert_slot, co
 /* Makes every expert of every layer resident (needs C == N) and waits for the copies. */
 int apex_warm_all(apex_ctx* ctx);
 /* Host-side fault hooks for tests: what = 1 the next copy issue fails (APEX_ECUDA path);
- * what = 2 the next slot-ready flag is withheld (device wait runs out); 0 clears. */
+ * what = 2 the next slot-ready flag is withheld (device wait runs out); what = 3 the candidate records of the next
+ * launched budget selection are withheld (the host's wait in apex_prefetch runs out); 0 clears. */
 int apex_test_inject(apex_ctx* ctx, int what);
 /* Number of kernels this library has launched on the context so far. */
 int64_t apex_launch_count(const apex_ctx* ctx);

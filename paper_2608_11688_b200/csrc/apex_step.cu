@@ -164,6 +164,10 @@ int fill_select(apex_ctx* ctx, int layer, int B, float tau, int32_t* cand_dev, i
   p->mbox_cand = mbox_i32(ctx, ctx->ml.off_cand);
   p->mbox_rec = const_cast<uint32_t*>(mbox_sel_rec(ctx));
   p->seq_value = ++ctx->sel_seq;
+  if (ctx->inject == 3) {
+    ctx->inject = 0;
+    --p->seq_value;
+  }
   p->stats = ctx->d_stats + layer;
   p->force = tau <= 0.f ? 1 : (tau >= 1.f ? 2 : 0);
   p->t_tau = p->force ? 0.f : (float)std::log((double)tau / (1.0 - (double)tau));
@@ -646,15 +650,13 @@ int apex_moe_ffn_end(apex_ctx* ctx, int layer) {
   return ffn_finalize(ctx, layer);
 }
 
+namespace {
+
 // Pipelined over layers: the host work that needs the gate's decision of layer l-1 (LRU stamps,
 // demand copies) is done after the kernels of layer l have been queued, so that on the hit path
 // the GPU never waits for the host.
-int apex_decode_token(apex_ctx* ctx, const float* h_dev, const float* hpost_dev, int B, float tau, int mode, float* y_dev,
-                      void* stream) {
-  CHECK_CTX(ctx);
-  if (!h_dev || !hpost_dev || !y_dev || B < 1 || B > ctx->cfg.max_batch) return fail(ctx, APEX_EINVAL, "apex_decode_token: bad argument");
-  if (decode_persistent_usable(ctx, B))  // one persistent kernel over all layers
-    return decode_token_persistent(ctx, h_dev, hpost_dev, tau, mode, y_dev, (cudaStream_t)stream);
+// *launched: layers whose expert FFN has been launched
+int decode_layers(apex_ctx* ctx, const float* h_dev, const float* hpost_dev, int B, float tau, int mode, float* y_dev, void* stream, int* launched) {
   const size_t step = (size_t)B * ctx->cfg.d;
   const size_t MB = ctx->cfg.max_batch, k = ctx->cfg.k, N = ctx->cfg.N;
   const bool standin = !(ctx->cfg.flags & APEX_FLAG_SKIP_STANDIN);
@@ -682,9 +684,34 @@ int apex_decode_token(apex_ctx* ctx, const float* h_dev, const float* hpost_dev,
     if ((r = ffn_launch(ctx, l, mode, hpost_dev + l * step, B, y_dev + l * step, ctx->d_exec_idx, ctx->d_exec_gate,
                         (cudaStream_t)stream)) != APEX_OK)
       return r;
+    *launched = l + 1;
     if (prefetching && settled && (r = apex_prefetch(ctx, l, B, nullptr)) != APEX_OK) return r;
   }
   return ffn_finalize(ctx, ctx->cfg.L - 1);
+}
+
+// An error in the middle of decode_layers leaves launched expert FFNs without their host half (one layer back, or this
+// layer's where it went out before the candidate records): their demand copies may be waited for, and a layer-step that stays
+// pending refuses every later one.  Each is completed here; the first error is the one that is reported.
+void complete_pending(apex_ctx* ctx, int launched) {
+  const std::string err = ctx->err;
+  for (int l = 0; l < launched; ++l)
+    if (ctx->step[l].pending) ffn_finalize(ctx, l);
+  ctx->err = err;
+}
+
+}  // namespace
+
+int apex_decode_token(apex_ctx* ctx, const float* h_dev, const float* hpost_dev, int B, float tau, int mode, float* y_dev,
+                      void* stream) {
+  CHECK_CTX(ctx);
+  if (!h_dev || !hpost_dev || !y_dev || B < 1 || B > ctx->cfg.max_batch) return fail(ctx, APEX_EINVAL, "apex_decode_token: bad argument");
+  if (decode_persistent_usable(ctx, B))  // one persistent kernel over all layers
+    return decode_token_persistent(ctx, h_dev, hpost_dev, tau, mode, y_dev, (cudaStream_t)stream);
+  int launched = 0;
+  const int r = decode_layers(ctx, h_dev, hpost_dev, B, tau, mode, y_dev, stream, &launched);
+  if (r != APEX_OK) complete_pending(ctx, launched);
+  return r;
 }
 
 int apex_decode_token_host(apex_ctx* ctx, const float* h_host, const float* hpost_host, int B, float tau, int mode,

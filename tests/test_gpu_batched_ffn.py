@@ -4,7 +4,7 @@ import pytest
 import torch
 
 from oracle import apex_oracle as ao
-from paper_2608_11688_b200 import synth
+from paper_2608_11688_b200 import binding, synth
 
 pytestmark = pytest.mark.gpu
 
@@ -88,3 +88,37 @@ def test_grouped_gemm_tiles(fmt, N, k, I, I_shared, B):
         assert rel <= 7.6e-6
     finally:
         ctx.destroy()
+
+
+def _decode_inputs(cfg, B):
+    hs = [synth.hidden_states(cfg, l, 1, B) for l in range(cfg.L)]
+    return tuple(torch.from_numpy(np.stack([x[i][0] for x in hs])).cuda() for i in (0, 1))
+
+
+@pytest.mark.parametrize("C", [6, 4])
+def test_decode_goes_on_after_candidate_records_that_never_arrived(C):
+    # C = N: the expert FFN of a layer is launched before its candidate records are waited for; C < N: after
+    import harness
+    B = 3
+    cfg = synth.tiny_config(d=256, N=6, k=2, I=128, C=C, L=2, T=1, cfg_id=323)
+    prob = harness.Problem(cfg)
+    h, hp = _decode_inputs(cfg, B)
+    out = []
+    for what in (0, 3):
+        ctx = prob.make_ctx(max_batch=B, wait_limit_ns=50_000_000)
+        try:
+            if C == cfg.N:
+                ctx.warm_all()
+            y = torch.zeros((cfg.L, B, cfg.d), device="cuda")
+            if what:
+                ctx.test_inject(what)
+                with pytest.raises(binding.ApexError) as ei:
+                    ctx.decode_token(h, hp, B, 0.9, "exact", y)
+                assert ei.value.code == binding.APEX_ETIMEOUT and "candidate" in str(ei.value)
+                torch.cuda.synchronize()
+            ctx.decode_token(h, hp, B, 0.9, "exact", y)
+            torch.cuda.synchronize()
+            out.append(y.cpu().numpy())
+        finally:
+            ctx.destroy()
+    np.testing.assert_allclose(out[1], out[0], rtol=0, atol=2e-6 * float(np.abs(out[0]).max()))  # (fp32 additions into y in another order)
