@@ -314,23 +314,37 @@ int apex_prefetch(apex_ctx* ctx, int layer, int B, void* copy_stream) {
   return APEX_OK;
 }
 
-int apex_attention_standin(apex_ctx* ctx, int layer, void* stream) {
-  CHECK_CTX(ctx);
-  CHECK_LAYER(ctx, layer);
+}  // extern "C"
+
+namespace {
+
+// wait_first: what is queued before the kernel is complete when its first CTA streams (and so before a kernel launched
+// behind it begins: the batched prefetch stage counts on it and has no wait of its own); otherwise when its last one exits.
+int launch_standin(apex_ctx* ctx, int layer, bool wait_first, cudaStream_t cs) {
   AttnParams p{};
   p.buf = ctx->d_attn + (size_t)(layer % ctx->attn_layers) * ctx->attn_bytes;
   p.bytes = ctx->attn_bytes;
   p.status = const_cast<unsigned*>(&mhdr(ctx)->status);
+  p.wait_first = wait_first ? 1 : 0;
+  CU_TRY(ctx, launch_attention(p, ctx->n_sm, cs));
+  ctx->last_was_ffn = false;
+  ctx->last_pred_layer = -1;
+  ctx->last_stream = cs;
+  ++ctx->launches;
+  return APEX_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+int apex_attention_standin(apex_ctx* ctx, int layer, void* stream) {
+  CHECK_CTX(ctx);
+  CHECK_LAYER(ctx, layer);
   // The attention block of a layer reads the layer's input, not the prefetch router's output: when the kernel
   // just before it on this stream is this layer-step's prefetch stage, the two may run side by side (Sec. IV-A:
   // prediction and prefetch are hidden under attention).  Anything else in front of it is waited for first.
-  p.wait_first = (ctx->last_stream == (cudaStream_t)stream && ctx->last_pred_layer == layer) ? 0 : 1;
-  CU_TRY(ctx, launch_attention(p, ctx->n_sm, (cudaStream_t)stream));
-  ctx->last_was_ffn = false;
-  ctx->last_pred_layer = -1;
-  ctx->last_stream = (cudaStream_t)stream;
-  ++ctx->launches;
-  return APEX_OK;
+  return launch_standin(ctx, layer, ctx->last_stream != (cudaStream_t)stream || ctx->last_pred_layer != layer, (cudaStream_t)stream);
 }
 
 int apex_route_topk(apex_ctx* ctx, int layer, const float* hpost_dev, int B, int32_t* idx_dev, float* alpha_dev, void* stream) {
@@ -670,7 +684,7 @@ int decode_layers(apex_ctx* ctx, const float* h_dev, const float* hpost_dev, int
     // the stand-in started 3 to 6 us later, a launch behind the router.  (One token: its candidate record is waited for
     // by the host, so its router, which is small, goes first.)
     const bool standin_first = standin && B > 1;
-    if (standin_first && (r = apex_attention_standin(ctx, l, stream)) != APEX_OK) return r;
+    if (standin_first && (r = launch_standin(ctx, l, true, (cudaStream_t)stream)) != APEX_OK) return r;
     if (prefetching && (r = predict_select_fused(ctx, l, h_dev + l * step, B, tau, ctx->d_cand, ctx->d_cand_ncand, standin_first, (cudaStream_t)stream)) != APEX_OK)
       return r;
     if (standin && !standin_first && (r = apex_attention_standin(ctx, l, stream)) != APEX_OK) return r;

@@ -122,3 +122,29 @@ def test_decode_goes_on_after_candidate_records_that_never_arrived(C):
         finally:
             ctx.destroy()
     np.testing.assert_allclose(out[1], out[0], rtol=0, atol=2e-6 * float(np.abs(out[0]).max()))  # (fp32 additions into y in another order)
+
+
+def test_decode_right_behind_a_prediction_of_its_first_layer():
+    # the prefetch stage of a batched step has no dependency wait of its own (the stand-in in front of it has): a prediction
+    # still running on the same scratch must be complete before it
+    import harness
+    B, cfg = 64, synth.tiny_config(d=2048, N=64, k=4, I=128, C=64, L=1, T=2, cfg_id=324)
+    prob = harness.Problem(cfg)
+    ctx = prob.make_ctx(max_batch=B)
+    try:
+        ctx.warm_all()
+        h, hp = _decode_inputs(cfg, B)
+        other = torch.flip(h, dims=(1,)).contiguous()
+        y = torch.zeros((1, B, cfg.d), device="cuda")
+        ctx.decode_token(h, hp, B, 0.9, "exact", y)
+        torch.cuda.synchronize()
+        want, y_want = ctx.read_prediction(B), y.cpu().numpy()
+        for _ in range(20):
+            ctx.predict(0, other[0], B)
+            ctx.decode_token(h, hp, B, 0.9, "exact", y)
+            torch.cuda.synchronize()
+            for a, b in zip(ctx.read_prediction(B), want):
+                np.testing.assert_array_equal(a, b)
+            np.testing.assert_allclose(y.cpu().numpy(), y_want, rtol=0, atol=2e-6 * float(np.abs(y_want).max()))
+    finally:
+        ctx.destroy()
