@@ -269,7 +269,8 @@ int apex_set_slot_table(apex_ctx* ctx, int layer, const int32_t* expert_slot, co
 int apex_warm_all(apex_ctx* ctx);
 /* Host-side fault hooks for tests: what = 1 the next copy issue fails (APEX_ECUDA path);
  * what = 2 the next slot-ready flag is withheld (device wait runs out); what = 3 the candidate records of the next
- * launched budget selection are withheld (the host's wait in apex_prefetch runs out); 0 clears. */
+ * launched budget selection are withheld (the host's wait in apex_prefetch runs out); what = 4 the next
+ * launched router of a batch waits for bytes that nobody sends (its device-side wait runs out); 0 clears. */
 int apex_test_inject(apex_ctx* ctx, int what);
 /* Number of kernels this library has launched on the context so far. */
 int64_t apex_launch_count(const apex_ctx* ctx);
@@ -294,6 +295,8 @@ int64_t apex_launch_count(const apex_ctx* ctx);
  * calls on a device share the array and it keeps the previous call's logits; the kernel overwrites
  * what it uses, so nothing has to be cleared, but two calls that overlap on the GPU (different
  * streams) race on it: serialise them.  First calls from several host threads are serialised inside.
+ * At B > 1 the kernel waits for its own loads, at most 2 s; should that run out (a GPU held that long), the tokens
+ * concerned get idx = -1 and alpha = NaN.
  * err (optional, err_len bytes, caller-owned) receives a text on failure.  Returns APEX_OK,
  * APEX_EINVAL or APEX_ECUDA. */
 int apex_route_topk_static(const float* W_r_dev, const float* b_r_dev, const float* hpost_dev, int N, int d, int k,

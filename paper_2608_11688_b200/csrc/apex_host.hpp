@@ -111,6 +111,7 @@ int issue_copy(apex_ctx* ctx, int layer, int e, int slot, cudaStream_t cs);
 int release_withheld(apex_ctx* ctx);
 SlotSnapshot make_snapshot(apex_ctx* ctx, int layer);
 int check_device_status(apex_ctx* ctx);
+int record_missing(apex_ctx* ctx, const char* what);
 
 // Persistent decode path (apex_decode.cu)
 int decode_setup(apex_ctx* ctx);

@@ -101,6 +101,9 @@ struct RouterParams {
   uint32_t seq_value;
   int C;
   int wait_last;      // 1: x does not come from the preceding kernel (the attention stand-in): wait for it before exiting only
+  volatile unsigned* status;  // mapped: 1 when a wait of the batched kernel ran out, or null
+  long long wait_limit_ns;    // bound of that wait
+  int starve;        // test hook: the batched kernel's first CTA waits for bytes that nobody sends
   int fuse_select;   // 1: the leader warp also runs the budget selection (sel) for its token
   SelectParams sel;
 };
@@ -412,7 +415,7 @@ struct apex_ctx {
   unsigned long long dec_epoch = 0;           // persistent launches since the counters were last cleared
   uint32_t dec_seq = 0;
   bool dec_dirty = false;                     // a launch gave up: counters and abort flag must be cleared before the next
-  int inject = 0;
+  int inject = 0;  // armed test hook (apex_test_inject)
   bool host_waves = false;  // B = 1 exact mode: misses are corrected by further launches, not by a wait inside the kernel
   int64_t launches = 0;
   void* fn_write_value32 = nullptr;  // cuStreamWriteValue32 when the driver offers it

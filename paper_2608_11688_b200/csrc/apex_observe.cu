@@ -116,7 +116,7 @@ int apex_warm_all(apex_ctx* ctx) {
 
 int apex_test_inject(apex_ctx* ctx, int what) {
   CHECK_CTX(ctx);
-  if (what < 0 || what > 3) return fail(ctx, APEX_EINVAL, "unknown injection");
+  if (what < 0 || what > 4) return fail(ctx, APEX_EINVAL, "unknown injection");
   ctx->inject = what;
   return APEX_OK;
 }

@@ -118,15 +118,31 @@ int check_device_status(apex_ctx* ctx) {
     // after the launch returns): from now on misses are corrected by further launches instead.
     ctx->host_waves = true;
     ctx->dec_dirty = true;  // a persistent decode launch that gave up leaves its counters short
-    return fail(ctx, APEX_ETIMEOUT, "a device-side wait on a slot-ready flag or a demand copy ran out");
+    return fail(ctx, APEX_ETIMEOUT, "a device-side wait (for a slot-ready flag, a demand copy or a kernel's own loads) ran out");
   }
   return APEX_OK;
+}
+
+// A record the host waited for did not come.  Where the device has reported why, that is taken note of here: left standing,
+// it would end the next step's waits as well.
+int record_missing(apex_ctx* ctx, const char* what) {
+  check_device_status(ctx);
+  return fail(ctx, APEX_ETIMEOUT, what);
 }
 
 }  // namespace apex
 
 namespace {
 
+// the batched router's bounded wait: its limit, where it reports, and the test hook
+void router_wait(apex_ctx* ctx, RouterParams* p) {
+  p->status = &mhdr(ctx)->status;
+  p->wait_limit_ns = ctx->cfg.wait_limit_ns;
+  if (ctx->inject == 4 && p->B > 1) {
+    ctx->inject = 0;
+    p->starve = 1;
+  }
+}
 
 int begin_predict(apex_ctx* ctx, int layer, const float* h_dev, int B, RouterParams* p) {
   if (!h_dev || B < 1 || B > ctx->cfg.max_batch) return fail(ctx, APEX_EINVAL, "apex_predict: bad h or B");
@@ -145,6 +161,7 @@ int begin_predict(apex_ctx* ctx, int layer, const float* h_dev, int B, RouterPar
   p->pi_out = ctx->d_pi;
   p->topk_out = B == 1 ? ctx->d_spec + (size_t)layer * APEX_MAX_TOPK : nullptr;  // the FFN's speculative first fill
   p->N = (int)N; p->d = (int)d; p->B = B; p->k = ctx->cfg.k; p->C = ctx->cfg.C;
+  router_wait(ctx, p);
   return APEX_OK;
 }
 
@@ -250,7 +267,7 @@ int apex_prefetch(apex_ctx* ctx, int layer, int B, void* copy_stream) {
   if (B == 1) {
     // one 16-byte record {mask lo, mask hi, ncand, seq}; the ranked list beside it is advisory
     volatile uint32_t* rec = mbox_sel_rec(ctx);
-    if (!host_wait_seq(ctx, rec + 3, ctx->sel_seq)) return fail(ctx, APEX_ETIMEOUT, "apex_prefetch: candidate set did not arrive");
+    if (!host_wait_seq(ctx, rec + 3, ctx->sel_seq)) return record_missing(ctx, "apex_prefetch: candidate set did not arrive");
     const uint64_t mask = ((uint64_t)rec[1] << 32) | rec[0];
     const int n = (int)rec[2];
     int32_t list[APEX_MAX_EXPERTS];
@@ -278,7 +295,7 @@ int apex_prefetch(apex_ctx* ctx, int layer, int B, void* copy_stream) {
     uint64_t plane[9] = {};  // counts up to APEX_MAX_BATCH
     volatile uint32_t* rec = mbox_sel_rec(ctx);
     for (int b = 0; b < B; ++b) {
-      if (!host_wait_seq(ctx, rec + 4 * b + 3, ctx->sel_seq)) return fail(ctx, APEX_ETIMEOUT, "apex_prefetch: a candidate set did not arrive");
+      if (!host_wait_seq(ctx, rec + 4 * b + 3, ctx->sel_seq)) return record_missing(ctx, "apex_prefetch: a candidate set did not arrive");
       uint64_t carry = ((uint64_t)rec[4 * b + 1] << 32) | rec[4 * b];
       for (int j = 0; carry; ++j) {
         const uint64_t c = plane[j] & carry;
@@ -374,6 +391,7 @@ int apex_route_topk(apex_ctx* ctx, int layer, const float* hpost_dev, int B, int
   p.pi_pred = st.selected ? ctx->d_pi : nullptr;
   p.ncand_pred = st.selected ? ctx->d_ncand : nullptr;
   p.stats = ctx->d_stats + layer;
+  router_wait(ctx, &p);
   if (B == 1) {  // K_r goes to the host from here: the expert FFN's host half finds it when it is called
     p.mbox_rec = const_cast<uint32_t*>(mbox_exec_rec(ctx, layer));
     p.seq_value = st.route_seq = ++ctx->exec_seq[layer];
@@ -541,7 +559,7 @@ int ffn_finalize(apex_ctx* ctx, int layer) {
   volatile uint32_t* rec = mbox_exec_rec(ctx, layer);
   if (!host_wait_seq(ctx, rec + 2, B == 1 ? st.route_seq : ctx->exec_seq[layer]) ||
       (st.pend_mode != APEX_MODE_EXACT && !host_wait_seq(ctx, rec + 6, ctx->exec_seq[layer])))
-    return fail(ctx, APEX_ETIMEOUT, "apex_moe_ffn: K_r did not arrive");
+    return record_missing(ctx, "apex_moe_ffn: K_r did not arrive");
   const uint64_t need = ((uint64_t)rec[1] << 32) | rec[0], ex_mask = ((uint64_t)rec[5] << 32) | rec[4];
   if (st.pend_mode == APEX_MODE_EXACT) {
     std::vector<SlotCopy> copies;

@@ -125,6 +125,21 @@ constexpr int kRouterWarps = 8;
 __host__ __device__ constexpr int router_tile_tok(int tt) { return tt < 4 ? tt : 4; }
 __host__ __device__ constexpr int router_tile_exp(int tt) { return tt <= 4 ? 1 : tt / 4; }
 
+// What a token gets whose logits could not be computed: nothing that looks like a routing.  No record goes to the host, which
+// stops waiting for it when it sees the status.
+__device__ __forceinline__ void router_failed(const RouterParams& p, int b, int lane) {
+  for (int e = lane; e < p.N; e += 32) {
+    p.z_out[(size_t)b * p.N + e] = p.q_out[(size_t)b * p.N + e] = __int_as_float(0x7fffffff);
+    if (p.pi_out) p.pi_out[(size_t)b * p.N + e] = e;  // (the gate indexes with it)
+  }
+  if (p.topk_out)
+    for (int j = lane; j < p.k; j += 32) p.topk_out[(size_t)b * p.k + j] = -1;
+  if (p.fuse_select) {
+    for (int j = lane; j < p.C; j += 32) p.sel.cand_out[(size_t)b * p.C + j] = -1;
+    if (lane == 0) p.sel.ncand_out[b] = p.sel.ncand_keep[b] = 0;
+  }
+}
+
 template <int TT>
 __global__ void __launch_bounds__(kRouterWarps * 32, 2) router_batched_kernel(const RouterParams p) {
   SPAN_BEGIN();
@@ -138,11 +153,13 @@ __global__ void __launch_bounds__(kRouterWarps * 32, 2) router_batched_kernel(co
   __shared__ int pis[kRouterWarps][APEX_MAX_EXPERTS];
   __shared__ int posp[kRouterWarps][APEX_MAX_EXPERTS];
   __shared__ uint64_t s_bar[2];
+  __shared__ int s_bad;                         // a wait of a CTA of the cluster ran out
   extern __shared__ __align__(128) float tiles[];  // [2][TT + 8][CH]: x rows, W rows
   const int b0 = blockIdx.y * TT, nt = min(TT, p.B - b0);
   const int e0 = (int)crank * p.warps_per_cta, ne = max(0, min(p.warps_per_cta, p.N - e0));
   const int n_chunks = (p.d + CH - 1) / CH;
   if (threadIdx.x == 0) {
+    s_bad = 0;
     mbar_init(&s_bar[0], 2);
     mbar_init(&s_bar[1], 2);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -150,7 +167,7 @@ __global__ void __launch_bounds__(kRouterWarps * 32, 2) router_batched_kernel(co
   __syncthreads();
   auto chunk_bytes = [&](int c) { return (uint32_t)(min(CH, p.d - c * CH) * 4); };
   auto load_w = [&](int c) {  // warp 0
-    if (lane == 0) mbar_expect_tx(&s_bar[c & 1], ne * chunk_bytes(c));
+    if (lane == 0) mbar_expect_tx(&s_bar[c & 1], ne * chunk_bytes(c) + (p.starve && c == 0 && blockIdx.x == 0 && blockIdx.y == 0 ? 16u : 0u));
     __syncwarp();
     if (lane < ne) bulk_g2s(tiles + ((c & 1) * (TT + 8) + TT + lane) * CH, p.W + (size_t)(e0 + lane) * p.d + c * CH, chunk_bytes(c), &s_bar[c & 1]);
   };
@@ -178,8 +195,15 @@ __global__ void __launch_bounds__(kRouterWarps * 32, 2) router_batched_kernel(co
   float acc[NT * NX];
 #pragma unroll
   for (int v = 0; v < NT * NX; ++v) acc[v] = 0.f;
+  // A wait that runs out (the GPU held for the length of the limit, say) does not end the loop, which has barriers: nothing more is
+  // waited for or loaded, and the cluster's tokens are marked below
+  bool dead = false;
+  int loaded = min(2, n_chunks);  // chunks asked for (warp 0)
   for (int c = 0; c < n_chunks; ++c) {
-    mbar_wait(&s_bar[c & 1], (c >> 1) & 1, nullptr, 2000000000ll);
+    if (!dead && !mbar_wait(&s_bar[c & 1], (c >> 1) & 1, &s_bad, p.wait_limit_ns)) {
+      dead = true;
+      *(volatile int*)&s_bad = 1;
+    }
     if (active) {
       const int nv = min(CH, p.d - c * CH) >> 2;
       const float4* xt = reinterpret_cast<const float4*>(tiles + ((c & 1) * (TT + 8) + t0) * CH) + lane;
@@ -209,10 +233,11 @@ __global__ void __launch_bounds__(kRouterWarps * 32, 2) router_batched_kernel(co
     }
     if (c + 2 < n_chunks) {
       __syncthreads();  // everybody has read this buffer
-      if (warp == 0) {
+      if (warp == 0 && !__any_sync(0xffffffffu, dead)) {
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         load_w(c + 2);
         load_x(c + 2);
+        loaded = c + 3;
       }
     }
   }
@@ -250,8 +275,20 @@ __global__ void __launch_bounds__(kRouterWarps * 32, 2) router_batched_kernel(co
     }
   }
   RTL(3);
+  if (__any_sync(0xffffffffu, dead)) {
+    if (lane < (int)csize) *cluster.map_shared_rank(&s_bad, lane) = 1;
+    if (warp == 0) {  // what is still on its way into this CTA's shared memory (bounded)
+      for (int c = max(0, loaded - 2); c < loaded; ++c) mbar_wait(&s_bar[c & 1], (c >> 1) & 1, nullptr, p.wait_limit_ns);
+      if (lane == 0 && p.status) *p.status = 1u;
+    }
+  }
   cluster.sync();
   RTL(4);
+  if (s_bad) {
+    for (int t = te; t < nt; t += kRouterWarps * (int)csize) router_failed(p, b0 + t, lane);
+    if (p.wait_last) pdl_wait();
+    return;
+  }
   if (te < nt) router_epilogue(p, ev, b0 + te, lane, zs[warp], qs[warp], pis[warp], posp[warp]);
   for (int t = te + kRouterWarps * (int)csize; t < nt; t += kRouterWarps * (int)csize) {  // (a cluster of one CTA: more tokens than warps)
     __syncwarp();
@@ -291,6 +328,7 @@ cudaError_t launch_router(const RouterParams& p, cudaStream_t s) {
   while (csize < 8 && csize * 8 < p.N) csize <<= 1;
   RouterParams q = p;
   q.warps_per_cta = (p.N + csize - 1) / csize;
+  if (q.wait_limit_ns <= 0) q.wait_limit_ns = 2000000000ll;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(csize, p.B, 1);
   cfg.blockDim = dim3(256, 1, 1);

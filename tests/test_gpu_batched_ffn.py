@@ -148,3 +148,43 @@ def test_decode_right_behind_a_prediction_of_its_first_layer():
             np.testing.assert_allclose(y.cpu().numpy(), y_want, rtol=0, atol=2e-6 * float(np.abs(y_want).max()))
     finally:
         ctx.destroy()
+
+
+@pytest.mark.parametrize("stage", ["prefetch", "gate"])
+def test_batched_router_reports_a_wait_that_ran_out(stage):
+    # one CTA of a batched router waits for bytes that nobody sends: its limit ends the wait, its cluster's tokens carry
+    # no routing, the call (or the next one) reports it, and the context goes on
+    import harness
+    B, cfg = 40, synth.tiny_config(d=2048, N=24, k=3, I=128, C=24, L=1, T=1, cfg_id=325)
+    prob = harness.Problem(cfg)
+    ctx = prob.make_ctx(max_batch=B, wait_limit_ns=50_000_000)
+    try:
+        ctx.warm_all()
+        h, hp = _decode_inputs(cfg, B)
+        y = torch.zeros((1, B, cfg.d), device="cuda")
+        ctx.decode_token(h, hp, B, 0.9, "exact", y)
+        torch.cuda.synchronize()
+        want = y.cpu().numpy()
+        if stage == "prefetch":
+            ctx.test_inject(4)
+            with pytest.raises(binding.ApexError) as ei:
+                ctx.decode_token(h, hp, B, 0.9, "exact", y)
+            assert ei.value.code == binding.APEX_ETIMEOUT
+        else:
+            idx = torch.full((B, cfg.k), 7, dtype=torch.int32, device="cuda")
+            alpha = torch.zeros((B, cfg.N), device="cuda")
+            ctx.test_inject(4)
+            ctx.route_topk(0, hp[0], B, idx, alpha)
+            torch.cuda.synchronize()
+            bad = (idx == -1).all(1)
+            assert bad.any() and not bad.all() and ((idx >= 0).all(1) == ~bad).all()
+            assert (torch.isnan(alpha).all(1) == bad).all() and torch.isfinite(alpha[~bad]).all()
+            with pytest.raises(binding.ApexError) as ei:
+                ctx.moe_ffn(0, "exact", hp[0], B, y[0])
+            assert ei.value.code == binding.APEX_ETIMEOUT
+        torch.cuda.synchronize()
+        ctx.decode_token(h, hp, B, 0.9, "exact", y)
+        torch.cuda.synchronize()
+        np.testing.assert_allclose(y.cpu().numpy(), want, rtol=0, atol=2e-6 * float(np.abs(want).max()))
+    finally:
+        ctx.destroy()
