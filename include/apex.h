@@ -272,6 +272,9 @@ int apex_warm_all(apex_ctx* ctx);
  * launched budget selection are withheld (the host's wait in apex_prefetch runs out); what = 4 the next
  * launched router of a batch waits for bytes that nobody sends (its device-side wait runs out); 0 clears. */
 int apex_test_inject(apex_ctx* ctx, int what);
+/* The same for apex_distill_router, which has no context: in the next call on this thread one CTA waits for an arrival that
+ * never comes (its device-side wait of 2 s runs out; APEX_ECUDA, W_host and b_host untouched). */
+int apex_test_starve_distill(void);
 /* Number of kernels this library has launched on the context so far. */
 int64_t apex_launch_count(const apex_ctx* ctx);
 

@@ -86,6 +86,7 @@ SIGNATURES = {
     "apex_set_slot_table": (_I, [_P, _I, _P, _P, C.c_int64]),
     "apex_warm_all": (_I, [_P]),
     "apex_test_inject": (_I, [_P, _I]),
+    "apex_test_starve_distill": (_I, []),
     "apex_launch_count": (C.c_int64, [_P]),
     "apex_route_topk_static": (_I, [_P, _P, _P, _I, _I, _I, _I, _P, _P, _P, C.c_char_p, C.c_size_t]),
     "apex_fit_cdf": (_I, [_P, _P, _I, _I, _I, _I, C.c_double, _P, _P, _P, C.c_char_p, C.c_size_t]),

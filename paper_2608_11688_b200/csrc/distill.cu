@@ -61,6 +61,8 @@ struct DistillParams {
   int T, N, d, ldw;
   int tok_warps;     // forward: tokens per CTA / 8: 1, 2, 4, 7 or 8
   int n_fwd, n_tiles, n_seg, seg_len;
+  int* status;       // 1: a wait of a ring ran out
+  int starve;        // test hook: the first forward CTA's ring expects an arrival that never comes
   double lr, c1, c2;  // step size; bias corrections 1 - 0.9^it, 1 - 0.999^it
 };
 
@@ -116,17 +118,29 @@ constexpr size_t bwd_smem_bytes(int ne) {
 
 struct Ring {
   uint64_t full[kStages], empty[kStages];
+  int dead;  // a wait ran out: everybody stops waiting, loading and multiplying; the host does not use the result
 };
-__device__ __forceinline__ void ring_init(Ring* r, int mma_warps) {
+__device__ __forceinline__ void ring_init(Ring* r, int mma_warps, int extra = 0) {
   if (threadIdx.x == 0) {
+    r->dead = 0;
     for (int s = 0; s < kStages; ++s) {
-      apex::mbar_init(&r->full[s], kProducers);
+      apex::mbar_init(&r->full[s], kProducers + extra);
       apex::mbar_init(&r->empty[s], mma_warps);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
 }
+
+// a whole warp (uniform result)
+__device__ __forceinline__ bool ring_wait(Ring* r, uint64_t* bar, uint32_t parity, int* status) {
+  if (__all_sync(0xffffffffu, apex::mbar_wait(bar, parity, &r->dead, kWaitLimitNs))) return true;
+  *(volatile int*)&r->dead = 1;
+  *(volatile int*)status = 1;
+  return false;
+}
+// the ring is reused behind the loops: a producer's copies must have landed, also where nobody waited for them any more
+__device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 template <int NE, bool VEC>
 __global__ void __launch_bounds__(kFwdThreads, 1) distill_fwd_kernel(const DistillParams p) {
@@ -137,7 +151,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) distill_fwd_kernel(const Disti
   const int t0 = blockIdx.x * toks;
   const int n_kt = (p.d + kKd - 1) / kKd;
   const size_t stage = fwd_stage_bytes(NE, toks);
-  ring_init(&ring, TW * KS);
+  ring_init(&ring, TW * KS, p.starve && blockIdx.x == 0 ? 1 : 0);
   const int mw = (tid - kProducers) >> 5;                // MMA warp
   const int tw = mw % TW, kslice = mw / TW;              // its eight tokens and its share of a stage's K steps
   const int fr = lane >> 2, fc = lane & 3;
@@ -147,7 +161,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) distill_fwd_kernel(const Disti
   if (tid < kProducers) {
     for (int kt = 0; kt < n_kt; ++kt) {
       const int s = kt % kStages;
-      if (kt >= kStages) apex::mbar_wait(&ring.empty[s], (kt / kStages - 1) & 1, nullptr, kWaitLimitNs);
+      if (kt >= kStages && !ring_wait(&ring, &ring.empty[s], (kt / kStages - 1) & 1, p.status)) break;
       float* th = reinterpret_cast<float*>(smem + s * stage);
       double* tw_ = reinterpret_cast<double*>(smem + s * stage + (size_t)toks * kLdH * 4);
       load_h<VEC>(th, kLdH, p, t0, toks, p.T, kt * kKd);
@@ -161,10 +175,11 @@ __global__ void __launch_bounds__(kFwdThreads, 1) distill_fwd_kernel(const Disti
         cp16(tw_ + r * kLdW + lane * 2, src, true);
       cp_arrive(&ring.full[s]);
     }
+    cp_wait_all();
   } else if (kslice < KS) {
     for (int kt = 0; kt < n_kt; ++kt) {
       const int s = kt % kStages;
-      apex::mbar_wait(&ring.full[s], (kt / kStages) & 1, nullptr, kWaitLimitNs);
+      if (!ring_wait(&ring, &ring.full[s], (kt / kStages) & 1, p.status)) break;
       const float* hp = reinterpret_cast<const float*>(smem + s * stage) + (tw * 8 + fr) * kLdH + fc;
       const double* wp = reinterpret_cast<const double*>(smem + s * stage + (size_t)toks * kLdH * 4) + fr * kLdW + fc;
 #pragma unroll 4
@@ -274,7 +289,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) distill_bwd_kernel(const Disti
   if (tid < kProducers) {
     for (int kt = 0; kt < n_kt; ++kt) {
       const int s = kt % kStages, t0 = t_lo + kt * kTokTile;
-      if (kt >= kStages) apex::mbar_wait(&ring.empty[s], (kt / kStages - 1) & 1, nullptr, kWaitLimitNs);
+      if (kt >= kStages && !ring_wait(&ring, &ring.empty[s], (kt / kStages - 1) & 1, p.status)) break;
       double* tg = reinterpret_cast<double*>(smem + s * stage);
       load_h<VEC>(reinterpret_cast<float*>(smem + s * stage + (size_t)kTokTile * LDG * 8), kLdHb, p, t0, kTokTile, t_hi, col0);
       if (kt == 0) {
@@ -290,10 +305,11 @@ __global__ void __launch_bounds__(kBwdThreads, 1) distill_bwd_kernel(const Disti
       }
       cp_arrive(&ring.full[s]);
     }
+    cp_wait_all();
   } else {
     for (int kt = 0; kt < n_kt; ++kt) {
       const int s = kt % kStages;
-      apex::mbar_wait(&ring.full[s], (kt / kStages) & 1, nullptr, kWaitLimitNs);
+      if (!ring_wait(&ring, &ring.full[s], (kt / kStages) & 1, p.status)) break;
       const double* gp = reinterpret_cast<const double*>(smem + s * stage) + fc * LDG + fr;                                  // A: experts x tokens
       const float* hp = reinterpret_cast<const float*>(smem + s * stage + (size_t)kTokTile * LDG * 8) + fc * kLdHb + cg * 16 + fr;  // B: tokens x columns
 #pragma unroll
@@ -407,6 +423,7 @@ cudaError_t run_iterations(DistillParams p, int iters, cudaStream_t cs) {
     cfg.blockDim = dim3(kStepThreads, 1, 1);
     cfg.dynamicSmemBytes = 0;
     if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, distill_step_kernel, p, 8 * NE);
+    p.starve = 0;
   }
   return e;
 }
@@ -425,11 +442,18 @@ cudaError_t run_iterations(const DistillParams& p, int ne, int iters, cudaStream
   }
 }
 
+thread_local bool starve_next = false;  // armed test hook
+
 void say(char* err, size_t err_len, const char* msg) {
   if (err && err_len) snprintf(err, err_len, "%s", msg);
 }
 
 }  // namespace
+
+extern "C" int apex_test_starve_distill(void) {
+  starve_next = true;
+  return APEX_OK;
+}
 
 extern "C" int apex_distill_router(const float* H_dev, const float* Qr_dev, int T, int N, int d, int iters, double lr,
                                    float* W_host, float* b_host, void* stream, char* err, size_t err_len) {
@@ -445,6 +469,8 @@ extern "C" int apex_distill_router(const float* H_dev, const float* Qr_dev, int 
   const int ne = (N + 7) / 8, rows = 8 * ne;
   DistillParams p{};
   p.H = H_dev; p.Qr = Qr_dev; p.T = T; p.N = N; p.d = d; p.lr = lr;
+  p.starve = starve_next ? 1 : 0;
+  starve_next = false;
   p.ldw = (d + kKd - 1) / kKd * kKd;
   // Forward: as few token tiles as fill the SMs once, 8 W tokens per CTA.  W = 7 (28 MMA warps, seven per scheduler)
   // turns T = 8192 into 147 tiles; W = 8 would leave 20 of 148 SMs idle there.
@@ -460,7 +486,7 @@ extern "C" int apex_distill_router(const float* H_dev, const float* Qr_dev, int 
   p.seg_len = (T + p.n_seg - 1) / p.n_seg;
   const size_t n_w = (size_t)rows * p.ldw, n_io = (size_t)N * d + N;
   // zeroed: parameters and moments; not zeroed: G, partial sums, the fp32 parameters
-  const size_t zeroed = 3 * (n_w + rows) * sizeof(double);
+  const size_t zeroed = (3 * (n_w + rows) + 2) * sizeof(double);  // (and the status word; G behind it is 16-byte aligned)
   const size_t n_rest = (size_t)T * rows + (size_t)p.n_fwd * rows + (size_t)p.n_tiles * p.n_seg * rows * kCols;
   uint8_t* buf = nullptr;
   cudaError_t e = cudaMalloc(&buf, zeroed + n_rest * sizeof(double) + n_io * sizeof(float));
@@ -470,6 +496,7 @@ extern "C" int apex_distill_router(const float* H_dev, const float* Qr_dev, int 
   }
   p.W = reinterpret_cast<double*>(buf); p.b = p.W + n_w;
   p.m = p.b + rows; p.v = p.m + n_w + rows;
+  p.status = reinterpret_cast<int*>(p.v + n_w + rows);
   p.G = reinterpret_cast<double*>(buf + zeroed);
   p.gb = p.G + (size_t)T * rows;
   p.partial = p.gb + (size_t)p.n_fwd * rows;
@@ -490,15 +517,21 @@ extern "C" int apex_distill_router(const float* H_dev, const float* Qr_dev, int 
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(host.data(), io, n_io * sizeof(float), cudaMemcpyDeviceToHost, cs);
+  int status = 0;
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&status, p.status, sizeof(int), cudaMemcpyDeviceToHost, cs);
   const cudaError_t e2 = cudaStreamSynchronize(cs);  // also after an error: nothing may still use the buffer
   if (e == cudaSuccess) e = e2;
-  if (e == cudaSuccess) {
+  if (e == cudaSuccess && status == 0) {
     for (size_t i = 0; i < (size_t)N * d; ++i) W_host[i] = host[i];
     for (int i = 0; i < N; ++i) b_host[i] = host[(size_t)N * d + i];
   }
   cudaFree(buf);
   if (e != cudaSuccess) {
     say(err, err_len, cudaGetErrorString(e));
+    return APEX_ECUDA;
+  }
+  if (status != 0) {
+    say(err, err_len, "apex_distill_router: a device-side wait ran out");
     return APEX_ECUDA;
   }
   return APEX_OK;

@@ -77,3 +77,19 @@ def test_distillation_rejects_bad_arguments():
     Q = torch.zeros((8, 70), dtype=torch.float32, device="cuda")
     with pytest.raises(binding.ApexError):
         binding.distill_router(H, Q, np.zeros((70, 16), np.float32), np.zeros(70, np.float32))      # N > 64
+
+
+def test_distillation_reports_a_wait_that_ran_out():
+    build.build()
+    rng = np.random.default_rng(7)
+    H = torch.from_numpy(rng.standard_normal((300, 128)).astype(np.float32)).cuda()
+    Qr = torch.softmax(torch.from_numpy(rng.standard_normal((300, 9)).astype(np.float32)), 1).cuda()
+    W0, b0 = rng.standard_normal((9, 128)).astype(np.float32), np.zeros(9, np.float32)
+    want = binding.distill_router(H, Qr, W0, b0, iters=3)
+    binding.load_library().apex_test_starve_distill()
+    with pytest.raises(binding.ApexError) as ei:
+        binding.distill_router(H, Qr, W0, b0, iters=3)
+    assert ei.value.code == binding.APEX_ECUDA and "wait" in str(ei.value)
+    got = binding.distill_router(H, Qr, W0, b0, iters=3)          # and the next call is not affected
+    for a, b in zip(got, want):
+        np.testing.assert_array_equal(a, b)
