@@ -362,6 +362,7 @@ ffn_tc_kernel(const __grid_constant__ TcWeightMaps tm_w, const __grid_constant__
       if (sl >= 0) r1 = (int32_t)(ld_acquire_sys(p.f.slot_ready + sl) - p.f.snap.need_gen[e1]) >= 0;
     }
     ready_mask = ((unsigned long long)__ballot_sync(0xffffffffu, r1) << 32) | __ballot_sync(0xffffffffu, r0);
+    __syncwarp();  // (every lane's acquires, before the loads of whichever lane)
     asm volatile("fence.proxy.async;" ::: "memory");  // the tensor-map loads below read what the flags cover
   }
   tc_fence_before();
@@ -680,6 +681,7 @@ ffn_tc_kernel(const __grid_constant__ TcWeightMaps tm_w, const __grid_constant__
             if (p.f.stats) atomicAdd(&p.f.stats->stall_ns, globaltimer_ns() - t0);
           }
           ready_mask |= 1ull << ud.expert;
+          __syncwarp();  // lane 0's acquire, before the loads of whichever lane
           asm volatile("fence.proxy.async;" ::: "memory");
         }
         ok = __all_sync(0xffffffffu, ok);
@@ -763,10 +765,13 @@ ffn_tc_kernel(const __grid_constant__ TcWeightMaps tm_w, const __grid_constant__
         if (lane == 0) {
           const unsigned want = ud.phase == 1 ? (unsigned)B : (unsigned)(p.geo[ud.expert >= N ? 1 : 0].blocks1 * ((s_grp[ud.group].n_tok + (1 << p.shift1) - 1) >> p.shift1));
           if (!wait_count(p.sync + (ud.phase == 1 ? kTcRows : kTcDone + ud.group), want)) ok = false;
-          asm volatile("fence.proxy.async;" ::: "memory");  // the bulk loads below read what other CTAs' threads have stored
         }
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
+        // The bulk loads below read what other CTAs' threads have stored, and any lane may issue one: lane 0's acquire reaches
+        // the others through the warp barrier (a vote or shuffle orders no memory), and each lane's fence its own loads
+        __syncwarp();
+        asm volatile("fence.proxy.async;" ::: "memory");
       }
       // The shared expert runs all tokens in order: plain boxes (32 gathers per stage were its pace, 1.3 us at 128 tokens)
       const int tiles = __shfl_sync(0xffffffffu, small ? WIDE : 1, 0);   // K tiles of a stage
@@ -1054,6 +1059,7 @@ ffn_tc_kernel(const __grid_constant__ TcWeightMaps tm_w, const __grid_constant__
           if (lane == 0) give_up();
           break;
         }
+        __syncwarp();  // lane 0's acquire, before every lane's additions into y
         rows_seen = true;
       }
       const bool shared = ud.expert >= N;

@@ -188,3 +188,28 @@ def test_batched_router_reports_a_wait_that_ran_out(stage):
         np.testing.assert_allclose(y.cpu().numpy(), want, rtol=0, atol=2e-6 * float(np.abs(want).max()))
     finally:
         ctx.destroy()
+
+
+@pytest.mark.parametrize("fmt", ["bf16", "fp4"])
+def test_grouped_gemm_reads_this_steps_activations_every_time(fmt):
+    # the rounded hidden states and the intermediate are written by some CTAs and read by the bulk loads of others; two
+    # inputs in turn, so that a load that came too early would read the other one's
+    import harness
+    B, cfg = 160, synth.tiny_config(d=1024, N=16, k=4, I=256, C=16, L=2, T=2, I_shared=384, cfg_id=326)
+    prob = harness.Problem(cfg, fp4=fmt == "fp4")
+    ctx = prob.make_ctx(max_batch=B)
+    try:
+        ctx.warm_all()
+        h, hp = _decode_inputs(cfg, B)
+        inputs = [(h, hp), (torch.flip(h, dims=(2,)).contiguous(), torch.flip(hp, dims=(2,)).contiguous())]
+        y = torch.zeros((cfg.L, B, cfg.d), device="cuda")
+        want = []
+        for n in range(60):
+            ctx.decode_token(*inputs[n % 2], B, 0.9, "exact", y)
+            torch.cuda.synchronize()
+            if n < 2:
+                want.append(y.clone())
+            else:
+                assert float((y - want[n % 2]).abs().max()) <= 2e-6 * float(want[n % 2].abs().max())
+    finally:
+        ctx.destroy()
