@@ -301,6 +301,7 @@ ffn_tc_kernel(const __grid_constant__ TcWeightMaps tm_w, const __grid_constant__
   __shared__ UnitDesc s_unit[kUnitRing];
   __shared__ uint32_t tmem_base_s;
   __shared__ int s_abort;
+  __shared__ uint2 s_end[3 + (QF ? kCvThreads / 32 : 0)];  // slot and parity at which each role that walks a ring has stopped: weights, activations, MMA, converters
   __shared__ int s_u[2][APEX_MAX_EXPERTS + 1], s_units[2];  // per projection: units before each group's in list order; all units
   __shared__ GroupDesc s_grp[APEX_MAX_EXPERTS + 1];         // executed experts, then the shared one
   constexpr int kTokWords = APEX_MAX_BATCH / 32;
@@ -743,6 +744,7 @@ ffn_tc_kernel(const __grid_constant__ TcWeightMaps tm_w, const __grid_constant__
       }
     }
     if (!ok && lane == 0) give_up();
+    if (lane == 0) s_end[0] = make_uint2(rp.s, rp.parity);
   } else if (warp == kBWarp) {
     // ================= activation loads: rows of X gathered by token index, or the group's rows of a_hi and a_lo
     RingPos rp;
@@ -829,6 +831,7 @@ ffn_tc_kernel(const __grid_constant__ TcWeightMaps tm_w, const __grid_constant__
       }
     }
     if (!ok && lane == 0) give_up();
+    if (lane == 0) s_end[1] = make_uint2(rp.s, rp.parity);
   } else if (warp == kMmaWarp) {
     // ================= MMA issuer: the whole warp walks the stages, one elected lane issues
     RingPos rp;
@@ -910,6 +913,7 @@ ffn_tc_kernel(const __grid_constant__ TcWeightMaps tm_w, const __grid_constant__
       if (lane == 0) TCTL(n, 2);
     }
     if (!ok && lane == 0) atomicExch(&s_abort, 1);
+    if (lane == 0) s_end[2] = make_uint2(rp.s, rp.parity);
   } else if (QF != 0 && warp >= kCvWarp0) {
     // ================= converters: the codes of a raw tile -> bf16 operand tiles of its SUB stages.  Gate and up go to
     // TMEM (lane = row, as the codes lie): a shared-memory tile is written once and read by its MMAs once at 128 bytes per
@@ -1042,6 +1046,7 @@ ffn_tc_kernel(const __grid_constant__ TcWeightMaps tm_w, const __grid_constant__
       }
     }
     if (!ok && lane == 0) atomicExch(&s_abort, 1);
+    if (lane == 0) s_end[3 + warp - kCvWarp0] = make_uint2(rp.s, rp.parity);
   } else {
     // ================= epilogue: warp w owns TMEM lanes 32*(w%4) .. +31
     const int quad = warp & 3;
@@ -1175,9 +1180,27 @@ ffn_tc_kernel(const __grid_constant__ TcWeightMaps tm_w, const __grid_constant__
   tc_fence_before();
   __syncthreads();
   if (*(volatile int*)&s_abort) {
-    // after an abort copies and MMAs may still be under way (everything they touch is this GPU's own memory: microseconds)
-    const unsigned long long t0 = globaltimer_ns();
-    while (globaltimer_ns() - t0 < 1000000ull) __nanosleep(1000);
+    // Copies into this CTA's shared memory and MMAs may still be under way: waited for (bounded), a ring slot per lane.  A role
+    // is never a round ahead of another on a slot, so where some have arrived in the barrier's current phase (the one whose
+    // parity has not completed) and others have not, the missing arrivals are made up for and the phase ends with its bytes.
+    if (warp == 0) {
+      auto last = [&](int role, uint32_t s) { return s < s_end[role].x ? s_end[role].y : s_end[role].y ^ 1u; };  // (1 before any: complete)
+      if (lane < NS) {
+        const uint32_t s = (uint32_t)lane, q = mbar_try_wait(&full[s], 0) ? 1u : 0u;
+        int in = 0, missing = 0;
+        auto arrived = [&](int role) { last(role, s) == q ? ++in : ++missing; };
+        arrived(1);
+        if (QF == 0) arrived(0);
+        for (int cw = 0; QF != 0 && cw < kCvThreads / 32; ++cw) arrived(3 + cw);
+        if (in > 0) {
+          for (; missing > 0; --missing) mbar_arrive(&full[s]);
+          mbar_wait(&full[s], q, nullptr, p.f.wait_limit_ns);
+        }
+        mbar_wait(&empty[s], last(2, s), nullptr, p.f.wait_limit_ns);
+      } else if (QF != 0 && lane >= 16 && lane < 16 + NR) {
+        mbar_wait(&rawfull[lane - 16], last(0, (uint32_t)lane - 16u), nullptr, p.f.wait_limit_ns);
+      }
+    }
     __syncthreads();
   }
   if (tid == 0) {  // the last CTA leaves the counters zero for the next launch (which waits for this one)

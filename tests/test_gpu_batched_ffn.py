@@ -213,3 +213,39 @@ def test_grouped_gemm_reads_this_steps_activations_every_time(fmt):
                 assert float((y - want[n % 2]).abs().max()) <= 2e-6 * float(want[n % 2].abs().max())
     finally:
         ctx.destroy()
+
+
+@pytest.mark.parametrize("fmt", ["bf16", "fp8", "fp4"])
+@pytest.mark.parametrize("I,I_shared", [(128, 0), (1024, 512)])
+def test_grouped_gemm_stops_with_copies_in_flight_and_the_context_goes_on(fmt, I, I_shared):
+    # one expert's slot-ready flag is withheld: the CTAs that wait for it run into the limit while others have weights,
+    # activations and MMAs under way.  Units of 32 rows (the first shape) and of 128
+    import harness
+    B, cfg = 24, synth.tiny_config(d=1024, N=4, k=2, I=I, C=4, L=1, T=1, I_shared=I_shared, cfg_id=327)
+    prob = harness.Problem(cfg, fp8=fmt == "fp8", fp4=fmt == "fp4")
+    h, hp = _decode_inputs(cfg, B)
+    y = torch.zeros((1, B, cfg.d), device="cuda")
+    ref = prob.make_ctx(max_batch=B)
+    try:
+        ref.warm_all()
+        ref.decode_token(h, hp, B, 0.9, "exact", y)
+        torch.cuda.synchronize()
+        want = y.cpu().numpy()
+    finally:
+        ref.destroy()
+    for _ in range(3):
+        ctx = prob.make_ctx(max_batch=B, wait_limit_ns=20_000_000)
+        try:
+            ctx.test_inject(2)
+            late = 0
+            for _ in range(3):
+                try:
+                    ctx.decode_token(h, hp, B, 1.0, "exact", y)
+                except binding.ApexError as e:
+                    assert e.code == binding.APEX_ETIMEOUT
+                    late += 1
+                torch.cuda.synchronize()
+            assert late > 0 and ctx.get_stats()["timeouts"] > 0
+            np.testing.assert_allclose(y.cpu().numpy(), want, rtol=0, atol=2e-6 * float(np.abs(want).max()))
+        finally:
+            ctx.destroy()
