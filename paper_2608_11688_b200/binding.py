@@ -1,7 +1,7 @@
 """ctypes binding of libapex.so: the same names as the C entry points, argument marshalling only.
 
-The calls of the decode step go through a small extension module (``_pycall``, csrc/pycall.c) that marshals in C; the
-others through ctypes.
+The calls of the decode step go through a small extension module (``_pycall``, csrc/pycall.c) that marshals in C, where it
+has been built (see ``build.build_pycall``); all others, and without it these too, through ctypes.
 
 Device buffers are torch CUDA tensors (``data_ptr()``), streams are ``torch.cuda.Stream`` objects
 (or None for the current stream).  There is no CPU fallback: loading fails loudly when the
@@ -14,14 +14,16 @@ import importlib.machinery
 import importlib.util
 import os
 import sys
+import sysconfig
 import threading
+import warnings
 from typing import Optional
 
 import numpy as np
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libapex.so")
-PYCALL_PATH = os.path.join(_HERE, "_pycall.so")
+PYCALL_PATH = os.path.join(_HERE, "_pycall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 
 APEX_OK, APEX_EINVAL, APEX_ENOMEM, APEX_ECUDA, APEX_ETIMEOUT, APEX_ESTATE, APEX_ENOTIMPL = 0, -1, -2, -3, -4, -5, -6
 MODE_EXACT, MODE_STALL_FREE = 0, 1
@@ -114,6 +116,8 @@ _pycall = None
 
 def _setup_pycall(with_stream=False):
     """Hands the extension module torch's types and getters (what there is of them yet: torch may be imported later)."""
+    if _pycall is None:
+        return
     torch = sys.modules.get("torch")
     tensor = getattr(torch, "Tensor", None)
     c = getattr(torch, "_C", None) if with_stream else None
@@ -123,16 +127,34 @@ def _setup_pycall(with_stream=False):
     _pycall.setup(_ptr, _stream, tensor, raw, dev)
 
 
+def _through_ctypes(address, name):
+    """What ``_pycall.make`` returns, without the extension module."""
+    res, types = SIGNATURES[name]
+    fn = C.CFUNCTYPE(res, *[C.c_void_p if t is C.c_char_p else t for t in types])(address)  # (text buffers come as addresses)
+    convert = [{"p": _ptr, "s": _stream}.get(c) for c in FAST[name]]
+
+    def call(*args):
+        if len(args) != len(convert):
+            raise TypeError(f"expected {len(convert)} arguments, got {len(args)}")
+        return fn(*[f(a) if f else a for f, a in zip(convert, args)])
+    return call
+
+
 def _load_pycall(lib):
     global _pycall
-    if not os.path.exists(PYCALL_PATH):
-        raise RuntimeError(f"{PYCALL_PATH} not found: build it with `python -m paper_2608_11688_b200.build`")
-    loader = importlib.machinery.ExtensionFileLoader("_pycall", PYCALL_PATH)
-    _pycall = importlib.util.module_from_spec(importlib.util.spec_from_loader("_pycall", loader))
-    loader.exec_module(_pycall)
+    _pycall = None
+    if os.path.exists(PYCALL_PATH):
+        try:
+            loader = importlib.machinery.ExtensionFileLoader("_pycall", PYCALL_PATH)
+            module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_pycall", loader))
+            loader.exec_module(module)
+            _pycall = module
+        except ImportError as e:
+            warnings.warn(f"{PYCALL_PATH} could not be loaded, the binding goes through ctypes: {e}", RuntimeWarning)
     _setup_pycall()
     for name, sig in FAST.items():
-        _fast[name] = _pycall.make(C.cast(getattr(lib, name), C.c_void_p).value, sig)
+        address = C.cast(getattr(lib, name), C.c_void_p).value
+        _fast[name] = _pycall.make(address, sig) if _pycall is not None else _through_ctypes(address, name)
 
 
 def load_library(path: str = LIB_PATH) -> C.CDLL:

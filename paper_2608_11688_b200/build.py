@@ -2,14 +2,18 @@
 from __future__ import annotations
 
 import os
+import platform
 import subprocess
 import sys
 import sysconfig
+import warnings
+from typing import Optional
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libapex.so")
-PYCALL = os.path.join(HERE, "_pycall.so")            # argument marshalling of the Python binding (csrc/pycall.c)
+# (named for the interpreter it is built for: another Python version builds and loads its own)
+PYCALL = os.path.join(HERE, "_pycall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))  # argument marshalling of the Python binding (csrc/pycall.c)
 TRACE_LIB = os.path.join(HERE, "libapex_trace.so")   # the same sources with the kernels' time stamps compiled in (trace.py)
 SOURCES = ["apex_ctx.cu", "apex_step.cu", "apex_observe.cu", "apex_decode.cu", "kernels_decode.cu", "kernels_router.cu", "kernels_ffn.cu", "kernels_plan.cu", "kernels_ffn_tc.cu", "apex_noalloc.cu", "fit_cdf.cu", "distill.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -31,17 +35,26 @@ def _stale(lib: str = LIB) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
-def build_pycall(force: bool = False) -> str:
-    """The binding's extension module (C, CPython API)."""
+def build_pycall(force: bool = False) -> Optional[str]:
+    """The binding's extension module (C, CPython API).  It is an accelerator: where it cannot be built (a host other than
+    x86-64, no C compiler, no Python headers) None is returned and the binding marshals through ctypes."""
+    if platform.machine().lower() not in ("x86_64", "amd64"):
+        return None
     src = os.path.join(CSRC, "pycall.c")
     if not force and os.path.exists(PYCALL) and os.path.getmtime(src) <= os.path.getmtime(PYCALL):
         return PYCALL
     cmd = [os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I" + sysconfig.get_paths()["include"], src, "-o", PYCALL]
-    r = subprocess.run(cmd, capture_output=True, text=True)
-    if r.returncode != 0:
-        sys.stderr.write(r.stdout + r.stderr)
-        raise RuntimeError("the compiler failed on pycall.c")
-    return PYCALL
+    try:
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        why = (r.stdout + r.stderr).strip() if r.returncode != 0 else None
+    except OSError as e:
+        why = str(e)
+    if why is None:
+        return PYCALL
+    if os.path.exists(PYCALL):   # built from an older source
+        os.remove(PYCALL)
+    warnings.warn(f"csrc/pycall.c was not built, the binding goes through ctypes: {why}", RuntimeWarning)
+    return None
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

@@ -179,3 +179,41 @@ def test_pycall_marshals_every_argument(sig, args, want):
         f(*[object()] * len(sig))
     with pytest.raises(AssertionError):
         binding._pycall.make(C.cast(entry, C.c_void_p).value, "p")(torch.zeros(4, 4).t())
+
+
+def test_binding_without_the_extension_module_goes_through_ctypes(lib, monkeypatch, tmp_path):
+    """No compiler (or another architecture): the build says so and goes on, the library loads, and the decode calls take
+    the same arguments to the same C functions."""
+    import ctypes as C
+    import torch
+    from paper_2608_11688_b200 import binding, build
+    monkeypatch.setattr(build, "PYCALL", str(tmp_path / "_pycall.so"))
+    monkeypatch.setenv("CC", str(tmp_path / "no_such_compiler"))
+    with pytest.warns(RuntimeWarning, match="pycall"):
+        assert build.build_pycall() is None
+    monkeypatch.setattr(build.platform, "machine", lambda: "aarch64")
+    assert build.build_pycall(force=True) is None
+
+    monkeypatch.setattr(binding, "PYCALL_PATH", build.PYCALL)
+    monkeypatch.setattr(binding, "_lib", None)
+    monkeypatch.setattr(binding, "_pycall", None)
+    monkeypatch.setattr(binding, "_fast", {})
+    assert binding.load_library() is not None and binding._pycall is None and set(binding._fast) == set(binding.FAST)
+    assert binding._fast["apex_moe_ffn_end"](0, 0) == binding.APEX_EINVAL            # reaches the library: no context
+    array, tensor, err, seen = np.zeros(4, np.float32), torch.zeros(4), C.create_string_buffer(8), []
+    for name, args, want in [
+            ("apex_select_candidates", (11, 2, 3, 0.5, tensor, array, 99), [11, 2, 3, 0.5, tensor.data_ptr(), array.ctypes.data, 99]),
+            ("apex_prefetch", (11, 2, 3, 0), [11, 2, 3, None]),
+            ("apex_route_topk_static", (tensor, None, array, 1, 2, 3, 4, tensor, tensor, 5, C.addressof(err), 8),
+             [tensor.data_ptr(), None, array.ctypes.data, 1, 2, 3, 4, tensor.data_ptr(), tensor.data_ptr(), 5, C.addressof(err), 8])]:
+        types = [C.c_void_p if t is C.c_char_p else t for t in binding.SIGNATURES[name][1]]
+        entry = C.CFUNCTYPE(C.c_int, *types)(lambda *a: seen.extend(a) or -5)
+        f = binding._through_ctypes(C.cast(entry, C.c_void_p).value, name)
+        seen.clear()
+        assert f(*args) == -5 and seen == want
+        with pytest.raises(TypeError):
+            f(*args, 0)
+        with pytest.raises(C.ArgumentError):
+            f(*[object() if c == "i" else a for a, c in zip(args, binding.FAST[name])])
+    with pytest.raises(AssertionError):
+        binding._through_ctypes(C.cast(entry, C.c_void_p).value, name)(torch.zeros(4, 4).t(), *args[1:])
