@@ -195,14 +195,12 @@ __global__ void __launch_bounds__(kRouterWarps * 32, 2) router_batched_kernel(co
   float acc[NT * NX];
 #pragma unroll
   for (int v = 0; v < NT * NX; ++v) acc[v] = 0.f;
-  // A wait that runs out (the GPU held for the length of the limit, say) does not end the loop, which has barriers: nothing more is
-  // waited for or loaded, and the cluster's tokens are marked below
-  bool dead = false;
+  // A wait that runs out (the GPU held for the length of the limit, say) does not end the loop, which has barriers: the cluster's
+  // flag is set, which ends its other waits, and the tokens are marked below
   int loaded = min(2, n_chunks);  // chunks asked for (warp 0)
   for (int c = 0; c < n_chunks; ++c) {
-    if (!dead && !mbar_wait(&s_bar[c & 1], (c >> 1) & 1, &s_bad, p.wait_limit_ns)) {
-      dead = true;
-      *(volatile int*)&s_bad = 1;
+    if (!mbar_wait(&s_bar[c & 1], (c >> 1) & 1, &s_bad, p.wait_limit_ns)) {
+      for (unsigned r = 0; r < csize; ++r) *(volatile int*)cluster.map_shared_rank(&s_bad, r) = 1;
     }
     if (active) {
       const int nv = min(CH, p.d - c * CH) >> 2;
@@ -233,7 +231,7 @@ __global__ void __launch_bounds__(kRouterWarps * 32, 2) router_batched_kernel(co
     }
     if (c + 2 < n_chunks) {
       __syncthreads();  // everybody has read this buffer
-      if (warp == 0 && !__any_sync(0xffffffffu, dead)) {
+      if (warp == 0 && !__shfl_sync(0xffffffffu, *(volatile int*)&s_bad, 0)) {  // (a buffer whose copies are still out is not filled again)
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         load_w(c + 2);
         load_x(c + 2);
@@ -275,16 +273,13 @@ __global__ void __launch_bounds__(kRouterWarps * 32, 2) router_batched_kernel(co
     }
   }
   RTL(3);
-  if (__any_sync(0xffffffffu, dead)) {
-    if (lane < (int)csize) *cluster.map_shared_rank(&s_bad, lane) = 1;
+  cluster.sync();
+  RTL(4);
+  if (s_bad) {
     if (warp == 0) {  // what is still on its way into this CTA's shared memory (bounded)
       for (int c = max(0, loaded - 2); c < loaded; ++c) mbar_wait(&s_bar[c & 1], (c >> 1) & 1, nullptr, p.wait_limit_ns);
       if (lane == 0 && p.status) *p.status = 1u;
     }
-  }
-  cluster.sync();
-  RTL(4);
-  if (s_bad) {
     for (int t = te; t < nt; t += kRouterWarps * (int)csize) router_failed(p, b0 + t, lane);
     if (p.wait_last) pdl_wait();
     return;
