@@ -364,7 +364,7 @@ ffn_tc_kernel(const __grid_constant__ TcWeightMaps tm_w, const __grid_constant__
     }
     ready_mask = ((unsigned long long)__ballot_sync(0xffffffffu, r1) << 32) | __ballot_sync(0xffffffffu, r0);
     __syncwarp();  // (every lane's acquires, before the loads of whichever lane)
-    asm volatile("fence.proxy.async;" ::: "memory");  // the tensor-map loads below read what the flags cover
+    asm volatile("fence.proxy.async.global;" ::: "memory");  // the tensor-map loads below read what the flags cover
   }
   tc_fence_before();
   __syncthreads();  // barriers initialised, TMEM allocated
@@ -683,7 +683,7 @@ ffn_tc_kernel(const __grid_constant__ TcWeightMaps tm_w, const __grid_constant__
           }
           ready_mask |= 1ull << ud.expert;
           __syncwarp();  // lane 0's acquire, before the loads of whichever lane
-          asm volatile("fence.proxy.async;" ::: "memory");
+          asm volatile("fence.proxy.async.global;" ::: "memory");
         }
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
@@ -772,8 +772,9 @@ ffn_tc_kernel(const __grid_constant__ TcWeightMaps tm_w, const __grid_constant__
         if (!ok) break;
         // The bulk loads below read what other CTAs' threads have stored, and any lane may issue one: lane 0's acquire reaches
         // the others through the warp barrier (a vote or shuffle orders no memory), and each lane's fence its own loads
+        // (of global memory only: over all state spaces a warp's fence took 0.4 us more per layer of a small step)
         __syncwarp();
-        asm volatile("fence.proxy.async;" ::: "memory");
+        asm volatile("fence.proxy.async.global;" ::: "memory");
       }
       // The shared expert runs all tokens in order: plain boxes (32 gathers per stage were its pace, 1.3 us at 128 tokens)
       const int tiles = __shfl_sync(0xffffffffu, small ? WIDE : 1, 0);   // K tiles of a stage
