@@ -109,8 +109,8 @@ int apex_create(const apex_config* cfg, apex_ctx** out) {
   CR(cudaMemset(ctx->d_tickets, 0, 64 * sizeof(unsigned int)));
   CR(dev_alloc(&ctx->d_spec, L * APEX_MAX_TOPK));
   CR(cudaMemset(ctx->d_spec, 0xff, L * APEX_MAX_TOPK * sizeof(int32_t)));
-  CR(dev_alloc(&ctx->d_counters, 2));
-  CR(cudaMemset(ctx->d_counters, 0, 2 * sizeof(unsigned long long)));
+  CR(dev_alloc(&ctx->d_zero_count, 1));
+  CR(cudaMemset(ctx->d_zero_count, 0, sizeof(unsigned long long)));
   CR(dev_alloc(&ctx->d_cand, MB * C));
   CR(dev_alloc(&ctx->d_idx, L * MB * k));
   CR(dev_alloc(&ctx->d_exec_idx, MB * k));
@@ -174,7 +174,6 @@ int apex_create(const apex_config* cfg, apex_ctx** out) {
     ctx->cur_copy_streams[i] = ctx->copy_streams[i];
   }
   CR(cudaEventCreateWithFlags(&ctx->ev_wave, cudaEventDisableTiming));
-  CR(cudaEventCreateWithFlags(&ctx->ev_in, cudaEventDisableTiming));
 #undef CR
   {
     void* fn = nullptr;
@@ -214,7 +213,7 @@ int apex_destroy(apex_ctx* ctx) {
   cudaDeviceSynchronize();
   cudaGetLastError();
   void* dev[] = {ctx->d_Wr, ctx->d_br, ctx->d_Wp, ctx->d_bp, ctx->d_w, ctx->d_theta, ctx->d_cache, ctx->d_slot_ready, ctx->d_zp,
-                 ctx->d_qp, ctx->d_zr, ctx->d_demand, ctx->d_pi, ctx->d_ncand, ctx->d_stats, ctx->d_counters, ctx->d_tickets, ctx->d_spec,
+                 ctx->d_qp, ctx->d_zr, ctx->d_demand, ctx->d_pi, ctx->d_ncand, ctx->d_stats, ctx->d_zero_count, ctx->d_tickets, ctx->d_spec,
                  ctx->d_pair_tok, ctx->d_pair_expert, ctx->d_pair_gate, ctx->d_n_pairs, ctx->d_tc_sync, ctx->d_sgate, ctx->d_xb, ctx->d_act, ctx->d_cand,
                  ctx->d_idx, ctx->d_exec_idx, ctx->d_alpha, ctx->d_exec_gate, ctx->d_cand_ncand, ctx->d_attn,
                  ctx->d_h_stage, ctx->d_hp_stage, ctx->d_y_stage};
@@ -230,7 +229,6 @@ int apex_destroy(apex_ctx* ctx) {
   for (cudaStream_t cs : ctx->copy_streams)
     if (cs) cudaStreamDestroy(cs);
   if (ctx->ev_wave) cudaEventDestroy(ctx->ev_wave);
-  if (ctx->ev_in) cudaEventDestroy(ctx->ev_in);
   delete ctx;
   return APEX_OK;
 }

@@ -308,7 +308,7 @@ struct apex_ctx {
   uint32_t* d_demand = nullptr;            // [L][N]
   int32_t *d_pi = nullptr, *d_ncand = nullptr;              // [maxB][N], [maxB]
   apex::DevStats* d_stats = nullptr;                        // [L]
-  unsigned long long* d_counters = nullptr;                 // [2]: -, zero
+  unsigned long long* d_zero_count = nullptr;               // CTAs of streaming launches that have zeroed their slice of y
   // batched path (max_batch > 1): the grouped GEMM's scratch, or the pair list of the streaming kernel
   bool tc_ok = false;
   int32_t *d_pair_tok = nullptr, *d_pair_expert = nullptr, *d_n_pairs = nullptr;
@@ -393,7 +393,7 @@ struct apex_ctx {
   cudaStream_t pred_stream = nullptr;   // stream of the last apex_predict
   uintptr_t last_ffn_y_lo = 0, last_ffn_y_hi = 0;  // output range of the last streaming-kernel launch
   int last_pred_layer = -1;             // layer whose prefetch stage (router, budget selection) was the last launch, else -1
-  cudaEvent_t ev_wave = nullptr, ev_in = nullptr;
+  cudaEvent_t ev_wave = nullptr;
   // persistent decode kernel (B = 1): device copies of the slot tables, mapped snapshots and records, counters
   int dec_clusters = 0;                       // clusters per launch; 0: the persistent path is not available
   apex::SlotSnapshot* d_dec_tab = nullptr;    // [L]

@@ -508,7 +508,7 @@ int ffn_launch(apex_ctx* ctx, int layer, int mode, const float* hpost_dev, int B
   p.pair_expert = ctx->d_pair_expert;
   p.pair_gate = ctx->d_pair_gate;
   p.n_pairs = ctx->d_n_pairs;
-  p.zero_counter = ctx->d_counters + 1;
+  p.zero_counter = ctx->d_zero_count;
   p.snap = make_snapshot(ctx, layer);
   p.slot_stride = ctx->expert_bytes;
   p.wait_limit_ns = ctx->cfg.wait_limit_ns;
