@@ -472,12 +472,14 @@ extern "C" int apex_distill_router(const float* H_dev, const float* Qr_dev, int 
   p.starve = starve_next ? 1 : 0;
   starve_next = false;
   p.ldw = (d + kKd - 1) / kKd * kKd;
-  // Forward: as few token tiles as fill the SMs once, 8 W tokens per CTA.  W = 7 (28 MMA warps, seven per scheduler)
-  // turns T = 8192 into 147 tiles; W = 8 would leave 20 of 148 SMs idle there.
+  // Forward: 8 W tokens per CTA, W the smallest of 1, 2, 4, 7, 8 that needs one round of the SMs (W = 7, 28 MMA warps, seven per
+  // scheduler, fills 147 of 148 SMs at T = 8192, where 8 fills 128).  Between the steps SMs stay idle: T = 5000 takes W = 7,
+  // 90 CTAs, where 5 would fill 125.
   const int want = (T + 8 * n_sm - 1) / (8 * n_sm);
   p.tok_warps = want <= 1 ? 1 : want <= 2 ? 2 : want <= 4 ? 4 : want <= 7 ? 7 : 8;
   p.n_fwd = (T + 8 * p.tok_warps - 1) / (8 * p.tok_warps);
-  // Backward: column tiles times segments fill the SMs once; a segment is at least one pipeline stage of tokens
+  // Backward: column tiles times segments within one round of the SMs; a segment is at least one pipeline stage of tokens, and there
+  // are at most kMaxSeg of them (the step kernel adds them up), so d = 256 takes 48 CTAs
   p.n_tiles = (d + kCols - 1) / kCols;
   p.n_seg = n_sm / p.n_tiles;
   const int most = (T + kTokTile - 1) / kTokTile;

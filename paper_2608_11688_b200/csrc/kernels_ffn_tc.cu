@@ -21,8 +21,8 @@
 // been counted in (its weights, which wait for nothing, are already on their way); the tickets are handed out in list
 // order, so whatever a unit waits for is already running somewhere and no co-residency is assumed.  As two kernels the
 // step lost a partial round of units at the end of each (748 units of 1 MB on 148 SMs: 5.05 rounds) and a pipeline
-// refill in between: 245 us against 187 at B = 256 (60 experts of 17 MB and a shared one of 69 MB: 1.16 GB), 107 against
-// 75 at B = 8.
+// refill in between; with the plan and gather kernels in front 256 us against 200 at B = 256 (60 experts of 17 MB and a shared
+// one of 69 MB: 1.11 GB), 124 against 93 at B = 8.
 //
 // A pipeline stage is 64 K values of two 128-row weight tiles (gate and up | the two column halves of downT: 32 KB) and
 // of the group's activations.  Roles: a warp loads weights and takes the tickets, a warp loads activations, a thread

@@ -1,5 +1,5 @@
 // Execution set of one token (S6) and small warp helpers, shared by the batch-1 kernels (every warp plans the token
-// itself); the batched kernel takes the shared expert's gate from here.
+// itself) and the plan kernel of batches that stream pairs; the grouped GEMM takes the shared expert's gate from here.
 #ifndef APEX_TOKEN_PLAN_CUH
 #define APEX_TOKEN_PLAN_CUH
 

@@ -249,3 +249,22 @@ def test_grouped_gemm_stops_with_copies_in_flight_and_the_context_goes_on(fmt, I
             np.testing.assert_allclose(y.cpu().numpy(), want, rtol=0, atol=2e-6 * float(np.abs(want).max()))
         finally:
             ctx.destroy()
+
+
+@pytest.mark.parametrize("mode,norm_topk", [("exact", 1), ("exact", 0), ("stall_free", 1)])
+@pytest.mark.parametrize("B,C", [(2, 12), (33, 6), (256, 6)])
+def test_pair_plan_in_lock_step(mode, norm_topk, B, C):
+    # the plan of batches that stream pairs: one warp's worth of tokens, a second CTA with one token, all eight CTAs of the
+    # cluster; demand waves (C < what the batch needs), substitution, and a gated shared expert
+    import harness
+    cfg = synth.tiny_config(d=512, N=12, k=3, I=72, C=C, L=2, T=2, I_shared=40, sigma_p=1.0, cfg_id=328)
+    prob = harness.Problem(cfg, gated_shared=True)
+    ctx = prob.make_ctx(C=C, max_batch=B, norm_topk=norm_topk)
+    try:
+        rep = harness.run_lockstep(prob, ctx, mode=mode, tau=0.8, T=2, B=B, C=C, norm_topk=bool(norm_topk), ffn_token_stride=max(1, B // 16))
+        stats = ctx.get_stats()
+        assert rep.near_ties == 0 and rep.worst_rel_l2 <= 3e-6
+        assert stats["hits_R"] == rep.hits_R and stats["substitutions"] == rep.n_subst
+        assert (stats["extra_waves"] > 0) == (mode == "exact" and rep.n_miss_steps > 0)
+    finally:
+        ctx.destroy()

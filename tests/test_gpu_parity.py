@@ -148,7 +148,7 @@ def test_batched_tokens(B, mode):
 @pytest.mark.parametrize("B", [16, 40, 97])
 @pytest.mark.parametrize("mode", ["exact", "stall_free"])
 def test_batched_tensor_core_path(B, mode):
-    # shapes the tcgen05 grouped GEMM accepts (d, I, I_shared multiples of 128), B >= 16
+    # shapes the tcgen05 grouped GEMM accepts (I, I_shared multiples of 128)
     cfg = synth.tiny_config(d=256, N=12, k=3, I=128, C=8, T=3, I_shared=256, sigma_p=1.0, cfg_id=230)
     rep, stats = _run(cfg, mode=mode, tau=0.8, T=3, B=B)
     assert stats["tokens"] == 3 * B and rep.ffn_checked >= 1 and rep.near_ties == 0
@@ -165,8 +165,8 @@ def test_batched_exact_mode_runs_in_waves_when_cache_is_smaller_than_need():
 @pytest.mark.parametrize("B,fmt", [(1, "bf16"), (1, "fp8"), (1, "fp4"), (5, "bf16"), (24, "bf16"), (24, "fp8")])
 @pytest.mark.parametrize("mode", ["exact", "stall_free"])
 def test_gated_shared_expert(B, fmt, mode):
-    # y = routed part + sigmoid(w_sg . h') * shared FFN: B = 1 the streaming kernel, B = 5 the streaming kernel per pair
-    # (gate value from the plan kernel), B = 24 the grouped GEMMs (gate value in the pair list)
+    # y = routed part + sigmoid(w_sg . h') * shared FFN: B = 1 the streaming kernel, B = 5 and 24 the grouped GEMM (the pairs of
+    # other sizes, with the gate value from the plan kernel: test_gpu_batched_ffn.py)
     cfg = synth.tiny_config(d=512, N=12, k=3, I=128, C=8, L=2, T=3, I_shared=256, sigma_p=1.0, cfg_id=290)
     hz = _harness()
     prob = hz.Problem(cfg, fp8=(fmt == "fp8"), fp4=(fmt == "fp4"), gated_shared=True)
@@ -207,6 +207,7 @@ def test_fp8_store_tiny_shapes(d, N, k, I, C, Ish, mode):
 
 
 def test_fp8_store_small_batch_runs_streaming_kernel():
+    # (these sizes run the grouped GEMM from two tokens on; batches that stream: test_gpu_batched_ffn.py)
     cfg = synth.tiny_config(d=512, N=12, k=3, I=128, C=8, T=3, I_shared=128, sigma_p=1.0, cfg_id=275)
     rep, stats = _run_fp8(cfg, mode="exact", tau=0.8, T=3, B=3)
     assert stats["tokens"] == 9
@@ -243,9 +244,8 @@ def test_fp8_store_of_subnormal_codes(B):
 @pytest.mark.parametrize("N,k,I,I_shared,B", [(4, 2, 72, 200, 2), (5, 2, 200, 0, 31), (3, 1, 130, 72, 130), (2, 2, 1100, 64, 256),
                                                   (6, 2, 700, 90, 40), (16, 3, 648, 200, 24)])
 def test_grouped_gemm_tile_edges(fmt, N, k, I, I_shared, B):
-    """Intermediate sizes off the 64- and 128-row tiles (the rest reads as zero), gate/up units of 32 rows (the first two, and
-    on the e4m3 store the fifth) and of 128, one and several chunks of K in the down projection, and groups of 2 to 256
-    tokens: one part or several, and on the quantised stores both accumulator layouts."""
+    """Intermediate sizes off the grouped GEMM's 64- and 128-row tiles, which stream their pairs instead, for groups of 2 to 256
+    tokens (the GEMM's own tile edges: test_grouped_gemm_tiles)."""
     cfg = synth.tiny_config(d=512, N=N, k=k, I=I, C=N, T=2, I_shared=I_shared, sigma_p=1.0, cfg_id=279)
     run = {"bf16": _run, "fp8": _run_fp8, "fp4": _run_fp4}[fmt]
     rep, stats = run(cfg, mode="exact", tau=0.8, T=2, B=B, ffn_token_stride=max(1, B // 16))
@@ -313,6 +313,7 @@ def test_fp4_store_tiny_shapes(d, N, k, I, C, Ish, mode):
 
 
 def test_fp4_store_small_batch_runs_streaming_kernel():
+    # (as above)
     cfg = synth.tiny_config(d=512, N=12, k=3, I=128, C=8, T=3, I_shared=128, sigma_p=1.0, cfg_id=315)
     rep, stats = _run_fp4(cfg, mode="exact", tau=0.8, T=3, B=5)
     assert stats["tokens"] == 15
