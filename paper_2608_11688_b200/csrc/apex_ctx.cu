@@ -1,6 +1,7 @@
 // C-ABI entry points, part 1: context creation and destruction, parameters (routers, confidence model, expert
 // stores).  No arithmetic of the path runs here.
 #include "apex_host.hpp"
+#include "workspace.hpp"
 
 using namespace apex;
 
@@ -49,6 +50,7 @@ int apex_create(const apex_config* cfg, apex_ctx** out) {
   }
   apex_ctx* ctx = new (std::nothrow) apex_ctx();
   if (!ctx) return APEX_ENOMEM;
+  workspace_trim();  // the memory is wanted here
   ctx->cfg = c;
   ctx->host_waves = (c.flags & APEX_FLAG_HOST_WAVES) != 0 || launches_may_block();
   if (ctx->cfg.wait_limit_ns <= 0) ctx->cfg.wait_limit_ns = 2000000000ll;
@@ -229,6 +231,7 @@ int apex_destroy(apex_ctx* ctx) {
   for (cudaStream_t cs : ctx->copy_streams)
     if (cs) cudaStreamDestroy(cs);
   if (ctx->ev_wave) cudaEventDestroy(ctx->ev_wave);
+  workspace_trim();
   delete ctx;
   return APEX_OK;
 }

@@ -25,6 +25,7 @@
 
 #include "apex_internal.hpp"
 #include "ptx.cuh"
+#include "workspace.hpp"
 
 namespace {
 
@@ -492,7 +493,7 @@ extern "C" int apex_distill_router(const float* H_dev, const float* Qr_dev, int 
   const size_t zeroed = ((3 * (n_w + rows) + 1) * sizeof(double) + 255) / 256 * 256;  // (and the status word; G behind it keeps whole lines)
   const size_t n_rest = (size_t)T * rows + (size_t)p.n_fwd * rows + (size_t)p.n_tiles * p.n_seg * rows * kCols;
   uint8_t* buf = nullptr;
-  cudaError_t e = cudaMalloc(&buf, zeroed + n_rest * sizeof(double) + n_io * sizeof(float));
+  cudaError_t e = apex::workspace_alloc(reinterpret_cast<void**>(&buf), zeroed + n_rest * sizeof(double) + n_io * sizeof(float), cs);
   if (e != cudaSuccess) {
     say(err, err_len, cudaGetErrorString(e));
     return e == cudaErrorMemoryAllocation ? APEX_ENOMEM : APEX_ECUDA;
@@ -528,7 +529,7 @@ extern "C" int apex_distill_router(const float* H_dev, const float* Qr_dev, int 
     for (size_t i = 0; i < (size_t)N * d; ++i) W_host[i] = host[i];
     for (int i = 0; i < N; ++i) b_host[i] = host[(size_t)N * d + i];
   }
-  cudaFree(buf);
+  apex::workspace_free(buf, cs);
   if (e != cudaSuccess) {
     say(err, err_len, cudaGetErrorString(e));
     return APEX_ECUDA;

@@ -31,6 +31,7 @@
 
 #include "apex_internal.hpp"
 #include "ptx.cuh"
+#include "workspace.hpp"
 
 namespace cg = cooperative_groups;
 
@@ -431,7 +432,7 @@ extern "C" int apex_fit_cdf(const double* X_dev, const int32_t* dstar_dev, int T
     cfg.gridDim = dim3(kCluster * clusters, 1, 1);
     cfg.numAttrs = 2;
     const size_t n_rec = 2 * (size_t)kMaxClusters * kMaxParams;
-    if ((e = cudaMalloc(&buf, n_rec * sizeof(ulonglong2) + (2 + 2 * (size_t)P + nth) * sizeof(double))) != cudaSuccess) { fail(e); break; }
+    if ((e = apex::workspace_alloc(reinterpret_cast<void**>(&buf), n_rec * sizeof(ulonglong2) + (2 + 2 * (size_t)P + nth) * sizeof(double), cs)) != cudaSuccess) { fail(e); break; }
     p.rec = reinterpret_cast<ulonglong2*>(buf);
     double* rest = reinterpret_cast<double*>(p.rec + n_rec);
     p.status = reinterpret_cast<int*>(rest);
@@ -459,6 +460,6 @@ extern "C" int apex_fit_cdf(const double* X_dev, const int32_t* dstar_dev, int T
       theta_host[j] = run;
     }
   } while (false);
-  if (buf) cudaFree(buf);
+  apex::workspace_free(buf, cs);
   return rc;
 }

@@ -93,3 +93,36 @@ def test_distillation_reports_a_wait_that_ran_out():
     got = binding.distill_router(H, Qr, W0, b0, iters=3)          # and the next call is not affected
     for a, b in zip(got, want):
         np.testing.assert_array_equal(a, b)
+
+
+def test_training_calls_from_two_threads_share_the_workspace_pool():
+    """Two threads on two streams, different sizes in turn: what each gets is what it gets alone."""
+    import threading
+    build.build()
+    g = torch.Generator(device="cuda").manual_seed(3)
+    jobs = []
+    for T, N, d in ((700, 9, 128), (3000, 40, 512)):
+        H = torch.randn((T, d), generator=g, device="cuda")
+        Qr = torch.softmax(torch.randn((T, N), generator=g, device="cuda"), 1).contiguous()
+        jobs.append((H, Qr, np.zeros((N, d), np.float32), np.zeros(N, np.float32)))
+    torch.cuda.synchronize()
+    alone = [binding.distill_router(*j, iters=5) for j in jobs]
+    got, errors = {}, []
+
+    def work(i):
+        try:
+            s = torch.cuda.Stream()
+            got[i] = [binding.distill_router(*jobs[(i + r) % 2], iters=5, stream=s) for r in range(6)]
+        except Exception as e:  # noqa: BLE001 (reported below)
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    for i in range(2):
+        for r in range(6):
+            for a, b in zip(got[i][r], alone[(i + r) % 2]):
+                np.testing.assert_array_equal(a, b)
