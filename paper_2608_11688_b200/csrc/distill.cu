@@ -38,7 +38,8 @@ constexpr int kKd = 64;         // columns of H and W per pipeline stage (forwar
 constexpr int kTokTile = 64;    // tokens per pipeline stage (backward)
 constexpr int kCols = 64;       // columns per CTA (backward)
 constexpr int kStages = 4;
-constexpr int kMaxSeg = 12;     // token segments (backward)
+constexpr int kMaxSeg = 37;     // token segments (backward)
+constexpr int kFewSeg = 12;     // (a shorter unrolled sum in the step kernel)
 // Row strides in shared memory: fragment loads touch 8 rows x 4 columns (or the transpose) at once; with these strides
 // the words of one access fall into different banks.
 constexpr int kLdH = kKd + 4, kLdW = kKd + 4, kLdHb = kCols + 8;
@@ -46,7 +47,7 @@ constexpr long long kWaitLimitNs = 2000000000ll;  // bound of the ring's waits (
 
 // K slices of a forward CTA: warps per eight tokens, a power of two (a stage has 16 K steps)
 __host__ __device__ constexpr int fwd_slices(int tok_warps) {
-  return tok_warps == 1 ? 16 : tok_warps == 2 ? 8 : tok_warps <= 7 ? 4 : 2;
+  return tok_warps == 1 ? 16 : tok_warps <= 3 ? 8 : tok_warps <= 7 ? 4 : 2;
 }
 
 struct DistillParams {
@@ -376,9 +377,16 @@ __global__ void __launch_bounds__(kStepThreads) distill_step_kernel(const Distil
   if (tile >= p.n_tiles || e >= p.N || j >= p.d) return;
   const double* part = p.partial + (size_t)tile * p.n_seg * n + r;
   double g = 0.0;
+  // in order; all loads in flight together (in turns of twelve 2 us more at 32 segments)
+  if (p.n_seg <= kFewSeg) {
 #pragma unroll
-  for (int s = 0; s < kMaxSeg; ++s)
-    if (s < p.n_seg) g += part[(size_t)s * n];
+    for (int s = 0; s < kFewSeg; ++s)
+      if (s < p.n_seg) g += part[(size_t)s * n];
+  } else {
+#pragma unroll
+    for (int s = 0; s < kMaxSeg; ++s)
+      if (s < p.n_seg) g += part[(size_t)s * n];
+  }
   const size_t at = (size_t)e * p.ldw + j;
   adam(p, p.W + at, p.m + at, p.v + at, g);
 }
@@ -474,20 +482,22 @@ extern "C" int apex_distill_router(const float* H_dev, const float* Qr_dev, int 
   p.starve = starve_next ? 1 : 0;
   starve_next = false;
   p.ldw = (d + kKd - 1) / kKd * kKd;
-  // Forward: 8 W tokens per CTA, W the smallest of 1, 2, 4, 7, 8 that needs one round of the SMs (W = 7, 28 MMA warps, seven per
-  // scheduler, fills 147 of 148 SMs at T = 8192, where 8 fills 128).  Between the steps SMs stay idle: T = 5000 takes W = 7,
-  // 90 CTAs, where 5 would fill 125.
+  // Forward: 8 W tokens per CTA, W the smallest that needs one round of the SMs, 8 at most (W = 7, 28 MMA warps, seven per
+  // scheduler, fills 147 of 148 SMs at T = 8192, where 8 fills 128).  With W from 1, 2, 4, 7 and 8 alone, T = 5800 took 7, 104 CTAs,
+  // where 5 fills 145: 75.6 us per iteration against 65.9 (d = 1536, N = 30).
   const int want = (T + 8 * n_sm - 1) / (8 * n_sm);
-  p.tok_warps = want <= 1 ? 1 : want <= 2 ? 2 : want <= 4 ? 4 : want <= 7 ? 7 : 8;
+  p.tok_warps = want < 8 ? want : 8;
   p.n_fwd = (T + 8 * p.tok_warps - 1) / (8 * p.tok_warps);
-  // Backward: column tiles times segments within one round of the SMs; a segment is at least one pipeline stage of tokens, and there
-  // are at most kMaxSeg of them (the step kernel adds them up), so d = 256 takes 48 CTAs
+  // Backward: column tiles times segments within one round of the SMs.  A segment is whole pipeline stages of tokens (a token
+  // more than a stage costs a stage), and there are at most kMaxSeg of them (the step kernel adds them up): the SMs of d = 256.
+  // With twelve at most, T = 8192, N = 40, d = 256 took 45.2 us per iteration on 48 CTAs, 38.8 on 148.
   p.n_tiles = (d + kCols - 1) / kCols;
   p.n_seg = n_sm / p.n_tiles;
-  const int most = (T + kTokTile - 1) / kTokTile;
+  const int stages = (T + kTokTile - 1) / kTokTile;
   p.n_seg = p.n_seg < 1 ? 1 : (p.n_seg > kMaxSeg ? kMaxSeg : p.n_seg);
-  p.n_seg = p.n_seg > most ? most : p.n_seg;
-  p.seg_len = (T + p.n_seg - 1) / p.n_seg;
+  const int per_seg = (stages + p.n_seg - 1) / p.n_seg;
+  p.n_seg = (stages + per_seg - 1) / per_seg;
+  p.seg_len = per_seg * kTokTile;
   const size_t n_w = (size_t)rows * p.ldw, n_io = (size_t)N * d + N;
   // zeroed: parameters and moments; not zeroed: G, partial sums, the fp32 parameters
   const size_t zeroed = ((3 * (n_w + rows) + 1) * sizeof(double) + 255) / 256 * 256;  // (and the status word; G behind it keeps whole lines)

@@ -95,6 +95,30 @@ def test_distillation_reports_a_wait_that_ran_out():
         np.testing.assert_array_equal(a, b)
 
 
+@pytest.mark.parametrize("T,N,d,iters", [
+    (2369, 12, 128, 3),    # three warps of tokens per forward CTA; 19 segments of two stages, the last one of a token
+    (4737, 20, 64, 3),     # five; one column tile, 37 segments
+    (7104, 8, 256, 3),     # six; 28 segments of four stages
+    (769, 40, 64, 3),      # thirteen segments of one stage: one more than the short sum of the step takes
+    (768, 40, 64, 3),      # twelve
+])
+def test_distillation_splits(T, N, d, iters):
+    """Warps per forward CTA and token segments of the backward pass, at the edges of their rules (fp64 on both sides, fp32
+    outputs: half an ulp of values below 8, and sums in another order, are well inside 2e-6)."""
+    from oracle import distill
+    build.build()
+    rng = np.random.default_rng(T)
+    H = rng.standard_normal((T, d)).astype(np.float32)
+    Z = rng.standard_normal((T, N))
+    Qr = (np.exp(Z) / np.exp(Z).sum(1, keepdims=True)).astype(np.float32)
+    W0 = (rng.standard_normal((N, d)) / np.sqrt(d)).astype(np.float32)
+    b0 = rng.standard_normal(N).astype(np.float32)
+    W_ref, b_ref = distill.distill(H, Qr, W0, b0, iters=iters, lr=0.01)
+    W, b = binding.distill_router(torch.from_numpy(H).cuda(), torch.from_numpy(Qr).cuda(), W0, b0, iters=iters, lr=0.01)
+    assert np.abs(W - W_ref).max() <= 2e-6 * max(1.0, float(np.abs(W_ref).max()))
+    assert np.abs(b - b_ref).max() <= 2e-6 * max(1.0, float(np.abs(b_ref).max()))
+
+
 def test_training_calls_from_two_threads_share_the_workspace_pool():
     """Two threads on two streams, different sizes in turn: what each gets is what it gets alone."""
     import threading
