@@ -15,7 +15,7 @@ LIB = os.path.join(HERE, "libapex.so")
 # (named for the interpreter it is built for: another Python version builds and loads its own)
 PYCALL = os.path.join(HERE, "_pycall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))  # argument marshalling of the Python binding (csrc/pycall.c)
 TRACE_LIB = os.path.join(HERE, "libapex_trace.so")   # the same sources with the kernels' time stamps compiled in (trace.py)
-SOURCES = ["apex_ctx.cu", "apex_step.cu", "apex_observe.cu", "apex_decode.cu", "kernels_decode.cu", "kernels_router.cu", "kernels_ffn.cu", "kernels_plan.cu", "kernels_ffn_tc.cu", "apex_noalloc.cu", "fit_cdf.cu", "distill.cu", "workspace.cu"]
+SOURCES = ["apex_ctx.cu", "apex_step.cu", "apex_observe.cu", "apex_decode.cu", "kernels_decode.cu", "kernels_decode_tiles.cu", "kernels_router.cu", "kernels_ffn.cu", "kernels_plan.cu", "kernels_ffn_tc.cu", "apex_noalloc.cu", "fit_cdf.cu", "distill.cu", "workspace.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "--use_fast_math=false"]
 

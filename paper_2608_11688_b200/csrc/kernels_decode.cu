@@ -1,3 +1,4 @@
+// (For rows this kernel takes: see kernels_decode_tiles.cu for the others.)
 // Persistent decode kernel: all L layer-steps of one token (B = 1) in ONE cooperative launch, so that no kernel
 // launch, no grid completion and no host round trip sits between the steps of the hit path (Sec. IV-D:
 // predict + budget before attention, prefetch during attention, exact gate after it, then the chosen
@@ -47,6 +48,7 @@
 #include <cuda_bf16.h>
 
 #include "apex_internal.hpp"
+#include "decode_common.cuh"
 #include "ptx.cuh"
 #include "router_common.cuh"
 #include "ffn_rows.cuh"
@@ -54,12 +56,16 @@
 
 namespace apex {
 
+#ifdef APEX_TIMELINE
+__device__ unsigned long long g_dec_tl[160][64][16];
+#endif
+
 namespace {
 
 constexpr int kDecMaxStages = 64;
 // Shared memory of a CTA: 227 KB, of which the kernel's static variables take 5 KB (a d = 1536 bf16 ring of 24 stages fills
 // the rest to the byte: the tests check that the token kernel is what ran) and the CTA's partial y 4 d bytes.
-constexpr int kDecSmemTotal = 227 * 1024, kDecSmemStatic = 5120;
+constexpr int kDecSmemStatic = 5120;
 
 __host__ __device__ constexpr int dec_ring_stages(uint32_t entry_bytes, int d) {
   int n = (kDecSmemTotal - kDecSmemStatic - 4 * d) / (int)entry_bytes;
@@ -67,53 +73,8 @@ __host__ __device__ constexpr int dec_ring_stages(uint32_t entry_bytes, int d) {
   return n / kDecWarps * kDecWarps;
 }
 
-#ifdef APEX_TIMELINE
-// per CTA and layer (the warp that writes last wins): 0 layer start, 1 W_p logit sent, 2 candidate mask out (poster),
-// 3 own attention share landed, 4 W_r logit sent, 5 gate logits complete, 6 plan done, 7 first expert row landed, 8 last
-// row consumed, 9 layer counted in, 10 candidate record posted (poster), 11 warps' partial y in shared memory, 12 cluster's
-// partial y complete, 13 y added, 14 both counters passed (W_r), 15 previous layer's counter passed (W_p)
-__device__ unsigned long long g_dec_tl[160][64][16];
-#define DTL(i) do { if (lane == 0 && blockIdx.x < 160 && l < 64) g_dec_tl[blockIdx.x][l][(i)] = globaltimer_ns(); } while (0)
-#else
-#define DTL(i) do { } while (0)
-#endif
-
 __device__ __forceinline__ float dbf16lo(uint32_t v) { return __uint_as_float(v << 16); }
 __device__ __forceinline__ float dbf16hi(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
-
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ void cluster_barrier() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// one 32-bit value into the shared memory of CTA `rank` of this cluster; the receiver's mbarrier counts its 4 bytes
-__device__ __forceinline__ void st_async_remote(void* local_dst, uint64_t* local_bar, uint32_t rank, float value) {
-  uint32_t ra, rb;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(smem_u32(local_dst)), "r"(rank));
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(smem_u32(local_bar)), "r"(rank));
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(ra), "r"(__float_as_uint(value)),
-               "r"(rb)
-               : "memory");
-}
-__device__ __forceinline__ void red_release_gpu_u64(unsigned long long* p, unsigned long long v) {
-  asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-__device__ __forceinline__ void red_relaxed_gpu_u64(unsigned long long* p, unsigned long long v) {
-  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-__device__ __forceinline__ uint32_t ld_acquire_gpu_u32(const uint32_t* p) {
-  uint32_t v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ unsigned ld_volatile_u32(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.volatile.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
 
 // Sum of the row weights of CTAs 0 .. cta-1.  16 per CTA; with the prefetch stage running, 14 for the CTAs of the first
 // cluster and 11 for its last CTA (the poster).
@@ -1246,13 +1207,8 @@ cudaError_t dispatch_quantised(const DecodeParams& p, int n_clusters, cudaStream
 cudaError_t dispatch(const DecodeParams& p, int n_clusters, cudaStream_t s, int* max_clusters_out) {
   if (p.fmt == kFmtE4m3) return dispatch_quantised<kFmtE4m3>(p, n_clusters, s, max_clusters_out);
   if (p.fmt == kFmtMxfp4) return dispatch_quantised<kFmtMxfp4>(p, n_clusters, s, max_clusters_out);
+  if (decode_in_tiles(p.d, p.fmt)) return launch_decode_tiles(p, n_clusters, s, max_clusters_out);
   switch (p.d) {
-    case 256: return launch_decode_t<1>(p, n_clusters, s, max_clusters_out);
-    case 512: return launch_decode_t<2>(p, n_clusters, s, max_clusters_out);
-    case 768: return launch_decode_t<3>(p, n_clusters, s, max_clusters_out);
-    case 1024: return launch_decode_t<4>(p, n_clusters, s, max_clusters_out);
-    case 1536: return launch_decode_t<6>(p, n_clusters, s, max_clusters_out);
-    case 2048: return launch_decode_t<8>(p, n_clusters, s, max_clusters_out);
     case 3072: return launch_decode_t<12>(p, n_clusters, s, max_clusters_out);
     case 4096: return launch_decode_t<16>(p, n_clusters, s, max_clusters_out);
   }

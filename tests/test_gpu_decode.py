@@ -269,3 +269,59 @@ def test_static_budget_baselines_against_the_oracle(delta):
     assert st["sum_delta_hat"] == delta * cfg.T * cfg.L == rep.sum_delta_hat and st["sum_ncand"] == (cfg.k + delta) * cfg.T * cfg.L
     rep, stats, _ = _decode(cfg, mode="stall_free", tau=0.9, T=cfg.T, prob=prob)
     assert stats["sum_delta_hat"] == delta * cfg.T * cfg.L
+
+
+@pytest.mark.parametrize("mode", ["exact", "stall_free"])
+@pytest.mark.parametrize("d,N,k,I,C,L,Ish", [
+    (256, 40, 16, 3, 30, 2, 0),      # a tile of 32 rows holds eleven experts; fewer rows than CTAs
+    (256, 9, 4, 1048, 9, 2, 249),    # tiles that end inside an expert, in the shared one and across both
+    (512, 12, 4, 479, 9, 2, 0),      # 16 rows a tile, one row in the last tile of some CTAs and 16 in others
+    (768, 16, 2, 1, 8, 2, 1),        # single rows
+    (1024, 10, 3, 641, 7, 2, 130),   # more tiles per CTA than the ring holds
+    (1536, 7, 7, 300, 7, 2, 0),      # all experts routed
+    (2048, 8, 1, 961, 4, 2, 0),      # two tiles in the ring
+])
+def test_token_kernel_tiles(d, N, k, I, C, L, Ish, mode):
+    """Rows in tiles: remainders, tiles over several experts, experts that have to be waited for."""
+    cfg = synth.tiny_config(d=d, N=N, k=k, I=I, C=C, L=L, T=4, I_shared=Ish, sigma_p=1.0, cfg_id=440 + N)
+    rep, stats, launches = _decode(cfg, mode=mode, tau=0.7, T=4)
+    assert rep.layer_steps == 4 * L and rep.ffn_checked == 4 * L
+    assert launches == 4 or not _harness().token_kernel_expected()
+
+
+@pytest.mark.parametrize("d", [256, 768, 2048])
+def test_token_kernel_special_values(d):
+    """h' of the largest and smallest magnitudes, infinities and NaN: finite and not where the per-layer kernels (fp32 products) are,
+    and as close to them as the two orders of summation are (a few hundred terms: 1e-5)."""
+    cfg = synth.tiny_config(d=d, N=6, k=2, I=40, C=6, L=1, T=1, sigma_p=0.5, cfg_id=455)
+    prob = _harness().Problem(cfg)
+    g = torch.Generator().manual_seed(d)
+    base = torch.randn((d,), generator=g) * 0.05
+    rows = [base.clone() for _ in range(6)]
+    rows[0][::7] *= 1e-30                      # parts far below the largest
+    rows[1][3] = 3.3e38                        # a rounded leading bf16 plane would overflow
+    rows[2] = rows[2] * 1e-38                  # subnormal planes
+    rows[3][5] = float("inf")
+    rows[4][7] = float("nan")
+    rows[4][9] = torch.tensor(0x7F800001, dtype=torch.int32).view(torch.float32)   # a NaN whose payload is in the low bits
+    rows[5][11] = -float("inf")
+    out = {}
+    for name, flags in (("tiles", 0), ("layers", binding.FLAG_LAYER_LAUNCHES)):
+        apex = prob.make_ctx(C=6, flags=flags)
+        try:
+            apex.warm_all()
+            ys = []
+            for r in rows:
+                h = base.cuda().view(1, 1, d).contiguous()
+                y = torch.full((1, 1, d), 7.0, device="cuda")
+                apex.decode_token(h, r.cuda().view(1, 1, d).contiguous(), 1, 0.8, "exact", y)
+                torch.cuda.synchronize()
+                ys.append(y.cpu().double().view(-1))
+            out[name] = ys
+        finally:
+            apex.destroy()
+    for i, (a, b) in enumerate(zip(out["tiles"], out["layers"])):
+        assert torch.equal(torch.isfinite(a), torch.isfinite(b)), i
+        m = torch.isfinite(b)
+        if m.any():
+            assert (a[m] - b[m]).norm() <= 1e-5 * b[m].norm() + 1e-45, i
