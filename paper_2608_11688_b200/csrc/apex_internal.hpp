@@ -280,7 +280,7 @@ bool ffn_quantised_shape_supported(int d);   // widths the e4m3 / e2m1 kernels w
 size_t ffn_row_bytes(int fmt, int d);        // bytes of one intermediate index (three vectors and their scales)
 int decode_max_clusters(int d, int fmt);     // clusters of kDecCluster CTAs the current device holds at once (0: not supported)
 cudaError_t launch_decode(const DecodeParams& p, int n_clusters, cudaStream_t s);
-bool decode_in_tiles(int d, int fmt);        // rows of this width and format are worked on in tiles (kernels_decode_tiles.cu)
+bool decode_in_tiles(int d);                 // rows of this width are worked on in tiles (kernels_decode_tiles.cu)
 cudaError_t launch_decode_tiles(const DecodeParams& p, int n_clusters, cudaStream_t s, int* max_clusters_out);  // (max_clusters_out: only that)
 
 }  // namespace apex

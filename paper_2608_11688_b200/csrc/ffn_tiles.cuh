@@ -14,6 +14,8 @@
 // columns; products of bf16 values are exact in fp32.  Error of y against 64 bits 1.5e-7 to 4e-7, as with fp32 products (of which
 // 1.5e-7 come from the gates).
 //
+// Quantised rows go the same way as fp16 (QuantTiles below).
+//
 // A tile's rows lie a multiple of 128 bytes plus 16 apart (tile_stride), so the eight rows an ldmatrix phase reads fall into
 // different banks.
 #ifndef APEX_FFN_TILES_CUH
@@ -176,6 +178,358 @@ struct RowTiles<D, kFmtBf16> {
         at[0] = lo;
         at[8] = hi;
       }
+    }
+  }
+};
+
+// ---- quantised rows: the codes become fp16 values, which hold both code sets exactly, two by one conversion.  What bounds them is
+// issue slots: a conversion is 1.7 cycles of a scheduler, a k16 MMA 16 (the e4m3 MMA of sm_100a, k32, takes 30 and no conversions, the
+// same; as bf16 a pair of codes would cost five integer operations).
+__device__ __forceinline__ void mma_f16_k16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"
+      : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
+}
+__device__ __forceinline__ void mma_f16_k8(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t b0) {
+  asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5}, {%6}, {%7, %7, %7, %7};"
+      : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+      : "r"(a0), "r"(a1), "r"(b0), "f"(0.f));
+}
+// the lower and the upper two of four e4m3 codes
+__device__ __forceinline__ void e4m3x4_to_f16(uint32_t v, uint32_t& lo, uint32_t& hi) {
+  asm("{\n.reg .b16 l, h;\nmov.b32 {l, h}, %2;\ncvt.rn.f16x2.e4m3x2 %0, l;\ncvt.rn.f16x2.e4m3x2 %1, h;\n}" : "=r"(lo), "=r"(hi) : "r"(v));
+}
+// eight e2m1 codes, two to a byte
+__device__ __forceinline__ void e2m1x8_to_f16(uint32_t v, uint32_t (&o)[4]) {
+  asm("{\n.reg .b8 b0, b1, b2, b3;\nmov.b32 {b0, b1, b2, b3}, %4;\ncvt.rn.f16x2.e2m1x2 %0, b0;\ncvt.rn.f16x2.e2m1x2 %1, b1;\n"
+      "cvt.rn.f16x2.e2m1x2 %2, b2;\ncvt.rn.f16x2.e2m1x2 %3, b3;\n}"
+      : "=r"(o[0]), "=r"(o[1]), "=r"(o[2]), "=r"(o[3])
+      : "r"(v));
+}
+
+// Activations beside them are cut into fp16 planes, three times eleven bits.  fp16's exponents do not reach far, so the values of a
+// group (a warp's columns of h', a tile's a) share a power of two that puts the largest between 2^14 and 2^15:
+//   x * up = p[0] + 2^-11 p[1] + 2^-22 p[2]
+// to the last bit of x, or to 2^-60 of the group's largest, whichever is coarser.
+struct PlaneScale {
+  float up, down;  // the power of two and its inverse
+};
+__device__ __forceinline__ PlaneScale plane_scale(uint32_t largest) {  // bits of the largest magnitude
+  const int f = min(268 - (int)(largest >> 23), 253);                  // (numbers below 2^-112 keep what 2^126 leaves them)
+  return PlaneScale{__uint_as_float((uint32_t)f << 23), __uint_as_float((uint32_t)(254 - f) << 23)};
+}
+__device__ __forceinline__ void f16_planes(float x, float up, __half (&p)[3]) {
+  const float s = x * up;
+  p[0] = __float2half_rn(s);
+  const float r1 = fabsf(s) < 65536.f ? (s - __half2float(p[0])) * 2048.f : 0.f;  // (an infinity or a NaN is p[0] alone)
+  p[1] = __float2half_rn(r1);
+  p[2] = __float2half_rn((r1 - __half2float(p[1])) * 2048.f);
+}
+// as join_planes; times the inverse of `up` the value
+__device__ __forceinline__ float join_f16_planes(float c0, float c1) {
+  const float third = __shfl_down_sync(0xffffffffu, c0, 1);
+  return fabsf(c0) <= 3.402823466e38f ? fmaf(fmaf(third, 0x1p-11f, c1), 0x1p-11f, c0) : c0;
+}
+
+// What the two quantised formats share: h' and a as fp16 planes.  K order of a step: an 8x8 matrix of ldmatrix gives a lane 4
+// consecutive bytes of a row, hence codes that follow one another, while the MMA wants columns 2t, 2t+1, 2t+8, 2t+9 in lane t:
+// h' is handed out in the order the codes arrive in, a sum does not mind.
+template <int D, int FMT>
+struct QuantTiles {
+  static constexpr int KW = D / 128;  // 16-column steps
+  static constexpr int KB = D / 256;  // 32-column blocks
+  static_assert(D % 512 == 0, "whole loads of four matrices");
+  uint32_t hb[KW][2];  // h', B operand of the gate and up products
+  float y[KW][4];      // accumulators of the down projection
+  float h_down;        // inverse of the power of two that the warp's h' was multiplied by
+
+  struct Raw {
+    float v[D / 256];
+  };
+  __device__ __forceinline__ static void ask_h(Raw& raw, const float* __restrict__ h, int warp, int lane) {
+#pragma unroll
+    for (int i = 0; i < D / 256; ++i) asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(raw.v[i]) : "l"(h + warp * (D / 8) + i * 32 + lane));
+  }
+  // (through 3 (d / 4 + 16) bytes of shared memory per warp)
+  __device__ __forceinline__ void take_h(const Raw& raw, uint8_t* scratch, int warp, int lane) {
+    constexpr int PLANE = D / 4 + 16;  // bytes
+    uint8_t* mine = scratch + warp * (3 * PLANE);
+    uint32_t largest = 0u;
+#pragma unroll
+    for (int i = 0; i < D / 256; ++i) largest = max(largest, __float_as_uint(raw.v[i]) & 0x7fffffffu);
+    const PlaneScale sc = plane_scale(__reduce_max_sync(0xffffffffu, largest));
+    h_down = sc.down;
+#pragma unroll
+    for (int i = 0; i < D / 256; ++i) {
+      __half x[3];
+      f16_planes(raw.v[i], sc.up, x);
+      __half* at = reinterpret_cast<__half*>(mine) + i * 32 + lane;
+      at[0] = x[0];
+      at[PLANE / 2] = x[1];
+      at[PLANE] = x[2];
+    }
+    __syncwarp();
+    const int plane = lane >> 2;
+    const uint8_t* src = mine + (plane < 3 ? plane : 0) * PLANE;
+#pragma unroll
+    for (int s = 0; s < KW; s += 2) {
+      // e4m3: step s has columns 16 s + 4 t .. + 3; e2m1: steps s and s + 1 have columns 16 s + 8 t .. + 3 and .. + 7
+      uint2 v0, v1;
+      if (FMT == kFmtE4m3) {
+        v0 = *reinterpret_cast<const uint2*>(src + s * 32 + (lane & 3) * 8);
+        v1 = *reinterpret_cast<const uint2*>(src + s * 32 + 32 + (lane & 3) * 8);
+      } else {
+        const uint4 v = *reinterpret_cast<const uint4*>(src + s * 32 + (lane & 3) * 16);
+        v0 = make_uint2(v.x, v.y);
+        v1 = make_uint2(v.z, v.w);
+      }
+      hb[s][0] = plane < 3 ? v0.x : 0u;
+      hb[s][1] = plane < 3 ? v0.y : 0u;
+      hb[s + 1][0] = plane < 3 ? v1.x : 0u;
+      hb[s + 1][1] = plane < 3 ? v1.y : 0u;
+    }
+  }
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int s = 0; s < KW; ++s) y[s][0] = y[s][1] = y[s][2] = y[s][3] = 0.f;
+  }
+  // The gated intermediate of ROWS rows (lane's row: lane mod ROWS) as the B operands of their 8-row blocks, and the inverse of
+  // their power of two; planes: the warp's scratch, 3 ROWS fp16 values.
+  template <int ROWS>
+  __device__ __forceinline__ static float take_a(float a, __half* planes, int lane, uint32_t (&b)[ROWS / 8]) {
+    const PlaneScale sc = plane_scale(__reduce_max_sync(0xffffffffu, __float_as_uint(a) & 0x7fffffffu));
+    __half x[3];
+    f16_planes(a, sc.up, x);
+    __syncwarp();  // (the tile before has been read)
+    if (lane < ROWS) {
+      planes[lane] = x[0];
+      planes[ROWS + lane] = x[1];
+      planes[2 * ROWS + lane] = x[2];
+    }
+    __syncwarp();
+    const int plane = lane >> 2;
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(planes + (plane < 3 ? plane : 0) * ROWS) + (lane & 3);
+#pragma unroll
+    for (int r = 0; r < ROWS / 8; ++r) b[r] = plane < 3 ? src[r * 4] : 0u;
+    return sc.down;
+  }
+};
+
+template <int D>
+struct RowTiles<D, kFmtE4m3> : QuantTiles<D, kFmtE4m3> {
+  using Base = QuantTiles<D, kFmtE4m3>;
+  using Base::KW;
+  using Base::hb;
+  using Base::y;
+  // shares of the dot products of rows' codes; see the bf16 rows.  tile: the eight rows' shared-memory address
+  __device__ __forceinline__ void gate_up(uint32_t tile, uint32_t stride, int warp, int lane, float& g, float& u) const {
+    // matrices: gate rows, up rows, columns 0 .. 15 of the step, then both of the next step
+    const uint32_t at = tile + (lane & 7) * stride + ((lane >> 3) & 1) * D + (lane >> 4) * 16 + warp * (D / 8);
+    float sum[4] = {};
+#pragma unroll
+    for (int s = 0; s < KW; s += 2) {
+      uint32_t v[4];
+      ldsm4(v, at + s * 16);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        uint32_t g0, g1, u0, u1;
+        float c[4];
+        e4m3x4_to_f16(v[2 * j], g0, g1);
+        e4m3x4_to_f16(v[2 * j + 1], u0, u1);
+        mma_f16_k16(c, g0, u0, g1, u1, hb[s + j][0], hb[s + j][1]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) sum[i] += c[i];
+      }
+    }
+    g = join_f16_planes(sum[0], sum[1]) * Base::h_down;
+    u = join_f16_planes(sum[2], sum[3]) * Base::h_down;
+  }
+  // a from the summed shares of a row: its scales are at the end of the row
+  __device__ __forceinline__ static float gated(const uint8_t* row, float gate, float g, float u) {
+    const float4 sc = *reinterpret_cast<const float4*>(row + 3 * D);
+    g *= sc.x;
+    return gate * g * __frcp_rn(1.f + expf(-g)) * (u * sc.y) * sc.z;
+  }
+  // y += downT^T a of ROWS rows, of which `here` exist
+  template <int ROWS>
+  __device__ __forceinline__ void down(uint32_t tile, uint32_t stride, int warp, int lane, const uint32_t (&b)[ROWS / 8], float unit, int here) {
+    constexpr bool PAIR = ROWS >= 16;  // two 8-row blocks to an MMA
+    // matrices: 8-row blocks 0 and 1 of a step, both of the next one | four steps of a block
+    const uint32_t at = tile + (lane & 7) * stride + 2 * D + warp * (D / 8) +
+                        (PAIR ? ((lane >> 3) & 1) * 8 * stride + (lane >> 4) * 16 : (lane >> 3) * 16);
+#pragma unroll
+    for (int r = 0; r < ROWS / 8; r += PAIR ? 2 : 1) {
+      uint32_t keep[2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int left = here - (r + i) * 8 - 2 * (lane & 3);
+        keep[i] = left >= 2 ? 0xffffffffu : left == 1 ? 0xffffu : 0u;
+      }
+#pragma unroll
+      for (int s = 0; s < KW; s += PAIR ? 2 : 4) {
+        uint32_t v[4];
+        ldsm4_t(v, at + r * 8 * stride + s * 16);
+        if (here != ROWS) {  // (what lies behind the rows may be a NaN's code)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) v[i] &= keep[PAIR ? i & 1 : 0];
+        }
+        // a register: columns 2g, 2g+1 of row 2t, then of row 2t+1.  As MMA rows: g column 2g, g + 8 column 2g+1
+        uint32_t a[4][2];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) e4m3x4_to_f16(__byte_perm(v[i], 0u, 0x3120), a[i][0], a[i][1]);
+#pragma unroll
+        for (int j = 0; j < (PAIR ? 2 : 4); ++j) {
+          float c[4];
+          if (PAIR) mma_f16_k16(c, a[2 * j][0], a[2 * j][1], a[(2 * j + 1) & 3][0], a[(2 * j + 1) & 3][1], b[r], b[PAIR ? r + 1 : r]);
+          else mma_f16_k8(c, a[j][0], a[j][1], b[r]);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) y[s + j][i] = fmaf(c[i], unit, y[s + j][i]);
+        }
+      }
+    }
+  }
+  __device__ __forceinline__ void store(float* dst, int warp, int lane) const {
+#pragma unroll
+    for (int s = 0; s < KW; ++s) {
+      const float lo = join_f16_planes(y[s][0], y[s][1]), hi = join_f16_planes(y[s][2], y[s][3]);
+      if ((lane & 3) == 0) *reinterpret_cast<float2*>(dst + warp * (D / 8) + s * 16 + (lane >> 2) * 2) = make_float2(lo, hi);
+    }
+  }
+};
+
+template <int D>
+struct RowTiles<D, kFmtMxfp4> : QuantTiles<D, kFmtMxfp4> {
+  using Base = QuantTiles<D, kFmtMxfp4>;
+  using Base::hb;
+  using Base::KB;
+  using Base::y;
+  static constexpr int SW = (KB + 3) / 4;  // words of scales of a warp's blocks
+  // scales (biased exponents) of the warp's blocks of a vector
+  __device__ __forceinline__ static void load_scales(uint32_t at, uint32_t (&sc)[SW]) {
+    if (KB == 8) {
+      asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(sc[0]), "=r"(sc[SW - 1]) : "r"(at) : "memory");
+    } else if (KB == 4) {
+      asm volatile("ld.shared.u32 %0, [%1];" : "=r"(sc[0]) : "r"(at) : "memory");
+    } else {
+#pragma unroll
+      for (int i = 0; i < KB; i += 2) {
+        uint16_t v;
+        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(at + i) : "memory");
+        if ((i & 2) == 0) sc[i / 4] = v;
+        else sc[i / 4] |= (uint32_t)v << 16;
+      }
+    }
+  }
+  __device__ __forceinline__ static uint32_t byte_of(const uint32_t (&sc)[SW], int i) { return __byte_perm(sc[i / 4], 0u, 0x4440 | (i & 3)); }
+
+  __device__ __forceinline__ void gate_up(uint32_t tile, uint32_t stride, int warp, int lane, float& g, float& u) const {
+    // matrices: gate rows, up rows of a block, then both of the next block
+    const uint32_t at = tile + (lane & 7) * stride + ((lane >> 3) & 1) * (D / 2) + (lane >> 4) * 16 + warp * (D / 16);
+    const uint32_t scales = tile + (lane >> 2) * stride + 3 * (D / 2) + warp * KB;
+    uint32_t sg[SW], su[SW];
+    load_scales(scales, sg);
+    load_scales(scales + D / 32, su);
+    float sum[4] = {};
+#pragma unroll
+    for (int b = 0; b < KB; b += 2) {
+      uint32_t v[4];
+      ldsm4(v, at + b * 16);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        uint32_t gw[4], uw[4];
+        float c0[4], c1[4];
+        e2m1x8_to_f16(v[2 * j], gw);
+        e2m1x8_to_f16(v[2 * j + 1], uw);
+        const int s = 2 * (b + j);
+        mma_f16_k16(c0, gw[0], uw[0], gw[1], uw[1], hb[s][0], hb[s][1]);
+        mma_f16_k16(c1, gw[2], uw[2], gw[3], uw[3], hb[s + 1][0], hb[s + 1][1]);
+        const float fg = __uint_as_float(byte_of(sg, b + j) << 23), fu = __uint_as_float(byte_of(su, b + j) << 23);
+        sum[0] = fmaf(c0[0] + c1[0], fg, sum[0]);
+        sum[1] = fmaf(c0[1] + c1[1], fg, sum[1]);
+        sum[2] = fmaf(c0[2] + c1[2], fu, sum[2]);
+        sum[3] = fmaf(c0[3] + c1[3], fu, sum[3]);
+      }
+    }
+    g = join_f16_planes(sum[0], sum[1]) * Base::h_down;
+    u = join_f16_planes(sum[2], sum[3]) * Base::h_down;
+  }
+  __device__ __forceinline__ static float gated(const uint8_t*, float gate, float g, float u) { return gate * g * __frcp_rn(1.f + expf(-g)) * u; }
+  // y += downT^T a.  A block's scale differs from row to row, along the sum, so it goes to the B operand: the row's planes times
+  // 2^(scale - largest scale of the block in these rows), exact down to 2^-39 of the largest value; the largest scale is
+  // applied to the result.
+  template <int ROWS>
+  __device__ __forceinline__ void down(uint32_t tile, uint32_t stride, int warp, int lane, const uint32_t (&b)[ROWS / 8], float unit, int here) {
+    constexpr bool PAIR = ROWS >= 16;
+    constexpr int RB = PAIR ? 2 : 1;  // 8-row blocks to an MMA
+    const uint32_t at = tile + (lane & 7) * stride + D + warp * (D / 16) +
+                        (PAIR ? ((lane >> 3) & 1) * 8 * stride + (lane >> 4) * 16 : (lane >> 3) * 16);
+    // lane 4 b + t works out the scales of block b in the rows 2t, 2t+1 of each 8-row block, and passes them on (every lane for
+    // itself and all blocks: 60 instructions per block instead of 5)
+    const uint32_t scales = tile + 2 * (lane & 3) * stride + 3 * (D / 2) + 2 * (D / 32) + warp * KB + min(lane >> 2, KB - 1);
+#pragma unroll
+    for (int r = 0; r < ROWS / 8; r += RB) {
+      uint32_t sc[2 * RB], top = 0u, e[RB];
+#pragma unroll
+      for (int i = 0; i < 2 * RB; ++i) {
+        const int row = (r + (i >> 1)) * 8 + (i & 1);
+        asm volatile("ld.shared.u8 %0, [%1];" : "=r"(sc[i]) : "r"(scales + row * stride) : "memory");
+        sc[i] = row + 2 * (lane & 3) < here ? sc[i] : 0u;
+        top = max(top, sc[i]);
+      }
+      top = max(top, __shfl_xor_sync(0xffffffffu, top, 1));
+      top = max(top, __shfl_xor_sync(0xffffffffu, top, 2));
+#pragma unroll
+      for (int i = 0; i < 2 * RB; ++i) {
+        // 2^-k in fp16, a subnormal from 15 on, zero from 25 on; a scale of zero is zero
+        const uint32_t k = top - sc[i];
+        const uint32_t v = sc[i] == 0u ? 0u : k < 15u ? (15u - k) << 10 : 0x400u >> min(k - 14u, 31u);
+        if (i & 1) e[i >> 1] |= v << 16;
+        else e[i >> 1] = v;
+      }
+      const float back = __uint_as_float(top << 23) * unit;
+      constexpr int STEP = PAIR || KB < 4 ? 2 : 4;  // blocks per load of four matrices (two of them unused where KB = 2 and 8 rows)
+#pragma unroll
+      for (int b0 = 0; b0 < KB; b0 += STEP) {
+        uint32_t v[4];
+        ldsm4_t(v, at + r * 8 * stride + b0 * 16);
+#pragma unroll
+        for (int j = 0; j < STEP; ++j) {
+          const int blk = b0 + j;
+          if (blk < KB) {
+            uint32_t bs[RB], a[RB][4];
+#pragma unroll
+            for (int i = 0; i < RB; ++i) {
+              const uint32_t es = __shfl_sync(0xffffffffu, e[i], blk * 4 + (lane & 3));
+              const __half2 t = __hmul2(*reinterpret_cast<const __half2*>(&b[r + i]), *reinterpret_cast<const __half2*>(&es));
+              bs[i] = *reinterpret_cast<const uint32_t*>(&t);
+              // a register: columns 4g .. 4g+3 of row 2t, then of row 2t+1, a nibble each: brought together by column
+              const uint32_t m = __byte_perm(v[PAIR ? 2 * j + i : j], 0u, 0x3120);
+              const uint32_t swap = (m ^ (m >> 4)) & 0x00f000f0u;
+              e2m1x8_to_f16(m ^ swap ^ (swap << 4), a[i]);
+            }
+            const float f = __shfl_sync(0xffffffffu, back, blk * 4);
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {  // columns 4g and 4g+1, then 4g+2 and 4g+3
+              float c[4];
+              if (PAIR) mma_f16_k16(c, a[0][2 * t], a[0][2 * t + 1], a[RB - 1][2 * t], a[RB - 1][2 * t + 1], bs[0], bs[RB - 1]);
+              else mma_f16_k8(c, a[0][2 * t], a[0][2 * t + 1], bs[0]);
+#pragma unroll
+              for (int i = 0; i < 4; ++i) y[2 * blk + t][i] = fmaf(c[i], f, y[2 * blk + t][i]);
+            }
+          }
+        }
+      }
+    }
+  }
+  __device__ __forceinline__ void store(float* dst, int warp, int lane) const {
+#pragma unroll
+    for (int b = 0; b < KB; ++b) {
+      float4 v;
+      v.x = join_f16_planes(y[2 * b][0], y[2 * b][1]);
+      v.y = join_f16_planes(y[2 * b][2], y[2 * b][3]);
+      v.z = join_f16_planes(y[2 * b + 1][0], y[2 * b + 1][1]);
+      v.w = join_f16_planes(y[2 * b + 1][2], y[2 * b + 1][3]);
+      if ((lane & 3) == 0) *reinterpret_cast<float4*>(dst + warp * (D / 8) + b * 32 + (lane >> 2) * 4) = v;
     }
   }
 };

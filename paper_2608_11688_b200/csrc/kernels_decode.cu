@@ -1,4 +1,4 @@
-// (For rows this kernel takes: see kernels_decode_tiles.cu for the others.)
+// (For the widths whose rows leave no room for tiles, d = 3072 and 4096; the narrower ones: kernels_decode_tiles.cu.)
 // Persistent decode kernel: all L layer-steps of one token (B = 1) in ONE cooperative launch, so that no kernel
 // launch, no grid completion and no host round trip sits between the steps of the hit path (Sec. IV-D:
 // predict + budget before attention, prefetch during attention, exact gate after it, then the chosen
@@ -16,8 +16,8 @@
 // allows instead -- a warp starts them as soon as its last expert rows of the previous layer have been requested, so
 // they arrive while that layer's tail, the reduction of y and the hand-over are still going on; faster, but the window
 // then overlaps the previous layer.  (Consumption stays in order, and everything derived from h or h' waits for the
-// counters below.)  The router rows do not go through the ring: narrow ones (d <= 1024) are held in registers from the
-// start of the layer, wide ones are prefetched into L2 and read when the dot product is taken (see load_row).
+// counters below.)  The router rows do not go through the ring: they are prefetched into L2 and read when the dot
+// product is taken.
 //
 //   prefetch router (S1-S3): CTA r of a cluster owns experts 8r .. 8r+7, one warp per expert.  Its dot product with h
 //     (reduction order of router_kernel: lane-strided fused multiply-adds, then the xor tree -- the logits are
@@ -63,8 +63,7 @@ __device__ unsigned long long g_dec_tl[160][64][16];
 namespace {
 
 constexpr int kDecMaxStages = 64;
-// Shared memory of a CTA: 227 KB, of which the kernel's static variables take 5 KB (a d = 1536 bf16 ring of 24 stages fills
-// the rest to the byte: the tests check that the token kernel is what ran) and the CTA's partial y 4 d bytes.
+// Shared memory of a CTA: 227 KB, of which the kernel's static variables take 5 KB and the CTA's partial y 4 d bytes.
 constexpr int kDecSmemStatic = 5120;
 
 __host__ __device__ constexpr int dec_ring_stages(uint32_t entry_bytes, int d) {
@@ -86,8 +85,8 @@ __device__ __forceinline__ long long row_weight_prefix(int cta, bool prefetching
 
 }  // namespace
 
-// NCH = d / 256; H_REGS: h' of the layer in registers; FMT: storage format of the expert rows (ffn_rows.cuh).
-template <int NCH, bool H_REGS, int FMT>
+// NCH = d / 256; FMT: storage format of the expert rows (ffn_rows.cuh).
+template <int NCH, int FMT>
 __global__ void __launch_bounds__(kDecThreads, 1) decode_token_kernel(const DecodeParams p) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ uint64_t s_full[kDecMaxStages];
@@ -279,55 +278,21 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_token_kernel(const Deco
     }
     return s;
   };
-  // A router row in registers: lane l holds float4 columns l, l + 32, ... (the order of router_kernel's reduction).
-  // Up to d = 1024 (8 float4 per lane and row) both rows are fetched at the start of the layer.  Wider rows are
-  // prefetched into L2 there instead: two rows of d = 2048 in registers spilled and cost 17 % of the layer-step
-  // (configs 2 and 4: 36.8 -> 29.8 and 42.3 -> 35.1 us without them), and even the 96 registers of two d = 1536 rows,
-  // which fit, cost the row loop more than the loads' latency costs the logits (config 1 without the stand-in:
-  // 19.3 -> 17.2 us per layer-step).  The prefetch router's wide row is read when its dot product is taken; the gate's
-  // row of d = 1536 comes into registers right before the wait for the attention window (the latency passes during the
-  // wait; + 3 % with the stand-in), and is read with x where there is no window to wait for.
-  constexpr int NVRP = NV <= 8 ? NV : 1;   // prefetch-router row
-  constexpr int NVRR = NV <= 12 ? NV : 1;  // gate row (9 to 12 float4 per lane: loaded late, see below; wider: not held)
-  constexpr bool WR_LATE = NV > 8 && NV <= 12;       // the gate row is fetched right before the wait for the attention window
-  auto load_row = [&](const float* __restrict__ W_row, auto& wr) {
-    constexpr int NVR = (int)(sizeof(wr) / sizeof(float4));
-    constexpr bool ROW_REGS = NVR > 1 || NV == 1;
-    if (!ROW_REGS) return;
-    const float4* rp = reinterpret_cast<const float4*>(W_row);
-#pragma unroll
-    for (int i = 0; i < NVR; ++i)  // volatile: keep the loads here, ahead of the waits
-      asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(wr[i].x), "=f"(wr[i].y), "=f"(wr[i].z), "=f"(wr[i].w) : "l"(rp + i * 32 + lane));
-  };
-  // dot product of the row with x (reduction order of router_kernel), plus bias; sent to CTAs [rank_lo, rank_hi) of the cluster
-  auto row_logit = [&](const float* __restrict__ W_row, const auto& wr, bool held, const float* __restrict__ x, float bias, float* zs,
-                       uint64_t* xbar, int rank_lo, int rank_hi) {
-    constexpr int NVR = (int)(sizeof(wr) / sizeof(float4));
-    constexpr bool ROW_REGS = NVR > 1 || NV == 1;
+  // Dot product of a router row with x (reduction order of router_kernel), plus bias; sent to CTAs [rank_lo, rank_hi) of the
+  // cluster.  The row has been prefetched into L2 at the start of the layer: held in registers from there, two rows of d = 2048
+  // spilled and cost 17 % of the layer-step.
+  auto row_logit = [&](const float* __restrict__ W_row, const float* __restrict__ x, float bias, float* zs, uint64_t* xbar, int rank_lo, int rank_hi) {
     const float4* __restrict__ xv = reinterpret_cast<const float4*>(x);
     const float4* __restrict__ rp = reinterpret_cast<const float4*>(W_row);
     float acc = 0.f;
-    if (ROW_REGS && held) {
-      float4 xr[NVR];
-#pragma unroll
-      for (int i = 0; i < NVR; ++i) xr[i] = __ldg(xv + i * 32 + lane);
-#pragma unroll
-      for (int i = 0; i < NVR; ++i) {
-        acc = fmaf(wr[i].x, xr[i].x, acc);
-        acc = fmaf(wr[i].y, xr[i].y, acc);
-        acc = fmaf(wr[i].z, xr[i].z, acc);
-        acc = fmaf(wr[i].w, xr[i].w, acc);
-      }
-    } else {
 #pragma unroll 8
-      for (int i = 0; i < NV; ++i) {
-        const float4 wv = __ldg(rp + i * 32 + lane);
-        const float4 v = __ldg(xv + i * 32 + lane);
-        acc = fmaf(wv.x, v.x, acc);
-        acc = fmaf(wv.y, v.y, acc);
-        acc = fmaf(wv.z, v.z, acc);
-        acc = fmaf(wv.w, v.w, acc);
-      }
+    for (int i = 0; i < NV; ++i) {
+      const float4 wv = __ldg(rp + i * 32 + lane);
+      const float4 v = __ldg(xv + i * 32 + lane);
+      acc = fmaf(wv.x, v.x, acc);
+      acc = fmaf(wv.y, v.y, acc);
+      acc = fmaf(wv.z, v.z, acc);
+      acc = fmaf(wv.w, v.w, acc);
     }
     acc = warp_sum_tree(acc);
     const float z = acc + bias;
@@ -363,11 +328,8 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_token_kernel(const Deco
     uint32_t f1 = sl1 >= 0 ? ld_relaxed_sys(slot_ready + sl1) : 0u;
     // parameters of this layer this warp will need: fetched now, used after the waits
     float bias_p = 0.f, bias_r = 0.f;
-    float4 wp_row[NVRP], wr_row[NVRR];
     const float* Wp_row = p.W_p + ((size_t)l * N + (has_row ? my_e : 0)) * d;
     const float* Wr_row = p.W_r + ((size_t)l * N + (has_row ? my_e : 0)) * d;
-    if (has_wp) load_row(Wp_row, wp_row);
-    if (has_wr && !has_wp && !WR_LATE) load_row(Wr_row, wr_row);  // (a warp with both rows fetches W_r after its W_p dot product)
     if (has_row) {
       if (has_wp) bias_p = __ldg(p.b_p + (size_t)l * N + my_e);
       bias_r = __ldg(p.b_r + (size_t)l * N + my_e);
@@ -377,9 +339,9 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_token_kernel(const Deco
         for (int i = 0; i < NV; ++i) {
           if (has_wp) prefetch_l2(reinterpret_cast<const float4*>(hl) + i * 32 + lane);
           prefetch_l2(reinterpret_cast<const float4*>(hpl) + i * 32 + lane);
-          // ... and so are the router rows that are not held in registers
-          if (NVRP == 1 && NV > 1 && has_wp) prefetch_l2(reinterpret_cast<const float4*>(Wp_row) + i * 32 + lane);
-          if (NVRR == 1 && NV > 1) prefetch_l2(reinterpret_cast<const float4*>(Wr_row) + i * 32 + lane);
+          // ... and so are the router rows
+          if (has_wp) prefetch_l2(reinterpret_cast<const float4*>(Wp_row) + i * 32 + lane);
+          prefetch_l2(reinterpret_cast<const float4*>(Wr_row) + i * 32 + lane);
         }
       }
     }
@@ -485,9 +447,8 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_token_kernel(const Deco
     if (ok && running) start_seg1(l, NSW);  // this layer's chunks: on their way while the prefetch logit is computed
     // prefetch router first of all: the sooner the candidate set is out, the more of the window the copies can use
     if (has_wp && running && ok) {
-      row_logit(Wp_row, wp_row, true, hl, bias_p, s_zp, &s_xbar[0], kDecCluster - 1, kDecCluster);  // to the poster only
+      row_logit(Wp_row, hl, bias_p, s_zp, &s_xbar[0], kDecCluster - 1, kDecCluster);  // to the poster only
       DTL(1);
-      if (has_wr && !WR_LATE) load_row(Wr_row, wr_row);
     }
     {
       int q_con = 0;
@@ -513,28 +474,14 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_token_kernel(const Deco
     // exact gate: this warp's logit, once the whole stand-in has been streamed (a real attention block would only then
     // have produced h') and the previous layer's y is complete
     if ((has_wr || (poller && (int)crank * kDecWarps < N)) && ok && !cta_stopped()) {
-      // (a wide gate row comes into registers only now, from L2: its latency passes while the counters are waited for,
-      // and the registers were free for the stand-in's segment and are free again for the expert rows)
-      if (WR_LATE && p.run_attn && has_wr) load_row(Wr_row, wr_row);  // (without a window to wait for, the row is read with x)
       // (without a stand-in: the previous layer's counter, which nobody may have waited for yet)
       bool go = true;
       if (p.run_attn) go = wait_counted(1, bar_attn, bar_prev_ffn, lpar);
       else if (bar_prev_ffn && !(J > 0 || has_wp || poller)) go = wait_counted(0, bar_prev_ffn, nullptr, (uint32_t)((l - 1) & 1));
       if (go) {
         DTL(14);
-        if (has_wr) row_logit(Wr_row, wr_row, !WR_LATE || p.run_attn != 0, hpl, bias_r, s_zr, &s_xbar[1], 0, kDecCluster);
+        if (has_wr) row_logit(Wr_row, hpl, bias_r, s_zr, &s_xbar[1], 0, kDecCluster);
         DTL(4);
-      }
-    }
-    // h' for the expert rows (the router rows' registers are free again)
-    float hreg[H_REGS ? NCH * 8 : 1];
-    if (H_REGS) {
-#pragma unroll
-      for (int c = 0; c < NCH; ++c) {
-        const float4 a = __ldg(reinterpret_cast<const float4*>(hpl) + (c * 32 + lane) * 2);
-        const float4 b2 = __ldg(reinterpret_cast<const float4*>(hpl) + (c * 32 + lane) * 2 + 1);
-        hreg[c * 8 + 0] = a.x; hreg[c * 8 + 1] = a.y; hreg[c * 8 + 2] = a.z; hreg[c * 8 + 3] = a.w;
-        hreg[c * 8 + 4] = b2.x; hreg[c * 8 + 5] = b2.y; hreg[c * 8 + 6] = b2.z; hreg[c * 8 + 7] = b2.w;
       }
     }
     // ------------------------------------------------------------ gate: routed set, execution set, row space
@@ -937,14 +884,9 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_token_kernel(const Deco
                   float gw[8], uw[8], hh[8];
                   load8<FMT>(gs, c * 32 + lane, gw);
                   load8<FMT>(us, c * 32 + lane, uw);
-                  if (H_REGS) {
-#pragma unroll
-                    for (int m = 0; m < 8; ++m) hh[m] = hreg[c * 8 + m];
-                  } else {
-                    const float4 a = __ldg(reinterpret_cast<const float4*>(hpl) + (c * 32 + lane) * 2);
-                    const float4 b2 = __ldg(reinterpret_cast<const float4*>(hpl) + (c * 32 + lane) * 2 + 1);
-                    hh[0] = a.x; hh[1] = a.y; hh[2] = a.z; hh[3] = a.w; hh[4] = b2.x; hh[5] = b2.y; hh[6] = b2.z; hh[7] = b2.w;
-                  }
+                  const float4 a = __ldg(reinterpret_cast<const float4*>(hpl) + (c * 32 + lane) * 2);
+                  const float4 b2 = __ldg(reinterpret_cast<const float4*>(hpl) + (c * 32 + lane) * 2 + 1);
+                  hh[0] = a.x; hh[1] = a.y; hh[2] = a.z; hh[3] = a.w; hh[4] = b2.x; hh[5] = b2.y; hh[6] = b2.z; hh[7] = b2.w;
                   float pg = 0.f, pu = 0.f;
 #pragma unroll
                   for (int m = 0; m < 8; ++m) pg = fmaf(gw[m], hh[m], pg);
@@ -989,14 +931,9 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_token_kernel(const Deco
                 const uint4 gv = reinterpret_cast<const uint4*>(gs)[c * 32 + lane];
                 const uint4 uv = reinterpret_cast<const uint4*>(us)[c * 32 + lane];
                 float hh[8];
-                if (H_REGS) {
-#pragma unroll
-                  for (int m = 0; m < 8; ++m) hh[m] = hreg[c * 8 + m];
-                } else {
-                  const float4 a = __ldg(reinterpret_cast<const float4*>(hpl) + (c * 32 + lane) * 2);
-                  const float4 b2 = __ldg(reinterpret_cast<const float4*>(hpl) + (c * 32 + lane) * 2 + 1);
-                  hh[0] = a.x; hh[1] = a.y; hh[2] = a.z; hh[3] = a.w; hh[4] = b2.x; hh[5] = b2.y; hh[6] = b2.z; hh[7] = b2.w;
-                }
+                const float4 a = __ldg(reinterpret_cast<const float4*>(hpl) + (c * 32 + lane) * 2);
+                const float4 b2 = __ldg(reinterpret_cast<const float4*>(hpl) + (c * 32 + lane) * 2 + 1);
+                hh[0] = a.x; hh[1] = a.y; hh[2] = a.z; hh[3] = a.w; hh[4] = b2.x; hh[5] = b2.y; hh[6] = b2.z; hh[7] = b2.w;
                 gp[0] = fmaf(dbf16lo(gv.x), hh[0], gp[0]); gp[1] = fmaf(dbf16hi(gv.x), hh[1], gp[1]);
                 gp[2] = fmaf(dbf16lo(gv.y), hh[2], gp[2]); gp[3] = fmaf(dbf16hi(gv.y), hh[3], gp[3]);
                 gp[0] = fmaf(dbf16lo(gv.z), hh[4], gp[0]); gp[1] = fmaf(dbf16hi(gv.z), hh[5], gp[1]);
@@ -1153,7 +1090,6 @@ namespace {
 
 template <int NCH, int FMT = 0>
 cudaError_t launch_decode_t(const DecodeParams& p, int n_clusters, cudaStream_t s, int* max_clusters_out) {
-  constexpr bool HR = NCH <= 8;
   constexpr uint32_t entry = fmt_entry_bytes(FMT, NCH * 256);
   constexpr int NS = dec_ring_stages(entry, NCH * 256);
   const size_t smem = (size_t)NS * entry + (size_t)NCH * 256 * sizeof(float);  // ring, then the CTA's partial y
@@ -1163,7 +1099,7 @@ cudaError_t launch_decode_t(const DecodeParams& p, int n_clusters, cudaStream_t 
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
   if (!configured[dev]) {
-    e = cudaFuncSetAttribute(decode_token_kernel<NCH, HR, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(decode_token_kernel<NCH, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     configured[dev] = true;
   }
@@ -1183,35 +1119,23 @@ cudaError_t launch_decode_t(const DecodeParams& p, int n_clusters, cudaStream_t 
     cfg.gridDim = dim3(kDecCluster, 1, 1);
     cfg.numAttrs = 1;
     int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, decode_token_kernel<NCH, HR, FMT>, &cfg);
+    e = cudaOccupancyMaxActiveClusters(&n, decode_token_kernel<NCH, FMT>, &cfg);
     *max_clusters_out = e == cudaSuccess ? n : 0;
     return e;
   }
   cfg.gridDim = dim3(kDecCluster * n_clusters, 1, 1);
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, decode_token_kernel<NCH, HR, FMT>, p);
-}
-
-template <int FMT>
-cudaError_t dispatch_quantised(const DecodeParams& p, int n_clusters, cudaStream_t s, int* max_clusters_out) {
-  switch (p.d) {  // the widths the quantised row decoders are built for
-    case 512: return launch_decode_t<2, FMT>(p, n_clusters, s, max_clusters_out);
-    case 1024: return launch_decode_t<4, FMT>(p, n_clusters, s, max_clusters_out);
-    case 1536: return launch_decode_t<6, FMT>(p, n_clusters, s, max_clusters_out);
-    case 2048: return launch_decode_t<8, FMT>(p, n_clusters, s, max_clusters_out);
-    case 4096: return launch_decode_t<16, FMT>(p, n_clusters, s, max_clusters_out);
-  }
-  return cudaErrorInvalidValue;
+  return cudaLaunchKernelEx(&cfg, decode_token_kernel<NCH, FMT>, p);
 }
 
 cudaError_t dispatch(const DecodeParams& p, int n_clusters, cudaStream_t s, int* max_clusters_out) {
-  if (p.fmt == kFmtE4m3) return dispatch_quantised<kFmtE4m3>(p, n_clusters, s, max_clusters_out);
-  if (p.fmt == kFmtMxfp4) return dispatch_quantised<kFmtMxfp4>(p, n_clusters, s, max_clusters_out);
-  if (decode_in_tiles(p.d, p.fmt)) return launch_decode_tiles(p, n_clusters, s, max_clusters_out);
-  switch (p.d) {
-    case 3072: return launch_decode_t<12>(p, n_clusters, s, max_clusters_out);
-    case 4096: return launch_decode_t<16>(p, n_clusters, s, max_clusters_out);
+  if (decode_in_tiles(p.d)) return launch_decode_tiles(p, n_clusters, s, max_clusters_out);
+  if (p.d == 4096) {
+    if (p.fmt == kFmtE4m3) return launch_decode_t<16, kFmtE4m3>(p, n_clusters, s, max_clusters_out);
+    if (p.fmt == kFmtMxfp4) return launch_decode_t<16, kFmtMxfp4>(p, n_clusters, s, max_clusters_out);
+    return launch_decode_t<16>(p, n_clusters, s, max_clusters_out);
   }
+  if (p.d == 3072 && p.fmt == kFmtBf16) return launch_decode_t<12>(p, n_clusters, s, max_clusters_out);
   return cudaErrorInvalidValue;
 }
 

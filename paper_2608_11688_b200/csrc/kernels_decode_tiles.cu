@@ -20,6 +20,9 @@
 // d = 256, I = 7000 323 -> 171; d = 512, I = 1500 and a shared expert of 500 134 -> 112; d = 768, I = 3000 212 -> 162; d = 1024,
 // I = 2500 208 -> 175; d = 2048, I = 3000 and 700 322 -> 318.  At d = 256 a copy per row is what is left: the copy engine takes one
 // every 85 cycles.
+// Quantised stores, 8 layers of 4 experts, against the row-per-warp kernel: e4m3 d = 512, I = 6000 314 -> 163; d = 1024, I = 2500
+// 203 -> 153; d = 1536, I = 1500 195 -> 160; d = 2048, I = 2500 294 -> 224 (61.6 MB of rows per layer, and 42 of the stand-in: 16 us of its 28
+// are bytes); e2m1, the same sizes, 316 -> 175, 202 -> 147, 194 -> 166, 299 -> 224: the conversions of the codes.
 #include <cuda_bf16.h>
 
 #include "apex_internal.hpp"
@@ -40,11 +43,14 @@ constexpr int kPlanRegs = 104, kWorkRegs = 200;
 static_assert(kPlanRegs * 128 + kWorkRegs * kDecThreads <= 168 * kTileThreads, "the split is served from the block's own registers");
 
 // Rows of a tile: enough for the chain of a tile (some 1 200 cycles) to be worth it, and three tiles in the ring at least where a
-// row allows it.
-__host__ __device__ constexpr int tile_blocks(int fmt, int d) { return fmt_entry_bytes(fmt, d) <= 1600u ? 4 : fmt_entry_bytes(fmt, d) <= 3200u ? 2 : 1; }
+// row allows it.  Quantised rows: two 8-row blocks make one MMA of the down projection, so 16 rows even where the ring holds two tiles
+// (e4m3 d = 2048, I = 2500: 224 us against 235 with eight rows); with 32 e2m1 d = 1024 takes 171 us instead of 182, d = 1536 213 instead of 193.
+__host__ __device__ constexpr int tile_blocks(int fmt, int d) {
+  return fmt_entry_bytes(fmt, d) <= 1700u ? 4 : fmt_entry_bytes(fmt, d) <= (fmt == kFmtBf16 ? 3200u : 6400u) ? 2 : 1;
+}
 // (the kernel's static variables: 3 KB and the exchange of a tile, twice; a d = 1536 bf16 ring of three tiles fills the rest)
 __host__ __device__ constexpr int tile_ring(int fmt, int d) {
-  const int n = (kDecSmemTotal - 3328 - 2 * 8 * tile_blocks(fmt, d) * kPartStride * 4 - 4 * d) / (int)(tile_stride(fmt_entry_bytes(fmt, d)) * 8 * tile_blocks(fmt, d));
+  const int n = (kDecSmemTotal - 3328 - 8 * tile_blocks(fmt, d) * (2 * kPartStride * 4 + (fmt == kFmtBf16 ? 0 : kTileWarps * 6)) - 4 * d) / (int)(tile_stride(fmt_entry_bytes(fmt, d)) * 8 * tile_blocks(fmt, d));
   return n > 8 ? 8 : n;
 }
 
@@ -156,6 +162,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) decode_tiles_kernel(const Dec
   __shared__ int s_abort;
   __shared__ int s_stop[2];                          // a worker has given up
   __shared__ __align__(16) float s_part[2][kRows * kPartStride];  // the warps' shares of a tile's dot products
+  __shared__ __align__(16) __half s_planes[FMT == kFmtBf16 ? 1 : kTileWarps][FMT == kFmtBf16 ? 2 : 3 * kRows];  // a worker's planes of a tile's gated intermediate
   float4* part4 = reinterpret_cast<float4*>(smem + (size_t)NT * tile_bytes);  // this CTA's partial y (behind the ring)
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -819,7 +826,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) decode_tiles_kernel(const Dec
           const int row = lane & (kRows - 1);
           for (int q = 0; q < tiles; ++q) {
             const int here = n - q * kRows < kRows ? n - q * kRows : kRows;
-            const uint32_t tile = smem_u32(smem) + s * tile_bytes + (lane & 7) * stride;
+            const uint32_t tile = smem_u32(smem) + s * tile_bytes;
             float* part = s_part[q & 1];
             const bool landed = warp_wait(&s_full[s], par);
             if (q == 0 && pass == 0) DTL(7);
@@ -827,7 +834,8 @@ __global__ void __launch_bounds__(kTileThreads, 1) decode_tiles_kernel(const Dec
 #pragma unroll
               for (int r = 0; r < R; ++r) {
                 float g, u;
-                rt.gate_up(tile + r * 8 * stride, warp, lane, g, u);
+                if constexpr (FMT == kFmtBf16) rt.gate_up(tile + (lane & 7) * stride + r * 8 * stride, warp, lane, g, u);
+                else rt.gate_up(tile + r * 8 * stride, stride, warp, lane, g, u);
                 if ((lane & 3) == 0) *reinterpret_cast<float2*>(part + (r * 8 + (lane >> 2)) * kPartStride + 2 * warp) = make_float2(g, u);
               }
             }
@@ -838,13 +846,21 @@ __global__ void __launch_bounds__(kTileThreads, 1) decode_tiles_kernel(const Dec
             const float gate = s_gate[e < N ? e : APEX_MAX_EXPERTS];
             float g, u;
             sum_shares(part, row, g, u);
-            float a = gate * g * __frcp_rn(1.f + expf(-g)) * u;
-            a = row < here ? a : 0.f;
+            if constexpr (FMT == kFmtBf16) {
+              float a = gate * g * __frcp_rn(1.f + expf(-g)) * u;
+              a = row < here ? a : 0.f;
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-              const int k0 = r * 8 + 2 * (lane & 3);
-              const float a0 = __shfl_sync(0xffffffffu, a, k0), a1 = __shfl_sync(0xffffffffu, a, k0 + 1);
-              rt.down(tile + r * 8 * stride, warp, lane, a0, a1, here - k0, here == kRows);
+              for (int r = 0; r < R; ++r) {
+                const int k0 = r * 8 + 2 * (lane & 3);
+                const float a0 = __shfl_sync(0xffffffffu, a, k0), a1 = __shfl_sync(0xffffffffu, a, k0 + 1);
+                rt.down(tile + ((lane & 7) + r * 8) * stride, warp, lane, a0, a1, here - k0, here == kRows);
+              }
+            } else {
+              float a = rt.gated(smem + s * tile_bytes + row * stride, gate, g, u);
+              a = row < here ? a : 0.f;
+              uint32_t b[R];
+              const float unit = rt.template take_a<kRows>(a, s_planes[warp], lane, b);
+              rt.template down<kRows>(tile, stride, warp, lane, b, unit, here);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&s_empty[s]);
@@ -944,11 +960,24 @@ cudaError_t launch_tiles_t(const DecodeParams& p, int n_clusters, cudaStream_t s
   return cudaLaunchKernelEx(&cfg, decode_tiles_kernel<NCH, FMT>, p);
 }
 
+template <int FMT>
+cudaError_t launch_quantised(const DecodeParams& p, int n_clusters, cudaStream_t s, int* max_clusters_out) {
+  switch (p.d) {
+    case 512: return launch_tiles_t<2, FMT>(p, n_clusters, s, max_clusters_out);
+    case 1024: return launch_tiles_t<4, FMT>(p, n_clusters, s, max_clusters_out);
+    case 1536: return launch_tiles_t<6, FMT>(p, n_clusters, s, max_clusters_out);
+    case 2048: return launch_tiles_t<8, FMT>(p, n_clusters, s, max_clusters_out);
+  }
+  return cudaErrorInvalidValue;
+}
+
 }  // namespace
 
-bool decode_in_tiles(int d, int fmt) { return fmt == kFmtBf16 && d <= 2048; }
+bool decode_in_tiles(int d) { return d <= 2048; }
 
 cudaError_t launch_decode_tiles(const DecodeParams& p, int n_clusters, cudaStream_t s, int* max_clusters_out) {
+  if (p.fmt == kFmtE4m3) return launch_quantised<kFmtE4m3>(p, n_clusters, s, max_clusters_out);
+  if (p.fmt == kFmtMxfp4) return launch_quantised<kFmtMxfp4>(p, n_clusters, s, max_clusters_out);
   switch (p.d) {
     case 256: return launch_tiles_t<1, kFmtBf16>(p, n_clusters, s, max_clusters_out);
     case 512: return launch_tiles_t<2, kFmtBf16>(p, n_clusters, s, max_clusters_out);

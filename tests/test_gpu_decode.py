@@ -289,12 +289,33 @@ def test_token_kernel_tiles(d, N, k, I, C, L, Ish, mode):
     assert launches == 4 or not _harness().token_kernel_expected()
 
 
+@pytest.mark.parametrize("fmt", ["fp8", "fp4"])
+@pytest.mark.parametrize("d,N,k,I,C,L,Ish", [
+    (512, 40, 16, 3, 30, 2, 0),      # a tile of 32 rows holds eleven experts; fewer rows than CTAs
+    (512, 9, 4, 1048, 9, 2, 249),    # tiles that end inside an expert, in the shared one and across both
+    (1024, 12, 4, 479, 9, 2, 0),     # 16 rows a tile, one row in the last tile of some CTAs and 16 in others
+    (1536, 7, 7, 641, 7, 2, 130),    # more tiles per CTA than the ring holds; all experts routed
+    (2048, 16, 2, 1, 8, 2, 1),       # single rows
+    (2048, 8, 1, 961, 4, 2, 0),      # two tiles in the ring; an expert that has to be waited for
+])
+def test_token_kernel_quantised_tiles(d, N, k, I, C, L, Ish, fmt):
+    """Quantised rows in tiles: remainders (what lies behind a tile's rows are codes of other rows), tiles over several experts."""
+    cfg = synth.tiny_config(d=d, N=N, k=k, I=I, C=C, L=L, T=4, I_shared=Ish, sigma_p=1.0, cfg_id=460 + N)
+    prob = _harness().Problem(cfg, fp8=(fmt == "fp8"), fp4=(fmt == "fp4"))
+    rep, stats, launches = _decode(cfg, mode="exact", tau=0.7, T=4, prob=prob)
+    assert rep.layer_steps == 4 * L and rep.ffn_checked == 4 * L
+    assert launches == 4 or not _harness().token_kernel_expected()
+
+
+@pytest.mark.parametrize("fmt", ["bf16", "fp8", "fp4"])
 @pytest.mark.parametrize("d", [256, 768, 2048])
-def test_token_kernel_special_values(d):
+def test_token_kernel_special_values(d, fmt):
     """h' of the largest and smallest magnitudes, infinities and NaN: finite and not where the per-layer kernels (fp32 products) are,
     and as close to them as the two orders of summation are (a few hundred terms: 1e-5)."""
+    if fmt != "bf16" and d != 2048:
+        pytest.skip("no quantised store of this width")
     cfg = synth.tiny_config(d=d, N=6, k=2, I=40, C=6, L=1, T=1, sigma_p=0.5, cfg_id=455)
-    prob = _harness().Problem(cfg)
+    prob = _harness().Problem(cfg, fp8=(fmt == "fp8"), fp4=(fmt == "fp4"))
     g = torch.Generator().manual_seed(d)
     base = torch.randn((d,), generator=g) * 0.05
     rows = [base.clone() for _ in range(6)]
