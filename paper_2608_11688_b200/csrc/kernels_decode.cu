@@ -95,7 +95,8 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_token_kernel(const Deco
   __shared__ uint64_t s_cbar[2];   // the CTA's polling warp has seen: the previous layer's y complete / the stand-in complete
   __shared__ uint64_t s_rbar;      // every warp has added its share of the gate's rank counts
   __shared__ unsigned s_rank[APEX_MAX_EXPERTS / 4];  // rank of each expert's gate logit, four 8-bit counts to a word (zero between layers)
-  __shared__ float s_zp[APEX_MAX_EXPERTS], s_zr[APEX_MAX_EXPERTS];
+  __shared__ __align__(16) float s_zp[APEX_MAX_EXPERTS];
+  __shared__ __align__(16) float s_zr[APEX_MAX_EXPERTS];
   __shared__ float s_q[APEX_MAX_EXPERTS];              // warp 0: prefetch probabilities by expert
   __shared__ int s_pi[1][APEX_MAX_EXPERTS];            // warp 0: expert by rank
   __shared__ int s_posp[APEX_MAX_EXPERTS];             // position of each expert in the prefetch ranking (warp 0)

@@ -151,7 +151,8 @@ __global__ void __launch_bounds__(kTileThreads, 1) decode_tiles_kernel(const Dec
   __shared__ uint64_t s_plan;        // the layer's tiles are known
   __shared__ uint64_t s_verdict;     // ... and whether they were requested from the right slot table
   __shared__ unsigned s_rank[APEX_MAX_EXPERTS / 4];  // rank of each expert's gate logit, four 8-bit counts to a word (zero between layers)
-  __shared__ float s_zp[APEX_MAX_EXPERTS], s_zr[APEX_MAX_EXPERTS];
+  __shared__ __align__(16) float s_zp[APEX_MAX_EXPERTS];
+  __shared__ __align__(16) float s_zr[APEX_MAX_EXPERTS];
   __shared__ float s_q[APEX_MAX_EXPERTS];            // clerk: prefetch probabilities by expert
   __shared__ int s_pi[APEX_MAX_EXPERTS];             // ... expert by rank
   __shared__ int s_posp[APEX_MAX_EXPERTS];           // ... position of each expert in the prefetch ranking

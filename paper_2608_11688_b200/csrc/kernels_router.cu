@@ -38,7 +38,7 @@ __global__ void __launch_bounds__(256) router_kernel(const RouterParams p) {
   const unsigned crank = cluster.block_rank();
   const int b = blockIdx.y;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __shared__ float zs[APEX_MAX_EXPERTS];
+  __shared__ __align__(16) float zs[APEX_MAX_EXPERTS];
   __shared__ float qs[APEX_MAX_EXPERTS];
   __shared__ int pis[APEX_MAX_EXPERTS];
   __shared__ int posp[APEX_MAX_EXPERTS];
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(kRouterWarps * 32, 2) router_batched_kernel(co
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr int CH = router_chunk(TT);
   constexpr int NT = router_tile_tok(TT), NX = router_tile_exp(TT);
-  __shared__ float zs[TT][APEX_MAX_EXPERTS];   // tokens finished here (at most all of them)
+  __shared__ __align__(16) float zs[TT][APEX_MAX_EXPERTS];   // tokens finished here (at most all of them)
   __shared__ float qs[kRouterWarps][APEX_MAX_EXPERTS];
   __shared__ int pis[kRouterWarps][APEX_MAX_EXPERTS];
   __shared__ int posp[kRouterWarps][APEX_MAX_EXPERTS];

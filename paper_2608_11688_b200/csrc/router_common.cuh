@@ -17,16 +17,12 @@ __device__ __forceinline__ float warp_sum_tree(float v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-__device__ __forceinline__ float warp_max_tree(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
+__device__ __forceinline__ float warp_max(float v) {  // (as fmaxf: a NaN is passed over)
+  float r;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
 }
-__device__ __forceinline__ int warp_max_int(int v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
+__device__ __forceinline__ int warp_max_int(int v) { return __reduce_max_sync(0xffffffffu, v); }
 
 // One cluster per token.  CTA r of the cluster owns experts r*wpc .. r*wpc+wpc-1, one warp per
 // expert; the logits are gathered in the leader CTA's shared memory through distributed shared
@@ -124,23 +120,46 @@ struct RankedLogits {
   int r0, r1;    // ranks
 };
 // the two halves of softmax_and_rank, for callers that need the ranks before the probabilities
+// (zs: 16-byte aligned)
 __device__ __forceinline__ void rank_lane_logits(const float* zs, int N, int lane, RankedLogits* R) {
   const int e0 = lane, e1 = lane + 32;
   const float NEG = -3.402823466e38f;
   R->z0 = e0 < N ? zs[e0] : NEG;
   R->z1 = e1 < N ? zs[e1] : NEG;
-  R->r0 = 0;
-  R->r1 = 0;
-#pragma unroll 8
-  for (int f = 0; f < N; ++f) {
-    const float zf = zs[f];
-    R->r0 += (zf > R->z0 || (zf == R->z0 && f < e0)) ? 1 : 0;
-    R->r1 += (zf > R->z1 || (zf == R->z1 && f < e1)) ? 1 : 0;
+  // The larger ones alone first, two instructions per comparison.  Without ties the ranks of the N experts add up to N (N - 1) / 2;
+  // a tie (or a NaN) leaves a pair out, and then the order of the indices is looked at too.  With that in every comparison, and
+  // the maximum by shuffles, barrier, ranking and softmax of 60 experts took 4 000 to 5 000 cycles of a router, 3 000 to 3 600 so; a token
+  // of 32 layers (d = 1536, N = 40) 658 us and 652.
+  int r0 = 0, r1 = 0;
+  auto count = [&](float zf) {
+    r0 += zf > R->z0 ? 1 : 0;
+    r1 += zf > R->z1 ? 1 : 0;
+  };
+  int f = 0;
+#pragma unroll 4
+  for (; f + 4 <= N; f += 4) {
+    const float4 v = *reinterpret_cast<const float4*>(zs + f);
+    count(v.x);
+    count(v.y);
+    count(v.z);
+    count(v.w);
   }
+  for (; f < N; ++f) count(zs[f]);
+  const int all = __reduce_add_sync(0xffffffffu, (e0 < N ? r0 : 0) + (e1 < N ? r1 : 0));
+  if (all != N * (N - 1) / 2) {
+    r0 = r1 = 0;
+    for (f = 0; f < N; ++f) {
+      const float zf = zs[f];
+      r0 += (zf > R->z0 || (zf == R->z0 && f < e0)) ? 1 : 0;
+      r1 += (zf > R->z1 || (zf == R->z1 && f < e1)) ? 1 : 0;
+    }
+  }
+  R->r0 = r0;
+  R->r1 = r1;
 }
 __device__ __forceinline__ void softmax_lane_logits(int N, int lane, RankedLogits* R) {
   const int e0 = lane, e1 = lane + 32;
-  const float m = warp_max_tree(fmaxf(R->z0, R->z1));
+  const float m = warp_max(fmaxf(R->z0, R->z1));
   const float x0 = e0 < N ? expf(R->z0 - m) : 0.f;
   const float x1 = e1 < N ? expf(R->z1 - m) : 0.f;
   const float sum = warp_sum_tree(x0 + x1);

@@ -147,3 +147,38 @@ def test_static_gate_refuses_sizes_beyond_its_scratch():
         binding.route_topk_static(torch.zeros((8, 258), device="cuda"), None, torch.zeros((1, 258), device="cuda"), 2,
                                   idx[:1].contiguous(), alpha[:1].contiguous())
     assert ei.value.code == binding.APEX_EINVAL
+
+
+@pytest.mark.parametrize("B", [1, 3])
+@pytest.mark.parametrize("N", [1, 3, 32, 33, 62, 64])
+@pytest.mark.parametrize("kind", ["distinct", "pairs", "all", "zeros", "nan"])
+def test_ranking_with_and_without_ties(N, B, kind):
+    """Equal logits are ranked by index (the signs of zeros do not count), and one tie is enough for it."""
+    build.build()
+    d, k = 256, min(16, N)
+    rng = np.random.default_rng(N)
+    W = rng.standard_normal((N, d)).astype(np.float32)
+    bias = np.zeros(N, np.float32)
+    if kind == "pairs":
+        W[N // 2:] = W[:N - N // 2]
+    elif kind == "all":
+        W[:] = W[0]
+    elif kind == "zeros":
+        W[:] = 0.0
+        bias[::2] = -0.0
+    hp = synth.round_to_bf16_values(rng.standard_normal((B, d)).astype(np.float32))
+    if kind == "nan":
+        bias[N // 2] = np.nan
+    idx = torch.full((B, k), -1, dtype=torch.int32, device="cuda")
+    alpha = torch.zeros((B, N), dtype=torch.float32, device="cuda")
+    binding.route_topk_static(torch.from_numpy(W).cuda(), torch.from_numpy(bias).cuda(), torch.from_numpy(hp).cuda(), k, idx, alpha)
+    torch.cuda.synchronize()
+    got, a = idx.cpu().numpy(), alpha.cpu().numpy()
+    for b in range(B):
+        if kind == "nan":      # a NaN is ordered before nobody and after nobody: it shares the first place
+            assert np.isnan(a[b]).any() and (got[b] < N).all()
+            continue
+        z = W.astype(np.float64) @ hp[b].astype(np.float64)
+        want = sorted(range(N), key=lambda e: (-z[e], e))[:k]      # (random rows: gaps far above fp32 rounding)
+        assert list(got[b]) == want, (b, list(got[b]), want)
+        assert abs(a[b].sum() - 1.0) < 1e-5
