@@ -83,6 +83,13 @@ struct SelectParams {
   int N, k, C, B;
 };
 
+struct AttnParams {
+  const uint8_t* buf;
+  size_t bytes;         // a multiple of 16
+  int wait_first;       // 1: wait for the preceding kernel before streaming; 0: stream beside it, wait before exiting
+  unsigned* status;     // mapped: 1 when a wait ran out
+};
+
 struct RouterParams {
   const float* W;     // [N][d]
   const float* bias;  // [N] or null
@@ -100,7 +107,7 @@ struct RouterParams {
   uint32_t* mbox_rec;  // mapped host, B == 1: {routed set lo, hi, sequence number, 0} in one 16-byte store, or null
   uint32_t seq_value;
   int C;
-  int wait_last;      // 1: x does not come from the preceding kernel (the attention stand-in): wait for it before exiting only
+  AttnParams attn;    // batched kernel: clusters behind the routers' stream these bytes (bytes = 0: none)
   volatile unsigned* status;  // mapped: 1 when a wait of the batched kernel ran out, or null
   long long wait_limit_ns;    // bound of that wait
   int starve;        // test hook: the batched kernel's first CTA waits for bytes that nobody sends
@@ -255,13 +262,6 @@ struct DecodeParams {
   size_t slot_stride, zr_stride, idx_stride;
   long long wait_limit_ns;
   int d, N, k, I, I_shared, C, L, mode, norm_topk, cache_reuse, n_sm;
-};
-
-struct AttnParams {
-  const uint8_t* buf;
-  size_t bytes;         // a multiple of 16
-  int wait_first;       // 1: wait for the preceding kernel before streaming; 0: stream beside it, wait before exiting
-  unsigned* status;     // mapped: 1 when a wait ran out
 };
 
 // launchers (kernels_*.cu).  Each returns the cudaError_t of the launch.

@@ -192,19 +192,27 @@ int fill_select(apex_ctx* ctx, int layer, int B, float tau, int32_t* cand_dev, i
   return APEX_OK;
 }
 
+AttnParams standin_params(apex_ctx* ctx, int layer) {
+  AttnParams p{};
+  p.buf = ctx->d_attn + (size_t)(layer % ctx->attn_layers) * ctx->attn_bytes;
+  p.bytes = ctx->attn_bytes;
+  p.status = const_cast<unsigned*>(&mhdr(ctx)->status);
+  return p;
+}
+
 // S1-S3 in one launch (used by apex_decode_token): the leader warp of the prefetch-router kernel
 // goes on with the budget selection of its token.
 int predict_select_fused(apex_ctx* ctx, int layer, const float* h_dev, int B, float tau, int32_t* cand_dev,
-                         int32_t* ncand_dev, bool beside_standin, cudaStream_t cs) {
+                         int32_t* ncand_dev, bool with_standin, cudaStream_t cs) {
   RouterParams p;
   int r = begin_predict(ctx, layer, h_dev, B, &p);
   if (r != APEX_OK) return r;
   if ((r = fill_select(ctx, layer, B, tau, cand_dev, ncand_dev, &p.sel)) != APEX_OK) return r;
   p.fuse_select = 1;
-  p.wait_last = beside_standin ? 1 : 0;
+  if (with_standin) p.attn = standin_params(ctx, layer);
   CU_TRY(ctx, launch_router(p, cs));
   ctx->last_was_ffn = false;
-  ctx->last_pred_layer = layer;
+  ctx->last_pred_layer = with_standin ? -1 : layer;
   ctx->last_stream = cs;
   ++ctx->launches;
   ctx->pred_stream = cs;
@@ -335,13 +343,9 @@ int apex_prefetch(apex_ctx* ctx, int layer, int B, void* copy_stream) {
 
 namespace {
 
-// wait_first: what is queued before the kernel is complete when its first CTA streams (and so before a kernel launched
-// behind it begins: the batched prefetch stage counts on it and has no wait of its own); otherwise when its last one exits.
+// wait_first: what is queued before the kernel is complete when its first CTA streams; otherwise when its last one exits.
 int launch_standin(apex_ctx* ctx, int layer, bool wait_first, cudaStream_t cs) {
-  AttnParams p{};
-  p.buf = ctx->d_attn + (size_t)(layer % ctx->attn_layers) * ctx->attn_bytes;
-  p.bytes = ctx->attn_bytes;
-  p.status = const_cast<unsigned*>(&mhdr(ctx)->status);
+  AttnParams p = standin_params(ctx, layer);
   p.wait_first = wait_first ? 1 : 0;
   CU_TRY(ctx, launch_attention(p, ctx->n_sm, cs));
   ctx->last_was_ffn = false;
@@ -697,15 +701,14 @@ int decode_layers(apex_ctx* ctx, const float* h_dev, const float* hpost_dev, int
     int32_t* idx = ctx->d_idx + (size_t)l * MB * k;
     float* alpha = ctx->d_alpha + (size_t)l * MB * N;
     const bool prefetching = !(tau < 0.f);  // tau < 0: the conventional scheme, expert loading on the critical path
-    // A batch: the stand-in goes first and waits for the previous layer (its window opens when that layer's output exists);
-    // the prefetch stage is launched when every CTA of it has passed that wait and runs beside it.  The other way round
-    // the stand-in started 3 to 6 us later, a launch behind the router.  (One token: its candidate record is waited for
-    // by the host, so its router, which is small, goes first.)
-    const bool standin_first = standin && B > 1;
-    if (standin_first && (r = launch_standin(ctx, l, true, (cudaStream_t)stream)) != APEX_OK) return r;
-    if (prefetching && (r = predict_select_fused(ctx, l, h_dev + l * step, B, tau, ctx->d_cand, ctx->d_cand_ncand, standin_first, (cudaStream_t)stream)) != APEX_OK)
+    // A batch: one launch streams the stand-in and runs the prefetch stage beside it.  As two launches the second came 3 to 6 us after the
+    // first, and the gate, which waits for both, a hand-over later: four layers of 60 experts (d = 2048) 424 -> 418 us at B = 8, 932 ->
+    // 914 at 256; six of 16 experts of 512 rows, B = 4, 278 -> 263.  (One token: its candidate record is waited for by the
+    // host, so its router, which is small, goes first.)
+    const bool together = standin && prefetching && B > 1;
+    if (prefetching && (r = predict_select_fused(ctx, l, h_dev + l * step, B, tau, ctx->d_cand, ctx->d_cand_ncand, together, (cudaStream_t)stream)) != APEX_OK)
       return r;
-    if (standin && !standin_first && (r = apex_attention_standin(ctx, l, stream)) != APEX_OK) return r;
+    if (standin && !together && (r = apex_attention_standin(ctx, l, stream)) != APEX_OK) return r;
     if ((r = apex_route_topk(ctx, l, hpost_dev + l * step, B, idx, alpha, stream)) != APEX_OK) return r;
     if (l > 0 && (r = ffn_finalize(ctx, l - 1)) != APEX_OK) return r;
     // With every expert of the layer in a slot no candidate set changes the table (only its LRU stamps): the expert FFN of a

@@ -63,8 +63,8 @@ __global__ void __launch_bounds__(256) router_kernel(const RouterParams p) {
   EpilogueVals ev;
   if (p.fuse_select && crank == 0 && warp == 0) ev.sel = load_select_vals(p.sel, lane);
   RTL(0);
-  if (!p.wait_last) pdl_wait();  // everything queued before this kernel is complete: x may be read
-  pdl_launch_dependents();       // the next kernel may begin its own prologue
+  pdl_wait();               // everything queued before this kernel is complete: x may be read
+  pdl_launch_dependents();  // the next kernel may begin its own prologue
   RTL(1);
   if (crank == 0 && warp == 0) load_prediction(p, b, lane, &ev);
 
@@ -97,15 +97,33 @@ __global__ void __launch_bounds__(256) router_kernel(const RouterParams p) {
   RTL(2);
   cluster.sync();
   RTL(3);
-  if (crank != 0 || warp != 0) {
-    if (p.wait_last) pdl_wait();
-    return;
-  }
+  if (crank != 0 || warp != 0) return;
 
   // ---- leader warp
   router_epilogue(p, ev, b, lane, zs, qs, pis, posp);
-  if (p.wait_last) pdl_wait();
   SPAN_END((p.fuse_select || !p.topk_out || !p.stats) ? 1 : 4);
+}
+
+// Streams the bytes of an attention block once, through shared memory by bulk copies: four threads keep a 16 KB copy
+// each in flight (64 KB per SM, 9.5 MB on the GPU against the 8 MB that latency times bandwidth asks for).  Few
+// registers and 64 KB, so a router's CTAs fit beside it; as 512-thread CTAs with loads in registers it took 12 to 17 us for the
+// 42 MB of d = 2048, and no router fitted beside two of them.
+constexpr int kAttnChunk = 16 * 1024, kAttnWarps = 4;
+
+// one of kAttnWarps warps of CTA `cta` of `ctas`; buf: its kAttnChunk bytes
+__device__ __forceinline__ void attn_stream(const AttnParams& p, uint8_t* buf, uint64_t* bar, int warp, int lane, int cta, int ctas) {
+  if (lane != 0) return;
+  uint32_t parity = 0;
+  const size_t stride = (size_t)ctas * kAttnWarps * kAttnChunk;
+  for (size_t off = ((size_t)warp * ctas + cta) * kAttnChunk; off < p.bytes; off += stride, parity ^= 1u) {
+    const uint32_t n = p.bytes - off < (size_t)kAttnChunk ? (uint32_t)(p.bytes - off) : (uint32_t)kAttnChunk;
+    mbar_expect_tx(bar, n);
+    bulk_g2s(buf, p.buf + off, n, bar);
+    if (!mbar_wait(bar, parity, nullptr, 2000000000ll)) {  // (bounded like every wait; a copy of this GPU's own memory)
+      *(volatile unsigned*)p.status = 1u;
+      break;
+    }
+  }
 }
 
 // The same for a batch (B > 1): a cluster takes TT tokens, its CTA r the experts r * wpc .. r * wpc + wpc - 1 (wpc <= 8).
@@ -119,7 +137,9 @@ __global__ void __launch_bounds__(256) router_kernel(const RouterParams p) {
 // serial epilogue.  As one token per pass over register-held rows it took 29 us at B = 256, N = 60, d = 2048.
 // columns per chunk: with 512 two of the largest CTAs share an SM (a GPU holds 15 clusters of eight CTAs, one to an SM, and
 // 16 are needed at B = 256: the last one ran behind the others)
-__host__ __device__ constexpr int router_chunk(int tt) { return tt >= 16 ? 512 : 1024; }
+__host__ __device__ constexpr int router_chunk(int tt) { return tt >= 8 ? 512 : 1024; }
+__host__ __device__ constexpr int router_smem(int tt) { return 2 * (tt + 8) * router_chunk(tt) * (int)sizeof(float); }
+static_assert(router_smem(1) >= kAttnWarps * kAttnChunk && router_smem(8) >= kAttnWarps * kAttnChunk, "a CTA of the stand-in runs in a router CTA's shared memory");
 constexpr int kRouterWarps = 8;
 
 __host__ __device__ constexpr int router_tile_tok(int tt) { return tt < 4 ? tt : 4; }
@@ -153,11 +173,25 @@ __global__ void __launch_bounds__(kRouterWarps * 32, 2) router_batched_kernel(co
   __shared__ int pis[kRouterWarps][APEX_MAX_EXPERTS];
   __shared__ int posp[kRouterWarps][APEX_MAX_EXPERTS];
   __shared__ uint64_t s_bar[2];
+  __shared__ uint64_t s_attn[kAttnWarps];
   __shared__ int s_bad;                         // a wait of a CTA of the cluster ran out
   extern __shared__ __align__(128) float tiles[];  // [2][TT + 8][CH]: x rows, W rows
   const int b0 = blockIdx.y * TT, nt = min(TT, p.B - b0);
   const int e0 = (int)crank * p.warps_per_cta, ne = max(0, min(p.warps_per_cta, p.N - e0));
   const int n_chunks = (p.d + CH - 1) / CH;
+  const int groups = (p.B + TT - 1) / TT;  // of tokens
+  if ((int)blockIdx.y >= groups) {  // the attention block's bytes, beside the routers
+    if (warp >= kAttnWarps) return;
+    if (lane == 0) {
+      mbar_init(&s_attn[warp], 1);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    pdl_wait();
+    pdl_launch_dependents();
+    attn_stream(p.attn, reinterpret_cast<uint8_t*>(tiles) + warp * kAttnChunk, &s_attn[warp], warp, lane, ((int)blockIdx.y - groups) * (int)csize + (int)crank,
+                ((int)gridDim.y - groups) * (int)csize);
+    return;
+  }
   if (threadIdx.x == 0) {
     s_bad = 0;
     mbar_init(&s_bar[0], 2);
@@ -182,7 +216,7 @@ __global__ void __launch_bounds__(kRouterWarps * 32, 2) router_batched_kernel(co
   EpilogueVals ev;
   if (p.fuse_select && te < nt) ev.sel = load_select_vals(p.sel, lane);
   RTL(0);
-  if (!p.wait_last) pdl_wait();
+  pdl_wait();
   pdl_launch_dependents();
   RTL(1);
   if (te < nt) load_prediction(p, b0 + te, lane, &ev);
@@ -281,7 +315,6 @@ __global__ void __launch_bounds__(kRouterWarps * 32, 2) router_batched_kernel(co
       if (lane == 0 && p.status) *p.status = 1u;
     }
     for (int t = te; t < nt; t += kRouterWarps * (int)csize) router_failed(p, b0 + t, lane);
-    if (p.wait_last) pdl_wait();
     return;
   }
   if (te < nt) router_epilogue(p, ev, b0 + te, lane, zs[warp], qs[warp], pis[warp], posp[warp]);
@@ -290,14 +323,21 @@ __global__ void __launch_bounds__(kRouterWarps * 32, 2) router_batched_kernel(co
     load_prediction(p, b0 + t, lane, &ev);
     router_epilogue(p, ev, b0 + t, lane, zs[t / csize], qs[warp], pis[warp], posp[warp]);
   }
-  if (p.wait_last) pdl_wait();
   RTL(6);
   SPAN_END((p.fuse_select || !p.topk_out || !p.stats) ? 1 : 4);
 }
 
+// Clusters that stream the attention block beside the routers: 128 CTAs (64 KB in flight each, 8.4 MB), fewer where it is short.  With
+// the routers' (120 CTAs at most) they are all resident, two CTAs to an SM.
+int attn_clusters(const AttnParams& a, int csize) {
+  const size_t ctas = (a.bytes + kAttnWarps * kAttnChunk - 1) / (kAttnWarps * kAttnChunk);
+  const size_t n = ctas < 128 ? ctas : 128;
+  return (int)((n + csize - 1) / csize);
+}
+
 template <int TT>
 cudaError_t launch_router_batched(const RouterParams& p, cudaLaunchConfig_t& cfg, int csize) {
-  constexpr int smem = 2 * (TT + 8) * router_chunk(TT) * (int)sizeof(float);
+  constexpr int smem = router_smem(TT);
   static bool configured[kMaxDevices];
   static std::mutex setup_mutex;  // contexts of several host threads (and the context-free gate) share this set-up
   int dev = 0;
@@ -312,7 +352,7 @@ cudaError_t launch_router_batched(const RouterParams& p, cudaLaunchConfig_t& cfg
     }
   }
   prefer_max_shared<router_batched_kernel<TT>>();
-  cfg.gridDim = dim3(csize, (p.B + TT - 1) / TT, 1);
+  cfg.gridDim = dim3(csize, (p.B + TT - 1) / TT + attn_clusters(p.attn, csize), 1);
   cfg.dynamicSmemBytes = smem;
   return cudaLaunchKernelEx(&cfg, router_batched_kernel<TT>, p);
 }
@@ -394,12 +434,6 @@ cudaError_t launch_select(const SelectParams& p, cudaStream_t s) {
   return cudaLaunchKernelEx(&cfg, select_kernel, p);
 }
 
-// Streams the bytes of an attention block once, through shared memory by bulk copies: four threads keep a 16 KB copy
-// each in flight (64 KB per SM, 9.5 MB on the GPU against the 8 MB that latency times bandwidth asks for).  Few
-// registers and 64 KB, so a router's CTAs fit beside it; as 512-thread CTAs with loads in registers it took 12 to 17 us for the
-// 42 MB of d = 2048, and no router fitted beside two of them.
-constexpr int kAttnChunk = 16 * 1024, kAttnWarps = 4;
-
 __global__ void __launch_bounds__(kAttnWarps * 32) attention_standin_kernel(const AttnParams p) {
   SPAN_BEGIN();
   extern __shared__ __align__(128) uint8_t attn_smem[];
@@ -411,19 +445,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32) attention_standin_kernel(cons
   }
   if (p.wait_first) pdl_wait();
   pdl_launch_dependents();
-  if (lane == 0) {
-    uint32_t parity = 0;
-    const size_t stride = (size_t)gridDim.x * kAttnWarps * kAttnChunk;
-    for (size_t off = ((size_t)warp * gridDim.x + blockIdx.x) * kAttnChunk; off < p.bytes; off += stride, parity ^= 1u) {
-      const uint32_t n = p.bytes - off < (size_t)kAttnChunk ? (uint32_t)(p.bytes - off) : (uint32_t)kAttnChunk;
-      mbar_expect_tx(&s_bar[warp], n);
-      bulk_g2s(attn_smem + warp * kAttnChunk, p.buf + off, n, &s_bar[warp]);
-      if (!mbar_wait(&s_bar[warp], parity, nullptr, 2000000000ll)) {  // (bounded like every wait; a copy of this GPU's own memory)
-        *(volatile unsigned*)p.status = 1u;
-        break;
-      }
-    }
-  }
+  attn_stream(p, attn_smem + warp * kAttnChunk, &s_bar[warp], warp, lane, blockIdx.x, gridDim.x);
   // Streamed beside the preceding kernel: wait for it now, so that whoever waits for this kernel has, as
   // always, everything before it on the stream complete.
   if (!p.wait_first) pdl_wait();
