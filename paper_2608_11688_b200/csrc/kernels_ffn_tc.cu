@@ -1327,23 +1327,33 @@ cudaError_t launch_ffn_tc(const TcParams& p_in, const TcMaps& m, int n_sm, cudaS
   p.nmax2 = b16 < 64 ? b16 : 64;
   p.shift1 = p.f.B <= p.nmax1 ? 20 : 7;  // (more tokens than a unit takes: the unit takes 128 or 64)
   p.shift2 = p.f.B <= p.nmax2 ? 20 : 6;
-  // Rows of I per gate/up unit: 32 where that still gives every CTA at most one unit, were all experts executed that B tokens
+  // Rows of I per gate/up unit: 32 where that gives every CTA two units at most, were all experts executed that B tokens
   // can ask for.  A unit is a chain over all of d, so with fewer units than CTAs the launch takes as long as one unit does,
   // and what a stage costs is the loops of its roles, 800 cycles whatever it holds: at d = 4096, I = 256 a step of
-  // two tokens was 79 us per layer (bf16) and 99 (e2m1) with 128 rows and one K tile per stage, 65 and 77 so.  With
-  // more units than CTAs 128 rows read the activations a quarter as often.  (More than 128 rows of X in a stage of several
-  // K tiles would leave no room for a ring.)
+  // two tokens was 79 us per layer (bf16) and 99 (e2m1) with 128 rows and one K tile per stage, 65 and 77 so.  Two rounds of
+  // 32 rows are half of one of 128: 256 units in six layers of d = 1024, B = 16 251 us (bf16) against 243, of d = 2048, B = 30 409
+  // against 387 (e2m1).  With more units 128 rows, which read the activations a quarter as often: at 512 units d = 1024, B = 32 takes 308 us,
+  // 325 with 32 rows.  (More than 128 rows of X in a stage of several K tiles would leave no room for a ring.)
   const int experts = p.f.N < p.f.B * p.f.k ? p.f.N : p.f.B * p.f.k;
   const int small_units = experts * (p.f.I / kRowsSmall) + (p.f.run_shared ? p.f.I_shared / kRowsSmall : 0);
-  const bool small = small_units <= n_sm && p.nmax1 * tc_wide(qf) <= 128;
+  const bool small = small_units <= 2 * n_sm && p.nmax1 * tc_wide(qf) <= 128;
   p.rows1 = small ? kRowsSmall : 128;
+  // Chunks of K per down unit: more where the units would leave half of the CTAs without one (a chunk keeps four tiles, and with many
+  // tokens its epilogue, one atomic per token and column, costs more than the idle CTAs).  64 units -> 128, six layers: d = 1024, I = 512,
+  // B = 16 243 -> 234 us (bf16), 285 -> 255 (e4m3); at B = 100 297 -> 309; 128 units -> 256, d = 4096, B = 8 429 -> 441.
+  const int most = qf ? kDownTilesQ : kDownTiles;
+  auto chunks = [&](int rows) { return (rows / kKTile + most - 1) / most; };
+  const int down_units = (p.f.d >> 8) * (experts * chunks(p.f.I) + (p.f.run_shared ? chunks(p.f.I_shared) : 0));
+  int split = 1;
+  while (p.f.B <= 32 && 2 * split * down_units <= n_sm) split *= 2;
   for (int q = 0; q < 2; ++q) {
     TcGeometry& g = p.geo[q];
-    const int rows = q ? p.f.I_shared : p.f.I, most = qf ? kDownTilesQ : kDownTiles, sub = tc_sub(qf);
+    const int rows = q ? p.f.I_shared : p.f.I, sub = tc_sub(qf);
     g.blocks1 = rows / p.rows1;
     g.tiles = rows / kKTile;
     if (!g.tiles) continue;
-    const int n = (g.tiles + most - 1) / most;
+    int n = chunks(rows);
+    if (n * split <= g.tiles / 4) n *= split;
     g.chunk = ((g.tiles + n - 1) / n + sub - 1) / sub * sub;  // whole raw tiles
     g.kch = (g.tiles + g.chunk - 1) / g.chunk;
     g.kch_inv = g.kch > 1 ? (uint32_t)((0x100000000ull + g.kch - 1) / g.kch) : 0u;

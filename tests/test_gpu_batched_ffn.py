@@ -95,6 +95,24 @@ def _decode_inputs(cfg, B):
     return tuple(torch.from_numpy(np.stack([x[i][0] for x in hs])).cuda() for i in (0, 1))
 
 
+@pytest.mark.parametrize("fmt", ["bf16", "fp8", "fp4"])
+@pytest.mark.parametrize("d,N,k,I,I_shared,B", [(512, 16, 3, 512, 0, 24), (256, 4, 4, 1152, 0, 32), (256, 3, 2, 512, 1024, 9), (1024, 9, 3, 1024, 0, 4)])
+def test_grouped_gemm_small_units(fmt, d, N, k, I, I_shared, B):
+    """Gate/up units of 32 rows, two to a CTA, and down projections cut into more chunks of K than their length asks for (equal
+    chunks or not).  Bounds as above."""
+    if fmt != "bf16" and d == 256:
+        d = 512
+    prob = _problem(fmt, d=d, N=N, k=k, I=I, I_shared=I_shared, cfg_id=329)
+    ctx = prob.make_ctx(max_batch=B)
+    try:
+        ctx.warm_all()
+        hp = torch.from_numpy(np.random.default_rng(329 + B).standard_normal((B, d)).astype(np.float32)).bfloat16().float().numpy()
+        y, ref = _step(prob, ctx, hp)
+        assert _rel(y, ref) <= 7.6e-6
+    finally:
+        ctx.destroy()
+
+
 @pytest.mark.parametrize("C", [6, 4])
 def test_decode_goes_on_after_candidate_records_that_never_arrived(C):
     # C = N: the expert FFN of a layer is launched before its candidate records are waited for; C < N: after
