@@ -88,6 +88,7 @@ struct AttnParams {
   size_t bytes;         // a multiple of 16
   int wait_first;       // 1: wait for the preceding kernel before streaming; 0: stream beside it, wait before exiting
   unsigned* status;     // mapped: 1 when a wait ran out
+  int n_sm;
 };
 
 struct RouterParams {

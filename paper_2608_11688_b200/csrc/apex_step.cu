@@ -197,6 +197,7 @@ AttnParams standin_params(apex_ctx* ctx, int layer) {
   p.buf = ctx->d_attn + (size_t)(layer % ctx->attn_layers) * ctx->attn_bytes;
   p.bytes = ctx->attn_bytes;
   p.status = const_cast<unsigned*>(&mhdr(ctx)->status);
+  p.n_sm = ctx->n_sm;
   return p;
 }
 

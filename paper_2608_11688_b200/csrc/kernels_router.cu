@@ -137,6 +137,8 @@ __device__ __forceinline__ void attn_stream(const AttnParams& p, uint8_t* buf, u
 // serial epilogue.  As one token per pass over register-held rows it took 29 us at B = 256, N = 60, d = 2048.
 // columns per chunk: with 512 two of the largest CTAs share an SM (a GPU holds 15 clusters of eight CTAs, one to an SM, and
 // 16 are needed at B = 256: the last one ran behind the others)
+// (The gate and the prefetch stage share a kernel on purpose: with one of its own each, for chunks of 1 024 columns at eight tokens,
+// the second came upon cold instructions and a layer took 2 to 3 us more.)
 __host__ __device__ constexpr int router_chunk(int tt) { return tt >= 8 ? 512 : 1024; }
 __host__ __device__ constexpr int router_smem(int tt) { return 2 * (tt + 8) * router_chunk(tt) * (int)sizeof(float); }
 static_assert(router_smem(1) >= kAttnWarps * kAttnChunk && router_smem(8) >= kAttnWarps * kAttnChunk, "a CTA of the stand-in runs in a router CTA's shared memory");
@@ -327,12 +329,14 @@ __global__ void __launch_bounds__(kRouterWarps * 32, 2) router_batched_kernel(co
   SPAN_END((p.fuse_select || !p.topk_out || !p.stats) ? 1 : 4);
 }
 
-// Clusters that stream the attention block beside the routers: 128 CTAs (64 KB in flight each, 8.4 MB), fewer where it is short.  With
-// the routers' (120 CTAs at most) they are all resident, two CTAs to an SM.
-int attn_clusters(const AttnParams& a, int csize) {
+// Clusters that stream the attention block beside the routers: a CTA per SM (64 KB in flight each), fewer where it is short.  All of
+// them are resident with the routers', two CTAs to an SM, as long as clusters of eight are no more than kMaxClusters8.
+constexpr int kMaxClusters8 = 31;
+int attn_clusters(const AttnParams& a, int csize, int groups) {
   const size_t ctas = (a.bytes + kAttnWarps * kAttnChunk - 1) / (kAttnWarps * kAttnChunk);
-  const size_t n = ctas < 128 ? ctas : 128;
-  return (int)((n + csize - 1) / csize);
+  if (ctas == 0) return 0;
+  const int n = ctas < (size_t)a.n_sm ? ((int)ctas + csize - 1) / csize : a.n_sm / csize;
+  return csize < 8 || n + groups <= kMaxClusters8 ? n : kMaxClusters8 - groups;
 }
 
 template <int TT>
@@ -352,7 +356,8 @@ cudaError_t launch_router_batched(const RouterParams& p, cudaLaunchConfig_t& cfg
     }
   }
   prefer_max_shared<router_batched_kernel<TT>>();
-  cfg.gridDim = dim3(csize, (p.B + TT - 1) / TT + attn_clusters(p.attn, csize), 1);
+  const int groups = (p.B + TT - 1) / TT;
+  cfg.gridDim = dim3(csize, groups + attn_clusters(p.attn, csize, groups), 1);
   cfg.dynamicSmemBytes = smem;
   return cudaLaunchKernelEx(&cfg, router_batched_kernel<TT>, p);
 }
@@ -382,9 +387,9 @@ cudaError_t launch_router(const RouterParams& p, cudaStream_t s) {
     prefer_max_shared<router_kernel>();
     return cudaLaunchKernelEx(&cfg, router_kernel, q);
   }
-  // Tokens per cluster: as few as let all clusters run at once (15 of eight CTAs), since a cluster's time grows with its
-  // tokens; at most 16
-  const int clusters = 120 / csize;
+  // Tokens per cluster: as few as let all clusters run at once (15 of eight CTAs; 128 CTAs of smaller ones), since a cluster's time
+  // grows with its tokens; at most 16
+  const int clusters = csize < 8 ? 128 / csize : 15;
   if (p.B <= clusters) return launch_router_batched<1>(q, cfg, csize);
   if (p.B <= 2 * clusters) return launch_router_batched<2>(q, cfg, csize);
   if (p.B <= 4 * clusters) return launch_router_batched<4>(q, cfg, csize);
