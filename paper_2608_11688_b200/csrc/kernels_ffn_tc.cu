@@ -1338,22 +1338,24 @@ cudaError_t launch_ffn_tc(const TcParams& p_in, const TcMaps& m, int n_sm, cudaS
   const int small_units = experts * (p.f.I / kRowsSmall) + (p.f.run_shared ? p.f.I_shared / kRowsSmall : 0);
   const bool small = small_units <= 2 * n_sm && p.nmax1 * tc_wide(qf) <= 128;
   p.rows1 = small ? kRowsSmall : 128;
-  // Chunks of K per down unit: more where the units would leave half of the CTAs without one (a chunk keeps four tiles, and with many
+  // Chunks of K per down unit: more where the units would leave half of the CTAs without one, or any of them on the quantised
+  // stores, whose stages take longer (d = 2048, I = 512, B = 30, e2m1 381 -> 358 us; d = 512, I = 1024, B = 12, e4m3 257 -> 238; d = 4096, B = 8,
+  // e2m1 345 -> 329; a chunk keeps four tiles, and with many
   // tokens its epilogue, one atomic per token and column, costs more than the idle CTAs).  64 units -> 128, six layers: d = 1024, I = 512,
   // B = 16 243 -> 234 us (bf16), 285 -> 255 (e4m3); at B = 100 297 -> 309; 128 units -> 256, d = 4096, B = 8 429 -> 441.
   const int most = qf ? kDownTilesQ : kDownTiles;
   auto chunks = [&](int rows) { return (rows / kKTile + most - 1) / most; };
   const int down_units = (p.f.d >> 8) * (experts * chunks(p.f.I) + (p.f.run_shared ? chunks(p.f.I_shared) : 0));
   int split = 1;
-  while (p.f.B <= 32 && 2 * split * down_units <= n_sm) split *= 2;
+  while (p.f.B <= 32 && (qf ? 1 : 2) * split * down_units <= n_sm) split *= 2;
   for (int q = 0; q < 2; ++q) {
     TcGeometry& g = p.geo[q];
     const int rows = q ? p.f.I_shared : p.f.I, sub = tc_sub(qf);
     g.blocks1 = rows / p.rows1;
     g.tiles = rows / kKTile;
     if (!g.tiles) continue;
-    int n = chunks(rows);
-    if (n * split <= g.tiles / 4) n *= split;
+    const int fewest = chunks(rows), finest = g.tiles / 4 > fewest ? g.tiles / 4 : fewest;
+    const int n = fewest * split < finest ? fewest * split : finest;
     g.chunk = ((g.tiles + n - 1) / n + sub - 1) / sub * sub;  // whole raw tiles
     g.kch = (g.tiles + g.chunk - 1) / g.chunk;
     g.kch_inv = g.kch > 1 ? (uint32_t)((0x100000000ull + g.kch - 1) / g.kch) : 0u;
