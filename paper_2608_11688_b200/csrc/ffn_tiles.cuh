@@ -231,6 +231,47 @@ __device__ __forceinline__ float join_f16_planes(float c0, float c1) {
   return fabsf(c0) <= 3.402823466e38f ? fmaf(fmaf(third, 0x1p-11f, c1), 0x1p-11f, c0) : c0;
 }
 
+// How many binades below the group's largest value its smallest one may still sink (by an fp16 factor, say) before a plane drops
+// bits: a value 36 binades down keeps its 24.  Negative: it does not, or the largest is so far from 1 that what the
+// planes' scales are multiplied by leaves fp32's exponents.
+__device__ __forceinline__ int plane_reach(uint32_t largest, uint32_t smallest) {  // bits of the magnitudes; smallest: of those above zero
+  const int top = (int)(largest >> 23);
+  return largest == 0u ? 36 : top < 77 || top > 187 ? -1 : 36 - (top - (int)(smallest >> 23));
+}
+
+// Four columns of a 32-column block of 16 rows' downT times a in fp32, a weight at a time, each scale applied to its own row: for
+// rows the planes do not hold.  at: the lane's codes of the first row's block (scale: its scale byte); a: of row lane mod 16
+// or 32; of the rows row0 .. row0 + 15 those below `here` exist.  The sums of the columns this lane group has in the
+// accumulators, in the lanes of plane 0 (zero in the others).  Out of line: it is hardly ever run.
+template <int FMT>
+__device__ __noinline__ float4 down_rows_fp32(const uint8_t* at, const uint8_t* scale, uint32_t stride, float a, int row0, int here) {
+  const int lane = threadIdx.x & 31;
+  float s[4] = {};
+#pragma unroll 1
+  for (int i = 0; i < 4; ++i) {
+    const int r = row0 + 4 * i + (lane & 3);
+    float ar = __shfl_sync(0xffffffffu, a, r);
+    if (r < here) {
+      uint32_t w[4];
+      e2m1x8_to_f16(*reinterpret_cast<const uint16_t*>(at + r * stride), w);
+      ar *= __uint_as_float((uint32_t)scale[r * stride] << 23);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[j]));
+        s[2 * j] = fmaf(ar, f.x, s[2 * j]);
+        s[2 * j + 1] = fmaf(ar, f.y, s[2 * j + 1]);
+      }
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    s[j] += __shfl_xor_sync(0xffffffffu, s[j], 1);
+    s[j] += __shfl_xor_sync(0xffffffffu, s[j], 2);
+    if (lane & 3) s[j] = 0.f;
+  }
+  return make_float4(s[0], s[1], s[2], s[3]);
+}
+
 // What the two quantised formats share: h' and a as fp16 planes.  K order of a step: an 8x8 matrix of ldmatrix gives a lane 4
 // consecutive bytes of a row, hence codes that follow one another, while the MMA wants columns 2t, 2t+1, 2t+8, 2t+9 in lane t:
 // h' is handed out in the order the codes arrive in, a sum does not mind.
@@ -294,10 +335,13 @@ struct QuantTiles {
     for (int s = 0; s < KW; ++s) y[s][0] = y[s][1] = y[s][2] = y[s][3] = 0.f;
   }
   // The gated intermediate of ROWS rows (lane's row: lane mod ROWS) as the B operands of their 8-row blocks, and the inverse of
-  // their power of two; planes: the warp's scratch, 3 ROWS fp16 values.
+  // their power of two; planes: the warp's scratch, 3 ROWS fp16 values; reach: see plane_reach.
   template <int ROWS>
-  __device__ __forceinline__ static float take_a(float a, __half* planes, int lane, uint32_t (&b)[ROWS / 8]) {
-    const PlaneScale sc = plane_scale(__reduce_max_sync(0xffffffffu, __float_as_uint(a) & 0x7fffffffu));
+  __device__ __forceinline__ static float take_a(float a, __half* planes, int lane, uint32_t (&b)[ROWS / 8], int& reach) {
+    const uint32_t bits = __float_as_uint(a) & 0x7fffffffu;
+    const uint32_t largest = __reduce_max_sync(0xffffffffu, bits);
+    reach = plane_reach(largest, __reduce_min_sync(0xffffffffu, bits == 0u ? 0xffffffffu : bits));
+    const PlaneScale sc = plane_scale(largest);
     __half x[3];
     f16_planes(a, sc.up, x);
     __syncwarp();  // (the tile before has been read)
@@ -352,7 +396,7 @@ struct RowTiles<D, kFmtE4m3> : QuantTiles<D, kFmtE4m3> {
   }
   // y += downT^T a of ROWS rows, of which `here` exist
   template <int ROWS>
-  __device__ __forceinline__ void down(uint32_t tile, uint32_t stride, int warp, int lane, const uint32_t (&b)[ROWS / 8], float unit, int here) {
+  __device__ __forceinline__ void down(const uint8_t*, uint32_t tile, uint32_t stride, int warp, int lane, const uint32_t (&b)[ROWS / 8], float unit, int here, float, int) {
     constexpr bool PAIR = ROWS >= 16;  // two 8-row blocks to an MMA
     // matrices: 8-row blocks 0 and 1 of a step, both of the next one | four steps of a block
     const uint32_t at = tile + (lane & 7) * stride + 2 * D + warp * (D / 8) +
@@ -455,10 +499,14 @@ struct RowTiles<D, kFmtMxfp4> : QuantTiles<D, kFmtMxfp4> {
   }
   __device__ __forceinline__ static float gated(const uint8_t*, float gate, float g, float u) { return gate * g * __frcp_rn(1.f + expf(-g)) * u; }
   // y += downT^T a.  A block's scale differs from row to row, along the sum, so it goes to the B operand: the row's planes times
-  // 2^(scale - largest scale of the block in these rows), exact down to 2^-39 of the largest value; the largest scale is
-  // applied to the result.
+  // 2^(scale - largest scale of the block in these rows); the largest scale is applied to the result.  A plane's last bit is 2^4 at the
+  // top of the reach and 2^-24 is fp16's, so nothing is cut where the smallest a lies with the smallest scale 28 binades
+  // below the largest of both.  Rows of one MMA whose scales (or a) span more, in any block, are taken in fp32: a row that sinks below the
+  // largest scale times the largest a, which no row need have together, may be all there is of a column.
   template <int ROWS>
-  __device__ __forceinline__ void down(uint32_t tile, uint32_t stride, int warp, int lane, const uint32_t (&b)[ROWS / 8], float unit, int here) {
+  __device__ __forceinline__ void down(const uint8_t* rows, uint32_t tile, uint32_t stride, int warp, int lane, const uint32_t (&b)[ROWS / 8], float unit, int here, float a,
+                                       int reach) {
+    static_assert(ROWS % 16 == 0, "two 8-row blocks to an MMA");
     constexpr bool PAIR = ROWS >= 16;
     constexpr int RB = PAIR ? 2 : 1;  // 8-row blocks to an MMA
     const uint32_t at = tile + (lane & 7) * stride + D + warp * (D / 16) +
@@ -478,6 +526,21 @@ struct RowTiles<D, kFmtMxfp4> : QuantTiles<D, kFmtMxfp4> {
       }
       top = max(top, __shfl_xor_sync(0xffffffffu, top, 1));
       top = max(top, __shfl_xor_sync(0xffffffffu, top, 2));
+      bool wide = false;
+#pragma unroll
+      for (int i = 0; i < 2 * RB; ++i) wide = wide || (sc[i] != 0u && ((int)(top - sc[i]) > reach - 8 || sc[i] - 64u > 127u));
+      if (__any_sync(0xffffffffu, wide)) {
+        const uint8_t* codes = rows + D + warp * (D / 16) + (lane >> 2) * 2;
+#pragma unroll
+        for (int blk = 0; blk < KB; ++blk) {
+          const float4 v = down_rows_fp32<kFmtMxfp4>(codes + blk * 16, rows + 3 * (D / 2) + 2 * (D / 32) + warp * KB + blk, stride, a, r * 8, here);
+          y[2 * blk][0] += v.x;
+          y[2 * blk][2] += v.y;
+          y[2 * blk + 1][0] += v.z;
+          y[2 * blk + 1][2] += v.w;
+        }
+        continue;
+      }
 #pragma unroll
       for (int i = 0; i < 2 * RB; ++i) {
         // 2^-k in fp16, a subnormal from 15 on, zero from 25 on; a scale of zero is zero

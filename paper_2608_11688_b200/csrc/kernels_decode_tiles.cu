@@ -860,8 +860,9 @@ __global__ void __launch_bounds__(kTileThreads, 1) decode_tiles_kernel(const Dec
               float a = rt.gated(smem + s * tile_bytes + row * stride, gate, g, u);
               a = row < here ? a : 0.f;
               uint32_t b[R];
-              const float unit = rt.template take_a<kRows>(a, s_planes[warp], lane, b);
-              rt.template down<kRows>(tile, stride, warp, lane, b, unit, here);
+              int reach;
+              const float unit = rt.template take_a<kRows>(a, s_planes[warp], lane, b, reach);
+              rt.template down<kRows>(smem + s * tile_bytes, tile, stride, warp, lane, b, unit, here, a, reach);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&s_empty[s]);

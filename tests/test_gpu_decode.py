@@ -346,3 +346,53 @@ def test_token_kernel_special_values(d, fmt):
         m = torch.isfinite(b)
         if m.any():
             assert (a[m] - b[m]).norm() <= 1e-5 * b[m].norm() + 1e-45, i
+
+
+def _one_layer_y(cfg, store, hp, *, fp4, flags=0):
+    """y of one token through apex_decode_token, all N = k experts resident and routed, each with the gate 1 / k (routers of zero
+    weights), and the same in 64 bits."""
+    d, N = cfg.d, cfg.N
+    pinned = torch.empty(store.shape, dtype=store.dtype, pin_memory=True)
+    pinned.copy_(store)
+    apex = binding.Apex(d=d, N=N, k=cfg.k, I=cfg.I, C_slots=N, L=1, max_batch=1, flags=(binding.FLAG_FP4_EXPERTS if fp4 else binding.FLAG_FP8_EXPERTS) | flags)
+    try:
+        zero = np.zeros((N, d), np.float32), np.zeros(N, np.float32)
+        apex.set_router(0, *zero)
+        apex.set_prefetch_router(0, *zero)
+        apex.set_cdf(0, *synth.handset_cdf_params(cfg))
+        apex.register_experts(0, pinned)
+        apex.warm_all()
+        y = torch.full((1, 1, d), 7.0, device="cuda")
+        apex.decode_token(hp.cuda().view(1, 1, d), hp.cuda().view(1, 1, d), 1, 0.8, "exact", y)
+        torch.cuda.synchronize()
+    finally:
+        apex.destroy()
+    w = (synth.dequantize_store_fp4 if fp4 else synth.dequantize_store_fp8)(store, d)   # [N][I][3][d], fp64
+    h64 = hp.double().numpy()
+    g, u = w[:, :, 0] @ h64, w[:, :, 1] @ h64
+    a = g / (1.0 + np.exp(-g)) * u / cfg.k
+    return y.cpu().double().numpy().reshape(-1), np.einsum("ei,eid->d", a, w[:, :, 2])
+
+
+@pytest.mark.parametrize("d", [512, 1024, 1536, 2048])
+@pytest.mark.parametrize("spread", [15, 24, 26, 40, 70, "saturated"])
+def test_token_kernel_block_scales_that_differ_between_rows(d, spread):
+    """e2m1 rows whose downT scales lie up to 2^70 apart while their shares of y do not (the up scales lie apart the other way round):
+    a row must not be measured by another one's scale.  "saturated": a downT scale 2^26 larger where SiLU leaves next to nothing.
+    3e-5: sums of up to 2048 fp32 products, and an error of g of a few 2^-24 of its 20 in a saturated SiLU."""
+    cfg = synth.tiny_config(d=d, N=2, k=2, I=150, C=2, L=1, T=1, cfg_id=470)
+    store = synth.expert_store_fp4(cfg, 0)
+    hp = torch.randn((d,), generator=torch.Generator().manual_seed(d)).bfloat16().float()
+    o, n = 3 * (d // 2), d // 32
+    rows = store[:, 1::2]
+    if spread == "saturated":
+        rows = store[:, 1::5]
+        code = torch.where(hp < 0, 2, 10).to(torch.uint8)              # -sign(h'): every product negative
+        rows[..., :d // 2] = code[0::2] | (code[1::2] << 4)
+        rows[..., o:o + n] = 127 + int(np.floor(np.log2(32.0 / float(hp.abs().sum()))))
+        rows[..., o + 2 * n:o + 3 * n] += 26
+    else:
+        rows[..., o + n:o + 2 * n] -= spread
+        rows[..., o + 2 * n:o + 3 * n] += spread
+    y, want = _one_layer_y(cfg, store, hp, fp4=True)
+    assert np.linalg.norm(y - want) <= 3e-5 * np.linalg.norm(want), np.linalg.norm(y - want) / np.linalg.norm(want)
