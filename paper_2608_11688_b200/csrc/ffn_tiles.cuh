@@ -210,7 +210,7 @@ __device__ __forceinline__ void e2m1x8_to_f16(uint32_t v, uint32_t (&o)[4]) {
 // Activations beside them are cut into fp16 planes, three times eleven bits.  fp16's exponents do not reach far, so the values of a
 // group (a warp's columns of h', a tile's a) share a power of two that puts the largest between 2^14 and 2^15:
 //   x * up = p[0] + 2^-11 p[1] + 2^-22 p[2]
-// to the last bit of x, or to 2^-60 of the group's largest, whichever is coarser.
+// to the last bit of x where the group spans no more than 36 binades; a group that spans more is worked on in fp32.
 struct PlaneScale {
   float up, down;  // the power of two and its inverse
 };
@@ -239,10 +239,11 @@ __device__ __forceinline__ int plane_reach(uint32_t largest, uint32_t smallest) 
   return largest == 0u ? 36 : top < 77 || top > 187 ? -1 : 36 - (top - (int)(smallest >> 23));
 }
 
-// Four columns of a 32-column block of 16 rows' downT times a in fp32, a weight at a time, each scale applied to its own row: for
-// rows the planes do not hold.  at: the lane's codes of the first row's block (scale: its scale byte); a: of row lane mod 16
-// or 32; of the rows row0 .. row0 + 15 those below `here` exist.  The sums of the columns this lane group has in the
-// accumulators, in the lanes of plane 0 (zero in the others).  Out of line: it is hardly ever run.
+// What the planes do not hold is worked on in fp32, a weight at a time, by the two functions below.  Out of line: they are hardly
+// ever run.
+// Four columns of a 32-column block of 16 rows' downT times a.  at: the lane's codes of the first row's block (scale: its scale byte,
+// e2m1); a: of row lane mod 16 or 32; of the rows row0 .. row0 + 15 those below `here` exist.  The sums of the columns this lane group
+// has in the accumulators, in the lanes of plane 0 (zero in the others).
 template <int FMT>
 __device__ __noinline__ float4 down_rows_fp32(const uint8_t* at, const uint8_t* scale, uint32_t stride, float a, int row0, int here) {
   const int lane = threadIdx.x & 31;
@@ -253,8 +254,13 @@ __device__ __noinline__ float4 down_rows_fp32(const uint8_t* at, const uint8_t* 
     float ar = __shfl_sync(0xffffffffu, a, r);
     if (r < here) {
       uint32_t w[4];
-      e2m1x8_to_f16(*reinterpret_cast<const uint16_t*>(at + r * stride), w);
-      ar *= __uint_as_float((uint32_t)scale[r * stride] << 23);
+      const uint16_t* codes = reinterpret_cast<const uint16_t*>(at + r * stride);
+      if (FMT == kFmtE4m3) {
+        e4m3x4_to_f16(codes[0] | (uint32_t)codes[8] << 16, w[0], w[1]);  // (two columns of each of two 16-column steps)
+      } else {
+        e2m1x8_to_f16(codes[0], w);
+        ar *= __uint_as_float((uint32_t)scale[r * stride] << 23);
+      }
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[j]));
@@ -272,6 +278,36 @@ __device__ __noinline__ float4 down_rows_fp32(const uint8_t* at, const uint8_t* 
   return make_float4(s[0], s[1], s[2], s[3]);
 }
 
+// The warp's shares of eight rows' gate and up dot products (before the e4m3 scales), in all lanes of row lane / 4.  row: the warp's
+// gate codes of that row, vec_bytes before the up codes; scales: of its gate blocks, scale_bytes before the up ones (e2m1); h: the warp's columns.
+template <int FMT>
+__device__ __noinline__ float2 gate_up_rows_fp32(const uint8_t* row, uint32_t vec_bytes, const uint8_t* scales, uint32_t scale_bytes, const float* __restrict__ h, int blocks) {
+  const int t = threadIdx.x & 3;
+  float g = 0.f, u = 0.f;
+#pragma unroll 1
+  for (int b = 0; b < blocks; ++b) {  // eight columns of every 32
+    float gw[8], uw[8], hh[8];
+    load8<FMT>(row, b * 4 + t, gw);
+    load8<FMT>(row + vec_bytes, b * 4 + t, uw);
+    const float4 h0 = __ldg(reinterpret_cast<const float4*>(h) + (b * 4 + t) * 2), h1 = __ldg(reinterpret_cast<const float4*>(h) + (b * 4 + t) * 2 + 1);
+    hh[0] = h0.x; hh[1] = h0.y; hh[2] = h0.z; hh[3] = h0.w; hh[4] = h1.x; hh[5] = h1.y; hh[6] = h1.z; hh[7] = h1.w;
+    float pg = 0.f, pu = 0.f;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+      pg = fmaf(gw[m], hh[m], pg);
+      pu = fmaf(uw[m], hh[m], pu);
+    }
+    g = fmaf(FMT == kFmtMxfp4 ? block_scale(scales, b * 4) : 1.f, pg, g);
+    u = fmaf(FMT == kFmtMxfp4 ? block_scale(scales + scale_bytes, b * 4) : 1.f, pu, u);
+  }
+#pragma unroll
+  for (int o = 1; o < 4; o <<= 1) {
+    g += __shfl_xor_sync(0xffffffffu, g, o);
+    u += __shfl_xor_sync(0xffffffffu, u, o);
+  }
+  return make_float2(g, u);
+}
+
 // What the two quantised formats share: h' and a as fp16 planes.  K order of a step: an 8x8 matrix of ldmatrix gives a lane 4
 // consecutive bytes of a row, hence codes that follow one another, while the MMA wants columns 2t, 2t+1, 2t+8, 2t+9 in lane t:
 // h' is handed out in the order the codes arrive in, a sum does not mind.
@@ -283,6 +319,7 @@ struct QuantTiles {
   uint32_t hb[KW][2];  // h', B operand of the gate and up products
   float y[KW][4];      // accumulators of the down projection
   float h_down;        // inverse of the power of two that the warp's h' was multiplied by
+  bool h_wide;         // the warp's h' are not all held: rows times h' in fp32
 
   struct Raw {
     float v[D / 256];
@@ -295,10 +332,16 @@ struct QuantTiles {
   __device__ __forceinline__ void take_h(const Raw& raw, uint8_t* scratch, int warp, int lane) {
     constexpr int PLANE = D / 4 + 16;  // bytes
     uint8_t* mine = scratch + warp * (3 * PLANE);
-    uint32_t largest = 0u;
+    uint32_t largest = 0u, smallest = 0xffffffffu;
 #pragma unroll
-    for (int i = 0; i < D / 256; ++i) largest = max(largest, __float_as_uint(raw.v[i]) & 0x7fffffffu);
-    const PlaneScale sc = plane_scale(__reduce_max_sync(0xffffffffu, largest));
+    for (int i = 0; i < D / 256; ++i) {
+      const uint32_t bits = __float_as_uint(raw.v[i]) & 0x7fffffffu;
+      largest = max(largest, bits);
+      smallest = min(smallest, bits == 0u ? 0xffffffffu : bits);
+    }
+    largest = __reduce_max_sync(0xffffffffu, largest);
+    h_wide = plane_reach(largest, __reduce_min_sync(0xffffffffu, smallest)) < 0;
+    const PlaneScale sc = plane_scale(largest);
     h_down = sc.down;
 #pragma unroll
     for (int i = 0; i < D / 256; ++i) {
@@ -365,8 +408,14 @@ struct RowTiles<D, kFmtE4m3> : QuantTiles<D, kFmtE4m3> {
   using Base::KW;
   using Base::hb;
   using Base::y;
-  // shares of the dot products of rows' codes; see the bf16 rows.  tile: the eight rows' shared-memory address
-  __device__ __forceinline__ void gate_up(uint32_t tile, uint32_t stride, int warp, int lane, float& g, float& u) const {
+  // shares of the dot products of rows' codes; see the bf16 rows.  tile: the eight rows' shared-memory address; h: h' in global memory
+  __device__ __forceinline__ void gate_up(const uint8_t* rows, uint32_t tile, uint32_t stride, int warp, int lane, const float* __restrict__ h, int, float& g, float& u) const {
+    if (Base::h_wide) {
+      const float2 v = gate_up_rows_fp32<kFmtE4m3>(rows + (lane >> 2) * stride + warp * (D / 8), D, nullptr, 0u, h + warp * (D / 8), D / 256);
+      g = v.x;
+      u = v.y;
+      return;
+    }
     // matrices: gate rows, up rows, columns 0 .. 15 of the step, then both of the next step
     const uint32_t at = tile + (lane & 7) * stride + ((lane >> 3) & 1) * D + (lane >> 4) * 16 + warp * (D / 8);
     float sum[4] = {};
@@ -396,7 +445,22 @@ struct RowTiles<D, kFmtE4m3> : QuantTiles<D, kFmtE4m3> {
   }
   // y += downT^T a of ROWS rows, of which `here` exist
   template <int ROWS>
-  __device__ __forceinline__ void down(const uint8_t*, uint32_t tile, uint32_t stride, int warp, int lane, const uint32_t (&b)[ROWS / 8], float unit, int here, float, int) {
+  __device__ __forceinline__ void down(const uint8_t* rows, uint32_t tile, uint32_t stride, int warp, int lane, const uint32_t (&b)[ROWS / 8], float unit, int here, float a_row,
+                                       int reach) {
+    if (reach < 0) {
+#pragma unroll
+      for (int r = 0; r < ROWS; r += 16) {
+#pragma unroll
+        for (int s = 0; s < KW; s += 2) {
+          const float4 v = down_rows_fp32<kFmtE4m3>(rows + 2 * D + warp * (D / 8) + s * 16 + (lane >> 2) * 2, nullptr, stride, a_row, r, here);
+          y[s][0] += v.x;
+          y[s][2] += v.y;
+          y[s + 1][0] += v.z;
+          y[s + 1][2] += v.w;
+        }
+      }
+      return;
+    }
     constexpr bool PAIR = ROWS >= 16;  // two 8-row blocks to an MMA
     // matrices: 8-row blocks 0 and 1 of a step, both of the next one | four steps of a block
     const uint32_t at = tile + (lane & 7) * stride + 2 * D + warp * (D / 8) +
@@ -466,13 +530,25 @@ struct RowTiles<D, kFmtMxfp4> : QuantTiles<D, kFmtMxfp4> {
   }
   __device__ __forceinline__ static uint32_t byte_of(const uint32_t (&sc)[SW], int i) { return __byte_perm(sc[i / 4], 0u, 0x4440 | (i & 3)); }
 
-  __device__ __forceinline__ void gate_up(uint32_t tile, uint32_t stride, int warp, int lane, float& g, float& u) const {
+  __device__ __forceinline__ void gate_up(const uint8_t* rows, uint32_t tile, uint32_t stride, int warp, int lane, const float* __restrict__ h, int here, float& g, float& u) const {
     // matrices: gate rows, up rows of a block, then both of the next block
     const uint32_t at = tile + (lane & 7) * stride + ((lane >> 3) & 1) * (D / 2) + (lane >> 4) * 16 + warp * (D / 16);
     const uint32_t scales = tile + (lane >> 2) * stride + 3 * (D / 2) + warp * KB;
     uint32_t sg[SW], su[SW];
     load_scales(scales, sg);
     load_scales(scales + D / 32, su);
+    // Scales between 2^-63 and 2^64 (and zero) leave the planes' sums inside fp32's exponents; each lane of a row
+    // (of the `here` that exist) looks at one word of them
+    const uint32_t w = (lane & 1) ? ((lane & 2) ? su[SW - 1] : su[0]) : ((lane & 2) ? sg[SW - 1] : sg[0]);
+    const uint32_t some = ((w & 0x3f3f3f3fu) + 0x3f3f3f3fu) << 1;  // bit 7 of a byte: its lower six bits are not zero; of w << 1: its bit 6
+    const bool far = (lane >> 2) < here && (((some & ~(w | w << 1)) | (w & w << 1)) & 0x80808080u) != 0u;
+    if (__any_sync(0xffffffffu, Base::h_wide || far)) {
+      const uint8_t* row = rows + (lane >> 2) * stride;
+      const float2 v = gate_up_rows_fp32<kFmtMxfp4>(row + warp * (D / 16), D / 2, row + 3 * (D / 2) + warp * KB, D / 32, h + warp * (D / 8), KB);
+      g = v.x;
+      u = v.y;
+      return;
+    }
     float sum[4] = {};
 #pragma unroll
     for (int b = 0; b < KB; b += 2) {

@@ -836,7 +836,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) decode_tiles_kernel(const Dec
               for (int r = 0; r < R; ++r) {
                 float g, u;
                 if constexpr (FMT == kFmtBf16) rt.gate_up(tile + (lane & 7) * stride + r * 8 * stride, warp, lane, g, u);
-                else rt.gate_up(tile + r * 8 * stride, stride, warp, lane, g, u);
+                else rt.gate_up(smem + s * tile_bytes + r * 8 * stride, tile + r * 8 * stride, stride, warp, lane, hpl, here - r * 8, g, u);
                 if ((lane & 3) == 0) *reinterpret_cast<float2*>(part + (r * 8 + (lane >> 2)) * kPartStride + 2 * warp) = make_float2(g, u);
               }
             }

@@ -396,3 +396,42 @@ def test_token_kernel_block_scales_that_differ_between_rows(d, spread):
         rows[..., o + 2 * n:o + 3 * n] += spread
     y, want = _one_layer_y(cfg, store, hp, fp4=True)
     assert np.linalg.norm(y - want) <= 3e-5 * np.linalg.norm(want), np.linalg.norm(y - want) / np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("fmt", ["fp8", "fp4"])
+@pytest.mark.parametrize("d", [512, 1024, 1536, 2048])
+@pytest.mark.parametrize("what", ["h", "a"])
+def test_token_kernel_values_far_below_the_largest_of_their_group(d, what, fmt):
+    """The warp's columns of h', a tile's gated intermediate: what lies 2^50 below the largest of its group keeps its 24 bits.  h: the
+    odd columns, and all that gate and up look at, are the small ones.  a: the odd rows, which alone make the odd columns of y.
+    (3e-5: sums of up to 2048 fp32 products.)"""
+    cfg = synth.tiny_config(d=d, N=2, k=2, I=150, C=2, L=1, T=1, cfg_id=471)
+    store = (synth.expert_store_fp4 if fmt == "fp4" else synth.expert_store_fp8)(cfg, 0)
+    hp = torch.randn((d,), generator=torch.Generator().manual_seed(d)).bfloat16().float()
+    vec = d // 2 if fmt == "fp4" else d
+
+    def scale(rows, v, by):                                        # v: 0 gate, 1 up, 2 downT
+        if fmt == "fp4":
+            rows[..., 3 * vec + v * (d // 32):3 * vec + (v + 1) * (d // 32)] += by
+        else:
+            rows[..., 3 * vec + 4 * v:3 * vec + 4 * v + 4] = (rows[..., 3 * vec + 4 * v:3 * vec + 4 * v + 4].contiguous().view(torch.float32) * 2.0 ** by).view(torch.uint8)
+
+    def drop(rows, v, odd):                                        # zero codes in the odd or the even columns
+        codes = rows[..., v * vec:(v + 1) * vec]
+        if fmt == "fp4":
+            codes &= 0x0F if odd else 0xF0
+        else:
+            codes[..., int(odd)::2] = 0
+
+    if what == "h":
+        hp[1::2] *= 2.0 ** -50
+        for v in (0, 1):
+            scale(store, v, 50)
+            drop(store, v, odd=False)
+    else:
+        scale(store[:, 1::2], 1, -50)
+        drop(store[:, 1::2], 2, odd=False)
+        drop(store[:, 0::2], 2, odd=True)
+    y, want = _one_layer_y(cfg, store, hp, fp4=fmt == "fp4")
+    for part in (slice(0, None, 2), slice(1, None, 2)):
+        assert np.linalg.norm(y[part] - want[part]) <= 3e-5 * np.linalg.norm(want[part]), np.linalg.norm(y[part] - want[part]) / np.linalg.norm(want[part])
