@@ -316,7 +316,7 @@ int apex_route_topk_static(const float* W_r_dev, const float* b_r_dev, const flo
  *   descending order); dstar_dev [T] int32 (device): its oracle budget delta* (Eq. (3)), 0 <= delta* <= N-k.
  *   w_host [N], theta_host [N-k+1] (host, fp32): the fitted parameters, theta made monotone again after
  *   the rounding to fp32 -- ready for apex_set_cdf.
- * Context-free; allocates and frees its own scratch; synchronises `stream` before it returns.
+ * Context-free; scratch: see apex_trim_scratch; synchronises `stream` before it returns.
  * N <= APEX_MAX_EXPERTS.  err (optional) receives a text on failure.  Returns APEX_OK, APEX_EINVAL,
  * APEX_ENOMEM or APEX_ECUDA. */
 int apex_fit_cdf(const double* X_dev, const int32_t* dstar_dev, int T, int N, int k, int iters, double lr,
@@ -330,10 +330,16 @@ int apex_fit_cdf(const double* X_dev, const int32_t* dstar_dev, int T, int N, in
  *   alpha output of apex_route_topk.
  *   W_host [N][d], b_host [N] (host, fp32): in: the starting point; out: the trained parameters, ready for
  *   apex_set_prefetch_router.
- * Context-free; allocates and frees its own scratch; synchronises `stream` before it returns.
+ * Context-free; scratch: see apex_trim_scratch; synchronises `stream` before it returns.
  * N <= APEX_MAX_EXPERTS.  Returns APEX_OK, APEX_EINVAL, APEX_ENOMEM or APEX_ECUDA. */
 int apex_distill_router(const float* H_dev, const float* Qr_dev, int T, int N, int d, int iters, double lr,
                         float* W_host, float* b_host, void* stream, char* err, size_t err_len);
+
+/* The two training calls above take their device scratch from a pool of the library and give it back before they return.
+ * Of what it was given the pool keeps up to 64 MB per device for the next call; creating or destroying a context on the device, and this
+ * call, hand that back to the system (of the current device; scratch of a call that is running stays).  Returns APEX_OK or
+ * APEX_ECUDA. */
+int apex_trim_scratch(void);
 
 /* ---- host-only slot planner (the state machine behind apex_prefetch / apex_moe_ffn) -------- */
 

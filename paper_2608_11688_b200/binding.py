@@ -93,6 +93,7 @@ SIGNATURES = {
     "apex_route_topk_static": (_I, [_P, _P, _P, _I, _I, _I, _I, _P, _P, _P, C.c_char_p, C.c_size_t]),
     "apex_fit_cdf": (_I, [_P, _P, _I, _I, _I, _I, C.c_double, _P, _P, _P, C.c_char_p, C.c_size_t]),
     "apex_distill_router": (_I, [_P, _P, _I, _I, _I, _I, C.c_double, _P, _P, _P, C.c_char_p, C.c_size_t]),
+    "apex_trim_scratch": (_I, []),
     "apex_slots_create": (_P, [_I, _I, _I]),
     "apex_slots_destroy": (None, [_P]),
     "apex_slots_begin_step": (_I, [_P]),
@@ -429,6 +430,13 @@ def distill_router(H_dev, Qr_dev, W0, b0, iters=200, lr=0.01, stream=None):
     if rc != APEX_OK:
         raise ApexError(rc, err.value.decode())
     return W, b
+
+
+def trim_scratch():
+    """apex_trim_scratch: the scratch memory that the training calls' pool keeps on the current device goes back to the system."""
+    rc = load_library().apex_trim_scratch()
+    if rc != APEX_OK:
+        raise ApexError(rc, "apex_trim_scratch")
 
 
 class Slots:

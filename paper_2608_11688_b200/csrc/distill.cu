@@ -533,13 +533,13 @@ extern "C" int apex_distill_router(const float* H_dev, const float* Qr_dev, int 
   if (e == cudaSuccess) e = cudaMemcpyAsync(host.data(), io, n_io * sizeof(float), cudaMemcpyDeviceToHost, cs);
   int status = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&status, p.status, sizeof(int), cudaMemcpyDeviceToHost, cs);
-  const cudaError_t e2 = cudaStreamSynchronize(cs);  // also after an error: nothing may still use the buffer
+  apex::workspace_free(buf, cs);                     // (in front of the synchronisation, at which the pool lets go of what it need not keep)
+  const cudaError_t e2 = cudaStreamSynchronize(cs);  // also after an error
   if (e == cudaSuccess) e = e2;
   if (e == cudaSuccess && status == 0) {
     for (size_t i = 0; i < (size_t)N * d; ++i) W_host[i] = host[i];
     for (int i = 0; i < N; ++i) b_host[i] = host[(size_t)N * d + i];
   }
-  apex::workspace_free(buf, cs);
   if (e != cudaSuccess) {
     say(err, err_len, cudaGetErrorString(e));
     return APEX_ECUDA;

@@ -446,6 +446,8 @@ extern "C" int apex_fit_cdf(const double* X_dev, const int32_t* dstar_dev, int T
     if ((e = cudaMemcpyAsync(out.data(), p.out, sizeof(double) * P, cudaMemcpyDeviceToHost, cs)) != cudaSuccess) { fail(e); break; }
     int status = 0;
     if ((e = cudaMemcpyAsync(&status, p.status, sizeof(int), cudaMemcpyDeviceToHost, cs)) != cudaSuccess) { fail(e); break; }
+    apex::workspace_free(buf, cs);  // (in front of the synchronisation, at which the pool lets go of what it need not keep)
+    buf = nullptr;
     if ((e = cudaStreamSynchronize(cs)) != cudaSuccess) { fail(e); break; }
     if (status != 0) {
       say(err, err_len, "apex_fit_cdf: a device-side wait ran out");
@@ -460,6 +462,9 @@ extern "C" int apex_fit_cdf(const double* X_dev, const int32_t* dstar_dev, int T
       theta_host[j] = run;
     }
   } while (false);
-  apex::workspace_free(buf, cs);
+  if (buf) {
+    apex::workspace_free(buf, cs);
+    cudaStreamSynchronize(cs);
+  }
   return rc;
 }

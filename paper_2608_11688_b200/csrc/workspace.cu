@@ -50,9 +50,12 @@ void workspace_free(void* p, cudaStream_t s) {
   if (p) cudaFreeAsync(p, s);
 }
 
-void workspace_trim() {
+cudaError_t workspace_trim() {
   cudaMemPool_t pool = nullptr;
-  if (pool_of_device(false, &pool) == cudaSuccess && pool) cudaMemPoolTrimTo(pool, 0);
+  const cudaError_t e = pool_of_device(false, &pool);
+  return e == cudaSuccess && pool ? cudaMemPoolTrimTo(pool, 0) : e;
 }
 
 }  // namespace apex
+
+extern "C" int apex_trim_scratch(void) { return apex::workspace_trim() == cudaSuccess ? APEX_OK : APEX_ECUDA; }

@@ -150,3 +150,22 @@ def test_training_calls_from_two_threads_share_the_workspace_pool():
         for r in range(6):
             for a, b in zip(got[i][r], alone[(i + r) % 2]):
                 np.testing.assert_array_equal(a, b)
+
+
+def test_training_scratch_goes_back():
+    """More than half a GB of scratch: at most 64 MB of it are kept when the call returns, and none after the trim."""
+    build.build()
+    H, Qr = torch.randn((1_000_000, 64), device="cuda"), torch.full((1_000_000, 64), 1.0 / 64, device="cuda")
+    W0, b0 = np.zeros((64, 64), np.float32), np.zeros(64, np.float32)
+    X, dstar = torch.softmax(torch.randn((500, 9), device="cuda", dtype=torch.float64), 1).sort(1, descending=True)[0].contiguous(), torch.zeros(500, dtype=torch.int32, device="cuda")
+    binding.distill_router(H[:1000], Qr[:1000], W0, b0, iters=1)      # (modules and the pool itself are there from here on)
+    binding.fit_cdf(X, dstar, 2, iters=2)
+    torch.cuda.synchronize()
+    binding.trim_scratch()
+    free = torch.cuda.mem_get_info()[0]
+    binding.distill_router(H, Qr, W0, b0, iters=1)
+    assert free - torch.cuda.mem_get_info()[0] <= 64 << 20
+    binding.fit_cdf(X, dstar, 2, iters=2)
+    assert free - torch.cuda.mem_get_info()[0] <= 64 << 20
+    binding.trim_scratch()
+    assert torch.cuda.mem_get_info()[0] == free
