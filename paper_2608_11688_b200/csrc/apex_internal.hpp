@@ -26,9 +26,11 @@ __device__ __forceinline__ unsigned long long span_now() {
   return t;
 }
 #define SPAN_BEGIN() const unsigned long long _span_t0 = span_now()
-#define SPAN_END(id)                                                                     \
+#define SPAN_END(id) SPAN_END_OF(id, 0)
+// (of the first block whose y is the given one: a launch of two roles logs both)
+#define SPAN_END_OF(id, by)                                                              \
   do {                                                                                   \
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {                         \
+    if (blockIdx.x == 0 && blockIdx.y == (unsigned)(by) && threadIdx.x == 0) {             \
       const unsigned long long _i = atomicAdd(&apex::g_spans.n, 1ull) & 4095ull;         \
       apex::g_spans.rec[_i][0] = (id);                                                   \
       apex::g_spans.rec[_i][1] = _span_t0;                                               \
@@ -38,6 +40,7 @@ __device__ __forceinline__ unsigned long long span_now() {
 #else
 #define SPAN_BEGIN() do { } while (0)
 #define SPAN_END(id) do { } while (0)
+#define SPAN_END_OF(id, by) do { } while (0)
 #endif
 
 // ---- mapped host mailbox: the kernels post small decision records here so that the host can

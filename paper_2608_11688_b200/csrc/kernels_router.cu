@@ -192,6 +192,7 @@ __global__ void __launch_bounds__(kRouterWarps * 32, 2) router_batched_kernel(co
     pdl_launch_dependents();
     attn_stream(p.attn, reinterpret_cast<uint8_t*>(tiles) + warp * kAttnChunk, &s_attn[warp], warp, lane, ((int)blockIdx.y - groups) * (int)csize + (int)crank,
                 ((int)gridDim.y - groups) * (int)csize);
+    SPAN_END_OF(3, groups);
     return;
   }
   if (threadIdx.x == 0) {

@@ -2,7 +2,8 @@
 
 A second build of the library (``build.build_trace()`` -> ``libapex_trace.so``: the same sources with
 ``-DAPEX_TIMELINE``) makes every kernel record, for its first block, a kernel id and the ``%globaltimer`` values at
-entry and at exit in a device-side log of 4096 records; the streaming expert-FFN kernel also stamps the phases of
+entry and at exit in a device-side log of 4096 records (the launch that streams the attention stand-in beside a batch's
+prefetch routers: one record for either); the streaming expert-FFN kernel also stamps the phases of
 every CTA.  The product library carries none of this.  Because a process can hold only one of the two libraries,
 ``use_trace_library()`` must be called before the first context is created.
 

@@ -84,6 +84,17 @@ def test_traced_decode_records_every_kernel_in_order():
 
 
 @pytest.mark.gpu
+def test_traced_batched_decode_records_the_standin_beside_the_routers():
+    r = subprocess.run([sys.executable, "bench.py", "--trace", "--config", "4", "--layers", "2", "--batch", "32", "--resident", "--warmup", "3"],
+                       cwd=ROOT, capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stderr[-2000:]
+    line = json.loads([l for l in r.stdout.splitlines() if l.startswith("{")][-1])
+    t, n = line["trace"], line["tokens_traced"] * line["layers"]
+    for kid in (1, 3, 4, 8):
+        assert t[trace.KERNEL_NAMES[kid]]["launches"] == n, t
+
+
+@pytest.mark.gpu
 def test_bench_line_carries_the_contract_keys():
     sys.path.insert(0, os.path.join(ROOT, "tests"))
     import harness
