@@ -363,6 +363,11 @@ def time_ffn_kernel(apex, cfg, h, hp, B, tokens):
     return statistics.mean(per_launch) * 1e-3, statistics.median(per_launch) * 1e-3, len(per_launch) * cfg.L
 
 
+def token_kernel_name(cfg):
+    """The kernel that runs a batch-1 token of this width (rows up to d = 2048 in tiles)."""
+    return "decode_tiles_kernel" if cfg.d <= 2048 else "decode_token_kernel"
+
+
 def time_token_kernel(cfg, prob, h, hp, y, tokens, standin):
     """Average device time of one launch of the persistent token kernel (all L layer-steps of a token: prefetch
     router, budget, gate, expert FFN, hand-over between layers), all experts resident, CUDA events on the launching
@@ -431,7 +436,7 @@ def other_config_rooflines(dev, peak, peak_kind):
                 if per_token == 1.0:
                     bytes_step, _ = algorithmic_bytes(cfg, 1)
                     bt = cfg.L * (bytes_step + cfg.d * 4)
-                    rec["decode_token_kernel"] = {"us_per_layer_step": sec_tok * 1e6 / cfg.L, "achieved": bt / sec_tok / 1e9,
+                    rec["token_kernel"] = {"kernel": token_kernel_name(cfg), "us_per_layer_step": sec_tok * 1e6 / cfg.L, "achieved": bt / sec_tok / 1e9,
                                                   "frac": bt / sec_tok / 1e9 / peak, "algorithmic_bytes_per_launch": bt}
             out[f"config{cfg_id}" + (f"_B{B}" if len(batches) > 1 else "")] = rec
             del h, hp
@@ -761,7 +766,7 @@ def main():
                     ach = bytes_tok / sec_tok / 1e9
                     sec_att, _ = time_token_kernel(cfg, prob, h_dev, hp_dev, y_dev, n_tok, standin=True)
                     attn_bytes = (4 * cfg.d * cfg.d + 2 * 1024 * cfg.d) * 2
-                    roof = {"bound": "hbm", "kernel": "decode_token_kernel", "achieved": ach, "peak": peak, "unit": "GB/s",
+                    roof = {"bound": "hbm", "kernel": token_kernel_name(cfg), "achieved": ach, "peak": peak, "unit": "GB/s",
                             "frac": ach / peak, "peak_kind": f"of {peak_kind}", "frac_of_8TBs": ach / NOMINAL_HBM_GBS,
                             "traffic": None, "algorithmic_bytes_per_launch": bytes_tok, "us_per_launch_mean": sec_tok * 1e6,
                             "us_per_layer_step": sec_tok * 1e6 / cfg.L, "launches_timed": n_tok,

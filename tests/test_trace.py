@@ -116,7 +116,7 @@ def test_bench_line_carries_the_contract_keys():
     e = d["e2e"]
     assert 5.0 < e["value"] < 1000.0 and e["h2d_bytes_per_step"] == 2 * 32 * 1536 * 4 and e["d2h_bytes_per_step"] == 32 * 1536 * 4
     rf = d["roofline"]
-    assert rf["bound"] == "hbm" and rf["kernel"] == "decode_token_kernel" and rf["unit"] == "GB/s"
+    assert rf["bound"] == "hbm" and rf["kernel"] == "decode_tiles_kernel" and rf["unit"] == "GB/s"
     assert abs(rf["frac"] - rf["achieved"] / rf["peak"]) < 1e-9 and 0.05 < rf["frac"] < 1.2 and "traffic" in rf
     assert rf["per_layer_ffn_kernel_alone"]["kernel"] == "moe_ffn_stream_kernel" and rf["per_layer_ffn_kernel_alone"]["traffic"] > 3.7e7
     c = d["cpu_baseline"]
