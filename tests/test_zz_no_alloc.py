@@ -176,7 +176,13 @@ def test_ranking_with_and_without_ties(N, B, kind):
     got, a = idx.cpu().numpy(), alpha.cpu().numpy()
     for b in range(B):
         if kind == "nan":      # a NaN is ordered before nobody and after nobody: it shares the first place
-            assert np.isnan(a[b]).any() and (got[b] < N).all()
+            assert np.isnan(a[b]).any()
+            z = W.astype(np.float64) @ hp[b].astype(np.float64) + bias
+            claims = [[] for _ in range(N)]
+            for e in range(N):
+                claims[sum(int(z[f] > z[e] or (z[f] == z[e] and f < e)) for f in range(N))].append(e)
+            for r in range(k):     # a place that several claim holds one of them, a place that nobody claims is not written
+                assert got[b][r] in (claims[r] or [-1]), (b, r, got[b][r], claims[r])
             continue
         z = W.astype(np.float64) @ hp[b].astype(np.float64)
         want = sorted(range(N), key=lambda e: (-z[e], e))[:k]      # (random rows: gaps far above fp32 rounding)
