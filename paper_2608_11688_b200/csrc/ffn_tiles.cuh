@@ -190,11 +190,6 @@ __device__ __forceinline__ void mma_f16_k16(float (&c)[4], uint32_t a0, uint32_t
       : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
 }
-__device__ __forceinline__ void mma_f16_k8(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t b0) {
-  asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5}, {%6}, {%7, %7, %7, %7};"
-      : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
-      : "r"(a0), "r"(a1), "r"(b0), "f"(0.f));
-}
 // the lower and the upper two of four e4m3 codes
 __device__ __forceinline__ void e4m3x4_to_f16(uint32_t v, uint32_t& lo, uint32_t& hi) {
   asm("{\n.reg .b16 l, h;\nmov.b32 {l, h}, %2;\ncvt.rn.f16x2.e4m3x2 %0, l;\ncvt.rn.f16x2.e4m3x2 %1, h;\n}" : "=r"(lo), "=r"(hi) : "r"(v));
@@ -447,6 +442,7 @@ struct RowTiles<D, kFmtE4m3> : QuantTiles<D, kFmtE4m3> {
   template <int ROWS>
   __device__ __forceinline__ void down(const uint8_t* rows, uint32_t tile, uint32_t stride, int warp, int lane, const uint32_t (&b)[ROWS / 8], float unit, int here, float a_row,
                                        int reach) {
+    static_assert(ROWS % 16 == 0, "two 8-row blocks to an MMA");
     if (reach < 0) {
 #pragma unroll
       for (int r = 0; r < ROWS; r += 16) {
@@ -461,12 +457,10 @@ struct RowTiles<D, kFmtE4m3> : QuantTiles<D, kFmtE4m3> {
       }
       return;
     }
-    constexpr bool PAIR = ROWS >= 16;  // two 8-row blocks to an MMA
-    // matrices: 8-row blocks 0 and 1 of a step, both of the next one | four steps of a block
-    const uint32_t at = tile + (lane & 7) * stride + 2 * D + warp * (D / 8) +
-                        (PAIR ? ((lane >> 3) & 1) * 8 * stride + (lane >> 4) * 16 : (lane >> 3) * 16);
+    // matrices: 8-row blocks 0 and 1 of a step, both of the next one
+    const uint32_t at = tile + ((lane & 7) + ((lane >> 3) & 1) * 8) * stride + 2 * D + warp * (D / 8) + (lane >> 4) * 16;
 #pragma unroll
-    for (int r = 0; r < ROWS / 8; r += PAIR ? 2 : 1) {
+    for (int r = 0; r < ROWS / 8; r += 2) {
       uint32_t keep[2];
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
@@ -474,22 +468,21 @@ struct RowTiles<D, kFmtE4m3> : QuantTiles<D, kFmtE4m3> {
         keep[i] = left >= 2 ? 0xffffffffu : left == 1 ? 0xffffu : 0u;
       }
 #pragma unroll
-      for (int s = 0; s < KW; s += PAIR ? 2 : 4) {
+      for (int s = 0; s < KW; s += 2) {
         uint32_t v[4];
         ldsm4_t(v, at + r * 8 * stride + s * 16);
         if (here != ROWS) {  // (what lies behind the rows may be a NaN's code)
 #pragma unroll
-          for (int i = 0; i < 4; ++i) v[i] &= keep[PAIR ? i & 1 : 0];
+          for (int i = 0; i < 4; ++i) v[i] &= keep[i & 1];
         }
         // a register: columns 2g, 2g+1 of row 2t, then of row 2t+1.  As MMA rows: g column 2g, g + 8 column 2g+1
         uint32_t a[4][2];
 #pragma unroll
         for (int i = 0; i < 4; ++i) e4m3x4_to_f16(__byte_perm(v[i], 0u, 0x3120), a[i][0], a[i][1]);
 #pragma unroll
-        for (int j = 0; j < (PAIR ? 2 : 4); ++j) {
+        for (int j = 0; j < 2; ++j) {
           float c[4];
-          if (PAIR) mma_f16_k16(c, a[2 * j][0], a[2 * j][1], a[(2 * j + 1) & 3][0], a[(2 * j + 1) & 3][1], b[r], b[PAIR ? r + 1 : r]);
-          else mma_f16_k8(c, a[j][0], a[j][1], b[r]);
+          mma_f16_k16(c, a[2 * j][0], a[2 * j][1], a[2 * j + 1][0], a[2 * j + 1][1], b[r], b[r + 1]);
 #pragma unroll
           for (int i = 0; i < 4; ++i) y[s + j][i] = fmaf(c[i], unit, y[s + j][i]);
         }
@@ -583,18 +576,15 @@ struct RowTiles<D, kFmtMxfp4> : QuantTiles<D, kFmtMxfp4> {
   __device__ __forceinline__ void down(const uint8_t* rows, uint32_t tile, uint32_t stride, int warp, int lane, const uint32_t (&b)[ROWS / 8], float unit, int here, float a,
                                        int reach) {
     static_assert(ROWS % 16 == 0, "two 8-row blocks to an MMA");
-    constexpr bool PAIR = ROWS >= 16;
-    constexpr int RB = PAIR ? 2 : 1;  // 8-row blocks to an MMA
-    const uint32_t at = tile + (lane & 7) * stride + D + warp * (D / 16) +
-                        (PAIR ? ((lane >> 3) & 1) * 8 * stride + (lane >> 4) * 16 : (lane >> 3) * 16);
+    const uint32_t at = tile + ((lane & 7) + ((lane >> 3) & 1) * 8) * stride + D + warp * (D / 16) + (lane >> 4) * 16;
     // lane 4 b + t works out the scales of block b in the rows 2t, 2t+1 of each 8-row block, and passes them on (every lane for
     // itself and all blocks: 60 instructions per block instead of 5)
     const uint32_t scales = tile + 2 * (lane & 3) * stride + 3 * (D / 2) + 2 * (D / 32) + warp * KB + min(lane >> 2, KB - 1);
 #pragma unroll
-    for (int r = 0; r < ROWS / 8; r += RB) {
-      uint32_t sc[2 * RB], top = 0u, e[RB];
+    for (int r = 0; r < ROWS / 8; r += 2) {
+      uint32_t sc[4], top = 0u, e[2];
 #pragma unroll
-      for (int i = 0; i < 2 * RB; ++i) {
+      for (int i = 0; i < 4; ++i) {
         const int row = (r + (i >> 1)) * 8 + (i & 1);
         asm volatile("ld.shared.u8 %0, [%1];" : "=r"(sc[i]) : "r"(scales + row * stride) : "memory");
         sc[i] = row + 2 * (lane & 3) < here ? sc[i] : 0u;
@@ -604,7 +594,7 @@ struct RowTiles<D, kFmtMxfp4> : QuantTiles<D, kFmtMxfp4> {
       top = max(top, __shfl_xor_sync(0xffffffffu, top, 2));
       bool wide = false;
 #pragma unroll
-      for (int i = 0; i < 2 * RB; ++i) wide = wide || (sc[i] != 0u && ((int)(top - sc[i]) > reach - 8 || sc[i] - 64u > 127u));
+      for (int i = 0; i < 4; ++i) wide = wide || (sc[i] != 0u && ((int)(top - sc[i]) > reach - 8 || sc[i] - 64u > 127u));
       if (__any_sync(0xffffffffu, wide)) {
         const uint8_t* codes = rows + D + warp * (D / 16) + (lane >> 2) * 2;
 #pragma unroll
@@ -618,7 +608,7 @@ struct RowTiles<D, kFmtMxfp4> : QuantTiles<D, kFmtMxfp4> {
         continue;
       }
 #pragma unroll
-      for (int i = 0; i < 2 * RB; ++i) {
+      for (int i = 0; i < 4; ++i) {
         // 2^-k in fp16, a subnormal from 15 on, zero from 25 on; a scale of zero is zero
         const uint32_t k = top - sc[i];
         const uint32_t v = sc[i] == 0u ? 0u : k < 15u ? (15u - k) << 10 : 0x400u >> min(k - 14u, 31u);
@@ -626,35 +616,31 @@ struct RowTiles<D, kFmtMxfp4> : QuantTiles<D, kFmtMxfp4> {
         else e[i >> 1] = v;
       }
       const float back = __uint_as_float(top << 23) * unit;
-      constexpr int STEP = PAIR || KB < 4 ? 2 : 4;  // blocks per load of four matrices (two of them unused where KB = 2 and 8 rows)
 #pragma unroll
-      for (int b0 = 0; b0 < KB; b0 += STEP) {
+      for (int b0 = 0; b0 < KB; b0 += 2) {  // blocks
         uint32_t v[4];
         ldsm4_t(v, at + r * 8 * stride + b0 * 16);
 #pragma unroll
-        for (int j = 0; j < STEP; ++j) {
+        for (int j = 0; j < 2; ++j) {
           const int blk = b0 + j;
-          if (blk < KB) {
-            uint32_t bs[RB], a[RB][4];
+          uint32_t bs[2], a[2][4];
 #pragma unroll
-            for (int i = 0; i < RB; ++i) {
-              const uint32_t es = __shfl_sync(0xffffffffu, e[i], blk * 4 + (lane & 3));
-              const __half2 t = __hmul2(*reinterpret_cast<const __half2*>(&b[r + i]), *reinterpret_cast<const __half2*>(&es));
-              bs[i] = *reinterpret_cast<const uint32_t*>(&t);
-              // a register: columns 4g .. 4g+3 of row 2t, then of row 2t+1, a nibble each: brought together by column
-              const uint32_t m = __byte_perm(v[PAIR ? 2 * j + i : j], 0u, 0x3120);
-              const uint32_t swap = (m ^ (m >> 4)) & 0x00f000f0u;
-              e2m1x8_to_f16(m ^ swap ^ (swap << 4), a[i]);
-            }
-            const float f = __shfl_sync(0xffffffffu, back, blk * 4);
+          for (int i = 0; i < 2; ++i) {
+            const uint32_t es = __shfl_sync(0xffffffffu, e[i], blk * 4 + (lane & 3));
+            const __half2 t = __hmul2(*reinterpret_cast<const __half2*>(&b[r + i]), *reinterpret_cast<const __half2*>(&es));
+            bs[i] = *reinterpret_cast<const uint32_t*>(&t);
+            // a register: columns 4g .. 4g+3 of row 2t, then of row 2t+1, a nibble each: brought together by column
+            const uint32_t m = __byte_perm(v[2 * j + i], 0u, 0x3120);
+            const uint32_t swap = (m ^ (m >> 4)) & 0x00f000f0u;
+            e2m1x8_to_f16(m ^ swap ^ (swap << 4), a[i]);
+          }
+          const float f = __shfl_sync(0xffffffffu, back, blk * 4);
 #pragma unroll
-            for (int t = 0; t < 2; ++t) {  // columns 4g and 4g+1, then 4g+2 and 4g+3
-              float c[4];
-              if (PAIR) mma_f16_k16(c, a[0][2 * t], a[0][2 * t + 1], a[RB - 1][2 * t], a[RB - 1][2 * t + 1], bs[0], bs[RB - 1]);
-              else mma_f16_k8(c, a[0][2 * t], a[0][2 * t + 1], bs[0]);
+          for (int t = 0; t < 2; ++t) {  // columns 4g and 4g+1, then 4g+2 and 4g+3
+            float c[4];
+            mma_f16_k16(c, a[0][2 * t], a[0][2 * t + 1], a[1][2 * t], a[1][2 * t + 1], bs[0], bs[1]);
 #pragma unroll
-              for (int i = 0; i < 4; ++i) y[2 * blk + t][i] = fmaf(c[i], f, y[2 * blk + t][i]);
-            }
+            for (int i = 0; i < 4; ++i) y[2 * blk + t][i] = fmaf(c[i], f, y[2 * blk + t][i]);
           }
         }
       }

@@ -97,8 +97,9 @@ def test_distillation_reports_a_wait_that_ran_out():
 
 @pytest.mark.parametrize("T,N,d,iters", [
     (2369, 12, 128, 3),    # three warps of tokens per forward CTA; 19 segments of two stages, the last one of a token
-    (4737, 20, 64, 3),     # five; one column tile, 37 segments
-    (7104, 8, 256, 3),     # six; 28 segments of four stages
+    (4737, 20, 64, 3),     # five; one column tile, 25 segments of three stages
+    (2368, 20, 64, 3),     # two; one column tile, 37 segments of one stage: the most there are
+    (7104, 8, 256, 3),     # six; four column tiles, 37 segments of three stages
     (769, 40, 64, 3),      # thirteen segments of one stage: one more than the short sum of the step takes
     (768, 40, 64, 3),      # twelve
 ])
