@@ -194,7 +194,11 @@ __device__ __forceinline__ void mma_f16_k16(float (&c)[4], uint32_t a0, uint32_t
 __device__ __forceinline__ void e4m3x4_to_f16(uint32_t v, uint32_t& lo, uint32_t& hi) {
   asm("{\n.reg .b16 l, h;\nmov.b32 {l, h}, %2;\ncvt.rn.f16x2.e4m3x2 %0, l;\ncvt.rn.f16x2.e4m3x2 %1, h;\n}" : "=r"(lo), "=r"(hi) : "r"(v));
 }
-// eight e2m1 codes, two to a byte
+// four e2m1 codes, two to a byte
+__device__ __forceinline__ void e2m1x4_to_f16(uint16_t v, uint32_t& lo, uint32_t& hi) {
+  asm("{\n.reg .b8 l, h;\nmov.b16 {l, h}, %2;\ncvt.rn.f16x2.e2m1x2 %0, l;\ncvt.rn.f16x2.e2m1x2 %1, h;\n}" : "=r"(lo), "=r"(hi) : "h"(v));
+}
+// eight of them; for whole words (a zero-extended half word gave zeroes for all four in down_rows_fp32, nvcc 12.9)
 __device__ __forceinline__ void e2m1x8_to_f16(uint32_t v, uint32_t (&o)[4]) {
   asm("{\n.reg .b8 b0, b1, b2, b3;\nmov.b32 {b0, b1, b2, b3}, %4;\ncvt.rn.f16x2.e2m1x2 %0, b0;\ncvt.rn.f16x2.e2m1x2 %1, b1;\n"
       "cvt.rn.f16x2.e2m1x2 %2, b2;\ncvt.rn.f16x2.e2m1x2 %3, b3;\n}"
@@ -248,12 +252,12 @@ __device__ __noinline__ float4 down_rows_fp32(const uint8_t* at, const uint8_t* 
     const int r = row0 + 4 * i + (lane & 3);
     float ar = __shfl_sync(0xffffffffu, a, r);
     if (r < here) {
-      uint32_t w[4];
+      uint32_t w[2];
       const uint16_t* codes = reinterpret_cast<const uint16_t*>(at + r * stride);
       if (FMT == kFmtE4m3) {
         e4m3x4_to_f16(codes[0] | (uint32_t)codes[8] << 16, w[0], w[1]);  // (two columns of each of two 16-column steps)
       } else {
-        e2m1x8_to_f16(codes[0], w);
+        e2m1x4_to_f16(codes[0], w[0], w[1]);
         ar *= __uint_as_float((uint32_t)scale[r * stride] << 23);
       }
 #pragma unroll

@@ -10,7 +10,8 @@
 // The workers take the router logits and the tiles, and nothing else: with every warp planning for itself and requesting its own
 // rows, a tile's chain was 2 400 cycles instead of 2 100, the first request came 1 us later, and the kernel's state did not
 // fit its registers.  The group of four gives registers to the workers (setmaxnreg); without that 400 bytes were spilled, and
-// d = 1536 took 754 us per token (32 layers, 8 of 40 experts of 512 rows) instead of 658.
+// d = 1536 took 754 us per token (32 layers, 8 of 40 experts of 512 rows) instead of 658.  With it none, or up to 20 bytes (bf16 d = 2048,
+// e4m3 from d = 1536 on, e2m1 d = 1536).
 //
 // Ring: NT tiles of kRows rows, used in order by stand-in pieces and by row tiles alike; `full` completes with a tile's bytes,
 // `empty` when the eight workers have read it (the planner stands in for them where it consumed a stand-in piece).
@@ -684,8 +685,9 @@ __global__ void __launch_bounds__(kTileThreads, 1) decode_tiles_kernel(const Dec
       return halted;
     };
     // Router rows (a worker's, one of W_p and one of W_r per layer): up to d = 1024 in registers from the start of the layer,
-    // wider ones prefetched into L2 there and read when the dot product is taken; the gate's row of d = 1536 comes into
-    // registers right before the wait for the attention window.  (kernels_decode.cu has the measurements.)
+    // wider ones prefetched into L2 there and read when the dot product is taken (two rows of d = 1536 held from the start of the
+    // layer cost the rows more than the loads cost the logits, 19.3 against 17.2 us per layer in the row-per-warp kernel; two of
+    // d = 2048 spilled); the gate's row of d = 1536 comes into registers right before the wait for the attention window (+ 3 %).
     constexpr int NVRP = NV <= 8 ? NV : 1;   // prefetch-router row
     constexpr int NVRR = NV <= 12 ? NV : 1;  // gate row
     constexpr bool WR_LATE = NV > 8 && NV <= 12;
