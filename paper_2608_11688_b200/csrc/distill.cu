@@ -61,7 +61,7 @@ struct DistillParams {
   double* gb;        // [forward CTAs][8 NE]: sums of G over a CTA's tokens
   double* partial;   // [column tiles][segments][8 NE][kCols]
   int T, N, d, ldw;
-  int tok_warps;     // forward: tokens per CTA / 8: 1, 2, 4, 7 or 8
+  int tok_warps;     // forward: tokens per CTA / 8, 1 to 8
   int n_fwd, n_tiles, n_seg, seg_len;
   int* status;       // 1: a wait of a ring ran out
   int starve;        // test hook: the first forward CTA's ring expects an arrival that never comes
@@ -489,8 +489,8 @@ extern "C" int apex_distill_router(const float* H_dev, const float* Qr_dev, int 
   p.tok_warps = want < 8 ? want : 8;
   p.n_fwd = (T + 8 * p.tok_warps - 1) / (8 * p.tok_warps);
   // Backward: column tiles times segments within one round of the SMs.  A segment is whole pipeline stages of tokens (a token
-  // more than a stage costs a stage), and there are at most kMaxSeg of them (the step kernel adds them up): the SMs of d = 256.
-  // With twelve at most, T = 8192, N = 40, d = 256 took 45.2 us per iteration on 48 CTAs, 38.8 on 148.
+  // more than a stage costs a stage), and there are at most kMaxSeg of them (the step kernel adds them up): the SMs per column tile of d = 256.
+  // With twelve at most, T = 8192, N = 40, d = 256 ran on 48 CTAs, now on 128 (32 segments of four stages).
   p.n_tiles = (d + kCols - 1) / kCols;
   p.n_seg = n_sm / p.n_tiles;
   const int stages = (T + kTokTile - 1) / kTokTile;
