@@ -88,6 +88,8 @@ struct RowTiles;
 template <int D>
 struct RowTiles<D, kFmtBf16> {
   static constexpr int KW = D / 128;  // 16-column steps
+  template <int ROWS>
+  struct Scales {};  // (see the e2m1 rows)
   static_assert(D % 256 == 0, "two steps of 16 columns per warp at least");
   uint32_t hb[KW][2];  // h', B operand of the gate and up products
   float y[KW][4];      // accumulators of the down projection
@@ -407,14 +409,18 @@ struct RowTiles<D, kFmtE4m3> : QuantTiles<D, kFmtE4m3> {
   using Base::KW;
   using Base::hb;
   using Base::y;
-  // shares of the dot products of rows' codes; see the bf16 rows.  tile: the eight rows' shared-memory address; h: h' in global memory
-  __device__ __forceinline__ void gate_up(const uint8_t* rows, uint32_t tile, uint32_t stride, int warp, int lane, const float* __restrict__ h, int, float& g, float& u) const {
-    if (Base::h_wide) {
-      const float2 v = gate_up_rows_fp32<kFmtE4m3>(rows + (lane >> 2) * stride + warp * (D / 8), D, nullptr, 0u, h + warp * (D / 8), D / 256);
-      g = v.x;
-      u = v.y;
-      return;
-    }
+  template <int ROWS>
+  struct Scales {};  // (see the e2m1 rows)
+  template <int ROWS>
+  __device__ __forceinline__ static Scales<ROWS> scales_of(uint32_t, uint32_t, int, int, int) { return Scales<ROWS>{}; }
+  template <int ROWS>
+  __device__ __forceinline__ bool needs_fp32(uint32_t, uint32_t, int, int, int) const { return Base::h_wide; }
+  // the same of eight rows in fp32; rows: their generic address, h: h' in global memory
+  __device__ __forceinline__ float2 gate_up_fp32(const uint8_t* rows, uint32_t stride, int warp, int lane, const float* __restrict__ h) const {
+    return gate_up_rows_fp32<kFmtE4m3>(rows + (lane >> 2) * stride + warp * (D / 8), D, nullptr, 0u, h + warp * (D / 8), D / 256);
+  }
+  // shares of the dot products of rows' codes; see the bf16 rows.  tile: the eight rows' shared-memory address
+  __device__ __forceinline__ void gate_up(uint32_t tile, uint32_t stride, int warp, int lane, float& g, float& u) const {
     // matrices: gate rows, up rows, columns 0 .. 15 of the step, then both of the next step
     const uint32_t at = tile + (lane & 7) * stride + ((lane >> 3) & 1) * D + (lane >> 4) * 16 + warp * (D / 8);
     float sum[4] = {};
@@ -445,10 +451,10 @@ struct RowTiles<D, kFmtE4m3> : QuantTiles<D, kFmtE4m3> {
   // y += downT^T a of ROWS rows, of which `here` exist
   template <int ROWS>
   __device__ __forceinline__ void down(const uint8_t* rows, uint32_t tile, uint32_t stride, int warp, int lane, const uint32_t (&b)[ROWS / 8], float unit, int here, float a_row,
-                                       int reach) {
+                                       int reach, const Scales<ROWS>&) {
     static_assert(ROWS % 16 == 0, "two 8-row blocks to an MMA");
     if (reach < 0) {
-#pragma unroll
+#pragma unroll 1
       for (int r = 0; r < ROWS; r += 16) {
 #pragma unroll
         for (int s = 0; s < KW; s += 2) {
@@ -527,25 +533,39 @@ struct RowTiles<D, kFmtMxfp4> : QuantTiles<D, kFmtMxfp4> {
   }
   __device__ __forceinline__ static uint32_t byte_of(const uint32_t (&sc)[SW], int i) { return __byte_perm(sc[i / 4], 0u, 0x4440 | (i & 3)); }
 
-  __device__ __forceinline__ void gate_up(const uint8_t* rows, uint32_t tile, uint32_t stride, int warp, int lane, const float* __restrict__ h, int here, float& g, float& u) const {
+  // Is anything in the tile's gate or up rows beyond the planes?  Scales between 2^-63 and 2^64 (and zero) leave the planes' sums inside fp32's
+  // exponents.  A lane looks at the scales of a row (of 16: at the gate's or the up row's).
+  template <int ROWS>
+  __device__ __forceinline__ bool needs_fp32(uint32_t tile, uint32_t stride, int warp, int lane, int here) const {
+    const int row = lane & (ROWS - 1);
+    const uint32_t at = tile + row * stride + 3 * (D / 2) + warp * KB;
+    uint32_t bits = 0u, sc[SW];
+    auto look = [&]() {
+#pragma unroll
+      for (int i = 0; i < SW; ++i) {
+        const uint32_t w = sc[i], some = ((w & 0x3f3f3f3fu) + 0x3f3f3f3fu) << 1;  // bit 7 of a byte: its lower six bits are not zero; of w << 1: its bit 6
+        bits |= (some & ~(w | w << 1)) | (w & w << 1);
+      }
+    };
+    load_scales(at + (ROWS == 32 ? 0 : (lane >> 4) * (D / 32)), sc);
+    look();
+    if (ROWS == 32) {
+      load_scales(at + D / 32, sc);
+      look();
+    }
+    return __any_sync(0xffffffffu, Base::h_wide || (row < here && (bits & 0x80808080u) != 0u));
+  }
+  __device__ __forceinline__ float2 gate_up_fp32(const uint8_t* rows, uint32_t stride, int warp, int lane, const float* __restrict__ h) const {
+    const uint8_t* row = rows + (lane >> 2) * stride;
+    return gate_up_rows_fp32<kFmtMxfp4>(row + warp * (D / 16), D / 2, row + 3 * (D / 2) + warp * KB, D / 32, h + warp * (D / 8), KB);
+  }
+  __device__ __forceinline__ void gate_up(uint32_t tile, uint32_t stride, int warp, int lane, float& g, float& u) const {
     // matrices: gate rows, up rows of a block, then both of the next block
     const uint32_t at = tile + (lane & 7) * stride + ((lane >> 3) & 1) * (D / 2) + (lane >> 4) * 16 + warp * (D / 16);
     const uint32_t scales = tile + (lane >> 2) * stride + 3 * (D / 2) + warp * KB;
     uint32_t sg[SW], su[SW];
     load_scales(scales, sg);
     load_scales(scales + D / 32, su);
-    // Scales between 2^-63 and 2^64 (and zero) leave the planes' sums inside fp32's exponents; each lane of a row
-    // (of the `here` that exist) looks at one word of them
-    const uint32_t w = (lane & 1) ? ((lane & 2) ? su[SW - 1] : su[0]) : ((lane & 2) ? sg[SW - 1] : sg[0]);
-    const uint32_t some = ((w & 0x3f3f3f3fu) + 0x3f3f3f3fu) << 1;  // bit 7 of a byte: its lower six bits are not zero; of w << 1: its bit 6
-    const bool far = (lane >> 2) < here && (((some & ~(w | w << 1)) | (w & w << 1)) & 0x80808080u) != 0u;
-    if (__any_sync(0xffffffffu, Base::h_wide || far)) {
-      const uint8_t* row = rows + (lane >> 2) * stride;
-      const float2 v = gate_up_rows_fp32<kFmtMxfp4>(row + warp * (D / 16), D / 2, row + 3 * (D / 2) + warp * KB, D / 32, h + warp * (D / 8), KB);
-      g = v.x;
-      u = v.y;
-      return;
-    }
     float sum[4] = {};
 #pragma unroll
     for (int b = 0; b < KB; b += 2) {
@@ -572,21 +592,27 @@ struct RowTiles<D, kFmtMxfp4> : QuantTiles<D, kFmtMxfp4> {
   }
   __device__ __forceinline__ static float gated(const uint8_t*, float gate, float g, float u) { return gate * g * __frcp_rn(1.f + expf(-g)) * u; }
   // y += downT^T a.  A block's scale differs from row to row, along the sum, so it goes to the B operand: the row's planes times
-  // 2^(scale - largest scale of the block in these rows); the largest scale is applied to the result.  A plane's last bit is 2^4 at the
-  // top of the reach and 2^-24 is fp16's, so nothing is cut where the smallest a lies with the smallest scale 28 binades
-  // below the largest of both.  Rows of one MMA whose scales (or a) span more, in any block, are taken in fp32: a row that sinks below the
+  // 2^(scale - largest scale of the block in the 16 rows of an MMA); the largest scale is applied to the result.  A plane's last bit is
+  // 2^4 at the top of the reach and 2^-24 is fp16's, so nothing is cut where the smallest a lies with the smallest scale 28 binades
+  // below the largest of both.  A tile whose scales (or a) span more, in any block, is taken in fp32: a row that sinks below the
   // largest scale times the largest a, which no row need have together, may be all there is of a column.
   template <int ROWS>
-  __device__ __forceinline__ void down(const uint8_t* rows, uint32_t tile, uint32_t stride, int warp, int lane, const uint32_t (&b)[ROWS / 8], float unit, int here, float a,
-                                       int reach) {
+  struct Scales {
+    uint32_t e[ROWS / 8], top[ROWS / 16];  // lane 4 b + t, block b: the factors of rows 2t, 2t+1 of each 8-row block; the largest scales
+    int span;                              // binades between the scales of a block, at most (any lane's)
+  };
+  // What does not depend on a: looked at in front of the exchange's barrier.  With the tests behind it, a branch for every eight rows, d = 512
+  // took 209 us (8 layers of 4 experts of 6000 rows), d = 2048 247 (2500 rows); 182 and 236 so, 175 and 221 without tests.
+  template <int ROWS>
+  __device__ __forceinline__ static Scales<ROWS> scales_of(uint32_t tile, uint32_t stride, int warp, int lane, int here) {
     static_assert(ROWS % 16 == 0, "two 8-row blocks to an MMA");
-    const uint32_t at = tile + ((lane & 7) + ((lane >> 3) & 1) * 8) * stride + D + warp * (D / 16) + (lane >> 4) * 16;
-    // lane 4 b + t works out the scales of block b in the rows 2t, 2t+1 of each 8-row block, and passes them on (every lane for
-    // itself and all blocks: 60 instructions per block instead of 5)
+    Scales<ROWS> f;
+    // a lane works out its block and passes the factors on (every lane for itself and all blocks: 60 instructions per block instead of 5)
     const uint32_t scales = tile + 2 * (lane & 3) * stride + 3 * (D / 2) + 2 * (D / 32) + warp * KB + min(lane >> 2, KB - 1);
+    uint32_t span = 0u;
 #pragma unroll
     for (int r = 0; r < ROWS / 8; r += 2) {
-      uint32_t sc[4], top = 0u, e[2];
+      uint32_t sc[4], top = 0u;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int row = (r + (i >> 1)) * 8 + (i & 1);
@@ -596,30 +622,42 @@ struct RowTiles<D, kFmtMxfp4> : QuantTiles<D, kFmtMxfp4> {
       }
       top = max(top, __shfl_xor_sync(0xffffffffu, top, 1));
       top = max(top, __shfl_xor_sync(0xffffffffu, top, 2));
-      bool wide = false;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) wide = wide || (sc[i] != 0u && ((int)(top - sc[i]) > reach - 8 || sc[i] - 64u > 127u));
-      if (__any_sync(0xffffffffu, wide)) {
-        const uint8_t* codes = rows + D + warp * (D / 16) + (lane >> 2) * 2;
-#pragma unroll
-        for (int blk = 0; blk < KB; ++blk) {
-          const float4 v = down_rows_fp32<kFmtMxfp4>(codes + blk * 16, rows + 3 * (D / 2) + 2 * (D / 32) + warp * KB + blk, stride, a, r * 8, here);
-          y[2 * blk][0] += v.x;
-          y[2 * blk][2] += v.y;
-          y[2 * blk + 1][0] += v.z;
-          y[2 * blk + 1][2] += v.w;
-        }
-        continue;
-      }
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         // 2^-k in fp16, a subnormal from 15 on, zero from 25 on; a scale of zero is zero
         const uint32_t k = top - sc[i];
         const uint32_t v = sc[i] == 0u ? 0u : k < 15u ? (15u - k) << 10 : 0x400u >> min(k - 14u, 31u);
-        if (i & 1) e[i >> 1] |= v << 16;
-        else e[i >> 1] = v;
+        if (i & 1) f.e[r + (i >> 1)] |= v << 16;
+        else f.e[r + (i >> 1)] = v;
+        span = max(span, sc[i] == 0u ? 0u : sc[i] - 64u > 127u ? 255u : k);
       }
-      const float back = __uint_as_float(top << 23) * unit;
+      f.top[r / 2] = top;
+    }
+    f.span = (int)__reduce_max_sync(0xffffffffu, span);
+    return f;
+  }
+  template <int ROWS>
+  __device__ __forceinline__ void down(const uint8_t* rows, uint32_t tile, uint32_t stride, int warp, int lane, const uint32_t (&b)[ROWS / 8], float unit, int here, float a_row,
+                                       int reach, const Scales<ROWS>& sc) {
+    if (sc.span > reach - 8) {
+      const uint8_t* codes = rows + D + warp * (D / 16) + (lane >> 2) * 2;
+#pragma unroll 1
+      for (int r = 0; r < ROWS; r += 16) {
+#pragma unroll
+        for (int blk = 0; blk < KB; ++blk) {
+          const float4 v = down_rows_fp32<kFmtMxfp4>(codes + blk * 16, rows + 3 * (D / 2) + 2 * (D / 32) + warp * KB + blk, stride, a_row, r, here);
+          y[2 * blk][0] += v.x;
+          y[2 * blk][2] += v.y;
+          y[2 * blk + 1][0] += v.z;
+          y[2 * blk + 1][2] += v.w;
+        }
+      }
+      return;
+    }
+    const uint32_t at = tile + ((lane & 7) + ((lane >> 3) & 1) * 8) * stride + D + warp * (D / 16) + (lane >> 4) * 16;
+#pragma unroll
+    for (int r = 0; r < ROWS / 8; r += 2) {
+      const float back = __uint_as_float(sc.top[r / 2] << 23) * unit;
 #pragma unroll
       for (int b0 = 0; b0 < KB; b0 += 2) {  // blocks
         uint32_t v[4];
@@ -630,7 +668,7 @@ struct RowTiles<D, kFmtMxfp4> : QuantTiles<D, kFmtMxfp4> {
           uint32_t bs[2], a[2][4];
 #pragma unroll
           for (int i = 0; i < 2; ++i) {
-            const uint32_t es = __shfl_sync(0xffffffffu, e[i], blk * 4 + (lane & 3));
+            const uint32_t es = __shfl_sync(0xffffffffu, sc.e[r + i], blk * 4 + (lane & 3));
             const __half2 t = __hmul2(*reinterpret_cast<const __half2*>(&b[r + i]), *reinterpret_cast<const __half2*>(&es));
             bs[i] = *reinterpret_cast<const uint32_t*>(&t);
             // a register: columns 4g .. 4g+3 of row 2t, then of row 2t+1, a nibble each: brought together by column

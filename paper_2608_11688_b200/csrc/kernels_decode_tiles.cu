@@ -833,13 +833,30 @@ __global__ void __launch_bounds__(kTileThreads, 1) decode_tiles_kernel(const Dec
             float* part = s_part[q & 1];
             const bool landed = warp_wait(&s_full[s], par);
             if (q == 0 && pass == 0) DTL(7);
+            float2* share = reinterpret_cast<float2*>(part + (lane >> 2) * kPartStride + 2 * warp);
+            constexpr int kShare8 = 8 * kPartStride / 2;  // (eight rows on)
+            [[maybe_unused]] typename RowTiles<d, FMT>::template Scales<kRows> scales;
             if (landed) {
+              bool fp32 = false;  // the planes do not hold all of h' or of the gate and up rows
+              if constexpr (FMT != kFmtBf16) {
+                scales = rt.template scales_of<kRows>(tile, stride, warp, lane, here);
+                fp32 = rt.template needs_fp32<kRows>(tile, stride, warp, lane, here);
+              }
 #pragma unroll
               for (int r = 0; r < R; ++r) {
                 float g, u;
                 if constexpr (FMT == kFmtBf16) rt.gate_up(tile + (lane & 7) * stride + r * 8 * stride, warp, lane, g, u);
-                else rt.gate_up(smem + s * tile_bytes + r * 8 * stride, tile + r * 8 * stride, stride, warp, lane, hpl, here - r * 8, g, u);
-                if ((lane & 3) == 0) *reinterpret_cast<float2*>(part + (r * 8 + (lane >> 2)) * kPartStride + 2 * warp) = make_float2(g, u);
+                else rt.gate_up(tile + r * 8 * stride, stride, warp, lane, g, u);
+                if ((lane & 3) == 0) share[r * kShare8] = make_float2(g, u);
+              }
+              if constexpr (FMT != kFmtBf16) {
+                if (fp32) {
+#pragma unroll 1
+                  for (int r = 0; r < R; ++r) {
+                    const float2 gu = rt.gate_up_fp32(smem + s * tile_bytes + r * 8 * stride, stride, warp, lane, hpl);
+                    if ((lane & 3) == 0) share[r * kShare8] = gu;
+                  }
+                }
               }
             }
             // (behind the last tile's barrier everybody knows whether the rows are to be repeated)
@@ -864,7 +881,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) decode_tiles_kernel(const Dec
               uint32_t b[R];
               int reach;
               const float unit = rt.template take_a<kRows>(a, s_planes[warp], lane, b, reach);
-              rt.template down<kRows>(smem + s * tile_bytes, tile, stride, warp, lane, b, unit, here, a, reach);
+              rt.template down<kRows>(smem + s * tile_bytes, tile, stride, warp, lane, b, unit, here, a, reach, scales);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&s_empty[s]);
